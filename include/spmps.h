@@ -73,10 +73,10 @@ typedef struct {
     int dav_max_sub;    /* Davidson subspace size before restart (default 20, max 32)         */
     int dav_max_iter;   /* Davidson iteration cap per two-site step (default 200)             */
     int device;         /* CUDA device ordinal (default 0)                                    */
-    int jacobi_smem_max; /* decimation blocks handled by one CTA (dimension <= 64 or > 256) up to
-                            this size are diagonalised in shared memory, larger ones in global
-                            memory (default and maximum 112; 0 = default); blocks of dimension
-                            65..256 always run on an 8-CTA thread-block cluster */
+    int jacobi_smem_max; /* largest decimation block whose FP32 start of the one-sided Jacobi may run in
+                            one CTA's shared memory; larger ones start in global memory on an 8-CTA
+                            cluster (0 = default; the default and maximum 112 set no limit of their
+                            own: every block that fits the shared memory takes it) */
     int precision;      /* bulk H_eff x block products: 0 = FP64 (default), 1 = TF32, 2 = 3xTF32
                            (tensor cores, FP32 accumulation).  N_eff x, environments, Davidson and
                            decimation stay FP64; with 1 or 2 each Davidson solve starts with

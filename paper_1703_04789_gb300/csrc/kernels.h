@@ -93,25 +93,13 @@ cudaError_t launch_restart_coef(const double* c_new, const double* c_old, int m,
 
 // ---- decimation -------------------------------------------------------------------------------
 
-// Symmetric eigen-decomposition of many small matrices by cyclic Jacobi, one CTA each.
-// mats: concatenated row-major n_i x n_i matrices (overwritten by the eigenvector matrices,
-// columns = vectors, sorted by descending eigenvalue), evals: concatenated eigenvalues.
-// vscratch: same size as mats (used for matrices above the shared-memory limit of 112).
-// Matrices up to min(smem_limit, 112) run in shared memory.  With cluster != 0, matrices of
-// dimension 65..256 run on a thread-block cluster of 8 CTAs each (rows distributed over the
-// CTAs' shared memory), the others on one CTA.
-cudaError_t launch_jacobi_batched(double* mats, double* vscratch, double* evals, const int64_t* mat_off,
-                                  const int64_t* val_off, const int* dims, int n_mats, int max_dim, int smem_limit,
-                                  int cluster, int* status, cudaStream_t st);
-
-// Ordered truncation of singular values sqrt(max(evals, 0)) (one CTA): values within
-// tie_rtol * max of their sorted predecessor form a cluster ordered by (n, 2m, index);
-// values below drop_abs are dropped; the first D kept.  keep_count[label] receives the
-// number kept per label (labels in bond order), keep_total[0] the total and discarded[0] the
-// discarded weight.
-cudaError_t launch_truncate(const double* evals, const int64_t* val_off, const int* dims, const int* label_n,
-                            const int* label_tm, int n_labels, int total, int D, double tie_rtol, double drop_abs,
-                            int* keep_count, int* keep_total, double* discarded, int* scratch_idx,
+// Ordered truncation of the singular values sqrt(max(evals, 0)): evals holds the values of all labels
+// in label order (label l from val_off[l]), labels ascending in (n, 2m).  Values within tie_rtol * max of
+// their sorted predecessor form a cluster ordered by (n, 2m, index); values below drop_abs are dropped;
+// the first D kept.  keep_count[label] receives the number kept per label, keep_total[0] the total and
+// discarded[0] the discarded weight.  Scratch: 3 total ints and 2 total doubles.
+cudaError_t launch_truncate(const double* evals, const int64_t* val_off, int n_labels, int total, int D, double tie_rtol,
+                            double drop_abs, int* keep_count, int* keep_total, double* discarded, int* scratch_idx,
                             double* scratch_val, cudaStream_t st);
 
 // Gather/scatter of sub-blocks: dst[(r)*ld_dst + c] = src[(r)*ld_src + c] * scale for a list.

@@ -1,0 +1,520 @@
+// Singular vectors of the decimation blocks: one-sided Jacobi, started in FP32 and finished in FP64.
+//
+// The FP64 pipe of this part executes 2 FMA per clock and SM (FP32: 128), so an FP64 Jacobi is bound
+// by that pipe of the few SMs a block occupies.  The bulk of the rotations therefore runs in FP32: for
+// the rows of Z (the block, or its transpose),
+//   1. k_osj<float>: one-sided Jacobi on an FP32 copy [Z | I] finds J with nearly orthogonal rows of J Z;
+//   2. two Newton-Schulz steps J <- (3/2 - 1/2 J J^T) J in FP64 (k_block_gemm, all SMs) make J orthonormal
+//      to FP64, and Z' = J Z is formed in FP64 from the unrounded block;
+//   3. k_osj<double>: one-sided Jacobi on Z' to FP64 convergence (two sweeps as a rule: the FP32 start
+//      leaves relative couplings of 1e-6, and the convergence is quadratic).
+// The singular values are the row norms of the result and come from Z itself, not from its Gram matrix,
+// so small ones keep the FP64 noise floor of Z (1e-16, not 1e-8).
+#include <cooperative_groups.h>
+
+#include "svd.h"
+
+namespace spmps {
+
+namespace {
+
+namespace cgx = cooperative_groups;
+
+constexpr int kOsjC = 8;             // CTAs per block of the global-memory form
+constexpr int kMaxSweeps = 40;
+constexpr double kNullRel = 1e-9;    // rows below this fraction of the block's norm are not separated further
+
+template <class T>
+__device__ __forceinline__ T ldc(const T* p) { return __ldcg(p); }
+
+template <class T>
+__device__ __forceinline__ T wsum(T v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// c = 1 / sqrt(1 + t^2): the hardware estimate polished to the precision of T, so that the rotation is
+// orthonormal in T (the angle itself may be rounded: the next sweep removes what it leaves).
+__device__ __forceinline__ float rotation_cos(float t) { return rsqrtf(fmaf(t, t, 1.0f)); }
+__device__ __forceinline__ double rotation_cos(double t) {
+    const double w = fma(t, t, 1.0);
+    double y = static_cast<double>(rsqrtf(static_cast<float>(w)));
+    y = y * fma(-0.5 * w, y * y, 1.5);
+    y = y * fma(-0.5 * w, y * y, 1.5);
+    return y;
+}
+
+// One-sided Jacobi on the rows of Z (R x W, row stride W): the first C columns are the block, the rest a
+// companion that receives the same rotations.  Round-robin pairs, one warp per pair and round.
+// SMEM: one CTA per block with the rows in shared memory (a round costs a __syncthreads); otherwise a
+// cluster of kOsjC CTAs with the rows in global memory (L2), a cluster barrier per round: in FP64 the
+// FP64 pipes of 8 SMs share the work.  NCH > 0 keeps the two rows of a pair in registers (W <= 32 NCH)
+// between the product and the update, NCH = 0 reads them twice.
+// Measured (GB300, middle decimation of the L = 24, D = 256 chain, blocks up to 136): see launch_svd.
+template <class T, bool SMEM, int NCH>
+__device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, int* conv, int rank, int ctas) {
+    const int lane = threadIdx.x & 31;
+    const int warp = (threadIdx.x >> 5) + rank * (blockDim.x >> 5);
+    const int warps = (blockDim.x >> 5) * ctas;
+    const int np = (R + 1) & ~1, half = np / 2;
+    constexpr bool kF64 = sizeof(T) == 8;
+    const T tol = kF64 ? T(1e-15) : T(3e-7);
+    const T done = kF64 ? T(1e-8) : T(1e-3);  // couplings below this square to the noise of T in one sweep
+    const T floor_abs = norm2_all * (kF64 ? T(1e-18) : T(1e-12));
+    const T null2 = norm2_all * (kF64 ? T(kNullRel * kNullRel) : T(1e-13));
+    const T inv_all = norm2_all > T(0) ? T(1) / norm2_all : T(0);  // keeps the angle's FP32 operands in range
+    auto barrier = [&]() {
+        if constexpr (SMEM)
+            __syncthreads();
+        else
+            cgx::this_cluster().sync();
+    };
+    auto ld = [&](const T* p) -> T {
+        if constexpr (SMEM)
+            return *p;
+        else
+            return ldc(p);
+    };
+    auto stg = [&](T* p, T v) {
+        if constexpr (SMEM)
+            *p = v;
+        else
+            __stcg(p, v);
+    };
+    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+        for (int r = warp; r < R; r += warps) {
+            T s = T(0);
+            for (int c = lane; c < C; c += 32) {
+                const T v = ld(Z + static_cast<int64_t>(r) * W + c);
+                s += v * v;
+            }
+            s = wsum(s);
+            if (lane == 0) stg(nrm2 + r, s);
+        }
+        barrier();
+        bool rough = false;
+        for (int round = 0; round < np - 1; ++round) {
+            for (int i = warp; i < half; i += warps) {
+                int p = i == 0 ? 0 : 1 + (i - 1 + round) % (np - 1);
+                int q = 1 + (np - 2 - i + round) % (np - 1);
+                if (p > q) {
+                    const int t = p;
+                    p = q;
+                    q = t;
+                }
+                if (q >= R) continue;
+                T* zp = Z + static_cast<int64_t>(p) * W;
+                T* zq = Z + static_cast<int64_t>(q) * W;
+                const T a = ld(nrm2 + p), b = ld(nrm2 + q);
+                if (!(a > null2) && !(b > null2)) continue;
+                T x[NCH > 0 ? NCH : 1], y[NCH > 0 ? NCH : 1];
+                T g = T(0);
+                if constexpr (NCH > 0) {
+#pragma unroll
+                    for (int k = 0; k < NCH; ++k) {
+                        const int c = lane + 32 * k;
+                        x[k] = c < W ? ld(zp + c) : T(0);
+                        y[k] = c < W ? ld(zq + c) : T(0);
+                    }
+#pragma unroll
+                    for (int k = 0; k < NCH; ++k)
+                        if (32 * k < C) g += lane + 32 * k < C ? x[k] * y[k] : T(0);
+                } else {
+                    for (int c = lane; c < C; c += 32) g += ld(zp + c) * ld(zq + c);
+                }
+                g = wsum(g);
+                // |g| <= tol sqrt(a b), compared by the squares
+                const T g2 = g * g, ab = a * b;
+                if (!(g2 > tol * tol * ab) || !(fabs(g) > floor_abs)) continue;
+                if (g2 > done * done * ab && a > null2 && b > null2) rough = true;
+                const float zeta = static_cast<float>((b - a) * inv_all) / (2.0f * static_cast<float>(g * inv_all));
+                const float tf = copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
+                const T t = static_cast<T>(tf);
+                const T cs = rotation_cos(t), sn = cs * t;
+                if constexpr (NCH > 0) {
+#pragma unroll
+                    for (int k = 0; k < NCH; ++k) {
+                        const int c = lane + 32 * k;
+                        if (c < W) {
+                            stg(zp + c, cs * x[k] - sn * y[k]);
+                            stg(zq + c, sn * x[k] + cs * y[k]);
+                        }
+                    }
+                } else {
+                    for (int c = lane; c < W; c += 32) {
+                        const T u = ld(zp + c), v = ld(zq + c);
+                        stg(zp + c, cs * u - sn * v);
+                        stg(zq + c, sn * u + cs * v);
+                    }
+                }
+                if (lane == 0) {
+                    // |p'|^2 = c^2 a - 2 c s g + s^2 b
+                    const T na = cs * cs * a - T(2) * cs * sn * g + sn * sn * b;
+                    const T nb = sn * sn * a + T(2) * cs * sn * g + cs * cs * b;
+                    stg(nrm2 + p, na > T(0) ? na : T(0));
+                    stg(nrm2 + q, nb > T(0) ? nb : T(0));
+                }
+            }
+            barrier();
+        }
+        if (rough && lane == 0) atomicOr(conv + sweep, 1);
+        if constexpr (!SMEM) __threadfence();
+        barrier();
+        if (!*reinterpret_cast<volatile int*>(conv + sweep)) break;  // uniform: read after the barrier
+    }
+}
+
+// FP32 start: [Z | I] of a block scaled to norm 1; J (R x R) leaves in FP64.
+template <bool SMEM>
+__device__ void osj32_block(const SvdBlock& B, const double* __restrict__ zraw, float* work, float* nrm2, double* J,
+                            int* conv, int rank, int ctas) {
+    __shared__ double red[32];
+    __shared__ double tot;
+    const int R = B.R, C = B.C, W = C + R;
+    const double* Zr = zraw + B.z_off;
+    double s = 0.0;
+    for (int e = threadIdx.x; e < R * C; e += blockDim.x) s = fma(Zr[e], Zr[e], s);
+    s = wsum(s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) t += red[i];
+        tot = t;
+    }
+    __syncthreads();
+    const double scale = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
+    for (int e = rank * blockDim.x + threadIdx.x; e < R * W; e += blockDim.x * ctas) {
+        const int r = e / W, c = e - r * W;
+        const float v = c < C ? static_cast<float>(Zr[static_cast<int64_t>(r) * C + c] * scale) : (c - C == r ? 1.0f : 0.0f);
+        if constexpr (SMEM)
+            work[e] = v;
+        else
+            __stcg(work + e, v);
+    }
+    if constexpr (SMEM)
+        __syncthreads();
+    else
+        cgx::this_cluster().sync();
+    if (W <= 256 && !SMEM)
+        osj_sweeps<float, SMEM, SMEM ? 0 : 8>(work, nrm2, R, C, W, 1.0f, conv, rank, ctas);
+    else
+        osj_sweeps<float, SMEM, 0>(work, nrm2, R, C, W, 1.0f, conv, rank, ctas);
+    for (int e = rank * blockDim.x + threadIdx.x; e < R * R; e += blockDim.x * ctas) {
+        const int r = e / R, c = e - r * R;
+        const float* p = work + static_cast<int64_t>(r) * W + C + c;
+        float v;
+        if constexpr (SMEM)
+            v = *p;
+        else
+            v = __ldcg(p);
+        J[B.j_off + e] = static_cast<double>(v);
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_osj32_smem(const SvdBlock* __restrict__ blocks, const double* __restrict__ zraw,
+                                                    double* __restrict__ J, int* __restrict__ conv, int smem_floats) {
+    extern __shared__ float sm32[];
+    const SvdBlock B = blocks[blockIdx.x];
+    if (B.R <= 0 || B.C <= 0 || B.smem == 0) return;
+    const int need = B.R * (B.C + B.R) + B.R;
+    if (need > smem_floats) return;  // never: the host marks only blocks that fit
+    osj32_block<true>(B, zraw, sm32, sm32 + B.R * (B.C + B.R), J, conv + blockIdx.x * 2 * kSvdConv, 0, 1);
+}
+
+__global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
+    k_osj32_global(const SvdBlock* __restrict__ blocks, const double* __restrict__ zraw, float* __restrict__ work,
+                   float* __restrict__ nrm, double* __restrict__ J, int* __restrict__ conv) {
+    const int b = blockIdx.x / kOsjC;
+    const SvdBlock B = blocks[b];
+    if (B.R <= 0 || B.C <= 0 || B.smem != 0) return;  // uniform over the cluster
+    osj32_block<false>(B, zraw, work + B.w_off, nrm + B.n_off, J, conv + b * 2 * kSvdConv,
+                       static_cast<int>(cgx::this_cluster().block_rank()), kOsjC);
+}
+
+// FP64 finish on Z' (R x W, W = C, or C + R with the companion J): singular values squared, sorted
+// descending, into evals (dim of them, zeros beyond the rank), and the wanted vectors as the columns of
+// mats (dim x dim): the companion's rows, or the normalised rows of Z'.
+__global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
+    k_osj64(const SvdBlock* __restrict__ blocks, double* __restrict__ z, double* __restrict__ nrm, int* __restrict__ conv,
+            double* __restrict__ mats, double* __restrict__ evals) {
+    __shared__ double red[32];
+    __shared__ double tot;
+    const int b = blockIdx.x / kOsjC;
+    const SvdBlock B = blocks[b];
+    if (B.dim <= 0) return;  // uniform over the cluster
+    const int rank = static_cast<int>(cgx::this_cluster().block_rank());
+    const int R = B.R, C = B.C, W = B.companion ? C + R : C;
+    double* Z = z + B.f_off;
+    double* nr = nrm + B.n_off;
+    double s = 0.0;
+    for (int e = threadIdx.x; e < R * C; e += blockDim.x) {
+        const int r = e / C, c = e - r * C;
+        const double v = __ldcg(Z + static_cast<int64_t>(r) * W + c);
+        s = fma(v, v, s);
+    }
+    s = wsum(s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) t += red[i];
+        tot = t;
+    }
+    cgx::this_cluster().sync();  // every CTA has read Z before any rotates it
+    int* cv = conv + (b * 2 + 1) * kSvdConv;
+    if (W <= 160)
+        osj_sweeps<double, false, 5>(Z, nr, R, C, W, tot, cv, rank, kOsjC);
+    else if (W <= 320)
+        osj_sweeps<double, false, 10>(Z, nr, R, C, W, tot, cv, rank, kOsjC);
+    else
+        osj_sweeps<double, false, 0>(Z, nr, R, C, W, tot, cv, rank, kOsjC);
+    // exact norms of the final rows, then the vectors by descending norm (ties by row)
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) + rank * (blockDim.x >> 5);
+    const int warps = (blockDim.x >> 5) * kOsjC;
+    for (int r = warp; r < R; r += warps) {
+        double t = 0.0;
+        for (int c = lane; c < C; c += 32) {
+            const double v = __ldcg(Z + static_cast<int64_t>(r) * W + c);
+            t = fma(v, v, t);
+        }
+        t = wsum(t);
+        if (lane == 0) __stcg(nr + r, t);
+    }
+    cgx::this_cluster().sync();
+    double* M = mats + B.m_off;
+    double* ev = evals + B.e_off;
+    const int n = B.dim;
+    for (int r = warp; r < R; r += warps) {
+        const double vr = __ldcg(nr + r);
+        int rk = 0;
+        for (int j = lane; j < R; j += 32) {
+            const double vj = __ldcg(nr + j);
+            rk += (vj > vr || (vj == vr && j < r)) ? 1 : 0;
+        }
+        rk = wsum(rk);
+        if (rk >= n) continue;  // rows beyond the rank of the block (more rows than columns): noise
+        if (lane == 0) ev[rk] = vr;
+        const double inv = B.companion ? 1.0 : (vr > 0.0 ? 1.0 / sqrt(vr) : 0.0);
+        const double* src = Z + static_cast<int64_t>(r) * W + (B.companion ? C : 0);
+        for (int c = lane; c < n; c += 32) M[static_cast<int64_t>(c) * n + rk] = __ldcg(src + c) * inv;
+    }
+    for (int rk = R + warp; rk < n; rk += warps) {  // fewer rows than the dimension: the rest is null
+        if (lane == 0) ev[rk] = 0.0;
+        for (int c = lane; c < n; c += 32) M[static_cast<int64_t>(c) * n + rk] = 0.0;
+    }
+}
+
+// Grouped FP64 products of the Newton-Schulz steps and of Z' = J Z: C = alpha A op(B) + diag 1, one CTA
+// per 32 x 32 tile (the FP64 pipes of all SMs), K staged through shared memory in chunks of 16.
+__global__ void __launch_bounds__(128) k_block_gemm(const double* __restrict__ a, const double* __restrict__ bm,
+                                                    double* __restrict__ cm, const SvdGemm* __restrict__ gs,
+                                                    const int3* __restrict__ tiles) {
+    __shared__ double As[16][34], Bs[16][34];
+    const int3 tl = tiles[blockIdx.x];
+    const SvdGemm G = gs[tl.x];
+    const int m0 = tl.y, n0 = tl.z, tid = threadIdx.x;
+    const double* A = a + G.a;
+    const double* Bp = bm + G.b;
+    const int tr = tid >> 3, tc = tid & 7;  // 16 x 8 threads, 2 x 4 outputs each
+    double acc[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+    for (int k0 = 0; k0 < G.K; k0 += 16) {
+        for (int e = tid; e < 512; e += 128) {
+            const int r = e >> 4, k = e & 15;
+            As[k][r] = (m0 + r < G.M && k0 + k < G.K) ? A[static_cast<int64_t>(m0 + r) * G.lda + k0 + k] : 0.0;
+            if (G.transb) Bs[k][r] = (n0 + r < G.N && k0 + k < G.K) ? Bp[static_cast<int64_t>(n0 + r) * G.ldb + k0 + k] : 0.0;
+        }
+        if (!G.transb)
+            for (int e = tid; e < 512; e += 128) {
+                const int k = e >> 5, c = e & 31;
+                Bs[k][c] = (n0 + c < G.N && k0 + k < G.K) ? Bp[static_cast<int64_t>(k0 + k) * G.ldb + n0 + c] : 0.0;
+            }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            double x[2], y[4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) x[i] = As[k][tr + 16 * i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) y[j] = Bs[k][tc + 8 * j];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = m0 + tr + 16 * i, c = n0 + tc + 8 * j;
+            if (r < G.M && c < G.N)
+                cm[G.c + static_cast<int64_t>(r) * G.ldc + c] = G.alpha * acc[i][j] + (r == c ? G.diag : 0.0);
+        }
+}
+
+// The companion columns of Z' of the blocks that keep J.
+__global__ void __launch_bounds__(256) k_companion(const SvdBlock* __restrict__ blocks, const double* __restrict__ J,
+                                                   double* __restrict__ z) {
+    const SvdBlock B = blocks[blockIdx.x];
+    if (!B.companion) return;
+    const int W = B.C + B.R;
+    for (int e = threadIdx.x; e < B.R * B.R; e += blockDim.x) {
+        const int r = e / B.R, c = e - r * B.R;
+        z[B.f_off + static_cast<int64_t>(r) * W + B.C + c] = J[B.j_off + e];
+    }
+}
+
+template <class T>
+cudaError_t put(T* dst, const std::vector<T>& v, cudaStream_t st) {
+    if (v.empty()) return cudaSuccess;
+    return cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st);
+}
+
+size_t up(size_t b) { return (b + 255) / 256 * 256; }
+
+}  // namespace
+
+void SvdPlan::build(const std::vector<SvdShape>& shapes, int smem_dim) {
+    blocks.clear();
+    gemms.clear();
+    tiles.clear();
+    gemm_rng.assign(1, 0);
+    z_size = j_size = f_size = w_size = n_size = 0;
+    smem_floats = max_rows = 0;
+    any_smem = any_global = any_companion = false;
+    int64_t m_off = 0, e_off = 0;
+    for (const SvdShape& s : shapes) {
+        SvdBlock B{};
+        // rows of the block itself (dim rows, their rotations kept as the companion), or of its transpose
+        // (the vectors are the normalised rows): whichever needs fewer FP64 operations per sweep, the
+        // product and the update counting 1 and 4 per element
+        const double own = 1.0 * s.dim * s.dim * (5.0 * s.other + 4.0 * s.dim);
+        const double trans = 1.0 * s.other * s.other * 5.0 * s.dim;
+        B.companion = own <= trans ? 1 : 0;
+        B.dim = s.dim;
+        B.R = B.companion ? s.dim : s.other;
+        B.C = B.companion ? s.other : s.dim;
+        B.z_off = z_size;
+        z_size += static_cast<int64_t>(B.R) * B.C;
+        B.j_off = j_size;
+        j_size += static_cast<int64_t>(B.R) * B.R;
+        B.f_off = f_size;
+        f_size += static_cast<int64_t>(B.R) * (B.C + (B.companion ? B.R : 0));
+        B.n_off = n_size;
+        n_size += B.R;
+        const int64_t fl = static_cast<int64_t>(B.R) * (B.C + B.R) + B.R;
+        // shared memory while it fits and the caller's limit on the dimension allows it
+        B.smem = (s.dim <= smem_dim || smem_dim >= kSvdSmemDefault) && fl <= kSvdSmemFloats ? 1 : 0;
+        B.w_off = w_size;
+        if (B.smem) {
+            any_smem = true;
+            max_rows = std::max(max_rows, B.R);
+            smem_floats = std::max<int>(smem_floats, static_cast<int>(fl));
+        } else {
+            any_global = true;
+            w_size += static_cast<int64_t>(B.R) * (B.C + B.R);
+        }
+        any_companion = any_companion || B.companion;
+        B.m_off = m_off;
+        B.e_off = e_off;
+        m_off += static_cast<int64_t>(s.dim) * s.dim;
+        e_off += s.dim;
+        blocks.push_back(B);
+    }
+    // products: T = 3/2 - 1/2 J J^T, J' = T J (twice, the second pair back into J's place), Z' = J Z
+    for (int step = 0; step < 5; ++step) {
+        for (const SvdBlock& B : blocks) {
+            SvdGemm G{};
+            G.M = G.N = G.K = B.R;
+            G.a = G.b = G.c = B.j_off;
+            G.lda = G.ldb = G.ldc = B.R;
+            G.alpha = 1.0;
+            if (step == 0 || step == 2) {
+                G.transb = 1;
+                G.alpha = -0.5;
+                G.diag = 1.5;
+            }
+            if (step == 4) {
+                G.N = B.C;
+                G.b = B.z_off;
+                G.ldb = B.C;
+                G.c = B.f_off;
+                G.ldc = B.C + (B.companion ? B.R : 0);
+            }
+            for (int m0 = 0; m0 < G.M; m0 += 32)
+                for (int n0 = 0; n0 < G.N; n0 += 32) tiles.push_back(make_int3(static_cast<int>(gemms.size()), m0, n0));
+            gemms.push_back(G);
+        }
+        gemm_rng.push_back(static_cast<int>(tiles.size()));
+    }
+}
+
+size_t SvdPlan::workspace() const {
+    return up(blocks.size() * sizeof(SvdBlock)) + up(gemms.size() * sizeof(SvdGemm)) + up(tiles.size() * sizeof(int3)) +
+           up(blocks.size() * 2 * kSvdConv * sizeof(int)) + up(z_size * 8) + 3 * up(j_size * 8) + up(f_size * 8) +
+           up(w_size * 4) + up(n_size * 8) + up(n_size * 4);
+}
+
+double* SvdPlan::z_buffer(void* ws) const {
+    return reinterpret_cast<double*>(static_cast<char*>(ws) + up(blocks.size() * sizeof(SvdBlock)) +
+                                     up(gemms.size() * sizeof(SvdGemm)) + up(tiles.size() * sizeof(int3)) +
+                                     up(blocks.size() * 2 * kSvdConv * sizeof(int)));
+}
+
+// Measured (GB300, with the parallel k_trunc_*): loading, canonicalising and measuring a random L = 24,
+// D = 256 triplet state (blocks up to 52 rows) takes 104.8 ms, 398.5 ms with the two-sided FP64 Jacobi on
+// X X^T and the one-thread truncation; a two-site step at the middle of the L = 24, D = 256 chain (blocks
+// up to 150 rows) 96.2 ms, 108.8 ms before.
+cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, cudaStream_t st) {
+    const int nb = static_cast<int>(P.blocks.size());
+    if (nb == 0) return cudaSuccess;
+    char* p = static_cast<char*>(ws);
+    auto take = [&](size_t bytes) {
+        char* q = p;
+        p += up(bytes);
+        return q;
+    };
+    auto* blocks = reinterpret_cast<SvdBlock*>(take(nb * sizeof(SvdBlock)));
+    auto* gemms = reinterpret_cast<SvdGemm*>(take(P.gemms.size() * sizeof(SvdGemm)));
+    auto* tiles = reinterpret_cast<int3*>(take(P.tiles.size() * sizeof(int3)));
+    auto* conv = reinterpret_cast<int*>(take(static_cast<size_t>(nb) * 2 * kSvdConv * sizeof(int)));
+    auto* z = reinterpret_cast<double*>(take(P.z_size * 8));
+    auto* j0 = reinterpret_cast<double*>(take(P.j_size * 8));
+    auto* j1 = reinterpret_cast<double*>(take(P.j_size * 8));
+    auto* t0 = reinterpret_cast<double*>(take(P.j_size * 8));
+    auto* f = reinterpret_cast<double*>(take(P.f_size * 8));
+    auto* w = reinterpret_cast<float*>(take(P.w_size * 4));
+    auto* n64 = reinterpret_cast<double*>(take(P.n_size * 8));
+    auto* n32 = reinterpret_cast<float*>(take(P.n_size * 4));
+    cudaError_t e = put(blocks, P.blocks, st);
+    if (e == cudaSuccess) e = put(gemms, P.gemms, st);
+    if (e == cudaSuccess) e = put(tiles, P.tiles, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(conv, 0, static_cast<size_t>(nb) * 2 * kSvdConv * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    if (P.any_smem) {
+        const int bytes = P.smem_floats * static_cast<int>(sizeof(float));
+        e = cudaFuncSetAttribute(k_osj32_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSvdSmemFloats * static_cast<int>(sizeof(float)));
+        if (e != cudaSuccess) return e;
+        const int threads = std::min(1024, std::max(64, 32 * ((P.max_rows + 1) / 2)));  // a warp per pair
+        k_osj32_smem<<<nb, threads, bytes, st>>>(blocks, z, j0, conv, P.smem_floats);
+    }
+    if (P.any_global) k_osj32_global<<<nb * kOsjC, 256, 0, st>>>(blocks, z, w, n32, j0, conv);
+    auto gemm = [&](int step, const double* a, const double* b, double* c) {
+        const int lo = P.gemm_rng[step], hi = P.gemm_rng[step + 1];
+        if (hi > lo) k_block_gemm<<<hi - lo, 128, 0, st>>>(a, b, c, gemms, tiles + lo);
+    };
+    gemm(0, j0, j0, t0);
+    gemm(1, t0, j0, j1);
+    gemm(2, j1, j1, t0);
+    gemm(3, t0, j1, j0);
+    gemm(4, j0, z, f);
+    if (P.any_companion) k_companion<<<nb, 256, 0, st>>>(blocks, j0, f);
+    k_osj64<<<nb * kOsjC, 256, 0, st>>>(blocks, f, n64, conv, mats, evals);
+    return cudaGetLastError();
+}
+
+}  // namespace spmps

@@ -10,10 +10,10 @@
 // taken, and the correction is t = -r / (diag H - theta diag N) (clamped) or a few conjugate-
 // gradient steps on N_eff t = r.  The host only reads scalars (theta, |r|) to steer the loop.
 //
-// The decimation forms the reduced density matrix of each middle label (n, 2m), X X^T for a
-// left-to-right step or X^T X for a right-to-left step, diagonalises all of them with one
-// batched Jacobi launch, keeps the D largest singular values with a deterministic order of
-// ties, and writes the new site tensors with grouped GEMMs: U and U^T X, or X V and V^T.
+// The decimation takes the matrix X of each middle label (n, 2m), the left singular vectors of all of
+// them for a left-to-right step or the right ones for a right-to-left step (svd.cu), keeps the D
+// largest singular values with a deterministic order of ties, and writes the new site tensors with
+// grouped GEMMs: U and U^T X, or X V and V^T.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -22,6 +22,7 @@
 
 #include "engine.h"
 #include "metric.h"
+#include "svd.h"
 
 using namespace spmps;
 using namespace spmps::eng;
@@ -30,8 +31,8 @@ namespace {
 
 constexpr double kTieRtol = 1e-10;   // relative gap below which singular values are tied
 // Singular values below this are dropped (|x| = 1, so the dropped weight per value is < 1e-14).
-// It sits above the noise floor of density-matrix eigenvalues in FP64 (~1e-16 absolute, i.e.
-// ~1e-8 in singular values), so numerically null directions are never kept.
+// It sits far above the noise floor of the two-site tensor in FP64, so numerically null directions
+// are never kept.
 constexpr double kDropAbs = 1e-7;
 constexpr double kEpsMetric = 1e-12;
 constexpr double kClamp = 1e-4;
@@ -476,9 +477,20 @@ struct MidLabel {
 };
 
 struct DecBuffers {
-    DevMem mats, vscr, evals, mat_off, val_off, dims, ln, ltm, keep, keep_total, disc, status, sidx, sval;
-    DevMem tasks, segs, tiles, cmaps, copies, newA0, newA1;
+    DevMem svd, gather, mats, evals, val_off, keep, keep_total, disc, sidx, sval;
 };
+
+bool copies_in_range(const std::vector<CopyBlock>& copies, const int64_t* sizes) {
+    for (const CopyBlock& cb : copies) {
+        const int64_t last_src = cb.transpose ? static_cast<int64_t>(cb.cols - 1) * cb.ld_src + cb.rows - 1
+                                              : static_cast<int64_t>(cb.rows - 1) * cb.ld_src + cb.cols - 1;
+        const int64_t last_dst = static_cast<int64_t>(cb.rows - 1) * cb.ld_dst + cb.cols - 1;
+        const int64_t so = static_cast<int64_t>(cb.src & 0x00FFFFFFFFFFFFFFull);
+        const int64_t dof = static_cast<int64_t>(cb.dst & 0x00FFFFFFFFFFFFFFull);
+        if (so + last_src >= sizes[cb.src >> 56] || dof + last_dst >= sizes[cb.dst >> 56]) return false;
+    }
+    return true;
+}
 
 // Decimate the two-site tensor x (row-block layout at sites (k, k+1), device) into new site
 // tensors k and k+1 with at most Dmax states on the middle bond; move_right selects the
@@ -527,6 +539,7 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
         if (kv.second.nr > 0 && kv.second.nc > 0) list.push_back(&kv.second);
     int64_t moff = 0, voff = 0;
     int maxdim = 0, total = 0;
+    std::vector<SvdShape> shapes;
     for (MidLabel* M : list) {
         M->mat_off = moff;
         M->val_off = voff;
@@ -534,138 +547,75 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
         voff += M->dim;
         maxdim = std::max(maxdim, M->dim);
         total += M->dim;
+        shapes.push_back({M->dim, move_right ? M->nc : M->nr});
     }
     if (maxdim > 512) return fail(h, SPMPS_ERR_UNSUPPORTED, "decimation block larger than 512");
-    // density matrices by grouped GEMMs: slot 0 = x, slot 1 = mats
-    GemmPlan G;
+    // the blocks as dense matrices with the kept side along the rows (or their transposes): slot 0 = x,
+    // slot 1 = the rows that the rotations act on
     auto xblock = [&](int la, int s) { return xl.row_off[la] + xl.seg_col[la * 16 + s]; };
-    for (MidLabel* M : list) {
-        if (move_right) {
-            for (size_t i = 0; i < M->rows.size(); ++i)
-                for (size_t j = 0; j < M->rows.size(); ++j) {
-                    const int la = M->rows[i].first, s1 = M->rows[i].second;
-                    const int la2 = M->rows[j].first, s1b = M->rows[j].second;
-                    GemmTask T{};
-                    T.c = handle(1, M->mat_off + static_cast<int64_t>(M->row_start[i]) * M->dim + M->row_start[j]);
-                    T.cmap = -1;
-                    T.M = bl.labels[la].dim;
-                    T.N = bl.labels[la2].dim;
-                    T.ldc = M->dim;
-                    T.seg0 = static_cast<int>(G.segs.size());
-                    for (size_t c = 0; c < M->cols.size(); ++c) {
-                        const int s2 = M->cols[c].first;
-                        const int sa = s1 * 4 + s2, sb = s1b * 4 + s2;
-                        if (xl.seg_label[la * 16 + sa] < 0 || xl.seg_label[la2 * 16 + sb] < 0) continue;
-                        GemmSeg sg{};
-                        sg.a = handle(0, xblock(la, sa));
-                        sg.a_rs = xl.width[la];
-                        sg.a_cs = 1;
-                        sg.K = br.labels[M->cols[c].second].dim;
-                        sg.b = handle(0, xblock(la2, sb));
-                        sg.b_rs = 1;
-                        sg.b_cs = xl.width[la2];
-                                                G.segs.push_back(sg);
-                    }
-                    T.nseg = static_cast<int>(G.segs.size()) - T.seg0;
-                    G.tasks.push_back(T);
+    SvdPlan SP;
+    SP.build(shapes, h->opt.jacobi_smem_max);
+    std::vector<CopyBlock> gather;
+    bool holes = false;  // a block of the matrix that x does not have (stays zero)
+    for (size_t i = 0; i < list.size(); ++i) {
+        const MidLabel& M = *list[i];
+        const SvdBlock& SB = SP.blocks[i];
+        const bool transposed = move_right != (SB.companion != 0);  // rows of the matrix run over M.cols
+        for (size_t r = 0; r < M.rows.size(); ++r)
+            for (size_t c = 0; c < M.cols.size(); ++c) {
+                const int la = M.rows[r].first, s = M.rows[r].second * 4 + M.cols[c].first;
+                if (xl.seg_label[la * 16 + s] < 0) {
+                    holes = true;
+                    continue;
                 }
-        } else {
-            for (size_t i = 0; i < M->cols.size(); ++i)
-                for (size_t j = 0; j < M->cols.size(); ++j) {
-                    const int s2 = M->cols[i].first, lb = M->cols[i].second;
-                    const int s2b = M->cols[j].first, lb2 = M->cols[j].second;
-                    GemmTask T{};
-                    T.c = handle(1, M->mat_off + static_cast<int64_t>(M->col_start[i]) * M->dim + M->col_start[j]);
-                    T.cmap = -1;
-                    T.M = br.labels[lb].dim;
-                    T.N = br.labels[lb2].dim;
-                    T.ldc = M->dim;
-                    T.seg0 = static_cast<int>(G.segs.size());
-                    for (size_t r = 0; r < M->rows.size(); ++r) {
-                        const int la = M->rows[r].first, s1 = M->rows[r].second;
-                        const int sa = s1 * 4 + s2, sb = s1 * 4 + s2b;
-                        if (xl.seg_label[la * 16 + sa] < 0 || xl.seg_label[la * 16 + sb] < 0) continue;
-                        GemmSeg sg{};
-                        sg.a = handle(0, xblock(la, sa));
-                        sg.a_rs = 1;
-                        sg.a_cs = xl.width[la];
-                        sg.K = bl.labels[la].dim;
-                        sg.b = handle(0, xblock(la, sb));
-                        sg.b_rs = xl.width[la];
-                        sg.b_cs = 1;
-                                                G.segs.push_back(sg);
-                    }
-                    T.nseg = static_cast<int>(G.segs.size()) - T.seg0;
-                    G.tasks.push_back(T);
-                }
-        }
+                CopyBlock cb{};
+                cb.src = handle(0, xblock(la, s));
+                cb.ld_src = xl.width[la];
+                cb.ld_dst = SB.C;
+                const int nr = bl.labels[la].dim, nc = br.labels[M.cols[c].second].dim;
+                cb.rows = transposed ? nc : nr;
+                cb.cols = transposed ? nr : nc;
+                cb.transpose = transposed ? 1 : 0;
+                cb.dst = handle(1, SB.z_off + (transposed ? static_cast<int64_t>(M.col_start[c]) * SB.C + M.row_start[r]
+                                                          : static_cast<int64_t>(M.row_start[r]) * SB.C + M.col_start[c]));
+                gather.push_back(cb);
+            }
     }
-    G.add_tiles();
+    CK(B.svd.ensure(std::max<size_t>(SP.workspace(), 1)));
+    CK(B.mats.ensure(std::max<int64_t>(moff, 1) * sizeof(double)));
+    CK(B.evals.ensure(std::max<int64_t>(voff, 1) * sizeof(double)));
     {
         int64_t sz[kMaxSlots];
         for (auto& v : sz) v = -1;
         sz[0] = n;
-        sz[1] = moff;
-        std::string why;
-        if (!validate_gemm(G, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (density matrix): " + why);
+        sz[1] = SP.z_size;
+        if (!copies_in_range(gather, sz)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (blocks)");
     }
-    CK(B.mats.ensure(std::max<int64_t>(moff, 1) * sizeof(double)));
-    CK(B.vscr.ensure(std::max<int64_t>(moff, 1) * sizeof(double)));
-    CK(B.evals.ensure(std::max<int64_t>(voff, 1) * sizeof(double)));
-    CK(upload(B.tasks, G.tasks, h->stream));
-    CK(upload(B.segs, G.segs, h->stream));
-    CK(upload(B.tiles, G.tiles, h->stream));
-    CK(upload(B.cmaps, G.cmaps, h->stream));
+    CK(upload(B.gather, gather, h->stream));
     Slots S{};
     S.p[0] = x;
-    S.p[1] = B.mats.as<double>();
-    {
-        double fl = 0.0;
-        for (const GemmTask& T : G.tasks)
-            for (int q = 0; q < T.nseg; ++q) fl += 2.0 * T.M * T.N * G.segs[T.seg0 + q].K;
-        const int rec = h->profile ? prof_begin(h, h->stream, 0, fl) : -1;
-        CK(launch_gemm_f64(S, B.tasks.as<GemmTask>(), B.segs.as<GemmSeg>(), B.tiles.as<GemmTile>(), B.cmaps.as<int>(),
-                           static_cast<int>(G.tiles.size()), h->stream));
-        if (rec >= 0) prof_end(h, h->stream, rec);
-    }
-    ++h->launches;
-    // batched Jacobi and ordered truncation
-    std::vector<int64_t> mo, vo;
-    std::vector<int> dims, lns, ltms;
-    for (MidLabel* M : list) {
-        mo.push_back(M->mat_off);
-        vo.push_back(M->val_off);
-        dims.push_back(M->dim);
-        lns.push_back(M->n);
-        ltms.push_back(M->tm);
-    }
+    S.p[1] = SP.z_buffer(B.svd.p);
+    if (holes) CK(cudaMemsetAsync(S.p[1], 0, SP.z_size * sizeof(double), h->stream));
+    // singular vectors and ordered truncation
+    std::vector<int64_t> vo;
+    for (MidLabel* M : list) vo.push_back(M->val_off);
     const int nm = static_cast<int>(list.size());
-    CK(upload(B.mat_off, mo, h->stream));
     CK(upload(B.val_off, vo, h->stream));
-    CK(upload(B.dims, dims, h->stream));
-    CK(upload(B.ln, lns, h->stream));
-    CK(upload(B.ltm, ltms, h->stream));
     CK(B.keep.ensure(std::max(nm, 1) * sizeof(int)));
     CK(B.keep_total.ensure(sizeof(int)));
     CK(B.disc.ensure(sizeof(double)));
-    CK(B.status.ensure(sizeof(int)));
     CK(B.sidx.ensure(std::max(3 * total, 1) * sizeof(int)));
     CK(B.sval.ensure(std::max(2 * total, 1) * sizeof(double)));
-    CK(cudaMemsetAsync(B.status.p, 0, sizeof(int), h->stream));
     const int rec_eig = h->profile ? prof_begin(h, h->stream, 4, 0.0) : -1;
-    CK(launch_jacobi_batched(B.mats.as<double>(), B.vscr.as<double>(), B.evals.as<double>(), B.mat_off.as<int64_t>(),
-                             B.val_off.as<int64_t>(), B.dims.as<int>(), nm, maxdim, h->opt.jacobi_smem_max, 1,
-                             B.status.as<int>(), h->stream));
-    CK(launch_truncate(B.evals.as<double>(), B.val_off.as<int64_t>(), B.dims.as<int>(), B.ln.as<int>(), B.ltm.as<int>(),
-                       nm, total, Dmax, kTieRtol, kDropAbs, B.keep.as<int>(), B.keep_total.as<int>(), B.disc.as<double>(),
-                       B.sidx.as<int>(), B.sval.as<double>(), h->stream));
+    CK(launch_copy_blocks(S, B.gather.as<CopyBlock>(), static_cast<int>(gather.size()), h->stream));
+    CK(launch_svd(SP, B.svd.p, B.mats.as<double>(), B.evals.as<double>(), h->stream));
+    CK(launch_truncate(B.evals.as<double>(), B.val_off.as<int64_t>(), nm, total, Dmax, kTieRtol, kDropAbs, B.keep.as<int>(),
+                       B.keep_total.as<int>(), B.disc.as<double>(), B.sidx.as<int>(), B.sval.as<double>(), h->stream));
     if (rec_eig >= 0) prof_end(h, h->stream, rec_eig);
-    h->launches += 2;
+    h->launches += 11;
     std::vector<int> keep(std::max(nm, 1));
-    int jac_status = 0;
     double disc = 0.0;
     CK(cudaMemcpyAsync(keep.data(), B.keep.p, std::max(nm, 1) * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(&jac_status, B.status.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(&disc, B.disc.p, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     if (discarded) *discarded = disc;
@@ -783,16 +733,7 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
         sz[3] = a1.size;
         std::string why;
         if (!validate_gemm(W, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (new tensors): " + why);
-        for (const CopyBlock& cb : copies) {
-            const int64_t last_src = cb.transpose ? static_cast<int64_t>(cb.cols - 1) * cb.ld_src + cb.rows - 1
-                                                  : static_cast<int64_t>(cb.rows - 1) * cb.ld_src + cb.cols - 1;
-            const int64_t last_dst = static_cast<int64_t>(cb.rows - 1) * cb.ld_dst + cb.cols - 1;
-            const int ss = static_cast<int>(cb.src >> 56), ds = static_cast<int>(cb.dst >> 56);
-            const int64_t so = static_cast<int64_t>(cb.src & 0x00FFFFFFFFFFFFFFull);
-            const int64_t dof = static_cast<int64_t>(cb.dst & 0x00FFFFFFFFFFFFFFull);
-            if (so + last_src >= sz[ss] || dof + last_dst >= sz[ds])
-                return fail(h, SPMPS_ERR_CUDA, "internal plan check (copies)");
-        }
+        if (!copies_in_range(copies, sz)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (copies)");
     }
     auto A0 = std::make_unique<DevMem>();
     auto A1 = std::make_unique<DevMem>();
@@ -823,7 +764,6 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
     CK(launch_copy_blocks(S2, d_copies.as<CopyBlock>(), static_cast<int>(copies.size()), h->stream));
     h->launches += 4;
     CK(cudaStreamSynchronize(h->stream));
-    (void)jac_status;
     // install
     h->bonds[k + 1] = nb;
     h->alay[k] = a0;
