@@ -6,8 +6,8 @@
 //   1. k_osj<float>: one-sided Jacobi on an FP32 copy [Z | I] finds J with nearly orthogonal rows of J Z;
 //   2. two Newton-Schulz steps J <- (3/2 - 1/2 J J^T) J in FP64 (k_block_gemm, all SMs) make J orthonormal
 //      to FP64, and Z' = J Z is formed in FP64 from the unrounded block;
-//   3. k_osj<double>: one-sided Jacobi on Z' to FP64 convergence (two sweeps as a rule: the FP32 start
-//      leaves relative couplings of 1e-6, and the convergence is quadratic).
+//   3. k_osj<double>: one-sided Jacobi on Z' to FP64 convergence (two or three sweeps as a rule: the FP32
+//      start leaves relative couplings of 1e-6, and the convergence is quadratic).
 // The singular values are the row norms of the result and come from Z itself, not from its Gram matrix,
 // so small ones keep the FP64 noise floor of Z (1e-16, not 1e-8).
 #include <cooperative_groups.h>
@@ -50,18 +50,18 @@ __device__ __forceinline__ double rotation_cos(double t) {
 // SMEM: one CTA per block with the rows in shared memory (a round costs a __syncthreads); otherwise a
 // cluster of kOsjC CTAs with the rows in global memory (L2), a cluster barrier per round: in FP64 the
 // FP64 pipes of 8 SMs share the work.  NCH > 0 keeps the two rows of a pair in registers (W <= 32 NCH)
-// between the product and the update, NCH = 0 reads them twice.
+// between the product and the update, NCH = 0 reads them twice.  The sweeps end after one that met no
+// relative coupling above `done` (what it leaves is the square of that over the relative gap).
 // Measured (GB300, middle decimation of the L = 24, D = 256 chain, blocks up to 136): see launch_svd.
 template <class T, bool SMEM, int NCH>
-__device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, int* conv, int rank, int ctas) {
+__device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T done, int* conv, int rank, int ctas) {
     const int lane = threadIdx.x & 31;
     const int warp = (threadIdx.x >> 5) + rank * (blockDim.x >> 5);
     const int warps = (blockDim.x >> 5) * ctas;
     const int np = (R + 1) & ~1, half = np / 2;
     constexpr bool kF64 = sizeof(T) == 8;
     const T tol = kF64 ? T(1e-15) : T(3e-7);
-    const T done = kF64 ? T(1e-8) : T(1e-3);  // couplings below this square to the noise of T in one sweep
-    const T floor_abs = norm2_all * (kF64 ? T(1e-18) : T(1e-12));
+    const T floor_abs = kF64 ? T(0) : norm2_all * T(1e-12);  // FP32: the noise of the block's largest rows
     const T null2 = norm2_all * (kF64 ? T(kNullRel * kNullRel) : T(1e-13));
     const T inv_all = norm2_all > T(0) ? T(1) / norm2_all : T(0);  // keeps the angle's FP32 operands in range
     auto barrier = [&]() {
@@ -198,9 +198,9 @@ __device__ void osj32_block(const SvdBlock& B, const double* __restrict__ zraw, 
     else
         cgx::this_cluster().sync();
     if (W <= 256 && !SMEM)
-        osj_sweeps<float, SMEM, SMEM ? 0 : 8>(work, nrm2, R, C, W, 1.0f, conv, rank, ctas);
+        osj_sweeps<float, SMEM, SMEM ? 0 : 8>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
     else
-        osj_sweeps<float, SMEM, 0>(work, nrm2, R, C, W, 1.0f, conv, rank, ctas);
+        osj_sweeps<float, SMEM, 0>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
     for (int e = rank * blockDim.x + threadIdx.x; e < R * R; e += blockDim.x * ctas) {
         const int r = e / R, c = e - r * R;
         const float* p = work + static_cast<int64_t>(r) * W + C + c;
@@ -264,12 +264,14 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
     }
     cgx::this_cluster().sync();  // every CTA has read Z before any rotates it
     int* cv = conv + (b * 2 + 1) * kSvdConv;
+    // the companion is orthonormal by construction; normalised rows only as far as they are uncoupled
+    const double done = B.companion ? 1e-11 : 1e-13;
     if (W <= 160)
-        osj_sweeps<double, false, 5>(Z, nr, R, C, W, tot, cv, rank, kOsjC);
+        osj_sweeps<double, false, 5>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     else if (W <= 320)
-        osj_sweeps<double, false, 10>(Z, nr, R, C, W, tot, cv, rank, kOsjC);
+        osj_sweeps<double, false, 10>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     else
-        osj_sweeps<double, false, 0>(Z, nr, R, C, W, tot, cv, rank, kOsjC);
+        osj_sweeps<double, false, 0>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     // exact norms of the final rows, then the vectors by descending norm (ties by row)
     const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) + rank * (blockDim.x >> 5);
     const int warps = (blockDim.x >> 5) * kOsjC;
