@@ -16,7 +16,6 @@
 #include <cstring>
 #include <array>
 #include <map>
-#include <unordered_map>
 
 #include "engine.h"
 
@@ -173,7 +172,19 @@ bool validate_tile_list(const GemmPlan& G, const std::vector<GemmTile>& tiles, s
     return true;
 }
 
-bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why) {
+bool validate_diag(const Plan& P, const int64_t* sizes, std::string* why) {
+    for (const DiagBlock& b : P.diag_blocks) {
+        for (int q = 0; q < b.nterm; ++q) {
+            const DiagTerm& t = P.diag_terms[b.term0 + q];
+            if (!in_range(t.l, static_cast<int64_t>(b.rows - 1) * t.l_step, sizes, why, "diag L")) return false;
+            if (!in_range(t.r, static_cast<int64_t>(b.cols - 1) * t.r_step, sizes, why, "diag R")) return false;
+        }
+    }
+    return true;
+}
+
+bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why, int G) {
+    if (!P.chan.pairs.empty() && !comb_check(P.chan, G, sizes[3], sizes[4], why)) return false;
     if (!validate_gemm(P.A, sizes, why) || !validate_gemm(P.C, sizes, why)) return false;
     for (const CombOut& o : P.B.outs) {
         if (o.rows <= 0 || o.cols <= 0 || o.cols > o.ld) { *why = "bad combination block"; return false; }
@@ -183,14 +194,7 @@ bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why) {
             if (!in_range(t.src, static_cast<int64_t>(o.rows - 1) * t.ld + o.cols - 1, sizes, why, "comb src")) return false;
         }
     }
-    for (const DiagBlock& b : P.diag_blocks) {
-        for (int q = 0; q < b.nterm; ++q) {
-            const DiagTerm& t = P.diag_terms[b.term0 + q];
-            if (!in_range(t.l, static_cast<int64_t>(b.rows - 1) * t.l_step, sizes, why, "diag L")) return false;
-            if (!in_range(t.r, static_cast<int64_t>(b.cols - 1) * t.r_step, sizes, why, "diag R")) return false;
-        }
-    }
-    return true;
+    return validate_diag(P, sizes, why);
 }
 
 // ---- plan upload and launch -------------------------------------------------------------------
@@ -226,8 +230,24 @@ spmps_status plan_upload(spmps_t* h, Plan& P) {
     CK(upload(P.d_cmapsC, P.C.cmaps, h->stream));
     CK(upload(P.d_tcA, P.A.tc_tiles, h->stream));
     CK(upload(P.d_tcC, P.C.tc_tiles, h->stream));
-    CK(upload(P.d_diag_blocks, P.diag_blocks, h->stream));
-    CK(upload(P.d_diag_terms, P.diag_terms, h->stream));
+    if (!P.chan.pairs.empty()) {
+        CombChan& N = P.chan;
+        CK(upload(P.d_chan[0], N.ins, h->stream));
+        CK(upload(P.d_chan[1], N.sets, h->stream));
+        CK(upload(P.d_chan[2], N.dsts, h->stream));
+        CK(upload(P.d_chan[3], N.coefs, h->stream));
+        CK(upload(P.d_chan[4], N.pairs, h->stream));
+        CK(upload(P.d_chan[5], N.lab, h->stream));
+        CK(upload(P.d_chan[6], N.units, h->stream));
+        CK(upload(P.d_chan[7], N.rots, h->stream));
+        std::vector<int> outs = N.outs;
+        outs.insert(outs.end(), N.shared_outs.begin(), N.shared_outs.end());
+        CK(upload(P.d_chan[8], outs, h->stream));
+        P.chan_dev = CombDev{P.d_chan[0].as<CombIn>(),   P.d_chan[1].as<CombSet>(), P.d_chan[2].as<CombDst>(),
+                             P.d_chan[3].as<CombCoef>(), P.d_chan[4].as<CombPair>(), P.d_chan[5].as<uint8_t>(),
+                             P.d_chan[6].as<int2>(),     P.d_chan[7].as<int2>(),    P.d_chan[8].as<int>(),
+                             static_cast<int>(N.outs.size()), h->d_rot.as<double>(),      N.stride};
+    }
     // tile and output ranges per (op, g): tasks were appended in (op, g) order
     auto ranges = [&](const std::vector<GemmTile>& tiles, const std::vector<int>& task_rng, std::vector<int>& out) {
         out.assign(task_rng.size(), 0);
@@ -254,7 +274,7 @@ spmps_status plan_upload(spmps_t* h, Plan& P) {
     };
     task_flops(P.A, a_task_rng, P.flopsA_rng);
     task_flops(P.C, c_task_rng, P.flopsC_rng);
-    P.flopsB_rng.assign(P.combB_rng.size(), 0.0);
+    if (P.chan.pairs.empty()) P.flopsB_rng.assign(P.combB_rng.size(), 0.0);
     for (size_t r = 0; r + 1 < P.combB_rng.size(); ++r)
         for (int o = P.combB_rng[r]; o < P.combB_rng[r + 1]; ++o)
             P.flopsB_rng[r] += 2.0 * P.B.outs[o].rows * P.B.outs[o].cols * P.B.outs[o].nterm;
@@ -319,9 +339,11 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
                       const SlotsF* split) {
     const bool batched = h->opt.batched != 0;
     if (ev) CK(cudaEventRecord(ev[0], st));
-    CK(cudaMemsetAsync(S.p[3], 0, std::max<int64_t>(1, P.t1_size) * sizeof(double), st));
+    if (P.zero_t1) {
+        CK(cudaMemsetAsync(S.p[3], 0, std::max<int64_t>(1, P.t1_size) * sizeof(double), st));
+        ++h->launches;
+    }
     if (ev) CK(cudaEventRecord(ev[1], st));
-    ++h->launches;
     // flops of a range of (op, g) entries, for the profiler
     auto range_flops = [&](const std::vector<double>& f, int a, int b) {
         double acc = 0.0;
@@ -331,6 +353,9 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
     // the H part (op 0) of a projected action may run on the tensor cores (precision 1 or 2)
     const int prec = P.reduce_nx > 0 ? h->apply_precision : 0;
     const int G = h->G;
+    // both operators in one launch per phase: N's phase A is part of H's where the operator allows it
+    // (its T1 is H's channel of identities; in FP64 only, N never runs in reduced precision)
+    const bool shared = batched && prec == 0 && P.chan.shares && r0 == 0 && r1 == 2 * G;
     auto gemm = [&](const DevMem& tasks, const DevMem& segs, const DevMem& tiles, const DevMem& cmaps,
                     const std::vector<int>& rng, const std::vector<double>& fl, const DevMem& tc,
                     const std::vector<int>& tc_rng, int a, int b) -> cudaError_t {
@@ -418,6 +443,14 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
         return gemm(P.d_tasksA, P.d_segsA, P.d_tilesA, P.d_cmapsA, P.tileA_rng, P.flopsA_rng, P.d_tcA, P.tcA_rng, a, b);
     };
     auto runB = [&](int a, int b) -> cudaError_t {
+        if (!P.chan.unit_rng.empty()) {  // (op, g) ranges: whole operators, or one beta point of one
+            const int rec = h->profile ? prof_begin(h, st, 1, range_flops(P.flopsB_rng, a, b)) : -1;
+            const bool single = b - a < G;
+            const cudaError_t e = launch_comb_chan(S, P.chan, P.chan_dev, a / G, single ? a / G + 1 : b / G, single ? a % G : 0,
+                                                   single ? b - a : G, shared, &h->launches, st);
+            if (rec >= 0) prof_end(h, st, rec);
+            return e;
+        }
         const int o0 = P.combB_rng[a], o1 = P.combB_rng[b];
         ++h->launches;
         const int rec = h->profile ? prof_begin(h, st, 1, range_flops(P.flopsB_rng, a, b)) : -1;
@@ -440,7 +473,7 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
         return launch_split_tf32(S.p[4], P.t2_size, split->p[4], st);
     };
     if (batched) {
-        CK(runA(r0, r1));
+        CK(runA(r0, shared ? G : r1));
         if (ev) CK(cudaEventRecord(ev[2], st));
         CK(runB(r0, r1));
         CK(split_t3());
@@ -456,16 +489,95 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
     }
     if (P.reduce_nx > 0) {
         // outputs of op: y (slot 1) from the partials in slot 8, z (slot 2) from slot 9
-        for (int op = r0 / G; op < (r1 + G - 1) / G && op < 2; ++op) {
-            CK(launch_sum_partials(S.p[8 + op], G, P.reduce_nx, S.p[1 + op], st));
-            ++h->launches;
-        }
+        CK(launch_sum_partials(S.p[8], S.p[9], P.weighted ? h->d_cg.as<double>() : nullptr, G, P.reduce_nx,
+                               r0 < G ? S.p[1] : nullptr, r1 > G ? S.p[2] : nullptr, st));
+        ++h->launches;
     }
     if (ev) CK(cudaEventRecord(ev[4], st));
     return SPMPS_OK;
 }
 
 // ---- environment update plans ------------------------------------------------------------------
+
+// Entries of one site's operator per output channel: the right channels (rows summed over the left ones)
+// or the left channels, by (input channel, s, t).
+std::vector<std::vector<ChanEntry>> site_entries(const MPO& m, int i, bool to_right) {
+    std::vector<std::vector<ChanEntry>> out(to_right ? m.dw[i + 1] : m.dw[i]);
+    auto put = [](std::vector<ChanEntry>& v, int w, const MpoEntry& e) {
+        for (int s = 0; s < 4; ++s)
+            for (int t = 0; t < 4; ++t)
+                if (e.op[s * 4 + t] != 0.0) v.push_back({w, s, t, e.op[s * 4 + t]});
+    };
+    if (to_right) {
+        for (const MpoEntry& e : m.E[i]) put(out[e.wr], e.wl, e);
+    } else {
+        for (int q : m.by_wl[i]) put(out[m.E[i][q].wl], m.E[i][q].wr, m.E[i][q]);
+    }
+    return out;
+}
+
+// Entries of two neighbouring sites' operators contracted over the bond between them, per right channel,
+// by (left channel, s, t) with s = 4 s1 + s2.
+std::vector<std::vector<ChanEntry>> pair_entries(const MPO& m, int k) {
+    const int dwl = m.dw[k], dwr = m.dw[k + 2];
+    std::vector<std::vector<ChanEntry>> out(dwr);
+    std::vector<int> place(dwl, -1);
+    std::vector<std::array<double, 256>> acc;
+    std::vector<int> ws;
+    for (int u = 0; u < dwr; ++u) {
+        acc.clear();
+        ws.clear();
+        for (int qb = m.wr_ptr[k + 1][u]; qb < m.wr_ptr[k + 1][u + 1]; ++qb) {
+            const MpoEntry& b = m.E[k + 1][qb];
+            const int v = b.wl;
+            for (int qa = m.wr_ptr[k][v]; qa < m.wr_ptr[k][v + 1]; ++qa) {
+                const MpoEntry& a = m.E[k][qa];
+                if (place[a.wl] < 0) {
+                    place[a.wl] = static_cast<int>(ws.size());
+                    ws.push_back(a.wl);
+                    acc.emplace_back();
+                    acc.back().fill(0.0);
+                }
+                std::array<double, 256>& dst = acc[place[a.wl]];
+                for (int s1 = 0; s1 < 4; ++s1)
+                    for (int t1 = 0; t1 < 4; ++t1) {
+                        const double av = a.op[s1 * 4 + t1];
+                        if (av == 0.0) continue;
+                        for (int s2 = 0; s2 < 4; ++s2)
+                            for (int t2 = 0; t2 < 4; ++t2) {
+                                const double bv = b.op[s2 * 4 + t2];
+                                if (bv != 0.0) dst[(s1 * 4 + s2) * 16 + t1 * 4 + t2] += av * bv;
+                            }
+                    }
+            }
+        }
+        std::vector<int> order = ws;
+        std::sort(order.begin(), order.end());
+        for (int w : order)
+            for (int q = 0; q < 256; ++q)
+                if (acc[place[w]][q] != 0.0) out[u].push_back({w, q >> 4, q & 15, acc[place[w]][q]});
+        for (int w : ws) place[w] = -1;
+    }
+    return out;
+}
+
+// The channel of bond k whose left environment is the identity operator's: every site before it is passed
+// by the identity alone.  -1: none.
+int identity_channel(const MPO& m, int k) {
+    int w = 0;
+    for (int i = 0; i < k; ++i) {
+        int next = -1;
+        for (int q = m.wl_ptr[i][w]; q < m.wl_ptr[i][w + 1] && next < 0; ++q) {
+            const MpoEntry& e = m.E[i][m.by_wl[i][q]];
+            bool one = m.wr_ptr[i][e.wr + 1] - m.wr_ptr[i][e.wr] == 1;  // its only entry
+            for (int s = 0; s < 16 && one; ++s) one = e.op[s] == (s % 5 == 0 ? 1.0 : 0.0);
+            if (one) next = e.wr;
+        }
+        if (next < 0) return -1;
+        w = next;
+    }
+    return w;
+}
 
 // Left update at site i: L(bond i+1) from L(bond i) and A[i].
 // Slots: 0 = A[i], 3 = T1, 4 = T2, 5 = L(bond i), 7 = L(bond i+1).
@@ -479,7 +591,7 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
     P.task_rng_kept = false;
     P.tileA_rng.assign(nops * G + 1, 0);
     P.tileC_rng.assign(nops * G + 1, 0);
-    P.combB_rng.assign(nops * G + 1, 0);
+    P.flopsB_rng.clear();
     // column maps of the site's row blocks into the N-dense T1 columns (depend on the label only)
     std::vector<int> cmap_off(bl.labels.size(), -1);
     for (size_t l = 0; l < bl.labels.size(); ++l) {
@@ -494,42 +606,84 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
             for (int j = 0; j < Lb.dim; ++j) P.A.cmaps.push_back(base + j);
         }
     }
+    // (left label, s) blocks of A that end in each right label, in order
+    std::vector<std::vector<std::pair<int, int>>> into(br.labels.size());
+    for (int la = 0; la < static_cast<int>(bl.labels.size()); ++la)
+        for (int q = 0; q < 4; ++q)
+            if (al.seg_label[la * 4 + q] >= 0) into[al.seg_label[la * 4 + q]].push_back({la, q});
     int64_t t1 = 0, t2 = 0;
-    std::vector<int64_t> t1_off, t2_off;  // [((op*G+g)*nw + w)*ngl + Ga]
-    std::vector<ColLayout> cl1, cl2;
+    P.chan.clear();
     for (int op = 0; op < nops; ++op) {
         const MPO& m = h->ops.mpo[op];
         const int dwl = m.dw[i], dwr = m.dw[i + 1];
         const std::vector<int>& cnl = m.cn[i];
         const std::vector<int>& cnr = m.cn[i + 1];
+        // blocks of T1[w][Ga] and T2[u][Ga] for beta point 0; the other points follow at equal distances
+        std::vector<int64_t> o1(static_cast<size_t>(dwl) * ngl, -1), o2(static_cast<size_t>(dwr) * ngl, -1);
+        std::vector<ColLayout> c1(o1.size()), c2(o2.size());
+        const int64_t t1_op = t1, t2_op = t2;
+        for (int w = 0; w < dwl; ++w)
+            for (int ga = 0; ga < ngl; ++ga) {
+                const int n0 = bl.groups[ga].n - cnl[w];
+                if (bl.group_of(n0) < 0 || Lo.lay[op].off[w * ngl + ga] < 0) continue;
+                ColLayout CL = make_col_layout(br, n0, 4, +1);
+                if (CL.width == 0) continue;
+                o1[w * ngl + ga] = t1;
+                t1 += static_cast<int64_t>(bl.groups[ga].dim) * CL.width;
+                c1[w * ngl + ga] = std::move(CL);
+            }
+        for (int u = 0; u < dwr; ++u)
+            for (int ga = 0; ga < ngl; ++ga) {
+                ColLayout CL = make_col_layout(br, bl.groups[ga].n - cnr[u], 4, +1);
+                if (CL.width == 0) continue;
+                o2[u * ngl + ga] = t2;
+                t2 += static_cast<int64_t>(bl.groups[ga].dim) * CL.width;
+                c2[u * ngl + ga] = std::move(CL);
+            }
+        const int64_t s1 = t1 - t1_op, s2 = t2 - t2_op;
+        t1 = t1_op + G * s1;
+        t2 = t2_op + G * s2;
+        // phase B: T2[u][Ga][:, s, :] = sum_{w,t} W[w,u,s,t] (r T1)[w][Ga][:, t, :]
+        P.chan.stride.t1[op] = s1;
+        P.chan.stride.t3[op] = s2;
+        const std::vector<std::vector<ChanEntry>> ent = site_entries(m, i, true);
+        CombSpec sp;
+        sp.op = op;
+        sp.legs = 1;
+        sp.sign = 1;
+        sp.row = &bl;
+        sp.col = &br;
+        sp.ket = &bl;
+        sp.cn_in = &cnl;
+        sp.cn_out = &cnr;
+        sp.o1 = &o1;
+        sp.o2 = &o2;
+        sp.c1 = &c1;
+        sp.c2 = &c2;
+        sp.entries = &ent;
+        sp.needed = [&](int la, int s) { return al.seg_label[la * 4 + s] >= 0; };
+        const double fb = comb_add(P.chan, sp);
+        P.B.flops += G * fb;
         for (int g = 0; g < G; ++g) {
-            const MPO& W = h->ops.rot[op][g];
             const int og = op * G + g;
+            P.flopsB_rng.push_back(fb);
             P.tileA_rng[og] = static_cast<int>(P.A.tasks.size());
-            P.combB_rng[og] = static_cast<int>(P.B.outs.size());
             P.tileC_rng[og] = static_cast<int>(P.C.tasks.size());
             // phase A
-            std::vector<int64_t> o1(static_cast<size_t>(dwl) * ngl, -1);
-            std::vector<ColLayout> c1(static_cast<size_t>(dwl) * ngl);
             for (int w = 0; w < dwl; ++w)
                 for (int ga = 0; ga < ngl; ++ga) {
-                    const int n0 = bl.groups[ga].n - cnl[w];
-                    const int gap = bl.group_of(n0);
+                    if (o1[w * ngl + ga] < 0) continue;
+                    const int gap = bl.group_of(bl.groups[ga].n - cnl[w]);
                     const int64_t loff = Lo.lay[op].off[w * ngl + ga];
-                    if (gap < 0 || loff < 0) continue;
-                    ColLayout CL = make_col_layout(br, n0, 4, +1);
-                    if (CL.width == 0) continue;
-                    const int M = bl.groups[ga].dim;
-                    o1[w * ngl + ga] = t1;
                     for (int l = bl.groups[gap].first; l < bl.groups[gap].first + bl.groups[gap].count; ++l) {
                         if (al.width[l] == 0) continue;
                         const Label& Ll = bl.labels[l];
                         GemmTask T{};
-                        T.c = handle(3, t1);
+                        T.c = handle(3, o1[w * ngl + ga] + g * s1);
                         T.cmap = cmap_off[l];
-                        T.M = M;
+                        T.M = bl.groups[ga].dim;
                         T.N = al.width[l];
-                        T.ldc = CL.width;
+                        T.ldc = c1[w * ngl + ga].width;
                         T.seg0 = static_cast<int>(P.A.segs.size());
                         T.nseg = 1;
                         GemmSeg sg{};
@@ -540,53 +694,10 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
                         sg.b = handle(0, al.row_off[l]);
                         sg.b_rs = al.width[l];
                         sg.b_cs = 1;
-                                                P.A.segs.push_back(sg);
+                        P.A.segs.push_back(sg);
                         P.A.tasks.push_back(T);
                         P.A.flops += 2.0 * T.M * T.N * sg.K;
                     }
-                    t1 += static_cast<int64_t>(M) * CL.width;
-                    c1[w * ngl + ga] = CL;
-                }
-            // phase B: T2[u][Ga][:, s, :] = sum_{w,t} W[w,u,s,t] T1[w][Ga][:, t, :]
-            std::vector<int64_t> o2(static_cast<size_t>(dwr) * ngl, -1);
-            std::vector<ColLayout> c2(static_cast<size_t>(dwr) * ngl);
-            for (int u = 0; u < dwr; ++u)
-                for (int ga = 0; ga < ngl; ++ga) {
-                    const int n0 = bl.groups[ga].n - cnr[u];
-                    ColLayout CL = make_col_layout(br, n0, 4, +1);
-                    if (CL.width == 0) continue;
-                    const int M = bl.groups[ga].dim;
-                    o2[u * ngl + ga] = t2;
-                    for (int s = 0; s < 4; ++s) {
-                        if (CL.col[s] < 0) continue;
-                        CombOut O{};
-                        O.dst = handle(4, t2 + CL.col[s]);
-                        O.rows = M;
-                        O.cols = br.groups[CL.group[s]].dim;
-                        O.ld = CL.width;
-                        O.term0 = static_cast<int>(P.B.terms.size());
-                        for (int ei = W.wr_ptr[i][u]; ei < W.wr_ptr[i][u + 1]; ++ei) {
-                            const MpoEntry& e = W.E[i][ei];
-                            const int w = e.wl;
-                            const int64_t s1 = o1[w * ngl + ga];
-                            if (s1 < 0) continue;
-                            const ColLayout& C1 = c1[w * ngl + ga];
-                            for (int t = 0; t < 4; ++t) {
-                                const double cf = e.op[s * 4 + t];
-                                if (cf == 0.0 || C1.col[t] < 0) continue;
-                                CombTerm tm{};
-                                tm.src = handle(3, s1 + C1.col[t]);
-                                tm.ld = C1.width;
-                                tm.coef = cf;
-                                P.B.terms.push_back(tm);
-                            }
-                        }
-                        O.nterm = static_cast<int>(P.B.terms.size()) - O.term0;
-                        P.B.flops += 2.0 * O.rows * O.cols * O.nterm;
-                        P.B.outs.push_back(O);
-                    }
-                    t2 += static_cast<int64_t>(M) * CL.width;
-                    c2[u * ngl + ga] = CL;
                 }
             // phase C: Lnew[u][Gb][lb rows, :] = sum_{la, s: la+q(s)=lb} A[la,s,lb]^T T2[u][Ga(la)][la rows, s cols]
             for (int u = 0; u < dwr; ++u)
@@ -603,34 +714,33 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
                         T.N = ldn;
                         T.ldc = ldn;
                         T.seg0 = static_cast<int>(P.C.segs.size());
-                        for (size_t la = 0; la < bl.labels.size(); ++la)
-                            for (int s = 0; s < 4; ++s) {
-                                if (al.seg_label[la * 4 + s] != lb) continue;
-                                const Label& La = bl.labels[la];
-                                const int ga = La.group;
-                                const int64_t s2 = o2[u * ngl + ga];
-                                if (s2 < 0) continue;
-                                const ColLayout& C2 = c2[u * ngl + ga];
-                                if (C2.col[s] < 0) continue;
-                                GemmSeg sg{};
-                                sg.a = handle(0, al.row_off[la] + al.seg_col[la * 4 + s]);
-                                sg.a_rs = 1;
-                                sg.a_cs = al.width[la];
-                                sg.K = La.dim;
-                                sg.b = handle(4, s2 + static_cast<int64_t>(La.off - bl.groups[ga].off) * C2.width + C2.col[s]);
-                                sg.b_rs = C2.width;
-                                sg.b_cs = 1;
-                                                                P.C.segs.push_back(sg);
-                                P.C.flops += 2.0 * T.M * T.N * sg.K;
-                            }
+                        for (const auto& ls : into[lb]) {
+                            const int la = ls.first, s = ls.second;
+                            const Label& La = bl.labels[la];
+                            const int ga = La.group;
+                            if (o2[u * ngl + ga] < 0) continue;
+                            const ColLayout& C2 = c2[u * ngl + ga];
+                            if (C2.col[s] < 0) continue;
+                            GemmSeg sg{};
+                            sg.a = handle(0, al.row_off[la] + al.seg_col[la * 4 + s]);
+                            sg.a_rs = 1;
+                            sg.a_cs = al.width[la];
+                            sg.K = La.dim;
+                            sg.b = handle(4, o2[u * ngl + ga] + g * s2 +
+                                                 static_cast<int64_t>(La.off - bl.groups[ga].off) * C2.width + C2.col[s]);
+                            sg.b_rs = C2.width;
+                            sg.b_cs = 1;
+                            P.C.segs.push_back(sg);
+                            P.C.flops += 2.0 * T.M * T.N * sg.K;
+                        }
                         T.nseg = static_cast<int>(P.C.segs.size()) - T.seg0;
                         P.C.tasks.push_back(T);
                     }
                 }
         }
     }
+    P.zero_t1 = P.chan.zero_t1;
     P.tileA_rng[nops * G] = static_cast<int>(P.A.tasks.size());
-    P.combB_rng[nops * G] = static_cast<int>(P.B.outs.size());
     P.tileC_rng[nops * G] = static_cast<int>(P.C.tasks.size());
     P.t1_size = t1;
     P.t2_size = t2;
@@ -649,32 +759,75 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
     P.task_rng_kept = false;
     P.tileA_rng.assign(nops * G + 1, 0);
     P.tileC_rng.assign(nops * G + 1, 0);
-    P.combB_rng.assign(nops * G + 1, 0);
+    P.flopsB_rng.clear();
     int64_t t1 = 0, t2 = 0;
+    P.chan.clear();
     for (int op = 0; op < nops; ++op) {
         const MPO& m = h->ops.mpo[op];
         const int dwl = m.dw[i], dwr = m.dw[i + 1];
         const std::vector<int>& cnl = m.cn[i];
         const std::vector<int>& cnr = m.cn[i + 1];
+        // blocks of T1[u][Gb] and T2[w][Gb] for beta point 0
+        std::vector<int64_t> o1(static_cast<size_t>(dwr) * ngr, -1), o2(static_cast<size_t>(dwl) * ngr, -1);
+        std::vector<ColLayout> c1(o1.size()), c2(o2.size());
+        const int64_t t1_op = t1, t2_op = t2;
+        for (int u = 0; u < dwr; ++u)
+            for (int gb = 0; gb < ngr; ++gb) {
+                const int n0 = br.groups[gb].n - cnr[u];
+                if (br.group_of(n0) < 0 || Ro.lay[op].off[u * ngr + gb] < 0) continue;
+                ColLayout CL = make_col_layout(bl, n0, 4, -1);
+                if (CL.width == 0) continue;
+                o1[u * ngr + gb] = t1;
+                t1 += static_cast<int64_t>(br.groups[gb].dim) * CL.width;
+                c1[u * ngr + gb] = std::move(CL);
+            }
+        for (int w = 0; w < dwl; ++w)
+            for (int gb = 0; gb < ngr; ++gb) {
+                ColLayout CL = make_col_layout(bl, br.groups[gb].n - cnl[w], 4, -1);
+                if (CL.width == 0) continue;
+                o2[w * ngr + gb] = t2;
+                t2 += static_cast<int64_t>(br.groups[gb].dim) * CL.width;
+                c2[w * ngr + gb] = std::move(CL);
+            }
+        const int64_t s1 = t1 - t1_op, s2 = t2 - t2_op;
+        t1 = t1_op + G * s1;
+        t2 = t2_op + G * s2;
+        // phase B: T2[w][Gb][:, s, :] = sum_{u,t} W[w,u,s,t] (r T1)[u][Gb][:, t, :]
+        P.chan.stride.t1[op] = s1;
+        P.chan.stride.t3[op] = s2;
+        const std::vector<std::vector<ChanEntry>> ent = site_entries(m, i, false);
+        CombSpec sp;
+        sp.op = op;
+        sp.legs = 1;
+        sp.sign = -1;
+        sp.row = &br;
+        sp.col = &bl;
+        sp.ket = &br;
+        sp.cn_in = &cnr;
+        sp.cn_out = &cnl;
+        sp.o1 = &o1;
+        sp.o2 = &o2;
+        sp.c1 = &c1;
+        sp.c2 = &c2;
+        sp.entries = &ent;
+        sp.needed = [&](int lb, int s) {
+            const int la = bl.find(br.labels[lb].n - kLocalN[s], br.labels[lb].tm - kLocal2M[s]);
+            return la >= 0 && al.seg_label[la * 4 + s] == lb;
+        };
+        const double fb = comb_add(P.chan, sp);
+        P.B.flops += G * fb;
         for (int g = 0; g < G; ++g) {
-            const MPO& W = h->ops.rot[op][g];
             const int og = op * G + g;
+            P.flopsB_rng.push_back(fb);
             P.tileA_rng[og] = static_cast<int>(P.A.tasks.size());
-            P.combB_rng[og] = static_cast<int>(P.B.outs.size());
             P.tileC_rng[og] = static_cast<int>(P.C.tasks.size());
             // phase A: T1[u][Gb][b, (t, a')] = sum_b' R[u][b, b'] A[a', t, b']
-            std::vector<int64_t> o1(static_cast<size_t>(dwr) * ngr, -1);
-            std::vector<ColLayout> c1(static_cast<size_t>(dwr) * ngr);
             for (int u = 0; u < dwr; ++u)
                 for (int gb = 0; gb < ngr; ++gb) {
-                    const int n0 = br.groups[gb].n - cnr[u];
-                    const int gbp = br.group_of(n0);
+                    if (o1[u * ngr + gb] < 0) continue;
+                    const int gbp = br.group_of(br.groups[gb].n - cnr[u]);
                     const int64_t roff = Ro.lay[op].off[u * ngr + gb];
-                    if (gbp < 0 || roff < 0) continue;
-                    ColLayout CL = make_col_layout(bl, n0, 4, -1);
-                    if (CL.width == 0) continue;
-                    const int M = br.groups[gb].dim;
-                    o1[u * ngr + gb] = t1;
+                    const ColLayout& CL = c1[u * ngr + gb];
                     for (int lbp = br.groups[gbp].first; lbp < br.groups[gbp].first + br.groups[gbp].count; ++lbp) {
                         const Label& Lbp = br.labels[lbp];
                         for (int t = 0; t < 4; ++t) {
@@ -682,9 +835,9 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                             if (lap < 0 || al.seg_label[lap * 4 + t] != lbp) continue;
                             const Label& Lap = bl.labels[lap];
                             GemmTask T{};
-                            T.c = handle(3, t1 + CL.col[t] + (Lap.off - bl.groups[Lap.group].off));
+                            T.c = handle(3, o1[u * ngr + gb] + g * s1 + CL.col[t] + (Lap.off - bl.groups[Lap.group].off));
                             T.cmap = -1;
-                            T.M = M;
+                            T.M = br.groups[gb].dim;
                             T.N = Lap.dim;
                             T.ldc = CL.width;
                             T.seg0 = static_cast<int>(P.A.segs.size());
@@ -697,54 +850,11 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                             sg.b = handle(0, al.row_off[lap] + al.seg_col[lap * 4 + t]);
                             sg.b_rs = 1;
                             sg.b_cs = al.width[lap];
-                                                        P.A.segs.push_back(sg);
+                            P.A.segs.push_back(sg);
                             P.A.tasks.push_back(T);
                             P.A.flops += 2.0 * T.M * T.N * sg.K;
                         }
                     }
-                    t1 += static_cast<int64_t>(M) * CL.width;
-                    c1[u * ngr + gb] = CL;
-                }
-            // phase B: T2[w][Gb][:, s, :] = sum_{u,t} W[w,u,s,t] T1[u][Gb][:, t, :]
-            std::vector<int64_t> o2(static_cast<size_t>(dwl) * ngr, -1);
-            std::vector<ColLayout> c2(static_cast<size_t>(dwl) * ngr);
-            for (int w = 0; w < dwl; ++w)
-                for (int gb = 0; gb < ngr; ++gb) {
-                    const int n0 = br.groups[gb].n - cnl[w];
-                    ColLayout CL = make_col_layout(bl, n0, 4, -1);
-                    if (CL.width == 0) continue;
-                    const int M = br.groups[gb].dim;
-                    o2[w * ngr + gb] = t2;
-                    for (int s = 0; s < 4; ++s) {
-                        if (CL.col[s] < 0) continue;
-                        CombOut O{};
-                        O.dst = handle(4, t2 + CL.col[s]);
-                        O.rows = M;
-                        O.cols = bl.groups[CL.group[s]].dim;
-                        O.ld = CL.width;
-                        O.term0 = static_cast<int>(P.B.terms.size());
-                        for (int q = W.wl_ptr[i][w]; q < W.wl_ptr[i][w + 1]; ++q) {
-                            const MpoEntry& e = W.E[i][W.by_wl[i][q]];
-                            const int u = e.wr;
-                            const int64_t s1 = o1[u * ngr + gb];
-                            if (s1 < 0) continue;
-                            const ColLayout& C1 = c1[u * ngr + gb];
-                            for (int t = 0; t < 4; ++t) {
-                                const double cf = e.op[s * 4 + t];
-                                if (cf == 0.0 || C1.col[t] < 0) continue;
-                                CombTerm tm{};
-                                tm.src = handle(3, s1 + C1.col[t]);
-                                tm.ld = C1.width;
-                                tm.coef = cf;
-                                P.B.terms.push_back(tm);
-                            }
-                        }
-                        O.nterm = static_cast<int>(P.B.terms.size()) - O.term0;
-                        P.B.flops += 2.0 * O.rows * O.cols * O.nterm;
-                        P.B.outs.push_back(O);
-                    }
-                    t2 += static_cast<int64_t>(M) * CL.width;
-                    c2[w * ngr + gb] = CL;
                 }
             // phase C: Rnew[w][Ga][la rows, :] = sum_s A[la, s, lb] T2[w][Gb(lb)][lb rows, s cols]
             for (int w = 0; w < dwl; ++w)
@@ -766,8 +876,7 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                             if (lb < 0) continue;
                             const Label& Lb = br.labels[lb];
                             const int gb = Lb.group;
-                            const int64_t s2 = o2[w * ngr + gb];
-                            if (s2 < 0) continue;
+                            if (o2[w * ngr + gb] < 0) continue;
                             const ColLayout& C2 = c2[w * ngr + gb];
                             if (C2.col[s] < 0) continue;
                             GemmSeg sg{};
@@ -775,10 +884,11 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                             sg.a_rs = al.width[la];
                             sg.a_cs = 1;
                             sg.K = Lb.dim;
-                            sg.b = handle(4, s2 + static_cast<int64_t>(Lb.off - br.groups[gb].off) * C2.width + C2.col[s]);
+                            sg.b = handle(4, o2[w * ngr + gb] + g * s2 +
+                                                 static_cast<int64_t>(Lb.off - br.groups[gb].off) * C2.width + C2.col[s]);
                             sg.b_rs = C2.width;
                             sg.b_cs = 1;
-                                                        P.C.segs.push_back(sg);
+                            P.C.segs.push_back(sg);
                             P.C.flops += 2.0 * T.M * T.N * sg.K;
                         }
                         T.nseg = static_cast<int>(P.C.segs.size()) - T.seg0;
@@ -787,8 +897,8 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                 }
         }
     }
+    P.zero_t1 = P.chan.zero_t1;
     P.tileA_rng[nops * G] = static_cast<int>(P.A.tasks.size());
-    P.combB_rng[nops * G] = static_cast<int>(P.B.outs.size());
     P.tileC_rng[nops * G] = static_cast<int>(P.C.tasks.size());
     P.t1_size = t1;
     P.t2_size = t2;
@@ -813,11 +923,9 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
     const int ngl = static_cast<int>(bl.groups.size()), ngr = static_cast<int>(br.groups.size());
     P.A.clear(); P.B.clear(); P.C.clear();
     P.task_rng_kept = false;
-    P.diag_blocks.clear();
-    P.diag_terms.clear();
     P.tileA_rng.assign(nops * G + 1, 0);
     P.tileC_rng.assign(nops * G + 1, 0);
-    P.combB_rng.assign(nops * G + 1, 0);
+    P.flopsB_rng.clear();
     for (double& f : P.flops_op) f = 0.0;
     std::vector<int> cmap_off(bl.labels.size(), -1);
     for (size_t l = 0; l < bl.labels.size(); ++l) {
@@ -832,97 +940,97 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
             for (int j = 0; j < Lb.dim; ++j) P.A.cmaps.push_back(base + j);
         }
     }
-    int64_t t1 = 0, t3 = 0, t1_op0 = 0, t3_op0 = 0;
-    std::vector<int64_t> t3_op_end(nops, 0), t3_op_begin(nops, 0);
-    // per (op, g): offsets of T3 blocks for the output phase, kept for all g
-    std::vector<std::vector<int64_t>> o3_all(static_cast<size_t>(nops) * G);
-    std::vector<std::vector<DiagPair>> diag_all(static_cast<size_t>(nops) * G);
-    std::vector<std::vector<ColLayout>> c3_all(static_cast<size_t>(nops) * G);
+    int64_t t1 = 0, t3 = 0;
+    P.chan.clear();
+    P.weighted = true;
+    // per op: T3 blocks of beta point 0, for the output phase
+    std::vector<std::vector<int64_t>> o3_op(nops);
+    std::vector<std::vector<ColLayout>> c3_op(nops);
     for (int op = 0; op < nops; ++op) {
         const MPO& m = h->ops.mpo[op];
         const int dwl = m.dw[k], dwr = m.dw[k + 2];
         const std::vector<int>& cnl = m.cn[k];
         const std::vector<int>& cnr = m.cn[k + 2];
-        t3_op_begin[op] = t3;
+        std::vector<int64_t> o1(static_cast<size_t>(dwl) * ngl, -1);
+        std::vector<int64_t>& o3 = o3_op[op];
+        std::vector<ColLayout>& c3 = c3_op[op];
+        o3.assign(static_cast<size_t>(dwr) * ngl, -1);
+        std::vector<ColLayout> c1(o1.size());
+        c3.resize(o3.size());
+        const int64_t t1_op = t1, t3_op = t3;
+        for (int w = 0; w < dwl; ++w)
+            for (int ga = 0; ga < ngl; ++ga) {
+                const int n0 = bl.groups[ga].n - cnl[w];
+                if (bl.group_of(n0) < 0 || Le.lay[op].off[w * ngl + ga] < 0) continue;
+                ColLayout CL = make_col_layout(br, n0, 16, +1);
+                if (CL.width == 0) continue;
+                o1[w * ngl + ga] = t1;
+                t1 += static_cast<int64_t>(bl.groups[ga].dim) * CL.width;
+                c1[w * ngl + ga] = std::move(CL);
+            }
+        for (int u = 0; u < dwr; ++u)
+            for (int ga = 0; ga < ngl; ++ga) {
+                ColLayout CL = make_col_layout(br, bl.groups[ga].n - cnr[u], 16, +1);
+                if (CL.width == 0) continue;
+                o3[u * ngl + ga] = t3;
+                t3 += static_cast<int64_t>(bl.groups[ga].dim) * CL.width;
+                c3[u * ngl + ga] = std::move(CL);
+            }
+        const int64_t s1 = t1 - t1_op, s3 = t3 - t3_op;
+        t1 = t1_op + G * s1;
+        t3 = t3_op + G * s3;
+        // phase B: T3[u][Ga][:, s, :] = sum_{w,t} WW[w,u,s,t] (r T1)[w][Ga][:, t, :]
+        P.chan.stride.t1[op] = s1;
+        P.chan.stride.t3[op] = s3;
+        const std::vector<std::vector<ChanEntry>> ent = pair_entries(m, k);
+        CombSpec sp;
+        sp.op = op;
+        sp.legs = 2;
+        sp.sign = 1;
+        sp.row = &bl;
+        sp.col = &br;
+        sp.ket = &bl;
+        sp.cn_in = &cnl;
+        sp.cn_out = &cnr;
+        sp.o1 = &o1;
+        sp.o2 = &o3;
+        sp.c1 = &c1;
+        sp.c2 = &c3;
+        sp.entries = &ent;
+        sp.needed = [&](int la, int s) { return xl.seg_label[la * 16 + s] >= 0; };
+        // T3 of the identity operator (one channel of charge 0), relative to its first block
+        std::vector<int64_t> n_o3(ngl, -1);
+        std::vector<ColLayout> n_c3(ngl);
+        if (op == 0 && nops == 2 && !screen && h->ops.mpo[1].dw[k] == 1 && h->ops.mpo[1].dw[k + 2] == 1)
+            sp.share = identity_channel(m, k);
+        if (sp.share >= 0) {
+            int64_t at = t3;  // operator 1's blocks follow operator 0's
+            for (int ga = 0; ga < ngl; ++ga) {
+                n_c3[ga] = make_col_layout(br, bl.groups[ga].n, 16, +1);
+                if (n_c3[ga].width == 0) continue;
+                n_o3[ga] = at;
+                at += static_cast<int64_t>(bl.groups[ga].dim) * n_c3[ga].width;
+            }
+            P.chan.stride.t3[1] = at - t3;
+            sp.share_o2 = &n_o3;
+            sp.share_c2 = &n_c3;
+        }
+        const double fb = comb_add(P.chan, sp);
+        P.B.flops += G * fb;
+        P.flopsB_op[op] += G * fb;
+        const double fa0 = P.A.flops;
         for (int g = 0; g < G; ++g) {
-            const MPO& W = h->ops.rot[op][g];
             const int og = op * G + g;
-            const double cgw = h->cg[g];
+            P.flopsB_rng.push_back(fb);
             P.tileA_rng[og] = static_cast<int>(P.A.tasks.size());
-            P.combB_rng[og] = static_cast<int>(P.B.outs.size());
-            const double fa0 = P.A.flops, fb0 = P.B.flops;
-            // WW[w][u][(s1 s2)][(t1 t2)] = c_g sum_v W_k[w,v,s1,t1] W_k+1[v,u,s2,t2], kept for the
-            // (w, u) pairs joined by some v; ww_u[u] lists (w, pair) ordered by w
-            std::unordered_map<uint64_t, int> ww_id;
-            std::vector<std::array<double, 256>> ww;
-            std::vector<std::vector<std::pair<int, int>>> ww_u(dwr);
-            for (const MpoEntry& a : W.E[k]) {
-                const int v = a.wr;
-                for (int q = W.wl_ptr[k + 1][v]; q < W.wl_ptr[k + 1][v + 1]; ++q) {
-                    const MpoEntry& b = W.E[k + 1][W.by_wl[k + 1][q]];
-                    const uint64_t key = (static_cast<uint64_t>(a.wl) << 32) | static_cast<uint32_t>(b.wr);
-                    auto it = ww_id.find(key);
-                    int id;
-                    if (it == ww_id.end()) {
-                        id = static_cast<int>(ww.size());
-                        ww_id.emplace(key, id);
-                        ww.emplace_back();
-                        ww.back().fill(0.0);
-                        ww_u[b.wr].push_back({a.wl, id});
-                    } else {
-                        id = it->second;
-                    }
-                    std::array<double, 256>& dst = ww[id];
-                    for (int s1 = 0; s1 < 4; ++s1)
-                        for (int t1i = 0; t1i < 4; ++t1i) {
-                            const double av = a.op[s1 * 4 + t1i];
-                            if (av == 0.0) continue;
-                            for (int s2 = 0; s2 < 4; ++s2)
-                                for (int t2i = 0; t2i < 4; ++t2i) {
-                                    const double bv = b.op[s2 * 4 + t2i];
-                                    if (bv == 0.0) continue;
-                                    dst[(s1 * 4 + s2) * 16 + (t1i * 4 + t2i)] += cgw * av * bv;
-                                }
-                        }
-                }
-            }
-            for (auto& lst : ww_u) std::sort(lst.begin(), lst.end());
-            // diagonal coefficients of the pairs between charge-0 channels, for the preconditioner
-            {
-                std::vector<DiagPair>& dp = diag_all[og];
-                dp.clear();
-                for (int u = 0; u < dwr; ++u) {
-                    if (cnr[u] != 0) continue;
-                    for (const auto& wp : ww_u[u]) {
-                        if (cnl[wp.first] != 0) continue;
-                        DiagPair d{};
-                        d.w = wp.first;
-                        d.u = u;
-                        bool any = false;
-                        for (int q = 0; q < 16; ++q) {
-                            d.c[q] = ww[wp.second][q * 16 + q];
-                            any = any || d.c[q] != 0.0;
-                        }
-                        if (any) dp.push_back(d);
-                    }
-                }
-                std::sort(dp.begin(), dp.end(), [](const DiagPair& a, const DiagPair& b) {
-                    return a.w != b.w ? a.w < b.w : a.u < b.u;
-                });
-            }
             // phase A
-            std::vector<int64_t> o1(static_cast<size_t>(dwl) * ngl, -1);
-            std::vector<ColLayout> c1(static_cast<size_t>(dwl) * ngl);
             for (int w = 0; w < dwl; ++w)
                 for (int ga = 0; ga < ngl; ++ga) {
-                    const int n0 = bl.groups[ga].n - cnl[w];
-                    const int gap = bl.group_of(n0);
+                    if (o1[w * ngl + ga] < 0) continue;
+                    const int gap = bl.group_of(bl.groups[ga].n - cnl[w]);
                     const int64_t loff = Le.lay[op].off[w * ngl + ga];
-                    if (gap < 0 || loff < 0) continue;
-                    ColLayout CL = make_col_layout(br, n0, 16, +1);
-                    if (CL.width == 0) continue;
-                    const int M = bl.groups[ga].dim;
-                    o1[w * ngl + ga] = t1;
+                    const int64_t t1_block = o1[w * ngl + ga] + g * s1;
+                    const int width = c1[w * ngl + ga].width;
                     const Group& Ga = bl.groups[ga];
                     for (int l = bl.groups[gap].first; l < bl.groups[gap].first + bl.groups[gap].count; ++l) {
                         if (xl.width[l] == 0) continue;
@@ -932,15 +1040,15 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
                         const int nsub = screen ? Ga.count : 1;
                         for (int q = 0; q < nsub; ++q) {
                             const int row0 = screen ? bl.labels[Ga.first + q].off - Ga.off : 0;
-                            const int rows = screen ? bl.labels[Ga.first + q].dim : M;
+                            const int rows = screen ? bl.labels[Ga.first + q].dim : Ga.dim;
                             if (screen && nL->dropped(op, g, w, ga, q, l - bl.groups[gap].first, tau)) continue;
                             GemmTask T{};
-                            T.c = handle(3, t1 + static_cast<int64_t>(row0) * CL.width);
+                            T.c = handle(3, t1_block + static_cast<int64_t>(row0) * width);
                             T.cmap = cmap_off[l];
                             T.M = rows;
                             T.N = xl.width[l];
                             T.key = static_cast<int>(l);  // all products of one ket label read x[l]
-                            T.ldc = CL.width;
+                            T.ldc = width;
                             T.seg0 = static_cast<int>(P.A.segs.size());
                             T.nseg = 1;
                             GemmSeg sg{};
@@ -957,62 +1065,15 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
                             P.A.flops += 2.0 * T.M * T.N * sg.K;
                         }
                     }
-                    t1 += static_cast<int64_t>(M) * CL.width;
-                    c1[w * ngl + ga] = CL;
                 }
-            // phase B: T3[u][Ga][:, s, :] = sum_{w,t} WW[w,u,s,t] T1[w][Ga][:, t, :]
-            std::vector<int64_t>& o3 = o3_all[og];
-            std::vector<ColLayout>& c3 = c3_all[og];
-            o3.assign(static_cast<size_t>(dwr) * ngl, -1);
-            c3.assign(static_cast<size_t>(dwr) * ngl, ColLayout{});
-            for (int u = 0; u < dwr; ++u)
-                for (int ga = 0; ga < ngl; ++ga) {
-                    const int n0 = bl.groups[ga].n - cnr[u];
-                    ColLayout CL = make_col_layout(br, n0, 16, +1);
-                    if (CL.width == 0) continue;
-                    const int M = bl.groups[ga].dim;
-                    o3[u * ngl + ga] = t3;
-                    for (int s = 0; s < 16; ++s) {
-                        if (CL.col[s] < 0) continue;
-                        CombOut O{};
-                        O.dst = handle(4, t3 + CL.col[s]);
-                        O.rows = M;
-                        O.cols = br.groups[CL.group[s]].dim;
-                        O.ld = CL.width;
-                        O.term0 = static_cast<int>(P.B.terms.size());
-                        for (const auto& wp : ww_u[u]) {
-                            const int w = wp.first;
-                            const int64_t s1 = o1[w * ngl + ga];
-                            if (s1 < 0) continue;
-                            const ColLayout& C1 = c1[w * ngl + ga];
-                            const std::array<double, 256>& cw = ww[wp.second];
-                            for (int t = 0; t < 16; ++t) {
-                                const double cf = cw[s * 16 + t];
-                                if (cf == 0.0 || C1.col[t] < 0) continue;
-                                CombTerm tm{};
-                                tm.src = handle(3, s1 + C1.col[t]);
-                                tm.ld = C1.width;
-                                tm.coef = cf;
-                                P.B.terms.push_back(tm);
-                            }
-                        }
-                        O.nterm = static_cast<int>(P.B.terms.size()) - O.term0;
-                        P.B.flops += 2.0 * O.rows * O.cols * O.nterm;
-                        P.B.outs.push_back(O);
-                    }
-                    t3 += static_cast<int64_t>(M) * CL.width;
-                    c3[u * ngl + ga] = CL;
-                }
-            P.flops_op[op] += (P.A.flops - fa0) + (P.B.flops - fb0);
-            P.flopsA_op[op] += P.A.flops - fa0;
-            P.flopsB_op[op] += P.B.flops - fb0;
         }
+        P.flopsA_op[op] += P.A.flops - fa0;
+        P.flops_op[op] += (P.A.flops - fa0) + G * fb;
         // algorithmic bytes of phase A for this op: its environment, x and T1, each once per g
-        P.bytesA_op[op] = 8.0 * (static_cast<double>(G) * (Le.lay[op].size + xl.size)) + 8.0 * static_cast<double>(t1 - t1_op0);
-        P.bytesB_op[op] = 8.0 * static_cast<double>((t1 - t1_op0) + (t3 - t3_op0));
-        t1_op0 = t1;
-        t3_op0 = t3;
+        P.bytesA_op[op] = 8.0 * (static_cast<double>(G) * (Le.lay[op].size + xl.size)) + 8.0 * static_cast<double>(G * s1);
+        P.bytesB_op[op] = 8.0 * static_cast<double>(G * (s1 + s3));
     }
+    P.zero_t1 = P.chan.zero_t1 || screen;  // screened products leave holes in T1
     // phase C: one task per (N, M)-allowed output block and beta point, writing the partial sum
     // over the channels u into the per-g slice of the partial buffer (slot 8 for y, 9 for z); a
     // deterministic reduction over g (launch_sum_partials) produces y and z
@@ -1041,9 +1102,9 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
                     T.ldc = xl.width[la];
                     T.seg0 = static_cast<int>(P.C.segs.size());
                     for (int u = 0; u < dwr; ++u) {
-                        const int64_t s3 = o3_all[og][u * ngl + ga];
-                        if (s3 < 0) continue;
-                        const ColLayout& C3 = c3_all[og][u * ngl + ga];
+                        if (o3_op[op][u * ngl + ga] < 0) continue;
+                        const int64_t s3 = o3_op[op][u * ngl + ga] + g * P.chan.stride.t3[op];
+                        const ColLayout& C3 = c3_op[op][u * ngl + ga];
                         if (C3.col[s] < 0) continue;
                         const int64_t roff = Re.lay[op].off[u * ngr + gb];
                         if (roff < 0) continue;
@@ -1078,19 +1139,56 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
         P.flops_op[op] += P.C.flops - fc0;
         P.flopsC_op[op] += P.C.flops - fc0;
         // phase C reads this op's T3 and right environment and writes G partial outputs
-        const int64_t t3_op = (op + 1 < nops ? t3_op_begin[op + 1] : t3) - t3_op_begin[op];
-        P.bytesC_op[op] = 8.0 * (static_cast<double>(t3_op) + static_cast<double>(G) * (Re.lay[op].size + nx));
+        P.bytesC_op[op] = 8.0 * static_cast<double>(G) * (P.chan.stride.t3[op] + Re.lay[op].size + nx);
     }
     P.reduce_nx = nx;
     P.tileA_rng[nops * G] = static_cast<int>(P.A.tasks.size());
-    P.combB_rng[nops * G] = static_cast<int>(P.B.outs.size());
     P.tileC_rng[nops * G] = static_cast<int>(P.C.tasks.size());
     P.t1_size = t1;
     P.t2_size = t3;
     P.flops = P.A.flops + P.B.flops + P.C.flops;
+}
 
-    // diagonal of the projected operators on the x layout: for each output block and beta point,
-    // the pairs (w, u) of charge-0 channels with a nonzero diagonal WW coefficient
+// Diagonal of the projected operators on the x layout, built by the first solve at the site: for each
+// output block and beta point, the pairs (w, u) of charge-0 channels with a nonzero diagonal coefficient
+// c_g (WW (r x r))[s, s].
+void build_diag(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re, Plan& P) {
+    const Bond& bl = h->bonds[k];
+    const Bond& br = h->bonds[k + 2];
+    const RowBlockLayout xl = make_row_block_layout(bl, br, 16);
+    const int G = h->G, nops = h->ops.n_ops();
+    const int ngl = static_cast<int>(bl.groups.size()), ngr = static_cast<int>(br.groups.size());
+    P.diag_blocks.clear();
+    P.diag_terms.clear();
+    std::vector<std::vector<DiagPair>> diag_all(static_cast<size_t>(nops) * G);
+    for (int op = 0; op < nops; ++op) {
+        const MPO& m = h->ops.mpo[op];
+        const std::vector<int>& cnl = m.cn[k];
+        const std::vector<int>& cnr = m.cn[k + 2];
+        const std::vector<std::vector<ChanEntry>> ent = pair_entries(m, k);
+        for (int g = 0; g < G; ++g) {
+            double r[16];
+            site_rotation(h->beta[g], r);
+            std::vector<DiagPair>& dp = diag_all[op * G + g];
+            for (int u = 0; u < m.dw[k + 2]; ++u) {
+                if (cnr[u] != 0) continue;
+                for (size_t q = 0; q < ent[u].size();) {
+                    const int w = ent[u][q].w;
+                    DiagPair d{};
+                    d.w = w;
+                    d.u = u;
+                    for (; q < ent[u].size() && ent[u][q].w == w; ++q) {
+                        const ChanEntry& e = ent[u][q];
+                        d.c[e.s] += h->cg[g] * e.coef * r[(e.t >> 2) * 4 + (e.s >> 2)] * r[(e.t & 3) * 4 + (e.s & 3)];
+                    }
+                    bool any = false;
+                    for (double c : d.c) any = any || c != 0.0;
+                    if (any && cnl[w] == 0) dp.push_back(d);
+                }
+            }
+            std::sort(dp.begin(), dp.end(), [](const DiagPair& x, const DiagPair& y) { return x.w != y.w ? x.w < y.w : x.u < y.u; });
+        }
+    }
     for (int op = 0; op < nops; ++op) {
         for (size_t la = 0; la < bl.labels.size(); ++la) {
             const Label& La = bl.labels[la];
@@ -1151,7 +1249,7 @@ spmps_status update_left(spmps_t* h, int i) {
         sz[5] = Lo.total;
         sz[7] = Ln.total;
         std::string why;
-        if (!validate_plan(P, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (left update): " + why);
+        if (!validate_plan(P, sz, &why, h->G)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (left update): " + why);
     }
     st = plan_upload(h, P);
     if (st != SPMPS_OK) return st;
@@ -1185,7 +1283,7 @@ spmps_status update_right(spmps_t* h, int i) {
         sz[6] = Ro.total;
         sz[7] = Rn.total;
         std::string why;
-        if (!validate_plan(P, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (right update): " + why);
+        if (!validate_plan(P, sz, &why, h->G)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (right update): " + why);
     }
     st = plan_upload(h, P);
     if (st != SPMPS_OK) return st;
@@ -1328,7 +1426,7 @@ spmps_status get_apply_plan(spmps_t* h, int k, Plan** out) {
             sz[6] = h->Renv[k + 2].total;
             sz[8] = sz[9] = static_cast<int64_t>(h->G) * nx;
             std::string why;
-            if (!validate_plan(*P, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (apply): " + why);
+            if (!validate_plan(*P, sz, &why, h->G)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (apply): " + why);
         }
         if (h->opt.autotune) {
             st = tune_apply_plan(h, k, *P);
@@ -1340,6 +1438,22 @@ spmps_status get_apply_plan(spmps_t* h, int k, Plan** out) {
         h->apply_plans[k] = std::move(P);
     }
     *out = h->apply_plans[k].get();
+    return SPMPS_OK;
+}
+
+spmps_status ensure_diag(spmps_t* h, int k, Plan& P) {
+    if (P.diag_ready) return SPMPS_OK;
+    build_diag(h, k, h->Lenv[k], h->Renv[k + 2], P);
+    int64_t sz[kMaxSlots];
+    for (auto& v : sz) v = -1;
+    sz[5] = h->Lenv[k].total;
+    sz[6] = h->Renv[k + 2].total;
+    std::string why;
+    if (!validate_diag(P, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (diagonal): " + why);
+    CK(upload(P.d_diag_blocks, P.diag_blocks, h->stream));
+    CK(upload(P.d_diag_terms, P.diag_terms, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    P.diag_ready = true;
     return SPMPS_OK;
 }
 
@@ -1444,13 +1558,6 @@ spmps_status build_opset(spmps_t* h, const MPO& Hin, OpSet* out) {
     out->mpo.clear();
     out->mpo.push_back(H);
     out->mpo.push_back(I);
-    out->rot.assign(2, {});
-    for (int op = 0; op < 2; ++op)
-        for (int g = 0; g < h->G; ++g) {
-            MPO r = mpo_rotated(out->mpo[op], h->beta[g]);
-            r.cn = out->mpo[op].cn;
-            out->rot[op].push_back(r);
-        }
     return SPMPS_OK;
 }
 
@@ -1546,6 +1653,16 @@ spmps_status spmps_create(int K, int N, int twoM, int twoS, int n_beta, int D, c
     h->Lenv.resize(K + 1);
     h->Renv.resize(K + 1);
     h->apply_plans.resize(K);
+    std::vector<double> rot;
+    for (double b : h->beta) {
+        rot.push_back(std::tan(0.25 * b));
+        rot.push_back(std::sin(0.5 * b));
+    }
+    if (upload(h->d_rot, rot, h->stream) != cudaSuccess || upload(h->d_cg, h->cg, h->stream) != cudaSuccess ||
+        cudaStreamSynchronize(h->stream) != cudaSuccess) {
+        delete h;
+        return fail(nullptr, SPMPS_ERR_OOM, "workspace");
+    }
     if (h->partial.ensure(kPartialDoubles * sizeof(double)) != cudaSuccess) {
         delete h;
         return fail(nullptr, SPMPS_ERR_OOM, "workspace");

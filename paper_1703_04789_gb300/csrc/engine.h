@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/spmps.h"
+#include "comb.h"
 #include "core.h"
 #include "kernels.h"
 #include "mlp.h"
@@ -58,8 +59,7 @@ EnvLayout make_env_layout(const Bond& b, const std::vector<int>& cn);
 // A set of operators sharing the environment machinery: H and the projector norm (identity)
 // for the energy; S^2 for its expectation value.
 struct OpSet {
-    std::vector<MPO> mpo;                  // per op, unrotated
-    std::vector<std::vector<MPO>> rot;     // [op][g], rotation on the ket leg
+    std::vector<MPO> mpo;                  // per op, unrotated (the plans rotate T1 instead)
     int n_ops() const { return static_cast<int>(mpo.size()); }
 };
 
@@ -97,7 +97,8 @@ struct EnvNorms {
 // A three-phase contraction plan (GEMM, MPO-leg combination, GEMM), uploaded to the device.
 struct Plan {
     GemmPlan A, C;
-    CombPlan B;
+    CombPlan B;     // explicit terms per beta point (the cross plans of excited states)
+    CombChan chan;  // phase B on unrotated operators (the plans of H and N)
     TilePolicy polA, polC;  // tile policies of phases A and C (autotuned per site, or the default)
     std::vector<int> tileA_rng, tileC_rng, combB_rng;  // [op * G + g] .. [op * G + g + 1]
     // the builders write task ranges into tileA_rng / tileC_rng; the first upload keeps them here
@@ -107,11 +108,15 @@ struct Plan {
     std::vector<double> flopsA_rng, flopsB_rng, flopsC_rng;  // algorithmic flops per range
     int64_t t1_size = 0, t2_size = 0;
     int64_t reduce_nx = 0;  // > 0: phase C writes per-beta partials of this length (slots 8, 9)
+    bool zero_t1 = true;    // T1 starts at zero (else phase B skips what phase A does not write)
+    bool weighted = false;  // the partials are summed with the weights c_g (else with 1)
     double flops = 0.0;
     double flops_op[4] = {0, 0, 0, 0};
     double bytesA_op[4] = {0, 0, 0, 0}, bytesB_op[4] = {0, 0, 0, 0}, bytesC_op[4] = {0, 0, 0, 0};
     double flopsA_op[4] = {0, 0, 0, 0}, flopsB_op[4] = {0, 0, 0, 0}, flopsC_op[4] = {0, 0, 0, 0};
     DevMem d_tasksA, d_segsA, d_tilesA, d_cmapsA, d_outsB, d_termsB, d_tasksC, d_segsC, d_tilesC, d_cmapsC;
+    DevMem d_chan[9];                        // the arrays of chan
+    CombDev chan_dev{};
     DevMem d_tcA, d_tcC;                     // tensor-core tile lists
     std::vector<int> tcA_rng, tcC_rng;       // their ranges per (op, g)
     TcPlan stA, stC;                         // tcgen05 stacks of the H part, phases A and C
@@ -121,6 +126,7 @@ struct Plan {
     // diagonal (apply plans only)
     std::vector<DiagBlock> diag_blocks;
     std::vector<DiagTerm> diag_terms;
+    bool diag_ready = false;  // built by the first solve at the site
     DevMem d_diag_blocks, d_diag_terms;
     bool ready = false;
     // environment versions the plan was built for (screened plans depend on their values)
@@ -188,6 +194,7 @@ struct spmps_t {
     std::vector<spmps::EnvStore> Lenv, Renv;  // per bond
     std::vector<std::unique_ptr<spmps::Plan>> apply_plans;  // per site
     spmps::DevMem work1, work2, work3, partial;
+    spmps::DevMem d_rot, d_cg;  // per beta point tan(beta / 4), sin(beta / 2); the weights c_g
     spmps::DevMem xbuf, ybuf, zbuf;  // host-API staging
     MlpState mlp;
     int apply_precision = 0;  // precision of the H part of projected actions issued now (0 = FP64)
@@ -219,7 +226,7 @@ cudaError_t upload(DevMem& m, const std::vector<T>& v, cudaStream_t st) {
     return cudaMemcpyAsync(m.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st);
 }
 
-bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why);
+bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why, int G = 1);
 bool validate_gemm(const GemmPlan& G, const int64_t* sizes, std::string* why);
 spmps_status plan_upload(spmps_t* h, Plan& P);
 spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t st, cudaEvent_t* ev = nullptr,
@@ -237,6 +244,7 @@ spmps_status update_right(spmps_t* h, int i);
 spmps_status ensure_envs(spmps_t* h, int k);
 void invalidate_all(spmps_t* h);
 spmps_status get_apply_plan(spmps_t* h, int k, Plan** out);
+spmps_status ensure_diag(spmps_t* h, int k, Plan& P);
 spmps_status do_apply(spmps_t* h, int k, const double* x, double* y, double* z, cudaStream_t st,
                       cudaEvent_t* ev = nullptr);
 spmps_status check_ready(spmps_t* h);

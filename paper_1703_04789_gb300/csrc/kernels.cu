@@ -171,12 +171,16 @@ __global__ void __launch_bounds__(128) k_gemm_f64(Slots S, const GemmTask* __res
 }
 
 // ---- beta reduction of the output partials ------------------------------------------------------
-__global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__ partial, int G, int64_t n,
-                                                      double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__ p0, const double* __restrict__ p1,
+                                                      const double* __restrict__ w, int G, int64_t n,
+                                                      double* __restrict__ out0, double* __restrict__ out1) {
+    const double* __restrict__ partial = blockIdx.y == 0 ? p0 : p1;
+    double* __restrict__ out = blockIdx.y == 0 ? out0 : out1;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         double acc = 0.0;
-        for (int g = 0; g < G; ++g) acc += partial[g * n + i];
+#pragma unroll 4
+        for (int g = 0; g < G; ++g) acc = fma(w ? __ldg(w + g) : 1.0, partial[g * n + i], acc);
         out[i] = acc;
     }
 }
@@ -860,9 +864,12 @@ cudaError_t launch_gemm_f64(const Slots& slots, const GemmTask* tasks, const Gem
     return cudaGetLastError();
 }
 
-cudaError_t launch_sum_partials(const double* partial, int G, int64_t n, double* out, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_sum_partials<<<grid_for(n, 256, 4096), 256, 0, st>>>(partial, G, n, out);
+cudaError_t launch_sum_partials(const double* partial0, const double* partial1, const double* w, int G, int64_t n,
+                                double* out0, double* out1, cudaStream_t st) {
+    if (n <= 0 || (!out0 && !out1)) return cudaSuccess;
+    const bool both = out0 && out1;
+    k_sum_partials<<<dim3(grid_for(n, 256, 4096), both ? 2 : 1), 256, 0, st>>>(out0 ? partial0 : partial1, partial1, w, G, n,
+                                                                             out0 ? out0 : out1, out1);
     return cudaGetLastError();
 }
 

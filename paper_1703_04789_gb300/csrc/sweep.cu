@@ -188,6 +188,8 @@ spmps_status davidson_stage(spmps_t* h, int k, const double* x0, DavBuffers& B, 
     st = get_apply_plan(h, k, &P);
     if (st != SPMPS_OK) return st;
     // diagonal of H_eff and N_eff for the preconditioner
+    st = ensure_diag(h, k, *P);
+    if (st != SPMPS_OK) return st;
     {
         Slots S{};
         S.p[5] = h->Lenv[k].buf.as<double>();
