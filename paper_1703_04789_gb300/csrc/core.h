@@ -175,6 +175,17 @@ struct TilePolicy {
 constexpr int kTileCandidates = 6;
 TilePolicy tile_candidate(int i);  // i = 0 is the default policy
 
+// Warp-block extents of an M x N output with at most `elems` (<= 256) outputs per warp: the even split of
+// both sides, parts of at most 32, that leaves the fewest lanes idle (a block's outputs are flattened over
+// the 32 lanes).
+struct BlockSplit {
+    int pm, pn;  // parts along M and N
+};
+BlockSplit split_block(int M, int N, int elems);
+// Outputs per warp for a launch of so many: at most `elems`, fewer (down to one per lane) where that would
+// leave sub-partitions of the chip without a warp.
+int fill_elems(int64_t outputs, int elems);
+
 struct GemmPlan {
     std::vector<GemmTask> tasks;
     std::vector<GemmSeg> segs;

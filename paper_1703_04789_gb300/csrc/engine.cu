@@ -326,6 +326,17 @@ spmps_status plan_upload(spmps_t* h, Plan& P) {
             P.ozA.ok = P.ozC.ok = false;
         }
     }
+    // phase C of an action on the FP64 pipe: stacked by right label
+    P.f64C.clear();
+    if (P.reduce_nx > 0 && !h->opt.fp64_tensor_cores && c_task_rng.size() > 1 &&
+        build_tc_plan(P.C, c_task_rng, static_cast<int>(c_task_rng.size()) - 1, 32, P.f64C)) {
+        stack_units(P.f64C, std::min(256, P.polC.wb_elems));
+        CK(upload(P.d_f64C[0], P.f64C.stacks, h->stream));
+        CK(upload(P.d_f64C[1], P.f64C.rows, h->stream));
+        CK(upload(P.d_f64C[2], P.f64C.segs, h->stream));
+        CK(upload(P.d_f64C[3], P.f64C.atab, h->stream));
+        CK(upload(P.d_f64C[4], P.f64C.units, h->stream));
+    }
     CK(h->work1.ensure(std::max<int64_t>(1, P.t1_size) * sizeof(double)));
     CK(h->work2.ensure(std::max<int64_t>(1, P.t2_size) * sizeof(double)));
     CK(cudaStreamSynchronize(h->stream));
@@ -371,6 +382,16 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
                                                       d[3].as<uint64_t>(), cmaps.as<int>(), d[4].as<int4>(),
                                                       OZ.unit_rng[lo], OZ.unit_rng[hi], h->tc_err.as<int>(),
                                                       h->opt.tc_wait_polls, st);
+                if (rec >= 0) prof_end(h, st, rec);
+                return e2;
+            }
+            if (!tf && &tasks == &P.d_tasksC && P.f64C.ok) {
+                ++h->launches;
+                const int rec = h->profile ? prof_begin(h, st, 0, range_flops(fl, lo, hi)) : -1;
+                const DevMem* d = P.d_f64C;
+                const cudaError_t e2 = launch_gemm_f64_stack(S, d[0].as<TcStack>(), d[1].as<TcRow>(), d[2].as<TcSeg>(),
+                                                             d[3].as<uint64_t>(), cmaps.as<int>(), d[4].as<int4>(),
+                                                             P.f64C.unit_rng[lo], P.f64C.unit_rng[hi], st);
                 if (rec >= 0) prof_end(h, st, rec);
                 return e2;
             }
@@ -489,7 +510,7 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
     }
     if (P.reduce_nx > 0) {
         // outputs of op: y (slot 1) from the partials in slot 8, z (slot 2) from slot 9
-        CK(launch_sum_partials(S.p[8], S.p[9], P.weighted ? h->d_cg.as<double>() : nullptr, G, P.reduce_nx,
+        CK(launch_sum_partials(S.p[8], S.p[9], P.weighted ? h->d_cg.as<double>() : nullptr, G, P.slices[0], P.slices[1], P.reduce_nx,
                                r0 < G ? S.p[1] : nullptr, r1 > G ? S.p[2] : nullptr, st));
         ++h->launches;
     }
@@ -911,6 +932,49 @@ struct DiagPair {
     double c[16];
 };
 
+// How many slices phase C's channel sum is divided into, per op.  An output block's reduction runs over all
+// channels of the right environment; where the blocks of all beta points are too few for the chip (a small
+// bond dimension, or hundreds of channels of an active-space Hamiltonian) to fill it once (tensor cores:
+// two CTAs of 128 x 32 outputs per SM; FP64 pipe: four warps of 256 outputs per SM sub-partition), the
+// channels are divided so that they fill it twice, each share with at least two K stages (64).  Measured
+// (GB300), phase C: K = 20, D = 100 (60 CTAs undivided) 2.7 ms, 8.1 ms undivided; K = 10, D = 61 on the
+// tensor cores 0.67 ms, 1.14 ms undivided.  With more than one wave there already, dividing costs more than it balances
+// (L = 24, D = 256, 392 CTAs per op: 456 us an action with two slices, 426 us with one).
+void choose_slices(spmps_t* h, int k, const RowBlockLayout& xl, const EnvStore& Re, int64_t t1, int64_t t3, Plan& P) {
+    const Bond& bl = h->bonds[k];
+    const Bond& br = h->bonds[k + 2];
+    const int nops = h->ops.n_ops(), G = h->G;
+    const int ngr = static_cast<int>(br.groups.size());
+    std::vector<int64_t> rows(br.labels.size(), 0);
+    int64_t warps = 0, units = 0;
+    for (size_t la = 0; la < bl.labels.size(); ++la)
+        for (int s = 0; s < 16; ++s) {
+            const int lb = xl.seg_label[la * 16 + s];
+            if (lb < 0) continue;
+            rows[lb] += bl.labels[la].dim;
+            warps += (static_cast<int64_t>(bl.labels[la].dim) * br.labels[lb].dim + 255) / 256;
+        }
+    for (size_t lb = 0; lb < br.labels.size(); ++lb) units += (rows[lb] + 127) / 128 * ((br.labels[lb].dim + 31) / 32);
+    for (int op = 0; op < nops && op < 2; ++op) {
+        const bool tc = h->opt.fp64_tensor_cores || (op == 0 && h->opt.precision > 0);
+        const int64_t have = std::max<int64_t>(1, G * (tc ? units : warps)), wave = tc ? 304 : 4 * 608;
+        // mean reduction length of an output block: channels times the width of a ket group
+        double elements = 0.0, rows_gb = 0.0;
+        for (int u = 0; u < h->ops.mpo[op].dw[k + 2]; ++u)
+            for (int gb = 0; gb < ngr; ++gb)
+                if (Re.lay[op].off[u * ngr + gb] >= 0) elements += static_cast<double>(br.groups[gb].dim) * Re.lay[op].ld[u * ngr + gb];
+        for (int gb = 0; gb < ngr; ++gb) rows_gb += br.groups[gb].dim;
+        const int64_t most = static_cast<int64_t>(elements / std::max(1.0, rows_gb) / 64.0);
+        P.slices[op] = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({have >= wave ? 1 : (2 * wave + have - 1) / have, most, 32,
+                                                                               static_cast<int64_t>(h->ops.mpo[op].dw[k + 2])})));
+    }
+    // an action that the fixed scratch of spmps_apply_heff_noalloc holds with one slice keeps fitting it
+    const int64_t part = G * xl.size;
+    while (P.slices[0] + P.slices[1] > 2 && noalloc_need(t1, t3, 2 * part) <= kNoAllocScratchDoubles - 64 &&
+           noalloc_need(t1, t3, (P.slices[0] + P.slices[1]) * part) > kNoAllocScratchDoubles - 64)
+        --P.slices[P.slices[0] > 1 ? 0 : 1];
+}
+
 // ---- the projected action plan ---------------------------------------------------------------
 // Slots: 0 = x, 1 = y, 2 = z, 3 = T1, 4 = T3, 5 = L(bond k), 6 = R(bond k+2).
 void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re, Plan& P, const EnvNorms* nL,
@@ -1074,17 +1138,36 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
         P.bytesB_op[op] = 8.0 * static_cast<double>(G * (s1 + s3));
     }
     P.zero_t1 = P.chan.zero_t1 || screen;  // screened products leave holes in T1
-    // phase C: one task per (N, M)-allowed output block and beta point, writing the partial sum
-    // over the channels u into the per-g slice of the partial buffer (slot 8 for y, 9 for z); a
-    // deterministic reduction over g (launch_sum_partials) produces y and z
+    // phase C: one task per (N, M)-allowed output block, beta point and slice of the channels u, writing
+    // its partial sum (slot 8 for y, 9 for z); a deterministic reduction (launch_sum_partials) produces
+    // y and z
     const int64_t nx = xl.size;
+    choose_slices(h, k, xl, Re, t1, t3, P);
+    const int nlab = static_cast<int>(br.labels.size());
     for (int op = 0; op < nops; ++op) {
         const MPO& m = h->ops.mpo[op];
-        const int dwr = m.dw[k + 2];
+        const int dwr = m.dw[k + 2], ks = P.slices[op];
         const double fc0 = P.C.flops;
+        // channels [u_of[q], u_of[q + 1]) to slice q: equal shares of the environment's elements
+        std::vector<int> u_of(ks + 1, dwr);
+        u_of[0] = 0;
+        {
+            std::vector<double> upto(dwr + 1, 0.0);
+            for (int u = 0; u < dwr; ++u) {
+                double n = 0.0;
+                for (int gb = 0; gb < ngr; ++gb)
+                    if (Re.lay[op].off[u * ngr + gb] >= 0) n += static_cast<double>(br.groups[gb].dim) * Re.lay[op].ld[u * ngr + gb];
+                upto[u + 1] = upto[u] + n;
+            }
+            for (int q = 1, u = 0; q < ks; ++q) {
+                while (u < dwr && upto[u] < upto[dwr] * q / ks) ++u;
+                u_of[q] = u;
+            }
+        }
         for (int g = 0; g < G; ++g) {
             const int og = op * G + g;
             P.tileC_rng[og] = static_cast<int>(P.C.tasks.size());
+            for (int slice = 0; slice < ks; ++slice)
             for (size_t la = 0; la < bl.labels.size(); ++la) {
                 const Label& La = bl.labels[la];
                 const int ga = La.group;
@@ -1094,14 +1177,14 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
                     const Label& Lb = br.labels[lb];
                     const int gb = Lb.group;
                     GemmTask T{};
-                    T.c = handle(8 + op, static_cast<int64_t>(g) * nx + xl.row_off[la] + xl.seg_col[la * 16 + s]);
+                    T.c = handle(8 + op, static_cast<int64_t>(g * ks + slice) * nx + xl.row_off[la] + xl.seg_col[la * 16 + s]);
                     T.cmap = -1;
                     T.M = La.dim;
                     T.N = Lb.dim;
-                    T.key = lb;  // all output blocks of one right label read its environment rows
+                    T.key = lb + nlab * slice;  // the output blocks of one right label read its environment rows
                     T.ldc = xl.width[la];
                     T.seg0 = static_cast<int>(P.C.segs.size());
-                    for (int u = 0; u < dwr; ++u) {
+                    for (int u = u_of[slice]; u < u_of[slice + 1]; ++u) {
                         if (o3_op[op][u * ngl + ga] < 0) continue;
                         const int64_t s3 = o3_op[op][u * ngl + ga] + g * P.chan.stride.t3[op];
                         const ColLayout& C3 = c3_op[op][u * ngl + ga];
@@ -1351,7 +1434,7 @@ spmps_status tune_apply_plan(spmps_t* h, int k, Plan& P) {
         const int64_t nx = std::max<int64_t>(1, P.reduce_nx);
         CK(h->tunebuf.ensure(3 * nx * sizeof(double)));
         CK(cudaMemsetAsync(h->tunebuf.p, 0, 3 * nx * sizeof(double), h->stream));
-        CK(h->work3.ensure(std::max<int64_t>(1, 2 * static_cast<int64_t>(h->G) * P.reduce_nx) * sizeof(double)));
+        CK(h->work3.ensure(std::max<int64_t>(1, P.partial_size(h->G)) * sizeof(double)));
         cudaEvent_t ev[5];
         for (auto& e : ev) CK(cudaEventCreate(&e));
         float best_a = INFINITY, best_c = INFINITY;
@@ -1370,7 +1453,7 @@ spmps_status tune_apply_plan(spmps_t* h, int k, Plan& P) {
             S.p[5] = h->Lenv[k].buf.as<double>();
             S.p[6] = h->Renv[k + 2].buf.as<double>();
             S.p[8] = h->work3.as<double>();
-            S.p[9] = h->work3.as<double>() + static_cast<int64_t>(h->G) * P.reduce_nx;
+            S.p[9] = h->work3.as<double>() + static_cast<int64_t>(P.slices[0]) * h->G * P.reduce_nx;
             float ta = 0.0f, tc = 0.0f;
             for (int rep = 0; rep < 3 && st == SPMPS_OK; ++rep) {
                 st = plan_run(h, P, S, 0, 2 * h->G, h->stream, ev);
@@ -1424,7 +1507,8 @@ spmps_status get_apply_plan(spmps_t* h, int k, Plan** out) {
             sz[4] = P->t2_size;
             sz[5] = h->Lenv[k].total;
             sz[6] = h->Renv[k + 2].total;
-            sz[8] = sz[9] = static_cast<int64_t>(h->G) * nx;
+            sz[8] = static_cast<int64_t>(P->slices[0]) * h->G * nx;
+            sz[9] = static_cast<int64_t>(P->slices[1]) * h->G * nx;
             std::string why;
             if (!validate_plan(*P, sz, &why, h->G)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (apply): " + why);
         }
@@ -1434,7 +1518,7 @@ spmps_status get_apply_plan(spmps_t* h, int k, Plan** out) {
         }
         st = plan_upload(h, *P);
         if (st != SPMPS_OK) return st;
-        CK(h->work3.ensure(std::max<int64_t>(1, 2 * static_cast<int64_t>(h->G) * P->reduce_nx) * sizeof(double)));
+        CK(h->work3.ensure(std::max<int64_t>(1, P->partial_size(h->G)) * sizeof(double)));
         h->apply_plans[k] = std::move(P);
     }
     *out = h->apply_plans[k].get();
@@ -1471,7 +1555,7 @@ spmps_status do_apply(spmps_t* h, int k, const double* x, double* y, double* z, 
     S.p[5] = h->Lenv[k].buf.as<double>();
     S.p[6] = h->Renv[k + 2].buf.as<double>();
     S.p[8] = h->work3.as<double>();
-    S.p[9] = h->work3.as<double>() + static_cast<int64_t>(h->G) * P->reduce_nx;
+    S.p[9] = h->work3.as<double>() + static_cast<int64_t>(P->slices[0]) * h->G * P->reduce_nx;
     const int G = h->G;
     SlotsF SF{};
     const SlotsF* split = nullptr;

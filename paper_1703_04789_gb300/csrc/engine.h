@@ -46,6 +46,10 @@ struct DevMem {
     template <class T> T* as() const { return static_cast<T*>(p); }
 };
 
+// Doubles of the fixed scratch of spmps_apply_heff_noalloc (32 MiB), and what an action needs of it.
+constexpr int64_t kNoAllocScratchDoubles = static_cast<int64_t>(4) << 20;
+constexpr int64_t noalloc_need(int64_t t1, int64_t t2, int64_t partials) { return t1 + t2 + partials + 64; }
+
 // Per-op layout of one environment tensor on one bond: block (w, G) of gdim(G) x gdim(G')
 // with G' the group of n(G) - cn[w]; -1 where absent.
 struct EnvLayout {
@@ -109,6 +113,8 @@ struct Plan {
     int64_t t1_size = 0, t2_size = 0;
     int64_t reduce_nx = 0;  // > 0: phase C writes per-beta partials of this length (slots 8, 9)
     bool zero_t1 = true;    // T1 starts at zero (else phase B skips what phase A does not write)
+    int slices[2] = {1, 1}; // per op: partials per beta point (phase C's channels are divided over them)
+    int64_t partial_size(int G) const { return static_cast<int64_t>(slices[0] + slices[1]) * G * reduce_nx; }
     bool weighted = false;  // the partials are summed with the weights c_g (else with 1)
     double flops = 0.0;
     double flops_op[4] = {0, 0, 0, 0};
@@ -122,6 +128,8 @@ struct Plan {
     TcPlan stA, stC;                         // tcgen05 stacks of the H part, phases A and C
     DevMem d_stA[5], d_stC[5];               // their stacks, rows, segments, A table, units
     TcPlan ozA, ozC;                         // stacks of all (op, g) ranges for the FP64-accurate
+    TcPlan f64C;                             // stacks of phase C on the FP64 pipe (actions only)
+    DevMem d_f64C[5];
     DevMem d_ozA[5], d_ozC[5];               // split-product GEMM (fp64_tensor_cores)
     // diagonal (apply plans only)
     std::vector<DiagBlock> diag_blocks;

@@ -5,6 +5,7 @@
 // sin(beta) d^S_MM(beta); Eq. pmpo evaluates it with Gauss-Legendre points in x = cos(beta).
 // The rotation of one site is the 4x4 matrix of Eq. expSy.
 #include <algorithm>
+#include <map>
 #include <cmath>
 #include <cstring>
 
@@ -106,31 +107,76 @@ TilePolicy tile_candidate(int i) {
     return p;
 }
 
+BlockSplit split_block(int M, int N, int elems) {
+    BlockSplit best{1, 1};
+    double best_cost = -1.0;
+    for (int pm = (M + 31) / 32; pm <= M; ++pm) {
+        const int tm = (M + pm - 1) / pm;
+        int pn = (N + 31) / 32;
+        while (tm * ((N + pn - 1) / pn) > elems && pn < N) ++pn;
+        const int tn = (N + pn - 1) / pn;
+        if (tm * tn <= elems || (tm == 1 && tn == 1)) {
+            // lanes of every tile (parts of a side differ by at most one) plus the staging of its operands
+            const int m_hi = M - (tm - 1) * pm, n_hi = N - (tn - 1) * pn;  // parts of the full extent
+            double cost = 0.0;
+            for (int i = 0; i < 2; ++i)
+                for (int j = 0; j < 2; ++j) {
+                    const int cnt = (i ? pm - m_hi : m_hi) * (j ? pn - n_hi : n_hi);
+                    const int em = tm - i, en = tn - j;
+                    if (cnt > 0 && em > 0 && en > 0) cost += cnt * (32.0 * ((em * en + 31) / 32) + em + en);
+                }
+            if (best_cost < 0.0 || cost < best_cost) {
+                best_cost = cost;
+                best = {pm, pn};
+            }
+        }
+        if (tm == 1) break;
+    }
+    return best;
+}
+
+// Warps that keep the chip's FP64 pipes busy: four per SM sub-partition of 152 SMs.
+constexpr int64_t kFillWarps = 4 * 4 * 152;
+
+// An FMA of a warp takes the FP64 pipe of its sub-partition for 64 clocks, so a launch of few outputs is
+// spread over as many warps as the chip holds rather than 256 outputs to a warp.  Measured (L = 8, D = 32
+// action, phase C with its sum): 37 us with 256 outputs to a warp, 22 us spread.
+int fill_elems(int64_t outputs, int elems) {
+    return static_cast<int>(std::min<int64_t>(std::min(elems, 256), std::max<int64_t>(32, (outputs / kFillWarps + 31) / 32 * 32)));
+}
+
 void GemmPlan::add_tiles(const TilePolicy& pol) {
-    // register-tiled shapes 0..4 (rows x cols per warp); shape 5 = warp block for long reductions
+    // register-tiled shapes 0..4 (rows x cols per warp); shape 5 = warp block
     static const int shp[5][2] = {{16, 16}, {4, 64}, {64, 4}, {32, 8}, {8, 32}};
     tiles.clear();
+    int64_t outputs = 0;
+    for (const GemmTask& T : tasks) outputs += static_cast<int64_t>(T.M) * T.N;
+    const int elems = fill_elems(outputs, pol.wb_elems);
+    const bool small = outputs < 128 * kFillWarps;
+    std::map<std::pair<int, int>, BlockSplit> splits;
     for (size_t t = 0; t < tasks.size(); ++t) {
         const GemmTask& T = tasks[t];
         int64_t ktot = 0;
         for (int q = 0; q < T.nseg; ++q) ktot += segs[T.seg0 + q].K;
-        if (ktot >= pol.wb_kmin && static_cast<int64_t>(T.M) * T.N <= pol.wb_mn_max) {
-            const int tm = T.M < 32 ? T.M : 32;
-            int tn = (pol.wb_elems < 256 ? pol.wb_elems : 256) / tm;  // the kernel holds <= 256 outputs
-            if (tn < 1) tn = 1;
-            if (tn > 32) tn = 32;
-            if (tn > T.N) tn = T.N;
-            for (int m0 = 0; m0 < T.M; m0 += tm)
-                for (int n0 = 0; n0 < T.N; n0 += tn) {
+        if (small || (ktot >= pol.wb_kmin && static_cast<int64_t>(T.M) * T.N <= pol.wb_mn_max)) {
+            BlockSplit& sp = splits.emplace(std::make_pair(T.M, T.N), BlockSplit{0, 0}).first->second;
+            if (sp.pm == 0) sp = split_block(T.M, T.N, elems);
+            for (int i = 0, m0 = 0; i < sp.pm; ++i) {
+                const int tm = T.M / sp.pm + (i < T.M % sp.pm ? 1 : 0);
+                for (int j = 0, n0 = 0; j < sp.pn; ++j) {
+                    const int tn = T.N / sp.pn + (j < T.N % sp.pn ? 1 : 0);
                     GemmTile g{};
                     g.task = static_cast<int>(t);
                     g.m0 = static_cast<int16_t>(m0);
                     g.n0 = static_cast<int16_t>(n0);
-                    g.tm = static_cast<int16_t>(T.M - m0 < tm ? T.M - m0 : tm);
-                    g.tn = static_cast<int16_t>(T.N - n0 < tn ? T.N - n0 : tn);
+                    g.tm = static_cast<int16_t>(tm);
+                    g.tn = static_cast<int16_t>(tn);
                     g.shape = 5;
                     tiles.push_back(g);
+                    n0 += tn;
                 }
+                m0 += tm;
+            }
             continue;
         }
         int best = 0;

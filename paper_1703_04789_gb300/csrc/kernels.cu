@@ -8,6 +8,7 @@
 #include <cmath>
 
 #include "kernels.h"
+#include "tc_gemm.h"
 
 namespace spmps {
 
@@ -15,6 +16,11 @@ namespace {
 
 __device__ __forceinline__ double* resolve(const Slots& S, uint64_t h) {
     return S.p[h >> 56] + static_cast<int64_t>(h & 0x00FFFFFFFFFFFFFFull);
+}
+
+__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src));
 }
 
 // ---- grouped FP64 GEMM ----------------------------------------------------------------------
@@ -77,20 +83,20 @@ __device__ __forceinline__ void gemm_tile(const Slots& S, const GemmTask& T, con
 }
 
 // Warp-block tile (shape 5): one warp computes a whole tm x tn output block (tm, tn <= 32,
-// tm * tn <= 256) of a task with a long reduction.  K is staged in chunks of 16 through the
-// warp's shared-memory slice with coalesced loads (two rows of 16 k per warp load), then every lane accumulates
-// its flattened outputs o = lane + 32 q (q < NQ) from shared memory, so the operand rows are read
-// once per block and no FMA is spent on padding beyond the last partial row of 32 outputs.
-constexpr int kWbK = 16;                    // K chunk
+// tm * tn <= 256).  K is staged in chunks of 8 through the warp's two shared-memory slices by asynchronous
+// copies (four rows of 8 k per warp step), the next chunk (of the same or the next segment) in flight while
+// every lane accumulates its flattened outputs o = lane + 32 q (q < NQ) from the current one, so the
+// operand rows are read once per block and no FMA is spent on padding beyond the last partial row of 32
+// outputs.
+constexpr int kWbK = 8;                     // K chunk
 constexpr int kWbStride = kWbK + 1;         // padded row stride of the staged chunks
-constexpr int kWbWarpSmem = 2 * 32 * kWbStride;  // doubles per warp (A rows and B rows)
+constexpr int kWbSlice = 2 * 32 * kWbStride;     // doubles of one stage (A rows and B rows)
+constexpr int kWbWarpSmem = 2 * kWbSlice;        // per warp
 
 template <int NQ>
 __device__ __forceinline__ void gemm_tile_wb(const Slots& S, const GemmTask& T, const GemmSeg* __restrict__ segs,
                                              const int* __restrict__ cmaps, int m0, int n0, int tm, int tn, int lane,
                                              double* __restrict__ sm) {
-    double* As = sm;
-    double* Bs = sm + 32 * kWbStride;
     const int nout = tm * tn;
     double v[NQ];
     int oa[NQ], ob[NQ];
@@ -100,29 +106,61 @@ __device__ __forceinline__ void gemm_tile_wb(const Slots& S, const GemmTask& T, 
         const int o = lane + 32 * q;
         const int oo = o < nout ? o : 0;
         oa[q] = (oo / tn) * kWbStride;
-        ob[q] = (oo % tn) * kWbStride;
+        ob[q] = (32 + oo % tn) * kWbStride;
     }
-    for (int sgi = 0; sgi < T.nseg; ++sgi) {
-        const GemmSeg sg = segs[T.seg0 + sgi];
-        const double* __restrict__ A = resolve(S, sg.a) + static_cast<int64_t>(m0) * sg.a_rs;
-        const double* __restrict__ B = resolve(S, sg.b) + static_cast<int64_t>(n0) * sg.b_cs;
-        const int kl = lane & 15, rl = lane >> 4;
-        for (int k0 = 0; k0 < sg.K; k0 += kWbK) {
-            const int kc = min(kWbK, sg.K - k0);
-            const bool kv = kl < kc;
-            const int64_t ka = static_cast<int64_t>(k0 + kl) * sg.a_cs;
-            const int64_t kb = static_cast<int64_t>(k0 + kl) * sg.b_rs;
-            for (int i = rl; i < tm; i += 2)
-                As[i * kWbStride + kl] = kv ? __ldg(A + static_cast<int64_t>(i) * sg.a_rs + ka) : 0.0;
-            for (int j = rl; j < tn; j += 2)
-                Bs[j * kWbStride + kl] = kv ? __ldg(B + kb + static_cast<int64_t>(j) * sg.b_cs) : 0.0;
+    const int kl = lane & (kWbK - 1), rl = lane >> 3;
+    GemmSeg sg{};
+    if (T.nseg > 0) sg = segs[T.seg0];
+    // chunk k0 of segment sg into slice buf
+    auto issue = [&](int k0, int buf) {
+        const double* A = resolve(S, sg.a) + static_cast<int64_t>(m0 + rl) * sg.a_rs + static_cast<int64_t>(k0 + kl) * sg.a_cs;
+        const double* B = resolve(S, sg.b) + static_cast<int64_t>(n0 + rl) * sg.b_cs + static_cast<int64_t>(k0 + kl) * sg.b_rs;
+        const bool kv = k0 + kl < sg.K;
+        double* As = sm + buf * kWbSlice + rl * kWbStride + kl;
+#pragma unroll 4
+        for (int i = 0; i < 8; ++i) {
+            if (rl + 4 * i < tm) {
+                if (kv)
+                    cp_async8(As + 4 * i * kWbStride, A + static_cast<int64_t>(4 * i) * sg.a_rs);
+                else
+                    As[4 * i * kWbStride] = 0.0;
+            }
+            if (rl + 4 * i < tn) {
+                double* Bs = As + 32 * kWbStride;
+                if (kv)
+                    cp_async8(Bs + 4 * i * kWbStride, B + static_cast<int64_t>(4 * i) * sg.b_cs);
+                else
+                    Bs[4 * i * kWbStride] = 0.0;
+            }
+        }
+    };
+    int sgi = 0, k0 = 0, kc = 0;  // kc: length of the chunk in flight
+    for (int t = 0;; ++t) {
+        int next = 0;
+        if (sgi < T.nseg) {
+            issue(k0, t & 1);
+            next = min(kWbK, sg.K - k0);
+            k0 += kWbK;
+            if (k0 >= sg.K) {
+                ++sgi;
+                k0 = 0;
+                if (sgi < T.nseg) sg = segs[T.seg0 + sgi];
+            }
+        }
+        asm volatile("cp.async.commit_group;");
+        if (t > 0) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
             __syncwarp();
+            const double* st = sm + ((t - 1) & 1) * kWbSlice;
+#pragma unroll 2
             for (int kk = 0; kk < kc; ++kk) {
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) v[q] = fma(As[oa[q] + kk], Bs[ob[q] + kk], v[q]);
+                for (int q = 0; q < NQ; ++q) v[q] = fma(st[oa[q] + kk], st[ob[q] + kk], v[q]);
             }
             __syncwarp();
         }
+        if (next == 0) break;
+        kc = next;
     }
     double* C = resolve(S, T.c);
     const int* cm = T.cmap >= 0 ? cmaps + T.cmap : nullptr;
@@ -137,7 +175,7 @@ __device__ __forceinline__ void gemm_tile_wb(const Slots& S, const GemmTask& T, 
     }
 }
 
-__global__ void __launch_bounds__(128) k_gemm_f64(Slots S, const GemmTask* __restrict__ tasks,
+__global__ void __launch_bounds__(128, 5) k_gemm_f64(Slots S, const GemmTask* __restrict__ tasks,
                                                   const GemmSeg* __restrict__ segs, const GemmTile* __restrict__ tiles,
                                                   const int* __restrict__ cmaps, int n_tiles) {
     __shared__ double wb_smem[4 * kWbWarpSmem];
@@ -170,17 +208,139 @@ __global__ void __launch_bounds__(128) k_gemm_f64(Slots S, const GemmTask* __res
     }
 }
 
+// ---- stacked FP64 GEMM ------------------------------------------------------------------------
+// The stacks of tc_gemm.h on the FP64 pipe, for the long reductions of phase C: every output row of all
+// blocks that read the same rows of the right environment, so that a warp's tile (tm x tn outputs of a
+// stack, <= 256) is full although most blocks are only a few rows high.  The K segments (one per channel)
+// are walked as one reduction in chunks of 8: lane kl of a chunk keeps its own position (segment, k), so
+// no chunk is cut short at a segment's end.  Double-buffered asynchronous copies as in gemm_tile_wb.  Bound by
+// the FP64 pipe.  Measured (GB300, phase C of the middle action of the L = 24, D = 256
+// chain, 494 Mflop): 0.494 ms; one block at a time per warp took 0.647 ms (28 % of the lanes idle).
+template <int NQ>
+__device__ __forceinline__ void stack_tile(const Slots& S, const TcStack& st, const TcRow* __restrict__ rows,
+                                           const TcSeg* __restrict__ segs, const uint64_t* __restrict__ atab,
+                                           const int* __restrict__ cmaps, int m0, int n0, int tm, int tn, int lane,
+                                           double* __restrict__ sm) {
+    const int nout = tm * tn;
+    double v[NQ];
+    int oa[NQ], ob[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        v[q] = 0.0;
+        const int o = lane + 32 * q;
+        const int oo = o < nout ? o : 0;
+        oa[q] = (oo / tn) * kWbStride;
+        ob[q] = (32 + oo % tn) * kWbStride;
+    }
+    const int kl = lane & (kWbK - 1), rl = lane >> 3;
+    int s = -1, k = kl, K = 0;  // this lane's segment and position in it; past the end: s = nseg
+    const double* B = nullptr;
+    int64_t b_ks = 0, b_ns = 0;
+    int left = st.ktot;  // of the whole reduction
+    int kc = 0;
+    for (int t = 0;; ++t) {
+        if (left > 0) {
+            while (s < st.nseg && k >= K) {
+                k -= K;
+                if (++s < st.nseg) {
+                    const TcSeg sg = segs[st.seg0 + s];
+                    K = sg.K;
+                    b_ks = sg.b_ks;
+                    b_ns = sg.b_ns;
+                    B = resolve(S, sg.b);
+                }
+            }
+            const bool kv = s < st.nseg;
+            const uint64_t* at = atab + st.atab0 + static_cast<int64_t>(m0 + rl) * st.nseg + (kv ? s : 0);
+            const double* bp = kv ? B + static_cast<int64_t>(n0 + rl) * b_ns + k * b_ks : nullptr;
+            double* As = sm + (t & 1) * kWbSlice + rl * kWbStride + kl;
+#pragma unroll 4
+            for (int i = 0; i < 8; ++i) {
+                if (rl + 4 * i < tm) {
+                    const uint64_t h = kv ? __ldg(at + static_cast<int64_t>(4 * i) * st.nseg) : kNoOperand;
+                    if (h != kNoOperand)
+                        cp_async8(As + 4 * i * kWbStride, resolve(S, h) + k);
+                    else
+                        As[4 * i * kWbStride] = 0.0;
+                }
+                if (rl + 4 * i < tn) {
+                    double* Bs = As + 32 * kWbStride;
+                    if (kv)
+                        cp_async8(Bs + 4 * i * kWbStride, bp + 4 * i * b_ns);
+                    else
+                        Bs[4 * i * kWbStride] = 0.0;
+                }
+            }
+            k += kWbK;
+        }
+        asm volatile("cp.async.commit_group;");
+        if (t > 0) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+            const double* sc = sm + ((t - 1) & 1) * kWbSlice;
+#pragma unroll 2
+            for (int kk = 0; kk < kc; ++kk) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) v[q] = fma(sc[oa[q] + kk], sc[ob[q] + kk], v[q]);
+            }
+            __syncwarp();
+        }
+        if (left <= 0) break;
+        kc = min(kWbK, left);
+        left -= kWbK;
+    }
+    const int* cm = st.cmap >= 0 ? cmaps + st.cmap : nullptr;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const int o = lane + 32 * q;
+        if (o < nout) {
+            const int i = o / tn, n = n0 + o % tn;
+            resolve(S, rows[st.row0 + m0 + i].c)[cm ? cm[n] : n] = v[q];
+        }
+    }
+}
+
+__global__ void __launch_bounds__(128, 5) k_gemm_f64_stack(Slots S, const TcStack* __restrict__ stacks,
+                                                           const TcRow* __restrict__ rows, const TcSeg* __restrict__ segs,
+                                                           const uint64_t* __restrict__ atab, const int* __restrict__ cmaps,
+                                                           const int4* __restrict__ units, int n_units) {
+    __shared__ double smem[4 * kWbWarpSmem];
+    const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (u >= n_units) return;
+    const int4 U = units[u];
+    const TcStack st = stacks[U.x];
+    const int tm = U.w & 0xFFFF, tn = U.w >> 16;
+    double* sm = smem + (threadIdx.x >> 5) * kWbWarpSmem;
+    switch ((tm * tn + 31) / 32) {
+        case 1: stack_tile<1>(S, st, rows, segs, atab, cmaps, U.y, U.z, tm, tn, lane, sm); break;
+        case 2: stack_tile<2>(S, st, rows, segs, atab, cmaps, U.y, U.z, tm, tn, lane, sm); break;
+        case 3:
+        case 4: stack_tile<4>(S, st, rows, segs, atab, cmaps, U.y, U.z, tm, tn, lane, sm); break;
+        case 5:
+        case 6: stack_tile<6>(S, st, rows, segs, atab, cmaps, U.y, U.z, tm, tn, lane, sm); break;
+        case 7: stack_tile<7>(S, st, rows, segs, atab, cmaps, U.y, U.z, tm, tn, lane, sm); break;
+        default: stack_tile<8>(S, st, rows, segs, atab, cmaps, U.y, U.z, tm, tn, lane, sm); break;
+    }
+}
+
 // ---- beta reduction of the output partials ------------------------------------------------------
+// Partials of beta point g: ks consecutive slices of n values (the slices of the channels).
 __global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__ p0, const double* __restrict__ p1,
-                                                      const double* __restrict__ w, int G, int64_t n,
+                                                      const double* __restrict__ w, int G, int ks0, int ks1, int64_t n,
                                                       double* __restrict__ out0, double* __restrict__ out1) {
     const double* __restrict__ partial = blockIdx.y == 0 ? p0 : p1;
     double* __restrict__ out = blockIdx.y == 0 ? out0 : out1;
+    const int ks = blockIdx.y == 0 ? ks0 : ks1;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         double acc = 0.0;
+        for (int g = 0; g < G; ++g) {
+            const double* __restrict__ p = partial + static_cast<int64_t>(g) * ks * n + i;
+            double s = p[0];
 #pragma unroll 4
-        for (int g = 0; g < G; ++g) acc = fma(w ? __ldg(w + g) : 1.0, partial[g * n + i], acc);
+            for (int k = 1; k < ks; ++k) s += p[k * n];
+            acc = fma(w ? __ldg(w + g) : 1.0, s, acc);
+        }
         out[i] = acc;
     }
 }
@@ -864,12 +1024,22 @@ cudaError_t launch_gemm_f64(const Slots& slots, const GemmTask* tasks, const Gem
     return cudaGetLastError();
 }
 
-cudaError_t launch_sum_partials(const double* partial0, const double* partial1, const double* w, int G, int64_t n,
-                                double* out0, double* out1, cudaStream_t st) {
+cudaError_t launch_gemm_f64_stack(const Slots& slots, const TcStack* stacks, const TcRow* rows, const TcSeg* segs,
+                                  const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, cudaStream_t st) {
+    if (u1 <= u0) return cudaSuccess;
+    k_gemm_f64_stack<<<(u1 - u0 + 3) / 4, 128, 0, st>>>(slots, stacks, rows, segs, atab, cmaps, units + u0, u1 - u0);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sum_partials(const double* partial0, const double* partial1, const double* w, int G, int ks0, int ks1,
+                                int64_t n, double* out0, double* out1, cudaStream_t st) {
     if (n <= 0 || (!out0 && !out1)) return cudaSuccess;
     const bool both = out0 && out1;
-    k_sum_partials<<<dim3(grid_for(n, 256, 4096), both ? 2 : 1), 256, 0, st>>>(out0 ? partial0 : partial1, partial1, w, G, n,
-                                                                             out0 ? out0 : out1, out1);
+    const dim3 grid(grid_for(n, 256, 4096), both ? 2 : 1);
+    if (out0)
+        k_sum_partials<<<grid, 256, 0, st>>>(partial0, partial1, w, G, ks0, ks1, n, out0, out1);
+    else
+        k_sum_partials<<<grid, 256, 0, st>>>(partial1, partial1, w, G, ks1, ks1, n, out1, out1);
     return cudaGetLastError();
 }
 

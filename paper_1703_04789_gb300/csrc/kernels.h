@@ -12,10 +12,10 @@ namespace spmps {
 cudaError_t launch_gemm_f64(const Slots& slots, const GemmTask* tasks, const GemmSeg* segs,
                             const GemmTile* tiles, const int* cmaps, int n_tiles, cudaStream_t st);
 
-// out[i] = sum_{g < G} w[g] partial[g * n + i] (fixed order; w null: 1) for one or two outputs (a null
-// output is left out).
-cudaError_t launch_sum_partials(const double* partial0, const double* partial1, const double* w, int G, int64_t n,
-                                double* out0, double* out1, cudaStream_t st);
+// out[i] = sum_{g < G} w[g] sum_{k < ks} partial[(g * ks + k) * n + i] (fixed order; w null: 1) for one or
+// two outputs (a null output is left out).
+cudaError_t launch_sum_partials(const double* partial0, const double* partial1, const double* w, int G, int ks0, int ks1,
+                                int64_t n, double* out0, double* out1, cudaStream_t st);
 
 // Same task lists on the tensor cores (m16n8k8 TF32, FP32 accumulation, FP64 in and out);
 // split3 != 0 uses the 3xTF32 split (hi*hi + hi*lo + lo*hi).

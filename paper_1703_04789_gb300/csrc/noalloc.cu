@@ -33,7 +33,6 @@ using namespace spmps::eng;
 
 namespace {
 
-constexpr size_t kNoAllocScratchDoubles = static_cast<size_t>(4) << 20;  // 32 MiB of doubles
 constexpr int kMaxDevices = 64;
 
 __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles];
@@ -67,8 +66,7 @@ extern "C" spmps_status spmps_apply_heff_noalloc(spmps_handle h, int site, const
     if (!P || !P->ready || !h->Lenv[site].valid || !h->Renv[site + 2].valid)
         return fail(h, SPMPS_ERR_STATE,
                     "no contraction plan for this site: call spmps_apply_heff once for it first (that call allocates)");
-    const size_t need = static_cast<size_t>(P->t1_size) + static_cast<size_t>(P->t2_size) +
-                        2 * static_cast<size_t>(h->G) * static_cast<size_t>(P->reduce_nx) + 64;
+    const int64_t need = noalloc_need(P->t1_size, P->t2_size, P->partial_size(h->G));
     if (need > kNoAllocScratchDoubles)
         return fail(h, SPMPS_ERR_BAD_INPUT, "intermediates need " + std::to_string(need) +
                                                 " doubles, above the fixed scratch of " +
@@ -97,8 +95,8 @@ extern "C" spmps_status spmps_apply_heff_noalloc(spmps_handle h, int site, const
     S.p[3] = base;
     S.p[4] = base + ((P->t1_size + 31) / 32) * 32;
     S.p[8] = S.p[4] + ((P->t2_size + 31) / 32) * 32;
-    S.p[9] = S.p[8] + static_cast<int64_t>(h->G) * P->reduce_nx;
-    if (static_cast<size_t>(S.p[9] - base) + static_cast<size_t>(h->G) * P->reduce_nx > kNoAllocScratchDoubles)
+    S.p[9] = S.p[8] + static_cast<int64_t>(P->slices[0]) * h->G * P->reduce_nx;
+    if (S.p[8] - base + P->partial_size(h->G) > kNoAllocScratchDoubles)
         return fail(h, SPMPS_ERR_BAD_INPUT, "intermediates do not fit the fixed scratch");
     S.p[5] = h->Lenv[site].buf.as<double>();
     S.p[6] = h->Renv[site + 2].buf.as<double>();

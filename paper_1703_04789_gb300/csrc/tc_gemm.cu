@@ -44,6 +44,7 @@ bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ra
                 }
             }
             S.nseg = static_cast<int>(P.segs.size()) - S.seg0;
+            for (int q = 0; q < S.nseg; ++q) S.ktot += P.segs[S.seg0 + q].K;
             S.atab0 = static_cast<int64_t>(P.atab.size());
             for (int t : ts) {
                 const GemmTask& T = G.tasks[t];
@@ -67,6 +68,7 @@ bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ra
             S.nrows = static_cast<int>(P.rows.size()) - S.row0;
             const int si = static_cast<int>(P.stacks.size());
             P.stacks.push_back(S);
+            P.stack_range.push_back(r);
             for (int m0 = 0; m0 < S.nrows; m0 += 128)
                 for (int n0 = 0; n0 < S.N; n0 += nt) P.units.push_back(make_int4(si, m0, n0, 0));
         }
@@ -74,6 +76,33 @@ bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ra
     P.unit_rng[n_ranges] = static_cast<int>(P.units.size());
     P.ok = true;
     return true;
+}
+
+void stack_units(TcPlan& P, int elems) {
+    std::map<std::pair<int, int>, BlockSplit> splits;
+    P.units.clear();
+    int64_t outputs = 0;
+    for (const TcStack& st : P.stacks) outputs += static_cast<int64_t>(st.nrows) * st.N;
+    elems = fill_elems(outputs, elems);
+    size_t si = 0;
+    for (size_t r = 0; r + 1 < P.unit_rng.size(); ++r) {
+        P.unit_rng[r] = static_cast<int>(P.units.size());
+        for (; si < P.stacks.size() && P.stack_range[si] == static_cast<int>(r); ++si) {
+            const TcStack& st = P.stacks[si];
+            BlockSplit& sp = splits.emplace(std::make_pair(st.nrows, st.N), BlockSplit{0, 0}).first->second;
+            if (sp.pm == 0) sp = split_block(st.nrows, st.N, elems);
+            for (int i = 0, m0 = 0; i < sp.pm; ++i) {
+                const int tm = st.nrows / sp.pm + (i < st.nrows % sp.pm ? 1 : 0);
+                for (int j = 0, n0 = 0; j < sp.pn; ++j) {
+                    const int tn = st.N / sp.pn + (j < st.N % sp.pn ? 1 : 0);
+                    P.units.push_back(make_int4(static_cast<int>(si), m0, n0, tm | (tn << 16)));
+                    n0 += tn;
+                }
+                m0 += tm;
+            }
+        }
+    }
+    P.unit_rng.back() = static_cast<int>(P.units.size());
 }
 
 namespace {

@@ -23,6 +23,7 @@ struct TcStack {
     int row0, nrows;  // stacked rows rows[row0 .. row0 + nrows)
     int seg0, nseg;   // K segments segs[seg0 ..)
     int N;            // columns
+    int ktot;         // sum of the segments' K
     int cmap;         // column map offset into the plan's cmaps, -1 for identity
     int64_t atab0;    // A handles atab[atab0 + r * nseg + s] for stacked row r and segment s
 };
@@ -41,11 +42,12 @@ struct TcPlan {
     std::vector<TcSeg> segs;
     std::vector<uint64_t> atab;   // A(r, s, k) = A[atab + k], contiguous along K
     std::vector<int4> units;      // (stack, m0, n0, 0): one CTA each
+    std::vector<int> stack_range; // per stack: its range
     std::vector<int> unit_rng;    // per beta range: units [unit_rng[g], unit_rng[g + 1])
     int nt = 64;                  // columns per CTA tile (32, 64 or 128)
     bool ok = false;              // every task of the range could be stacked
     void clear() {
-        stacks.clear(); rows.clear(); segs.clear(); atab.clear(); units.clear(); unit_rng.clear();
+        stacks.clear(); stack_range.clear(); rows.clear(); segs.clear(); atab.clear(); units.clear(); unit_rng.clear();
         ok = false;
     }
 };
@@ -54,6 +56,12 @@ struct TcPlan {
 // nt = columns per CTA.  Returns false (and leaves P.ok false) when a task does not fit the stacked
 // form (A not contiguous along K).
 bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ranges, int nt, TcPlan& P);
+
+// Units of the FP64 pipe's kernel instead (one warp each: (stack, m0, n0, tm | tn << 16), tm tn <= elems):
+// the even split of every stack that leaves the fewest lanes idle.
+void stack_units(TcPlan& P, int elems);
+cudaError_t launch_gemm_f64_stack(const Slots& slots, const TcStack* stacks, const TcRow* rows, const TcSeg* segs,
+                                  const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, cudaStream_t st);
 
 // One launch over units [u0, u1): C = sum over segments of A B^T for every unit tile, with A and B
 // read from the pre-split (hi, lo) TF32 buffers; split3 != 0 accumulates hi*hi + hi*lo + lo*hi,
