@@ -425,6 +425,31 @@ __global__ void k_multidot_final(const double* __restrict__ partial, int nb, dou
     if (lane == 0) out[j] = acc;
 }
 
+// The same for two right-hand sides (blockIdx.z) in one launch each.
+__global__ void __launch_bounds__(256) k_multidot2_partial(const double* __restrict__ V, int64_t ldv,
+                                                           const double* __restrict__ x0, const double* __restrict__ x1,
+                                                           int64_t n, double* __restrict__ partial) {
+    __shared__ double sh[32];
+    const int j = blockIdx.y;
+    const double* v = V + j * ldv;
+    const double* x = blockIdx.z == 0 ? x0 : x1;
+    double acc = 0.0;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        acc = fma(v[i], x[i], acc);
+    acc = block_sum(acc, sh);
+    if (threadIdx.x == 0) partial[(blockIdx.z * gridDim.y + j) * kRedBlocks + blockIdx.x] = acc;
+}
+__global__ void k_multidot2_final(const double* __restrict__ partial, int nb, double* __restrict__ out0,
+                                  double* __restrict__ out1) {
+    const int j = blockIdx.x, lane = threadIdx.x;
+    const double* p = partial + (blockIdx.y * gridDim.x + j) * kRedBlocks;
+    double acc = 0.0;
+    for (int b = lane; b < nb; b += 32) acc += p[b];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) (blockIdx.y == 0 ? out0 : out1)[j] = acc;
+}
+
 __global__ void __launch_bounds__(256) k_gemv(const double* __restrict__ V, int64_t ldv, int m,
                                               const double* __restrict__ c, int64_t n, double* __restrict__ y,
                                               int sub) {
@@ -478,19 +503,113 @@ __global__ void __launch_bounds__(256) k_scale_inv_sqrt(double* __restrict__ x, 
         x[i] *= s;
 }
 
-__global__ void __launch_bounds__(256) k_residual_diag(const double* __restrict__ hx, const double* __restrict__ nx,
-                                                       const double* __restrict__ dh, const double* __restrict__ dn,
-                                                       const double* __restrict__ scal, double clamp, int64_t n,
-                                                       double* __restrict__ r, double* __restrict__ t) {
+// The vectors of one Davidson iteration in one pass over the bases: x = V c, H x = HV c, N x = NV c, the
+// residual r, its diagonal correction t (also into t2 where given) and block sums of |r|^2.  Bound by the
+// 3 m vectors it reads (L2 at the sizes of a chain).  Measured (GB300, L = 16, D = 64 step): the vector
+// kernels of an iteration take 39 us in 6 launches, 79 us in 14 launches and copies before.
+__global__ void __launch_bounds__(256) k_ritz_vectors(const double* __restrict__ V, const double* __restrict__ HV,
+                                                      const double* __restrict__ NV, int64_t n, int m,
+                                                      const double* __restrict__ coef, const double* __restrict__ dh,
+                                                      const double* __restrict__ dn, const double* __restrict__ scal,
+                                                      double clamp, double* __restrict__ x, double* __restrict__ hx,
+                                                      double* __restrict__ nx, double* __restrict__ r,
+                                                      double* __restrict__ t, double* __restrict__ t2,
+                                                      double* __restrict__ sums) {
+    __shared__ double cs[32], sh[32];
+    if (threadIdx.x < m) cs[threadIdx.x] = coef[threadIdx.x];
+    __syncthreads();
     const double theta = scal[0];
+    double rr = 0.0;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const double ri = hx[i] - theta * nx[i];
+        double a = 0.0, b = 0.0, c = 0.0;
+#pragma unroll 4
+        for (int j = 0; j < m; ++j) {
+            a = fma(V[j * n + i], cs[j], a);
+            b = fma(HV[j * n + i], cs[j], b);
+            c = fma(NV[j * n + i], cs[j], c);
+        }
+        x[i] = a;
+        hx[i] = b;
+        nx[i] = c;
+        const double ri = b - theta * c;
         r[i] = ri;
         double den = dh[i] - theta * dn[i];
         if (fabs(den) < clamp) den = den < 0.0 ? -clamp : clamp;
-        t[i] = -ri / den;
+        const double ti = -ri / den;
+        t[i] = ti;
+        if (t2) t2[i] = ti;
+        rr = fma(ri, ri, rr);
     }
+    rr = block_sum(rr, sh);
+    if (threadIdx.x == 0) sums[blockIdx.x] = rr;
+}
+
+// y -= V d with d_j the sum of the nb block sums of k_multidot_partial (same order as k_multidot_final);
+// block sums of |y|^2 where `sums` is given.
+__global__ void __launch_bounds__(256) k_project(const double* __restrict__ V, int64_t n, int m,
+                                                 const double* __restrict__ partial, int nb, double* __restrict__ y,
+                                                 double* __restrict__ sums) {
+    __shared__ double cs[32], sh[32];
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x >> 5; j < m; j += 8) {
+        double d = 0.0;
+        for (int b = lane; b < nb; b += 32) d += partial[j * kRedBlocks + b];
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+        if (lane == 0) cs[j] = d;
+    }
+    __syncthreads();
+    double yy = 0.0;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        double acc = 0.0;
+#pragma unroll 4
+        for (int j = 0; j < m; ++j) acc = fma(V[j * n + i], cs[j], acc);
+        const double v = y[i] - acc;
+        y[i] = v;
+        yy = fma(v, v, yy);
+    }
+    if (sums) {
+        yy = block_sum(yy, sh);
+        if (threadIdx.x == 0) sums[blockIdx.x] = yy;
+    }
+}
+
+// Sum of nb block sums by one warp, fixed order (valid in lane 0).
+__device__ __forceinline__ double sum_blocks(const double* __restrict__ s, int nb) {
+    double v = 0.0;
+    for (int b = threadIdx.x & 31; b < nb; b += 32) v += s[b];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// out[0] = sum of the block sums.
+__global__ void k_sum_blocks(const double* __restrict__ s, int nb, double* __restrict__ out) {
+    const double v = sum_blocks(s, nb);
+    if (threadIdx.x == 0) out[0] = v;
+}
+
+// y scaled to norm 1 by the block sums of |y|^2 (nyb of them), which also goes to yy; where rsums is
+// given, the sum of those goes to rr.
+__global__ void __launch_bounds__(256) k_normalise(double* __restrict__ y, int64_t n, const double* __restrict__ ysums,
+                                                   int nyb, const double* __restrict__ rsums, int nrb,
+                                                   double* __restrict__ yy, double* __restrict__ rr) {
+    __shared__ double sc;
+    if (threadIdx.x < 32) {
+        const double v = sum_blocks(ysums, nyb);
+        if (threadIdx.x == 0) {
+            sc = v > 1e-300 ? 1.0 / sqrt(v) : 0.0;
+            if (blockIdx.x == 0) *yy = v;
+        }
+    } else if (threadIdx.x < 64 && blockIdx.x == 0 && rsums) {
+        const double v = sum_blocks(rsums, nrb);
+        if (threadIdx.x == 32) *rr = v;
+    }
+    __syncthreads();
+    const double s = sc;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        y[i] *= s;
 }
 
 // out = v / (diag H - theta diag N), the denominator clamped as in k_residual_diag
@@ -526,93 +645,6 @@ __global__ void __launch_bounds__(256) k_xpby_ratio(double* __restrict__ p, cons
         p[i] = fma(b, p[i], r[i]);
 }
 
-// ---- one-warp cyclic Jacobi in FP32 --------------------------------------------------------------
-// Round-robin pairs, rows then columns, on one warp with warp-level synchronisation; A (n x n, row stride ld) symmetric, V receives the
-// rotations (eigenvectors as columns).  Used for the eigenbasis of the Ritz problem, whose lowest
-// pair is then refined in FP64.
-__device__ __forceinline__ float warp_sumf(float v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ void jacobi_warp_f32(float* A, float* V, int ld, int n, float* cs, int* pq) {
-    const int lane = threadIdx.x & 31;
-    for (int e = lane; e < n * n; e += 32) {
-        const int i = e / n, j = e - i * n;
-        V[i * ld + j] = i == j ? 1.0f : 0.0f;
-    }
-    __syncwarp();
-    if (n <= 1) return;
-    const int np = (n + 1) & ~1;
-    const int half = np / 2;
-    float off_prev = INFINITY;
-    for (int sweep = 0; sweep < 30; ++sweep) {
-        float off = 0.0f, tot = 0.0f;
-        for (int e = lane; e < n * n; e += 32) {
-            const int i = e / n, j = e - i * n;
-            const float v = A[i * ld + j];
-            tot += v * v;
-            if (i != j) off += v * v;
-        }
-        off = warp_sumf(off);
-        tot = warp_sumf(tot);
-        // off-diagonal below 3e-5 of the matrix (the FP64 refinement of the lowest pair reduces
-        // its error by about that factor per correction), or no longer decreasing
-        if (off <= 1e-9f * tot || off == 0.0f || (off <= 1e-6f * tot && off > 0.25f * off_prev)) break;
-        off_prev = off;
-        const float tiny = 1e-10f * sqrtf(tot);
-        for (int round = 0; round < np - 1; ++round) {
-            if (lane < half) {
-                auto player = [&](int k) { return k == 0 ? 0 : 1 + ((k - 1 + round) % (np - 1)); };
-                int p = player(lane), q = player(np - 1 - lane);
-                if (p > q) {
-                    const int t = p;
-                    p = q;
-                    q = t;
-                }
-                float c = 1.0f, s = 0.0f;
-                if (q < n && fabsf(A[p * ld + q]) > tiny) {
-                    const float apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
-                    const float theta = (aqq - app) / (2.0f * apq);
-                    const float t = (theta >= 0.0f ? 1.0f : -1.0f) / (fabsf(theta) + sqrtf(theta * theta + 1.0f));
-                    c = 1.0f / sqrtf(t * t + 1.0f);
-                    s = t * c;
-                } else {
-                    q = -1;
-                }
-                pq[2 * lane] = p;
-                pq[2 * lane + 1] = q;
-                cs[2 * lane] = c;
-                cs[2 * lane + 1] = s;
-            }
-            __syncwarp();
-            for (int e = lane; e < half * n; e += 32) {  // rows p, q
-                const int i = e / n, j = e - i * n;
-                const int p = pq[2 * i], q = pq[2 * i + 1];
-                if (q < 0) continue;
-                const float c = cs[2 * i], s = cs[2 * i + 1];
-                const float ap = A[p * ld + j], aq = A[q * ld + j];
-                A[p * ld + j] = c * ap - s * aq;
-                A[q * ld + j] = s * ap + c * aq;
-            }
-            __syncwarp();
-            for (int e = lane; e < half * n; e += 32) {  // columns p, q of A and V
-                const int i = e / n, j = e - i * n;
-                const int p = pq[2 * i], q = pq[2 * i + 1];
-                if (q < 0) continue;
-                const float c = cs[2 * i], s = cs[2 * i + 1];
-                const float ap = A[j * ld + p], aq = A[j * ld + q];
-                A[j * ld + p] = c * ap - s * aq;
-                A[j * ld + q] = s * ap + c * aq;
-                const float vp = V[j * ld + p], vq = V[j * ld + q];
-                V[j * ld + p] = c * vp - s * vq;
-                V[j * ld + q] = s * vp + c * vq;
-            }
-            __syncwarp();
-        }
-    }
-}
-
 constexpr int kRitzMax = 32;
 
 // ---- incremental Ritz step --------------------------------------------------------------------
@@ -621,96 +653,210 @@ constexpr int kRitzMax = 32;
 // Adding basis vector v_m: classical Gram-Schmidt of e_m against X in the n inner product,
 // twice; the direction is kept when its n-norm^2 exceeds eps * max(diag n) (numerically null
 // directions of the metric are dropped, as in canonical orthogonalisation).  hp grows by one row
-// and column; its eigenbasis is re-solved by one-warp FP32 Jacobi started from the previous
-// eigenvectors (so only the new coupling has to be rotated away), and the lowest pair is refined in
-// FP64 against hp (below).
+// and column; its eigenbasis is re-solved by FP32 Jacobi started from the previous eigenvectors (so only
+// the new coupling has to be rotated away), and the lowest pair is refined in FP64 against hp (below).
+//
+// One CTA of 16 warps, bound by latency: every FP64 instruction of a warp holds its sub-partition's FP64
+// pipe for 64 clocks.  The FP64 products of vectors of 32 run on four warps, one per sub-partition, each
+// taking a quarter of the sum; every thread of the CTA owns two elements of the FP32 matrices, so a Jacobi
+// round (the two rotations of an element's row and column, recomputed by each thread) is one barrier.
+// Measured (GB300, ncu, L = 16, D = 64 step, subspaces up to 20): 48 us; one warp took 93 us.
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-// Incremental Ritz step (one CTA of 128 threads: one warp per SM sub-partition for the
-// Gram-Schmidt and the products; the Jacobi sweeps and the FP64 refinement run on warp 0).
 constexpr double kMetricFloor = 1e-14;
+constexpr int kRitzThreads = 512;
+constexpr int kRitzLd = RitzState::kR + 1;
 
-__global__ void __launch_bounds__(128) k_ritz_inc(const double* __restrict__ h, const double* __restrict__ nm, int ldm,
-                                                  int m, int reset, double eps, RitzState* __restrict__ st,
-                                                  double* __restrict__ coef, double* __restrict__ scal) {
-    constexpr int R = RitzState::kR;
+// sum_l M[lane, l] v_l for l < n (v_l held by lane l; M[lane, l] = mat[lane * rs + l * cs]) on the four warps
+// of threads 0 .. 127, whose `slot` of shared memory (128 doubles) no warp may still be reading.
+__device__ __forceinline__ double matvec4(const double* mat, int rs, int cs, double v, int n, double* slot) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double acc = 0.0;
+    for (int l = w; l < n; l += 4) acc = fma(mat[lane * rs + l * cs], __shfl_sync(0xffffffffu, v, l), acc);
+    slot[w * 32 + lane] = acc;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    return (slot[lane] + slot[32 + lane]) + (slot[64 + lane] + slot[96 + lane]);
+}
+
+// Cyclic Jacobi (round-robin pairs) on the n x n symmetric matrix in a (row stride kRitzLd), the rotations
+// accumulated in v (the identity at first); a2, v2: second buffers.  Returns with the results in a and v.
+__device__ void jacobi_cta_f32(float*& a, float*& v, float*& a2, float*& v2, int n, float* red) {
+    const int tid = threadIdx.x, np = (n + 1) & ~1;
+    if (n <= 1) return;
+    // the two elements of this thread and the round-robin positions of their row and column
+    int ei[2], ej[2], ki[2], kj[2];
+    bool own[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int e = tid + q * kRitzThreads;
+        own[q] = e < n * n;
+        ei[q] = own[q] ? e / n : 0;
+        ej[q] = own[q] ? e - ei[q] * n : 0;
+    }
+    float off_prev = INFINITY;
+    for (int sweep = 0; sweep < 30; ++sweep) {
+        float off = 0.0f, tot = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            if (own[q]) {
+                const float x = a[ei[q] * kRitzLd + ej[q]];
+                tot = fmaf(x, x, tot);
+                if (ei[q] != ej[q]) off = fmaf(x, x, off);
+            }
+        for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        }
+        if ((tid & 31) == 0) {
+            red[tid >> 5] = off;
+            red[16 + (tid >> 5)] = tot;
+        }
+        __syncthreads();
+        off = tot = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kRitzThreads / 32; ++w) {
+            off += red[w];
+            tot += red[16 + w];
+        }
+        // off-diagonal below 3e-5 of the matrix (the FP64 refinement of the lowest pair reduces
+        // its error by about that factor per correction), or no longer decreasing
+        if (off <= 1e-9f * tot || off == 0.0f || (off <= 1e-6f * tot && off > 0.25f * off_prev)) break;
+        off_prev = off;
+        const float tiny = 1e-10f * sqrtf(tot);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            ki[q] = ei[q];
+            kj[q] = ej[q];
+        }
+        for (int round = 0; round < np - 1; ++round) {
+            // the player at position k plays the one at np - 1 - k; position 0 is player 0, positions
+            // 1 .. np - 1 move on by one player per round
+            auto opponent = [&](int k) {
+                const int o = np - 1 - k;
+                if (o == 0) return 0;
+                const int x = o - 1 + round;
+                return 1 + (x >= np - 1 ? x - (np - 1) : x);
+            };
+            // rotation of index i with p: its own factor, and the one of its opponent's entry
+            auto rotation = [&](int i, int p, float& c, float& s) {
+                c = 1.0f;
+                s = 0.0f;
+                if (p >= n || p == i) return;
+                const int lo = min(i, p), hi = max(i, p);
+                const float apq = a[lo * kRitzLd + hi];
+                if (!(fabsf(apq) > tiny)) return;
+                const float z = __fdividef(a[hi * kRitzLd + hi] - a[lo * kRitzLd + lo], 2.0f * apq);
+                const float t = copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f)));
+                c = rsqrtf(fmaf(t, t, 1.0f));
+                s = i == lo ? -t * c : t * c;
+            };
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (own[q]) {
+                    const int i = ei[q], j = ej[q];
+                    const int pi = opponent(ki[q]), pj = opponent(kj[q]);
+                    float ci, si, cj, sj;
+                    rotation(i, pi, ci, si);
+                    rotation(j, pj, cj, sj);
+                    const int ii = i * kRitzLd, pp = (pi < n ? pi : i) * kRitzLd, jj = pj < n ? pj : j;
+                    const float x = fmaf(sj, a[ii + jj], cj * a[ii + j]), y = fmaf(sj, a[pp + jj], cj * a[pp + j]);
+                    a2[ii + j] = fmaf(si, y, ci * x);
+                    v2[ii + j] = fmaf(sj, v[ii + jj], cj * v[ii + j]);
+                    ki[q] = ki[q] == 0 ? 0 : (ki[q] == 1 ? np - 1 : ki[q] - 1);
+                    kj[q] = kj[q] == 0 ? 0 : (kj[q] == 1 ? np - 1 : kj[q] - 1);
+                }
+            }
+            __syncthreads();
+            float* t = a;
+            a = a2;
+            a2 = t;
+            t = v;
+            v = v2;
+            v2 = t;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kRitzThreads) k_ritz_inc(const double* __restrict__ h, const double* __restrict__ nm,
+                                                           int ldm, int m, int reset, double eps,
+                                                           RitzState* __restrict__ st, double* __restrict__ coef,
+                                                           double* __restrict__ coef_prev, double* __restrict__ scal) {
+    constexpr int R = RitzState::kR, L = kRitzLd, MM = R * L;
     extern __shared__ double rs_smem[];
-    double* X = rs_smem;           // n-orthonormal coefficient basis, X[i + j*R]
-    double* HP = X + R * R;        // X^T h X
-    double* CC = HP + R * R;       // previous eigenvectors of HP (columns)
-    double* A = CC + R * R;
-    double* T = A + R * R;
-    double* NS = T + R * R;        // n, full symmetric, NS[i*R + j]
-    double* HS = NS + R * R;       // h, full symmetric
-    __shared__ double cs_sh[R + 2], red_sh[40];
-    __shared__ int pq_sh[R + 2];
+    double* X = rs_smem;      // n-orthonormal coefficient basis, X[i * L + j]
+    double* HP = X + MM;      // X^T h X
+    double* NS = HP + MM;     // n, full symmetric; later the eigenbasis in FP64
+    double* HS = NS + MM;     // h, full symmetric
+    float* Af = reinterpret_cast<float*>(HS + MM);
+    float* A2 = Af + MM;
+    float* Vf = A2 + MM;
+    float* V2 = Vf + MM;
+    float* W0 = V2 + MM;      // start basis
+    float* Hf = W0 + MM;      // X^T h X in FP32
+    __shared__ double slots[2][128];
+    __shared__ float red[32];
     __shared__ int k_sh;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
     int k = 0, m0 = 0, kc = 0;
     if (!reset) {
         k = st->k;
         m0 = st->m;
         kc = st->kc;
-        for (int e = tid; e < R * R; e += nt) {
-            X[e] = st->X[e];
-            HP[e] = st->hp[e];
-            CC[e] = st->C[e];
-        }
     }
-    for (int e = tid; e < m * m; e += nt) {
-        const int i = e / m, j = e - i * m;
+    for (int e = tid; e < R * R; e += kRitzThreads) {
+        const int i = e / R, j = e % R;
+        X[i * L + j] = reset ? 0.0 : st->X[i + j * R];
+        HP[i * L + j] = reset ? 0.0 : st->hp[e];
+        W0[i * L + j] = i < kc && j < kc ? st->C[e] : (i == j ? 1.0f : 0.0f);
+        const bool in = i < m && j < m;
         const int hi = i > j ? i : j, lo = i > j ? j : i;
-        NS[i * R + j] = nm[hi * ldm + lo];
-        HS[i * R + j] = h[hi * ldm + lo];
+        NS[i * L + j] = in ? nm[hi * ldm + lo] : 0.0;
+        HS[i * L + j] = in ? h[hi * ldm + lo] : 0.0;
     }
+    // the coefficients of the previous Ritz vector, kept for the restart
+    if (tid < R) coef_prev[tid] = coef[tid];
     __syncthreads();
-    // new columns of the n-orthonormal basis (32-long vectors: warp 0)
-    if (tid < 32) {
-        double dmax = 0.0;
-        for (int i = 0; i < m; ++i) dmax = fmax(dmax, NS[i * R + i]);
+    int turn = 0;
+    if (tid < 128) {  // four warps with the same values
+        auto mv = [&](const double* mat, int rs, int cs, double v, int n) {
+            turn ^= 1;
+            return matvec4(mat, rs, cs, v, n, slots[turn]);
+        };
+        double dmax = lane < m ? NS[lane * L + lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
         for (int col = m0; col < m; ++col) {
             // y = e_col - X (X^T n y), twice, in the n inner product (lane i holds y_i, i <= col)
-            double y = lane == col ? 1.0 : 0.0;
+            double y = lane == col ? 1.0 : 0.0, ny;
             for (int pass = 0; pass < 2; ++pass) {
-                double ny = 0.0;
-                for (int l = 0; l <= col; ++l) {
-                    const double yl = __shfl_sync(0xffffffffu, y, l);
-                    if (lane <= col) ny = fma(NS[lane * R + l], yl, ny);
-                }
-                double corr = 0.0;
-                for (int j = 0; j < k; ++j) {
-                    const double cj = warp_sum(lane <= col ? X[lane + j * R] * ny : 0.0);
-                    if (lane <= col) corr = fma(X[lane + j * R], cj, corr);
-                }
-                y -= corr;
+                ny = mv(NS, L, 1, y, col + 1);
+                if (lane > col) ny = 0.0;
+                const double c = mv(X, 1, L, ny, col + 1);  // lane j: X_j . n y
+                const double corr = mv(X, L, 1, c, k);
+                if (lane <= col) y -= corr;
             }
-            double ny = 0.0;
-            for (int l = 0; l <= col; ++l) {
-                const double yl = __shfl_sync(0xffffffffu, y, l);
-                if (lane <= col) ny = fma(NS[lane * R + l], yl, ny);
-            }
+            ny = mv(NS, L, 1, y, col + 1);
             const double nu2 = warp_sum(lane <= col ? y * ny : 0.0);
             // the basis vectors have unit norm and |N_eff| <= 1: below kMetricFloor the metric is
             // numerically zero (no state of the target spin is reachable), whatever eps says
             if (nu2 > eps * dmax && nu2 > kMetricFloor) {
-                const double inv = 1.0 / sqrt(nu2);
-                X[lane + k * R] = lane <= col ? y * inv : 0.0;
-                __syncwarp();
-                double hx = 0.0;
-                for (int l = 0; l <= col; ++l)
-                    if (lane <= col) hx = fma(HS[lane * R + l], X[l + k * R], hx);
-                for (int j = 0; j <= k; ++j) {
-                    const double v = warp_sum(lane <= col ? X[lane + j * R] * hx : 0.0);
-                    if (lane == 0) { HP[j * R + k] = v; HP[k * R + j] = v; }
+                const double xk = lane <= col ? y * (1.0 / sqrt(nu2)) : 0.0;
+                double hx = mv(HS, L, 1, xk, col + 1);
+                if (lane > col) hx = 0.0;
+                if (tid < 32) X[lane * L + k] = xk;
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                const double hk = mv(X, 1, L, hx, col + 1);  // lane j: X_j . h x_k
+                if (tid < 32 && lane <= k) {
+                    HP[lane * L + k] = hk;
+                    HP[k * L + lane] = hk;
                 }
                 ++k;
+                asm volatile("bar.sync 1, 128;" ::: "memory");
             }
-            __syncwarp();
         }
-        if (lane == 0) k_sh = k;
+        if (tid == 0) k_sh = k;
     }
     __syncthreads();
     k = k_sh;
@@ -718,55 +864,48 @@ __global__ void __launch_bounds__(128) k_ritz_inc(const double* __restrict__ h, 
     // identity (so only the new row and column have to be rotated away), gives the eigenbasis W of
     // HP to FP32 accuracy; the lowest pair is then refined in FP64 against HP itself: Rayleigh
     // quotient y^T HP y / y^T y, residual r = HP y - theta y, and the correction
-    // sum_{j != min} w_j (w_j^T r) / (theta - lambda_j) through W's spectrum, three times, so theta
+    // sum_{j != min} w_j (w_j^T r) / (theta - lambda_j) through W's spectrum, up to three times, so theta
     // and the coefficients are FP64-accurate while the O(k^3) work runs in FP32.
-    constexpr int LF = R + 1;
-    float* Af = reinterpret_cast<float*>(A);   // W0^T HP W0, then its Jacobi-diagonalised form
-    float* Vf = reinterpret_cast<float*>(T);   // HP W0, then the Jacobi rotations
-    float* W0 = reinterpret_cast<float*>(NS);  // start basis
-    float* Wf = reinterpret_cast<float*>(HS);  // eigenbasis W = W0 V
-    __shared__ float cs32[2 * R];
-    __shared__ int pq32[2 * R];
-    for (int e = tid; e < k * k; e += nt) {
+    for (int e = tid; e < k * k; e += kRitzThreads) {
         const int i = e / k, j = e - i * k;
-        W0[i * LF + j] = (i < kc && j < kc) ? static_cast<float>(CC[i * R + j]) : (i == j ? 1.0f : 0.0f);
+        Hf[i * L + j] = static_cast<float>(HP[i * L + j]);
     }
     __syncthreads();
-    for (int e = tid; e < k * k; e += nt) {  // HP W0
+    for (int e = tid; e < k * k; e += kRitzThreads) {  // HP W0
         const int i = e / k, j = e - i * k;
         float acc = 0.0f;
-        for (int l = 0; l < k; ++l) acc = fmaf(static_cast<float>(HP[i * R + l]), W0[l * LF + j], acc);
-        Vf[i * LF + j] = acc;
+        for (int l = 0; l < k; ++l) acc = fmaf(Hf[i * L + l], W0[l * L + j], acc);
+        A2[i * L + j] = acc;
     }
     __syncthreads();
-    for (int e = tid; e < k * k; e += nt) {  // W0^T (HP W0)
+    for (int e = tid; e < k * k; e += kRitzThreads) {  // W0^T (HP W0), one triangle
         const int i = e / k, j = e - i * k;
-        float acc = 0.0f;
-        for (int l = 0; l < k; ++l) acc = fmaf(W0[l * LF + i], Vf[l * LF + j], acc);
-        Af[i * LF + j] = acc;
-    }
-    __syncthreads();
-    for (int e = tid; e < k * k; e += nt) {  // symmetrise
-        const int i = e / k, j = e - i * k;
-        if (i < j) {
-            const float v = 0.5f * (Af[i * LF + j] + Af[j * LF + i]);
-            Af[i * LF + j] = v;
-            Af[j * LF + i] = v;
+        if (i <= j) {
+            float acc = 0.0f;
+            for (int l = 0; l < k; ++l) acc = fmaf(W0[l * L + i], A2[l * L + j], acc);
+            Af[i * L + j] = acc;
+            Af[j * L + i] = acc;
         }
+        Vf[i * L + j] = i == j ? 1.0f : 0.0f;
     }
     __syncthreads();
-    if (tid < 32) jacobi_warp_f32(Af, Vf, LF, k, cs32, pq32);
+    jacobi_cta_f32(Af, Vf, A2, V2, k, red);
     __syncthreads();
-    for (int e = tid; e < k * k; e += nt) {  // W = W0 V
+    for (int e = tid; e < k * k; e += kRitzThreads) {  // W = W0 V
         const int i = e / k, j = e - i * k;
         float acc = 0.0f;
-        for (int l = 0; l < k; ++l) acc = fmaf(W0[i * LF + l], Vf[l * LF + j], acc);
-        Wf[i * LF + j] = acc;
+        for (int l = 0; l < k; ++l) acc = fmaf(W0[i * L + l], Vf[l * L + j], acc);
+        Hf[i * L + j] = acc;
+        NS[i * L + j] = static_cast<double>(acc);
     }
     __syncthreads();
-    if (tid < 32) {
+    if (tid < 128) {
+        auto mv = [&](const double* mat, int rs, int cs, double v, int n) {
+            turn ^= 1;
+            return matvec4(mat, rs, cs, v, n, slots[turn]);
+        };
         // lowest diagonal entry of the rotated matrix
-        float lam = lane < k ? Af[lane * LF + lane] : INFINITY;
+        const float lam = lane < k ? Af[lane * L + lane] : INFINITY;
         float best = lam;
         int jmin = lane < k ? lane : R;
         for (int o = 16; o > 0; o >>= 1) {
@@ -777,54 +916,46 @@ __global__ void __launch_bounds__(128) k_ritz_inc(const double* __restrict__ h, 
                 jmin = oj;
             }
         }
-        double y = (lane < k && jmin < R) ? static_cast<double>(Wf[lane * LF + jmin]) : 0.0;
+        double y = (lane < k && jmin < R) ? NS[lane * L + jmin] : 0.0;
         double theta = 0.0;
-        for (int it = 0; it <= 3; ++it) {
-            double hy = 0.0;
-            for (int l = 0; l < k; ++l) {
-                const double yl = __shfl_sync(0xffffffffu, y, l);
-                if (lane < k) hy = fma(HP[lane * R + l], yl, hy);
+        bool last = false;
+        for (int it = 0;; ++it) {
+            double hy = mv(HP, L, 1, y, k);
+            if (lane >= k) hy = 0.0;
+            double yy = y * y, yhy = y * hy;
+            for (int o = 16; o > 0; o >>= 1) {
+                yy += __shfl_xor_sync(0xffffffffu, yy, o);
+                yhy += __shfl_xor_sync(0xffffffffu, yhy, o);
             }
-            const double yy = warp_sum(y * y), yhy = warp_sum(y * hy);
             theta = yy > 0.0 ? yhy / yy : 0.0;
-            if (it == 3) {
+            if (last) {
                 y = yy > 0.0 ? y / sqrt(yy) : 0.0;
                 break;
             }
             const double r = lane < k ? hy - theta * y : 0.0;
-            double c = 0.0;  // lane j: w_j^T r
-            for (int i = 0; i < k; ++i) {
-                const double ri = __shfl_sync(0xffffffffu, r, i);
-                if (lane < k) c = fma(static_cast<double>(Wf[i * LF + lane]), ri, c);
-            }
+            double c = mv(NS, 1, L, r, k);  // lane j: w_j^T r
             const double den = theta - static_cast<double>(lam);
             // components (nearly) degenerate with the lowest one are left as they are
             const bool use = lane < k && lane != jmin && fabs(den) > 1e-7 * (fabs(theta) + fabs(static_cast<double>(lam)) + 1e-300);
             c = use ? c / den : 0.0;
-            double d = 0.0;
-            for (int j = 0; j < k; ++j) {
-                const double cj = __shfl_sync(0xffffffffu, c, j);
-                if (lane < k) d = fma(static_cast<double>(Wf[lane * LF + j]), cj, d);
-            }
-            y += d;
+            const double d = mv(NS, L, 1, c, k);
+            if (lane < k) y += d;
+            // a correction leaves 3e-5 of itself: below 1e-11 the next one is rounding
+            last = it == 2 || !__any_sync(0xffffffffu, fabsf(static_cast<float>(c)) > 1e-11f);
         }
-        if (lane == 0) {
+        if (tid == 0) {
             scal[0] = k > 0 ? theta : 0.0;
             scal[1] = static_cast<double>(k);
         }
         // coefficients of the Ritz vector in the basis V: X y
-        double acc = 0.0;
-        for (int j = 0; j < k; ++j) {
-            const double yj = __shfl_sync(0xffffffffu, y, j);
-            if (lane < m) acc = fma(X[lane + j * R], yj, acc);
-        }
-        if (lane < m) coef[lane] = k > 0 ? acc : 0.0;
+        const double acc = mv(X, L, 1, y, k);
+        if (tid < R) coef[tid] = tid < m && k > 0 ? acc : 0.0;
     }
-    for (int e = tid; e < R * R; e += nt) {
-        const int i = e / R, j = e - i * R;
-        st->C[e] = (i < k && j < k) ? static_cast<double>(Wf[i * LF + j]) : 0.0;
-        st->X[e] = X[e];
-        st->hp[e] = HP[e];
+    for (int e = tid; e < R * R; e += kRitzThreads) {
+        const int i = e / R, j = e % R;
+        st->C[e] = (i < k && j < k) ? Hf[i * L + j] : 0.0f;
+        st->X[i + j * R] = X[i * L + j];
+        st->hp[e] = HP[i * L + j];
     }
     if (tid == 0) {
         st->k = k;
@@ -833,8 +964,9 @@ __global__ void __launch_bounds__(128) k_ritz_inc(const double* __restrict__ h, 
     }
 }
 
-// Orthonormal restart coefficients from [c_new, c_old] (Gram-Schmidt, twice).
-__global__ void k_restart_coef(const double* __restrict__ cn, const double* __restrict__ co, int m,
+// Orthonormal restart coefficients from [c_new, c_old] (Gram-Schmidt, twice); c_new is replaced by the
+// coefficients of the same vector in the restarted basis.
+__global__ void k_restart_coef(double* __restrict__ cn, const double* __restrict__ co, int m,
                                double* __restrict__ Q, double* __restrict__ out) {
     if (threadIdx.x != 0) return;
     double a[kRitzMax], b[kRitzMax];
@@ -863,8 +995,7 @@ __global__ void k_restart_coef(const double* __restrict__ cn, const double* __re
     // coefficients of the current Ritz vector in the rotated basis: Q^T c_new
     double d0 = 0.0, d1 = 0.0;
     for (int i = 0; i < m; ++i) { d0 += Q[i] * cn[i]; if (k == 2) d1 += Q[m + i] * cn[i]; }
-    out[1] = d0;
-    out[2] = d1;
+    for (int i = 0; i < kRitzMax; ++i) cn[i] = i == 0 ? d0 : (i == 1 ? d1 : 0.0);
 }
 
 // ---- ordered truncation ---------------------------------------------------------------------------
@@ -1011,6 +1142,9 @@ int grid_for(int64_t n, int threads, int cap) {
     return static_cast<int>(g);
 }
 
+// Blocks of the elementwise kernels that also sum (one partial sum each): up to kNormBlocks.
+int norm_blocks(int64_t n) { return grid_for(n, 256, kNormBlocks); }
+
 }  // namespace
 
 // ---- launch wrappers ----------------------------------------------------------------------------
@@ -1083,9 +1217,9 @@ cudaError_t launch_basis_rotate(const double* src, int64_t ld, int m, const doub
 
 
 cudaError_t launch_ritz_inc(const double* h, const double* nmat, int ldm, int m, int reset, double eps_metric,
-                            RitzState* state, double* coef, double* scal, cudaStream_t st) {
+                            RitzState* state, double* coef, double* coef_prev, double* scal, cudaStream_t st) {
     if (m > RitzState::kR) return cudaErrorInvalidValue;
-    constexpr int smem = 7 * RitzState::kR * RitzState::kR * static_cast<int>(sizeof(double));
+    constexpr int smem = RitzState::kR * kRitzLd * (4 * static_cast<int>(sizeof(double)) + 6 * static_cast<int>(sizeof(float)));
     static int attr_device = -1;  // the attribute is per device; set it once per device in use
     int dev = 0;
     cudaGetDevice(&dev);
@@ -1094,17 +1228,45 @@ cudaError_t launch_ritz_inc(const double* h, const double* nmat, int ldm, int m,
         if (e != cudaSuccess) return e;
         attr_device = dev;
     }
-    k_ritz_inc<<<1, 128, smem, st>>>(h, nmat, ldm, m, reset, eps_metric, state, coef, scal);
+    k_ritz_inc<<<1, kRitzThreads, smem, st>>>(h, nmat, ldm, m, reset, eps_metric, state, coef, coef_prev, scal);
     return cudaGetLastError();
 }
 
-cudaError_t launch_residual_diag(const double* hx, const double* nx, const double* dh, const double* dn,
-                                 const double* scal, double clamp, int64_t n, double* r, double* t, double* red,
-                                 double* partial, cudaStream_t st) {
-    k_residual_diag<<<grid_for(n, 256, 2048), 256, 0, st>>>(hx, nx, dh, dn, scal, clamp, n, r, t);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_norm2(r, n, red, partial, st);
+cudaError_t launch_ritz_vectors(const double* V, const double* HV, const double* NV, int64_t n, int m, const double* coef,
+                                const double* dh, const double* dn, const double* scal, double clamp, double* x,
+                                double* hx, double* nx, double* r, double* t, double* t2, double* sums, cudaStream_t st) {
+    if (m > kRitzMax) return cudaErrorInvalidValue;
+    k_ritz_vectors<<<norm_blocks(n), 256, 0, st>>>(V, HV, NV, n, m, coef, dh, dn, scal, clamp, x, hx, nx, r, t, t2, sums);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_project(const double* V, int64_t n, int m, double* y, double* partial, double* sums, cudaStream_t st) {
+    if (m > kRitzMax) return cudaErrorInvalidValue;
+    const int nb = grid_for(n, 256, kRedBlocks);
+    if (m > 0) k_multidot_partial<<<dim3(nb, m), 256, 0, st>>>(V, n, y, n, partial);
+    k_project<<<norm_blocks(n), 256, 0, st>>>(V, n, m, partial, nb, y, sums);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sum_blocks(const double* sums, int64_t n, double* out, cudaStream_t st) {
+    k_sum_blocks<<<1, 32, 0, st>>>(sums, norm_blocks(n), out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_normalise(double* y, int64_t n, const double* ysums, const double* rsums, double* yy, double* rr,
+                             cudaStream_t st) {
+    k_normalise<<<norm_blocks(n), 256, 0, st>>>(y, n, ysums, norm_blocks(n), rsums, norm_blocks(n), yy, rr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_multidot2(const double* V, int64_t ldv, int m, const double* x0, const double* x1, int64_t n,
+                             double* out0, double* out1, double* partial, cudaStream_t st) {
+    if (m <= 0) return cudaSuccess;
+    if (m > kRitzMax) return cudaErrorInvalidValue;
+    const int nb = grid_for(n, 256, kRedBlocks);
+    k_multidot2_partial<<<dim3(nb, m, 2), 256, 0, st>>>(V, ldv, x0, x1, n, partial);
+    k_multidot2_final<<<dim3(m, 2), 32, 0, st>>>(partial, nb, out0, out1);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_precond_apply(const double* v, const double* dh, const double* dn, const double* scal,
@@ -1137,7 +1299,7 @@ cudaError_t launch_xpby_ratio(double* p, const double* r, int64_t n, const doubl
     return cudaGetLastError();
 }
 
-cudaError_t launch_restart_coef(const double* c_new, const double* c_old, int m, double* Qout, double* scal_out,
+cudaError_t launch_restart_coef(double* c_new, const double* c_old, int m, double* Qout, double* scal_out,
                                 cudaStream_t st) {
     if (m > kRitzMax) return cudaErrorInvalidValue;
     k_restart_coef<<<1, 32, 0, st>>>(c_new, c_old, m, Qout, scal_out);

@@ -46,7 +46,8 @@ cudaError_t launch_diag_f64(const Slots& slots, const DiagBlock* blocks, const D
 
 // out[j] = sum_i V[j*ldv + i] * x[i] for j < m (plus a scale); multi-dot with block reduction.
 // `partial` is a per-caller scratch of kPartialDoubles doubles.
-constexpr int kPartialDoubles = 64 * 32;
+constexpr int kPartialDoubles = 2 * 64 * 32;
+constexpr int kNormBlocks = 304;  // partial sums of launch_ritz_vectors / launch_project (two CTAs per SM)
 cudaError_t launch_multidot(const double* V, int64_t ldv, int m, const double* x, int64_t n, double* out,
                             double* partial, cudaStream_t st);
 // y[i] = sum_j V[j*ldv + i] * c[j]  (c on the device), optionally y -= (when sub != 0).
@@ -56,25 +57,36 @@ cudaError_t launch_gemv(const double* V, int64_t ldv, int m, const double* c, in
 cudaError_t launch_basis_rotate(const double* src, int64_t ld, int m, const double* Q, int ldq, int k,
                                 int64_t n, double* dst, cudaStream_t st);
 
-// Incremental Ritz step of the Davidson solver (one CTA of 128 threads) on the stored subspace
+// Incremental Ritz step of the Davidson solver (one CTA) on the stored subspace
 // matrices h, n (m x m, leading dim ldm, upper triangles column by column): lowest Ritz pair in the
 // range of n kept above eps_metric * max diag(n).  The state is kept across the iterations of one
-// solve; reset != 0 rebuilds it from the m stored columns.  Writes coef[0..m) and scal[0] = theta,
-// scal[1] = number of kept metric directions (0 = singular).
+// solve; reset != 0 rebuilds it from the m stored columns.  Writes coef[0..32) (zeros beyond m; the previous
+// contents go to coef_prev) and scal[0] = theta, scal[1] = number of kept metric directions (0 = singular).
 struct RitzState {
     static constexpr int kR = 32;
     double X[kR * kR];   // n-orthonormal coefficient basis, X[i + j*kR]
     double hp[kR * kR];  // X^T h X
-    double C[kR * kR];   // eigenvectors of hp (columns)
+    float C[kR * kR];    // eigenvectors of hp (columns)
     int k, m, kc, pad;
 };
 cudaError_t launch_ritz_inc(const double* h, const double* nmat, int ldm, int m, int reset, double eps_metric,
-                            RitzState* state, double* coef, double* scal, cudaStream_t st);
+                            RitzState* state, double* coef, double* coef_prev, double* scal, cudaStream_t st);
 
-// r = hx - theta * nx, t = preconditioned correction, scal[2] = ||r||^2.
-cudaError_t launch_residual_diag(const double* hx, const double* nx, const double* dh, const double* dn,
-                                 const double* scal, double clamp, int64_t n, double* r, double* t,
-                                 double* red, double* partial, cudaStream_t st);
+// One pass over the bases (leading dimension n): x = V c, hx = HV c, nx = NV c, r = hx - theta nx (theta =
+// scal[0]), t = -r / (diag H - theta diag N) clamped (also into t2 unless null), block sums of |r|^2.
+cudaError_t launch_ritz_vectors(const double* V, const double* HV, const double* NV, int64_t n, int m, const double* coef,
+                                const double* dh, const double* dn, const double* scal, double clamp, double* x,
+                                double* hx, double* nx, double* r, double* t, double* t2, double* sums, cudaStream_t st);
+// y -= V V^T y (one pass of classical Gram-Schmidt against m vectors); block sums of |y|^2 unless null.
+cudaError_t launch_project(const double* V, int64_t n, int m, double* y, double* partial, double* sums, cudaStream_t st);
+// *out = sum of the block sums of a vector of length n.
+cudaError_t launch_sum_blocks(const double* sums, int64_t n, double* out, cudaStream_t st);
+// y /= |y| from the block sums of |y|^2 (their sum to *yy); the sum of rsums (unless null) to *rr.
+cudaError_t launch_normalise(double* y, int64_t n, const double* ysums, const double* rsums, double* yy, double* rr,
+                             cudaStream_t st);
+// out0[j] = V_j . x0 and out1[j] = V_j . x1 for j < m.
+cudaError_t launch_multidot2(const double* V, int64_t ldv, int m, const double* x0, const double* x1, int64_t n,
+                             double* out0, double* out1, double* partial, cudaStream_t st);
 // sum of squares into *out (two-pass deterministic reduction).
 cudaError_t launch_norm2(const double* x, int64_t n, double* out, double* partial, cudaStream_t st);
 // x *= 1/sqrt(*nrm2) (device scalar)
@@ -89,8 +101,9 @@ cudaError_t launch_axpy_ratio(double* x, const double* y, int64_t n, const doubl
 cudaError_t launch_xpby_ratio(double* p, const double* r, int64_t n, const double* num, const double* den,
                               cudaStream_t st);
 // Two-vector orthonormal restart coefficients in the current basis: Qout (m x 2) from the
-// Ritz coefficients c_new and c_old (m each); returns the count in scal_out[0].
-cudaError_t launch_restart_coef(const double* c_new, const double* c_old, int m, double* Qout, double* scal_out,
+// Ritz coefficients c_new and c_old (m each); the count to scal_out[0]; c_new (32 entries) becomes the
+// coefficients of the same vector in the restarted basis.
+cudaError_t launch_restart_coef(double* c_new, const double* c_old, int m, double* Qout, double* scal_out,
                                 cudaStream_t st);
 
 // ---- decimation -------------------------------------------------------------------------------

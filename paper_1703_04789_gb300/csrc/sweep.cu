@@ -47,7 +47,7 @@ int64_t x_size(spmps_t* h, int k) { return make_row_block_layout(h->bonds[k], h-
 
 // Device work buffers of the Davidson solver.
 struct DavBuffers {
-    DevMem V, HV, NV, hm, nm, coef, coef_prev, scal, x, hx, nx, r, t, dh, dn, Q, tmp, cg_p, cg_ap, cg_res, dot, ritz;
+    DevMem V, HV, NV, hm, nm, coef, coef_prev, scal, x, hx, nx, r, t, dh, dn, Q, tmp, cg_p, cg_ap, cg_res, dot, ritz, sums;
     MetricState metric;  // factors of the metric blocks (precond == 4)
     DevMem Vc;           // orthonormal constraint vectors (excited states, Eq. orthoB)
     int ncon = 0;
@@ -79,17 +79,17 @@ spmps_status ensure_dav(spmps_t* h, DavBuffers& B, int64_t n, int ms) {
     CK(B.scal.ensure(sizeof(double) * 16));
     CK(B.dot.ensure(sizeof(double) * 64));
     CK(B.ritz.ensure(sizeof(RitzState)));
+    CK(B.sums.ensure(sizeof(double) * 2 * kNormBlocks));
+    CK(cudaMemsetAsync(B.coef.p, 0, sizeof(double) * 64, h->stream));
     return SPMPS_OK;
 }
 
 // Subspace matrix columns for basis column j: h[j*ms + i] = V_i . HV_j (i <= j), same for n.
 spmps_status subspace_column(spmps_t* h, DavBuffers& B, int64_t n, int ms, int j) {
     double* V = B.V.as<double>();
-    CK(launch_multidot(V, n, j + 1, B.HV.as<double>() + j * n, n, B.hm.as<double>() + j * ms, h->partial.as<double>(),
-                       h->stream));
-    CK(launch_multidot(V, n, j + 1, B.NV.as<double>() + j * n, n, B.nm.as<double>() + j * ms, h->partial.as<double>(),
-                       h->stream));
-    h->launches += 4;
+    CK(launch_multidot2(V, n, j + 1, B.HV.as<double>() + j * n, B.NV.as<double>() + j * n, n, B.hm.as<double>() + j * ms,
+                        B.nm.as<double>() + j * ms, h->partial.as<double>(), h->stream));
+    h->launches += 2;
     return SPMPS_OK;
 }
 
@@ -99,13 +99,10 @@ spmps_status apply_column(spmps_t* h, int k, DavBuffers& B, int64_t n, int j) {
 
 // t <- t - V (V^T t), twice; returns |t|^2 (host)
 spmps_status orthogonalise(spmps_t* h, DavBuffers& B, int64_t n, int m, double* t, double* nrm2) {
-    for (int pass = 0; pass < 2; ++pass) {
-        CK(launch_multidot(B.V.as<double>(), n, m, t, n, B.dot.as<double>(), h->partial.as<double>(), h->stream));
-        CK(launch_gemv(B.V.as<double>(), n, m, B.dot.as<double>(), n, t, 1, h->stream));
-        h->launches += 3;
-    }
-    CK(launch_norm2(t, n, B.scal.as<double>() + 3, h->partial.as<double>(), h->stream));
-    h->launches += 2;
+    for (int pass = 0; pass < 2; ++pass)
+        CK(launch_project(B.V.as<double>(), n, m, t, h->partial.as<double>(), pass ? B.sums.as<double>() : nullptr, h->stream));
+    CK(launch_sum_blocks(B.sums.as<double>(), n, B.scal.as<double>() + 3, h->stream));
+    h->launches += 5;
     CK(cudaMemcpyAsync(nrm2, B.scal.as<double>() + 3, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     return SPMPS_OK;
@@ -282,16 +279,25 @@ spmps_status davidson_stage(spmps_t* h, int k, const double* x0, DavBuffers& B, 
         // metric range kept before the switch to FP64 is cut well above that error
         const double eps_metric = switched ? kEpsMetric : (h->apply_precision == 1 ? 1e-2 : 1e-6);
         CK(launch_ritz_inc(B.hm.as<double>(), B.nm.as<double>(), ms, m, reset, eps_metric, B.ritz.as<RitzState>(),
-                           B.coef.as<double>(), sc, h->stream));
+                           B.coef.as<double>(), B.coef_prev.as<double>(), sc, h->stream));
         if (rec >= 0) prof_end(h, h->stream, rec);
         reset = 0;
         rec = h->profile ? prof_begin(h, h->stream, 3, 0.0) : -1;
-        CK(launch_gemv(V, n, m, B.coef.as<double>(), n, B.x.as<double>(), 0, h->stream));
-        CK(launch_gemv(B.HV.as<double>(), n, m, B.coef.as<double>(), n, B.hx.as<double>(), 0, h->stream));
-        CK(launch_gemv(B.NV.as<double>(), n, m, B.coef.as<double>(), n, B.nx.as<double>(), 0, h->stream));
-        CK(launch_residual_diag(B.hx.as<double>(), B.nx.as<double>(), B.dh.as<double>(), B.dn.as<double>(), sc, kClamp,
-                                n, B.r.as<double>(), B.t.as<double>(), sc + 2, h->partial.as<double>(), h->stream));
-        h->launches += 7;
+        // the diagonal correction goes straight to the new basis column where nothing stands between
+        double* tcol = V + static_cast<int64_t>(m) * n;
+        double* rsums = B.sums.as<double>();
+        double* ysums = rsums + kNormBlocks;
+        const bool direct = m < ms && h->opt.precond == 0 && B.ncon == 0;
+        CK(launch_ritz_vectors(V, B.HV.as<double>(), B.NV.as<double>(), n, m, B.coef.as<double>(), B.dh.as<double>(),
+                               B.dn.as<double>(), sc, kClamp, B.x.as<double>(), B.hx.as<double>(), B.nx.as<double>(),
+                               B.r.as<double>(), B.t.as<double>(), direct ? tcol : nullptr, rsums, h->stream));
+        h->launches += 2;
+        // |r|^2 (sc[2]) now where the iteration reads it, else with the norm of the new direction
+        const bool rr_now = B.ncon == 0 && (harvest || learned_on);
+        if (rr_now) {
+            CK(launch_sum_blocks(rsums, n, sc + 2, h->stream));
+            ++h->launches;
+        }
         if (B.ncon > 0) {
             // the residual within the range of Q, its norm and the diagonal correction of it
             st = project_constraints(h, B, n, B.r.as<double>());
@@ -363,26 +369,18 @@ spmps_status davidson_stage(spmps_t* h, int k, const double* x0, DavBuffers& B, 
                 if (st != SPMPS_OK) return st;
             }
             reset = 1;
-            // coefficients of the current Ritz vector in the rotated basis: (scal[5], scal[6], 0, ...)
-            CK(cudaMemsetAsync(B.coef_prev.p, 0, 64 * sizeof(double), h->stream));
-            CK(cudaMemcpyAsync(B.coef_prev.p, sc + 5, 2 * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-        } else {
-            CK(cudaMemsetAsync(B.coef_prev.p, 0, 64 * sizeof(double), h->stream));
-            CK(cudaMemcpyAsync(B.coef_prev.p, B.coef.p, m * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
+            tcol = V + static_cast<int64_t>(m) * n;
         }
         // new direction into column m: t orthogonalised twice against V, normalised
-        double* tcol = V + static_cast<int64_t>(m) * n;
-        CK(cudaMemcpyAsync(tcol, tsrc, n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-        st = project_constraints(h, B, n, tcol);
-        if (st != SPMPS_OK) return st;
-        for (int pass = 0; pass < 2; ++pass) {
-            CK(launch_multidot(V, n, m, tcol, n, B.dot.as<double>(), h->partial.as<double>(), h->stream));
-            CK(launch_gemv(V, n, m, B.dot.as<double>(), n, tcol, 1, h->stream));
-            h->launches += 3;
+        if (!direct) {
+            CK(cudaMemcpyAsync(tcol, tsrc, n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
+            st = project_constraints(h, B, n, tcol);
+            if (st != SPMPS_OK) return st;
         }
-        CK(launch_norm2(tcol, n, sc + 3, h->partial.as<double>(), h->stream));
-        CK(launch_scale_inv_sqrt(tcol, n, sc + 3, h->stream));
-        h->launches += 3;
+        for (int pass = 0; pass < 2; ++pass)
+            CK(launch_project(V, n, m, tcol, h->partial.as<double>(), pass ? ysums : nullptr, h->stream));
+        CK(launch_normalise(tcol, n, ysums, B.ncon > 0 || rr_now ? nullptr : rsums, sc + 3, sc + 2, h->stream));
+        h->launches += 5;
         if (rec >= 0) prof_end(h, h->stream, rec);
         // one host read per iteration: theta, kept metric directions, |r|^2, |t|^2
         CK(cudaMemcpyAsync(host, sc, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
