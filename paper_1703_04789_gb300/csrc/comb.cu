@@ -64,7 +64,7 @@ __device__ __forceinline__ void rotate(double* v, int m, double t, double s) {
 constexpr int kStageIns = kFusedInputs, kStageDsts = 64, kStageCoefs = 128;
 
 template <int LEGS>
-__global__ void __launch_bounds__(kFusedThreads) k_comb_pair(Slots S, CombDev D, int unit0, int g0, int shared) {
+__global__ void __launch_bounds__(kFusedThreads) k_comb_pair(const __grid_constant__ Slots S, const __grid_constant__ CombDev D, int unit0, int g0, int shared) {
     extern __shared__ double vin[];
     __shared__ CombIn sins[kStageIns];
     __shared__ CombSet ssets[kStageIns];
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_comb_pair(Slots S, CombDev D,
 
 // Separate rotation of T1 in place for classes of many inputs: one CTA per (pair, channel).
 template <int LEGS>
-__global__ void __launch_bounds__(256) k_comb_rotate(Slots S, CombDev D, int rot0, int g0) {
+__global__ void __launch_bounds__(256) k_comb_rotate(const __grid_constant__ Slots S, const __grid_constant__ CombDev D, int rot0, int g0) {
     const int2 U = D.rots[rot0 + blockIdx.x];
     const CombPair P = D.pairs[U.x];
     const CombSet st = D.sets[P.set0 + U.y];
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) k_comb_rotate(Slots S, CombDev D, int rot
 // per output on average at K = 20); the inputs of a beta point come from L2.  Measured (K = 20, D = 100,
 // n_beta = 12, middle action): 25.2 ms for the phase, 95.7 ms with rotated coefficients (2.2 times the
 // nonzeros) and without leaving out the rows that phase C does not read.
-__global__ void __launch_bounds__(128) k_comb_list(Slots S, CombDev D, int out0, int n_out, int g0) {
+__global__ void __launch_bounds__(128) k_comb_list(const __grid_constant__ Slots S, const __grid_constant__ CombDev D, int out0, int n_out, int g0) {
     constexpr int E = 4;
     const int ob = blockIdx.x;  // operator 0's (or 1's) blocks, then operator 1's on operator 0's T1
     const CombDst d = D.dsts[D.outs[ob < n_out ? out0 + ob : D.shared0 + ob - n_out]];

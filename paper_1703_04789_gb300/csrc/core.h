@@ -113,6 +113,17 @@ struct Slots {
     double* p[kMaxSlots];
 };
 
+// Elements between consecutive beta points in the buffer of each slot, per operator: the lists of a plan
+// hold one beta point, and the kernels add g times this to every base pointer.
+struct BetaStride {
+    int64_t s[2][kMaxSlots] = {};
+};
+// Beta points [g0, g0 + ng) of a launch whose tiles (units) from `split` on belong to operator 1.
+struct BetaRun {
+    BetaStride stride;
+    int split = 1 << 30, g0 = 0, ng = 1;
+};
+
 // C (M x N) = sum over segments of A(M x K) B(K x N); C(i, j) is stored at
 // C[i*ldc + cmap[j]] (cmap = -1: j).  A(i, k) = A[i*a_rs + k*a_cs], B(k, j) = B[k*b_rs + j*b_cs].
 struct GemmTask {
@@ -192,7 +203,8 @@ struct GemmPlan {
     std::vector<GemmTile> tiles;
     std::vector<int> cmaps;
     double flops = 0.0;
-    void add_tiles(const TilePolicy& pol = TilePolicy());
+    // `copies`: beta points that run per launch of these tasks
+    void add_tiles(const TilePolicy& pol = TilePolicy(), int copies = 1);
     // tiles for the tensor-core kernel: regions of at most 32 x 32 outputs (one MMA sub-tile per
     // warp), shape 6
     std::vector<GemmTile> tc_tiles;

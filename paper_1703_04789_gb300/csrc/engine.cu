@@ -76,7 +76,7 @@ spmps_status env_prepare(spmps_t* h, EnvStore& E, const Bond& b, int bond) {
         }
     }
     E.total = off;
-    CK(E.buf.ensure(std::max<int64_t>(1, off) * sizeof(double)));
+    CK(ensure_idle(E.buf, std::max<int64_t>(1, off) * sizeof(double), h->stream));
     return SPMPS_OK;
 }
 
@@ -117,8 +117,13 @@ bool in_range(uint64_t hd, int64_t last, const int64_t* sizes, std::string* why,
 
 bool validate_tiles(const GemmPlan& G, std::string* why);
 
-bool validate_gemm(const GemmPlan& G, const int64_t* sizes, std::string* why) {
-    for (const GemmTask& T : G.tasks) {
+bool validate_gemm(const GemmPlan& G, const int64_t* sizes, std::string* why, const BetaStride* stride, int op1, int copies) {
+    // distance from the listed beta point to the last one, per handle's slot
+    auto far = [&](uint64_t hd, int task) -> int64_t {
+        return stride ? (copies - 1) * stride->s[task >= op1 ? 1 : 0][(hd >> 56) & (kMaxSlots - 1)] : 0;
+    };
+    for (int ti = 0; ti < static_cast<int>(G.tasks.size()); ++ti) {
+        const GemmTask& T = G.tasks[ti];
         if (T.M <= 0 || T.N <= 0) { *why = "empty GEMM task"; return false; }
         int64_t maxc = T.N - 1;
         if (T.cmap >= 0) {
@@ -130,14 +135,14 @@ bool validate_gemm(const GemmPlan& G, const int64_t* sizes, std::string* why) {
             }
         }
         if (maxc >= T.ldc && T.M > 1) { *why = "column beyond leading dimension"; return false; }
-        if (!in_range(T.c, static_cast<int64_t>(T.M - 1) * T.ldc + maxc, sizes, why, "GEMM C")) return false;
+        if (!in_range(T.c, far(T.c, ti) + static_cast<int64_t>(T.M - 1) * T.ldc + maxc, sizes, why, "GEMM C")) return false;
         for (int q = 0; q < T.nseg; ++q) {
             const GemmSeg& sg = G.segs[T.seg0 + q];
             if (sg.K <= 0 || sg.a_rs < 0 || sg.a_cs < 0 || sg.b_rs < 0 || sg.b_cs < 0) { *why = "bad segment"; return false; }
-            if (!in_range(sg.a, static_cast<int64_t>(T.M - 1) * sg.a_rs + static_cast<int64_t>(sg.K - 1) * sg.a_cs, sizes,
+            if (!in_range(sg.a, far(sg.a, ti) + static_cast<int64_t>(T.M - 1) * sg.a_rs + static_cast<int64_t>(sg.K - 1) * sg.a_cs, sizes,
                           why, "GEMM A"))
                 return false;
-            if (!in_range(sg.b, static_cast<int64_t>(sg.K - 1) * sg.b_rs + static_cast<int64_t>(T.N - 1) * sg.b_cs, sizes,
+            if (!in_range(sg.b, far(sg.b, ti) + static_cast<int64_t>(sg.K - 1) * sg.b_rs + static_cast<int64_t>(T.N - 1) * sg.b_cs, sizes,
                           why, "GEMM B"))
                 return false;
         }
@@ -185,7 +190,11 @@ bool validate_diag(const Plan& P, const int64_t* sizes, std::string* why) {
 
 bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why, int G) {
     if (!P.chan.pairs.empty() && !comb_check(P.chan, G, sizes[3], sizes[4], why)) return false;
-    if (!validate_gemm(P.A, sizes, why) || !validate_gemm(P.C, sizes, why)) return false;
+    const BetaStride* bs = P.per_op ? &P.stride : nullptr;
+    const int copies = P.per_op ? G : 1;
+    if (!validate_gemm(P.A, sizes, why, bs, P.per_op ? P.tileA_rng[1] : 1 << 30, copies) ||
+        !validate_gemm(P.C, sizes, why, bs, P.per_op ? P.tileC_rng[1] : 1 << 30, copies))
+        return false;
     for (const CombOut& o : P.B.outs) {
         if (o.rows <= 0 || o.cols <= 0 || o.cols > o.ld) { *why = "bad combination block"; return false; }
         if (!in_range(o.dst, static_cast<int64_t>(o.rows - 1) * o.ld + o.cols - 1, sizes, why, "comb dst")) return false;
@@ -199,7 +208,9 @@ bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why, int G)
 
 // ---- plan upload and launch -------------------------------------------------------------------
 
-spmps_status plan_upload(spmps_t* h, Plan& P) {
+// Work lists of the plan's kernels, packed into `lists` (the plan's own buffer, or the handle's for plans that
+// run once) with one copy.  Only the lists that the handle's options can launch are made.
+spmps_status plan_upload(spmps_t* h, Plan& P, DevMem& lists) {
     const auto t0 = std::chrono::steady_clock::now();
     struct Done {
         spmps_t* h;
@@ -210,45 +221,50 @@ spmps_status plan_upload(spmps_t* h, Plan& P) {
             h->prof_ms[5] += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
     } done{h, t0};
-    P.A.add_tiles(P.polA);
-    P.C.add_tiles(P.polC);
-    P.A.add_tc_tiles();
-    P.C.add_tc_tiles();
+    if (!P.task_rng_kept) {
+        P.taskA_rng = P.tileA_rng;
+        P.taskC_rng = P.tileC_rng;
+        P.task_rng_kept = true;
+    }
+    const int nr = static_cast<int>(P.taskA_rng.size()) - 1, copies = P.per_op ? h->G : 1;
+    const bool action = P.reduce_nx > 0 && nr > 0 && !P.chan.pairs.empty();
+    const bool oz = action && h->opt.fp64_tensor_cores, reduced = action && h->opt.precision > 0;
+    // stacks by the shared operand: phase A by ket label (x rows shared), phase C by right label
+    P.stackA.clear();
+    P.stackC.clear();
+    if (action && (oz || reduced)) build_tc_plan(P.A, P.taskA_rng, nr, P.stackA);
+    if (action) build_tc_plan(P.C, P.taskC_rng, nr, P.stackC);
+    const bool stacked = P.stackA.ok && P.stackC.ok;
+    for (TcUnits* u : {&P.tcA, &P.tcC, &P.ozA, &P.ozC, &P.f64C}) *u = TcUnits();
+    if (reduced && stacked && h->opt.tensor_core_kernel == 0) {
+        tile_units(P.stackA, 128, P.tcA);
+        tile_units(P.stackC, 64, P.tcC);
+    }
+    if (oz && stacked) {
+        tile_units(P.stackA, gemm_oz_columns(), P.ozA);
+        tile_units(P.stackC, gemm_oz_columns(), P.ozC);
+        if (!h->tc_err.p) {  // its status word, so that running the plan allocates nothing
+            CK(h->tc_err.ensure(sizeof(int)));
+            CK(cudaMemsetAsync(h->tc_err.p, 0, sizeof(int), h->stream));
+        }
+    } else if (P.stackC.ok) {
+        stack_units(P.stackC, std::min(256, P.polC.wb_elems), copies, P.f64C);
+    }
+    P.A.tiles.clear();
+    P.C.tiles.clear();
+    P.A.tc_tiles.clear();
+    P.C.tc_tiles.clear();
+    if (P.ozA.rng.empty()) P.A.add_tiles(P.polA, copies);
+    if (P.ozC.rng.empty() && P.f64C.rng.empty()) P.C.add_tiles(P.polC, copies);
+    if (reduced && P.tcA.rng.empty()) {
+        P.A.add_tc_tiles();
+        P.C.add_tc_tiles();
+    }
     {
         std::string why;
         if (!validate_tiles(P.A, &why) || !validate_tiles(P.C, &why)) return fail(h, SPMPS_ERR_CUDA, "internal tile check: " + why);
     }
-    CK(upload(P.d_tasksA, P.A.tasks, h->stream));
-    CK(upload(P.d_segsA, P.A.segs, h->stream));
-    CK(upload(P.d_tilesA, P.A.tiles, h->stream));
-    CK(upload(P.d_cmapsA, P.A.cmaps, h->stream));
-    CK(upload(P.d_outsB, P.B.outs, h->stream));
-    CK(upload(P.d_termsB, P.B.terms, h->stream));
-    CK(upload(P.d_tasksC, P.C.tasks, h->stream));
-    CK(upload(P.d_segsC, P.C.segs, h->stream));
-    CK(upload(P.d_tilesC, P.C.tiles, h->stream));
-    CK(upload(P.d_cmapsC, P.C.cmaps, h->stream));
-    CK(upload(P.d_tcA, P.A.tc_tiles, h->stream));
-    CK(upload(P.d_tcC, P.C.tc_tiles, h->stream));
-    if (!P.chan.pairs.empty()) {
-        CombChan& N = P.chan;
-        CK(upload(P.d_chan[0], N.ins, h->stream));
-        CK(upload(P.d_chan[1], N.sets, h->stream));
-        CK(upload(P.d_chan[2], N.dsts, h->stream));
-        CK(upload(P.d_chan[3], N.coefs, h->stream));
-        CK(upload(P.d_chan[4], N.pairs, h->stream));
-        CK(upload(P.d_chan[5], N.lab, h->stream));
-        CK(upload(P.d_chan[6], N.units, h->stream));
-        CK(upload(P.d_chan[7], N.rots, h->stream));
-        std::vector<int> outs = N.outs;
-        outs.insert(outs.end(), N.shared_outs.begin(), N.shared_outs.end());
-        CK(upload(P.d_chan[8], outs, h->stream));
-        P.chan_dev = CombDev{P.d_chan[0].as<CombIn>(),   P.d_chan[1].as<CombSet>(), P.d_chan[2].as<CombDst>(),
-                             P.d_chan[3].as<CombCoef>(), P.d_chan[4].as<CombPair>(), P.d_chan[5].as<uint8_t>(),
-                             P.d_chan[6].as<int2>(),     P.d_chan[7].as<int2>(),    P.d_chan[8].as<int>(),
-                             static_cast<int>(N.outs.size()), h->d_rot.as<double>(),      N.stride};
-    }
-    // tile and output ranges per (op, g): tasks were appended in (op, g) order
+    // tile ranges: tasks were appended range by range
     auto ranges = [&](const std::vector<GemmTile>& tiles, const std::vector<int>& task_rng, std::vector<int>& out) {
         out.assign(task_rng.size(), 0);
         size_t t = 0;
@@ -257,89 +273,57 @@ spmps_status plan_upload(spmps_t* h, Plan& P) {
             out[r] = static_cast<int>(t);
         }
     };
-    if (!P.task_rng_kept) {
-        P.taskA_rng = P.tileA_rng;
-        P.taskC_rng = P.tileC_rng;
-        P.task_rng_kept = true;
+    ranges(P.A.tiles, P.taskA_rng, P.tileA_rng);
+    ranges(P.C.tiles, P.taskC_rng, P.tileC_rng);
+    ranges(P.A.tc_tiles, P.taskA_rng, P.warpA_rng);
+    ranges(P.C.tc_tiles, P.taskC_rng, P.warpC_rng);
+    {  // flops of a range's one copy, for the profiler
+        auto task_flops = [](const GemmPlan& gp, const std::vector<int>& rng, std::vector<double>& out) {
+            out.assign(rng.size(), 0.0);
+            for (size_t r = 0; r + 1 < rng.size(); ++r)
+                for (int t = rng[r]; t < rng[r + 1]; ++t) {
+                    const GemmTask& T = gp.tasks[t];
+                    for (int q = 0; q < T.nseg; ++q) out[r] += 2.0 * T.M * T.N * gp.segs[T.seg0 + q].K;
+                }
+        };
+        task_flops(P.A, P.taskA_rng, P.flopsA_rng);
+        task_flops(P.C, P.taskC_rng, P.flopsC_rng);
     }
-    const std::vector<int>& a_task_rng = P.taskA_rng;
-    const std::vector<int>& c_task_rng = P.taskC_rng;
-    auto task_flops = [](const GemmPlan& gp, const std::vector<int>& rng, std::vector<double>& out) {
-        out.assign(rng.size(), 0.0);
-        for (size_t r = 0; r + 1 < rng.size(); ++r)
-            for (int t = rng[r]; t < rng[r + 1]; ++t) {
-                const GemmTask& T = gp.tasks[t];
-                for (int q = 0; q < T.nseg; ++q) out[r] += 2.0 * T.M * T.N * gp.segs[T.seg0 + q].K;
-            }
-    };
-    task_flops(P.A, a_task_rng, P.flopsA_rng);
-    task_flops(P.C, c_task_rng, P.flopsC_rng);
     if (P.chan.pairs.empty()) P.flopsB_rng.assign(P.combB_rng.size(), 0.0);
     for (size_t r = 0; r + 1 < P.combB_rng.size(); ++r)
         for (int o = P.combB_rng[r]; o < P.combB_rng[r + 1]; ++o)
             P.flopsB_rng[r] += 2.0 * P.B.outs[o].rows * P.B.outs[o].cols * P.B.outs[o].nterm;
-    ranges(P.A.tiles, a_task_rng, P.tileA_rng);
-    ranges(P.C.tiles, c_task_rng, P.tileC_rng);
-    ranges(P.A.tc_tiles, a_task_rng, P.tcA_rng);
-    ranges(P.C.tc_tiles, c_task_rng, P.tcC_rng);
-    // tcgen05 stacks of the H part (op 0) of an apply plan: phase A by ket label (x rows shared),
-    // phase C by right label (environment rows shared)
-    P.stA.clear();
-    P.stC.clear();
-    if (P.reduce_nx > 0 && static_cast<int>(a_task_rng.size()) > h->G && static_cast<int>(c_task_rng.size()) > h->G) {
-        const bool okA = build_tc_plan(P.A, a_task_rng, h->G, 128, P.stA);
-        const bool okC = build_tc_plan(P.C, c_task_rng, h->G, 64, P.stC);
-        if (okA && okC) {
-            for (TcPlan* T : {&P.stA, &P.stC}) {
-                DevMem* d = T == &P.stA ? P.d_stA : P.d_stC;
-                CK(upload(d[0], T->stacks, h->stream));
-                CK(upload(d[1], T->rows, h->stream));
-                CK(upload(d[2], T->segs, h->stream));
-                CK(upload(d[3], T->atab, h->stream));
-                CK(upload(d[4], T->units, h->stream));
-            }
-        } else {
-            P.stA.ok = P.stC.ok = false;
-        }
-    }
-    // stacks of every (op, g) range for the FP64-accurate split-product GEMM; its status word is
-    // allocated here so that running the plan allocates nothing
-    P.ozA.clear();
-    P.ozC.clear();
-    if (P.reduce_nx > 0 && h->opt.fp64_tensor_cores && a_task_rng.size() > 1 && c_task_rng.size() > 1) {
-        const bool okA = build_tc_plan(P.A, a_task_rng, static_cast<int>(a_task_rng.size()) - 1, gemm_oz_columns(), P.ozA);
-        const bool okC = build_tc_plan(P.C, c_task_rng, static_cast<int>(c_task_rng.size()) - 1, gemm_oz_columns(), P.ozC);
-        if (okA && okC) {
-            for (TcPlan* T : {&P.ozA, &P.ozC}) {
-                DevMem* d = T == &P.ozA ? P.d_ozA : P.d_ozC;
-                CK(upload(d[0], T->stacks, h->stream));
-                CK(upload(d[1], T->rows, h->stream));
-                CK(upload(d[2], T->segs, h->stream));
-                CK(upload(d[3], T->atab, h->stream));
-                CK(upload(d[4], T->units, h->stream));
-            }
-            if (!h->tc_err.p) {
-                CK(h->tc_err.ensure(sizeof(int)));
-                CK(cudaMemsetAsync(h->tc_err.p, 0, sizeof(int), h->stream));
-            }
-        } else {
-            P.ozA.ok = P.ozC.ok = false;
-        }
-    }
-    // phase C of an action on the FP64 pipe: stacked by right label
-    P.f64C.clear();
-    if (P.reduce_nx > 0 && !h->opt.fp64_tensor_cores && c_task_rng.size() > 1 &&
-        build_tc_plan(P.C, c_task_rng, static_cast<int>(c_task_rng.size()) - 1, 32, P.f64C)) {
-        stack_units(P.f64C, std::min(256, P.polC.wb_elems));
-        CK(upload(P.d_f64C[0], P.f64C.stacks, h->stream));
-        CK(upload(P.d_f64C[1], P.f64C.rows, h->stream));
-        CK(upload(P.d_f64C[2], P.f64C.segs, h->stream));
-        CK(upload(P.d_f64C[3], P.f64C.atab, h->stream));
-        CK(upload(P.d_f64C[4], P.f64C.units, h->stream));
-    }
-    CK(h->work1.ensure(std::max<int64_t>(1, P.t1_size) * sizeof(double)));
-    CK(h->work2.ensure(std::max<int64_t>(1, P.t2_size) * sizeof(double)));
-    CK(cudaStreamSynchronize(h->stream));
+    // one image, one copy; tasks and segments only where their kernels run
+    static const std::vector<GemmTask> no_tasks;
+    static const std::vector<GemmSeg> no_segs;
+    const bool listA = !P.A.tiles.empty() || !P.A.tc_tiles.empty(), listC = !P.C.tiles.empty() || !P.C.tc_tiles.empty();
+    Packer K(h->staging);
+    CombChan& N = P.chan;
+    std::vector<int> outs = N.outs;
+    outs.insert(outs.end(), N.shared_outs.begin(), N.shared_outs.end());
+    const size_t o[] = {K.add(listA ? P.A.tasks : no_tasks), K.add(listC ? P.C.tasks : no_tasks),
+                        K.add(listA ? P.A.segs : no_segs), K.add(listC ? P.C.segs : no_segs),
+                        K.add(P.A.tiles), K.add(P.C.tiles), K.add(P.A.tc_tiles), K.add(P.C.tc_tiles),
+                        K.add(P.A.cmaps), K.add(P.C.cmaps), K.add(P.B.outs), K.add(P.B.terms),
+                        K.add(P.stackA.stacks), K.add(P.stackC.stacks), K.add(P.stackA.rows), K.add(P.stackC.rows),
+                        K.add(P.stackA.segs), K.add(P.stackC.segs), K.add(P.stackA.atab), K.add(P.stackC.atab),
+                        K.add(P.tcA.units), K.add(P.tcC.units), K.add(P.ozA.units), K.add(P.ozC.units), K.add(P.f64C.units),
+                        K.add(N.ins), K.add(N.sets), K.add(N.dsts), K.add(N.coefs), K.add(N.pairs), K.add(N.lab),
+                        K.add(N.units), K.add(N.rots), K.add(outs)};
+    CK(K.put(lists, h->stream));
+    const DevMem& L = lists;
+    P.dev = Plan::Dev{at<GemmTask>(L, o[0]),  at<GemmTask>(L, o[1]),  at<GemmSeg>(L, o[2]),   at<GemmSeg>(L, o[3]),
+                      at<GemmTile>(L, o[4]),  at<GemmTile>(L, o[5]),  at<GemmTile>(L, o[6]),  at<GemmTile>(L, o[7]),
+                      at<int>(L, o[8]),       at<int>(L, o[9]),       at<CombOut>(L, o[10]),  at<CombTerm>(L, o[11]),
+                      at<TcStack>(L, o[12]),  at<TcStack>(L, o[13]),  at<TcRow>(L, o[14]),    at<TcRow>(L, o[15]),
+                      at<TcSeg>(L, o[16]),    at<TcSeg>(L, o[17]),    at<uint64_t>(L, o[18]), at<uint64_t>(L, o[19]),
+                      at<int4>(L, o[20]),     at<int4>(L, o[21]),     at<int4>(L, o[22]),     at<int4>(L, o[23]),
+                      at<int4>(L, o[24])};
+    P.chan_dev = CombDev{at<CombIn>(L, o[25]),  at<CombSet>(L, o[26]), at<CombDst>(L, o[27]), at<CombCoef>(L, o[28]),
+                         at<CombPair>(L, o[29]), at<uint8_t>(L, o[30]), at<int2>(L, o[31]),    at<int2>(L, o[32]),
+                         at<int>(L, o[33]),      static_cast<int>(N.outs.size()), h->d_rot.as<double>(), N.stride};
+    CK(ensure_idle(h->work1, std::max<int64_t>(1, P.t1_size) * sizeof(double), h->stream));
+    CK(ensure_idle(h->work2, std::max<int64_t>(1, P.t2_size) * sizeof(double), h->stream));
     P.ready = true;
     return SPMPS_OK;
 }
@@ -355,78 +339,84 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
         ++h->launches;
     }
     if (ev) CK(cudaEventRecord(ev[1], st));
-    // flops of a range of (op, g) entries, for the profiler
-    auto range_flops = [&](const std::vector<double>& f, int a, int b) {
-        double acc = 0.0;
-        for (int r = a; r < b && r < static_cast<int>(f.size()); ++r) acc += f[r];
-        return acc;
-    };
     // the H part (op 0) of a projected action may run on the tensor cores (precision 1 or 2)
     const int prec = P.reduce_nx > 0 ? h->apply_precision : 0;
     const int G = h->G;
     // both operators in one launch per phase: N's phase A is part of H's where the operator allows it
     // (its T1 is H's channel of identities; in FP64 only, N never runs in reduced precision)
     const bool shared = batched && prec == 0 && P.chan.shares && r0 == 0 && r1 == 2 * G;
-    auto gemm = [&](const DevMem& tasks, const DevMem& segs, const DevMem& tiles, const DevMem& cmaps,
-                    const std::vector<int>& rng, const std::vector<double>& fl, const DevMem& tc,
-                    const std::vector<int>& tc_rng, int a, int b) -> cudaError_t {
-        auto one = [&](int lo, int hi, int tf) -> cudaError_t {
-            if (hi <= lo) return cudaSuccess;
-            const TcPlan& OZ = &tasks == &P.d_tasksA ? P.ozA : P.ozC;
-            if (!tf && OZ.ok && h->opt.fp64_tensor_cores && h->tc_err.p) {
-                // FP64-accurate split products on the tensor cores over the units of [lo, hi)
-                const DevMem* d = &tasks == &P.d_tasksA ? P.d_ozA : P.d_ozC;
-                ++h->launches;
-                const int rec = h->profile ? prof_begin(h, st, 9, range_flops(fl, lo, hi)) : -1;
-                const cudaError_t e2 = launch_gemm_oz(S, d[0].as<TcStack>(), d[1].as<TcRow>(), d[2].as<TcSeg>(),
-                                                      d[3].as<uint64_t>(), cmaps.as<int>(), d[4].as<int4>(),
-                                                      OZ.unit_rng[lo], OZ.unit_rng[hi], h->tc_err.as<int>(),
-                                                      h->opt.tc_wait_polls, st);
-                if (rec >= 0) prof_end(h, st, rec);
-                return e2;
-            }
-            if (!tf && &tasks == &P.d_tasksC && P.f64C.ok) {
-                ++h->launches;
-                const int rec = h->profile ? prof_begin(h, st, 0, range_flops(fl, lo, hi)) : -1;
-                const DevMem* d = P.d_f64C;
-                const cudaError_t e2 = launch_gemm_f64_stack(S, d[0].as<TcStack>(), d[1].as<TcRow>(), d[2].as<TcSeg>(),
-                                                             d[3].as<uint64_t>(), cmaps.as<int>(), d[4].as<int4>(),
-                                                             P.f64C.unit_rng[lo], P.f64C.unit_rng[hi], st);
-                if (rec >= 0) prof_end(h, st, rec);
-                return e2;
-            }
-            const TcPlan& TP = &tasks == &P.d_tasksA ? P.stA : P.stC;
-            if (tf && split && TP.ok && h->opt.tensor_core_kernel == 0 && hi <= G) {
-                // stacked tcgen05 GEMM over the units of the H-part ranges [lo, hi)
-                const DevMem* d = &tasks == &P.d_tasksA ? P.d_stA : P.d_stC;
-                ++h->launches;
-                const int rec = h->profile ? prof_begin(h, st, 8, range_flops(fl, lo, hi)) : -1;
-                cudaError_t e2 = cudaSuccess;
-                if (!h->tc_err.p) {
-                    e2 = h->tc_err.ensure(sizeof(int));
-                    if (e2 == cudaSuccess) e2 = cudaMemsetAsync(h->tc_err.p, 0, sizeof(int), st);
-                }
-                if (e2 == cudaSuccess)
-                    e2 = launch_gemm_tc(S, *split, d[0].as<TcStack>(), d[1].as<TcRow>(), d[2].as<TcSeg>(),
-                                        d[3].as<uint64_t>(), cmaps.as<int>(), d[4].as<int4>(), TP.unit_rng[lo],
-                                        TP.unit_rng[hi], TP.nt, tf == 2, h->tc_err.as<int>(), h->opt.tc_wait_polls, st);
-                if (rec >= 0) prof_end(h, st, rec);
-                return e2;
-            }
-            const bool use_tc = tf && split;
-            const int t0 = use_tc ? tc_rng[lo] : rng[lo], t1 = use_tc ? tc_rng[hi] : rng[hi];
+    // ranges and beta points of the (op, g) range [a, b): whole operators, or beta points of one
+    struct Part {
+        int lo, hi, g0, ng;
+    };
+    auto part = [&](int a, int b) -> Part {
+        if (!P.per_op) return {a, b, 0, 1};
+        return b - a < G ? Part{a / G, a / G + 1, a % G, b - a} : Part{a / G, b / G, 0, G};
+    };
+    auto beta_run = [&](const Part& p, const std::vector<int>& rng) {
+        BetaRun r;
+        r.g0 = p.g0;
+        r.ng = p.ng;
+        if (P.per_op) {
+            r.stride = P.stride;
+            if (rng.size() > 2) r.split = rng[1];
+        }
+        return r;
+    };
+    auto range_flops = [&](const std::vector<double>& f, int lo, int hi, int ng) {
+        double acc = 0.0;
+        for (int r = lo; r < hi && r < static_cast<int>(f.size()); ++r) acc += ng * f[r];
+        return acc;
+    };
+    auto gemm = [&](bool isA, int a, int b) -> cudaError_t {
+        const Plan::Dev& D = P.dev;
+        const TcStack* stacks = isA ? D.stacksA : D.stacksC;
+        const TcRow* rows = isA ? D.rowsA : D.rowsC;
+        const TcSeg* tsegs = isA ? D.tsegsA : D.tsegsC;
+        const uint64_t* atab = isA ? D.atabA : D.atabC;
+        const int* cmaps = isA ? D.cmapsA : D.cmapsC;
+        auto one = [&](int from, int to, int tf) -> cudaError_t {
+            if (to <= from) return cudaSuccess;
+            const Part p = part(from, to);
+            const TcUnits& OZ = isA ? P.ozA : P.ozC;
+            const TcUnits& TC = isA ? P.tcA : P.tcC;
+            const bool use_oz = !tf && !OZ.rng.empty() && h->tc_err.p, use_stack = !tf && !isA && !P.f64C.rng.empty();
+            const bool use_tc = tf && split && !TC.rng.empty();
             ++h->launches;
-            const int rec = h->profile ? prof_begin(h, st, tf ? 8 : 0, range_flops(fl, lo, hi)) : -1;
-            cudaError_t e;
-            if (use_tc)
-                e = launch_gemm_tf32s(S, *split, tasks.as<GemmTask>(), segs.as<GemmSeg>(), tc.as<GemmTile>() + t0,
-                                      cmaps.as<int>(), t1 - t0, tf == 2, st);
-            else if (tf)
-                e = launch_gemm_tf32(S, tasks.as<GemmTask>(), segs.as<GemmSeg>(), tiles.as<GemmTile>() + t0,
-                                     cmaps.as<int>(), t1 - t0, tf == 2, st);
-            else
-                e = launch_gemm_f64(S, tasks.as<GemmTask>(), segs.as<GemmSeg>(), tiles.as<GemmTile>() + t0,
-                                    cmaps.as<int>(), t1 - t0, st);
+            const int rec = h->profile ? prof_begin(h, st, use_oz ? 9 : (tf ? 8 : 0),
+                                                    range_flops(isA ? P.flopsA_rng : P.flopsC_rng, p.lo, p.hi, p.ng))
+                                       : -1;
+            cudaError_t e = cudaSuccess;
+            if (use_oz) {
+                // FP64-accurate split products on the tensor cores
+                e = launch_gemm_oz(S, stacks, rows, tsegs, atab, cmaps, isA ? D.ozA : D.ozC, OZ.rng[p.lo], OZ.rng[p.hi],
+                                   h->tc_err.as<int>(), h->opt.tc_wait_polls, st, beta_run(p, OZ.rng));
+            } else if (use_stack) {
+                e = launch_gemm_f64_stack(S, stacks, rows, tsegs, atab, cmaps, D.f64C, P.f64C.rng[p.lo], P.f64C.rng[p.hi], st,
+                                          beta_run(p, P.f64C.rng));
+            } else if (use_tc) {
+                // stacked tcgen05 GEMM of the H part
+                if (!h->tc_err.p) {
+                    e = h->tc_err.ensure(sizeof(int));
+                    if (e == cudaSuccess) e = cudaMemsetAsync(h->tc_err.p, 0, sizeof(int), st);
+                }
+                if (e == cudaSuccess)
+                    e = launch_gemm_tc(S, *split, stacks, rows, tsegs, atab, cmaps, isA ? D.tcA : D.tcC, TC.rng[p.lo],
+                                       TC.rng[p.hi], TC.nt, tf == 2, h->tc_err.as<int>(), h->opt.tc_wait_polls, st,
+                                       beta_run(p, TC.rng));
+            } else if (tf && split) {
+                const std::vector<int>& rng = isA ? P.warpA_rng : P.warpC_rng;
+                BetaRun r = beta_run(p, rng);
+                r.split -= rng[p.lo];
+                e = launch_gemm_tf32s(S, *split, isA ? D.tasksA : D.tasksC, isA ? D.segsA : D.segsC,
+                                      (isA ? D.warpA : D.warpC) + rng[p.lo], cmaps, rng[p.hi] - rng[p.lo], tf == 2, st, r);
+            } else {
+                const std::vector<int>& rng = isA ? P.tileA_rng : P.tileC_rng;
+                BetaRun r = beta_run(p, rng);
+                r.split -= rng[p.lo];
+                e = launch_gemm_f64(S, isA ? D.tasksA : D.tasksC, isA ? D.segsA : D.segsC,
+                                    (isA ? D.tilesA : D.tilesC) + rng[p.lo], cmaps, rng[p.hi] - rng[p.lo], st, r);
+            }
             if (rec >= 0) prof_end(h, st, rec);
             return e;
         };
@@ -460,27 +450,23 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
         if (e != cudaSuccess) return e;
         return cudaStreamWaitEvent(st, h->aux_join, 0);
     };
-    auto runA = [&](int a, int b) -> cudaError_t {
-        return gemm(P.d_tasksA, P.d_segsA, P.d_tilesA, P.d_cmapsA, P.tileA_rng, P.flopsA_rng, P.d_tcA, P.tcA_rng, a, b);
-    };
+    auto runA = [&](int a, int b) -> cudaError_t { return gemm(true, a, b); };
+    auto runC = [&](int a, int b) -> cudaError_t { return gemm(false, a, b); };
     auto runB = [&](int a, int b) -> cudaError_t {
-        if (!P.chan.unit_rng.empty()) {  // (op, g) ranges: whole operators, or one beta point of one
-            const int rec = h->profile ? prof_begin(h, st, 1, range_flops(P.flopsB_rng, a, b)) : -1;
+        if (!P.chan.unit_rng.empty()) {
             const bool single = b - a < G;
-            const cudaError_t e = launch_comb_chan(S, P.chan, P.chan_dev, a / G, single ? a / G + 1 : b / G, single ? a % G : 0,
-                                                   single ? b - a : G, shared, &h->launches, st);
+            const Part p = single ? Part{a / G, a / G + 1, a % G, b - a} : Part{a / G, b / G, 0, G};
+            const int rec = h->profile ? prof_begin(h, st, 1, range_flops(P.flopsB_rng, a, b, 1)) : -1;
+            const cudaError_t e = launch_comb_chan(S, P.chan, P.chan_dev, p.lo, p.hi, p.g0, p.ng, shared, &h->launches, st);
             if (rec >= 0) prof_end(h, st, rec);
             return e;
         }
         const int o0 = P.combB_rng[a], o1 = P.combB_rng[b];
         ++h->launches;
-        const int rec = h->profile ? prof_begin(h, st, 1, range_flops(P.flopsB_rng, a, b)) : -1;
-        cudaError_t e = launch_comb_f64(S, P.d_outsB.as<CombOut>() + o0, P.d_termsB.as<CombTerm>(), o1 - o0, st);
+        const int rec = h->profile ? prof_begin(h, st, 1, range_flops(P.flopsB_rng, a, b, 1)) : -1;
+        cudaError_t e = launch_comb_f64(S, P.dev.outsB + o0, P.dev.termsB, o1 - o0, st);
         if (rec >= 0) prof_end(h, st, rec);
         return e;
-    };
-    auto runC = [&](int a, int b) -> cudaError_t {
-        return gemm(P.d_tasksC, P.d_segsC, P.d_tilesC, P.d_cmapsC, P.tileC_rng, P.flopsC_rng, P.d_tcC, P.tcC_rng, a, b);
     };
     // tensor-core phases read pre-split operands: x before phase A, the phase-B output before C
     const bool pre_split = prec > 0 && split && r0 < G;
@@ -610,8 +596,10 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
     const int ngl = static_cast<int>(bl.groups.size()), ngr = static_cast<int>(br.groups.size());
     P.A.clear(); P.B.clear(); P.C.clear();
     P.task_rng_kept = false;
-    P.tileA_rng.assign(nops * G + 1, 0);
-    P.tileC_rng.assign(nops * G + 1, 0);
+    P.per_op = true;
+    P.stride = BetaStride();
+    P.tileA_rng.assign(nops + 1, 0);
+    P.tileC_rng.assign(nops + 1, 0);
     P.flopsB_rng.clear();
     // column maps of the site's row blocks into the N-dense T1 columns (depend on the label only)
     std::vector<int> cmap_off(bl.labels.size(), -1);
@@ -685,11 +673,15 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
         sp.needed = [&](int la, int s) { return al.seg_label[la * 4 + s] >= 0; };
         const double fb = comb_add(P.chan, sp);
         P.B.flops += G * fb;
-        for (int g = 0; g < G; ++g) {
-            const int og = op * G + g;
-            P.flopsB_rng.push_back(fb);
-            P.tileA_rng[og] = static_cast<int>(P.A.tasks.size());
-            P.tileC_rng[og] = static_cast<int>(P.C.tasks.size());
+        P.flopsB_rng.insert(P.flopsB_rng.end(), G, fb);
+        P.stride.s[op][3] = s1;
+        P.stride.s[op][4] = s2;
+        P.stride.s[op][5] = Lo.lay[op].size;
+        P.stride.s[op][7] = Ln.lay[op].size;
+        {
+            const int og = op * G;  // beta point 0 stands for all
+            P.tileA_rng[op] = static_cast<int>(P.A.tasks.size());
+            P.tileC_rng[op] = static_cast<int>(P.C.tasks.size());
             // phase A
             for (int w = 0; w < dwl; ++w)
                 for (int ga = 0; ga < ngl; ++ga) {
@@ -700,7 +692,7 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
                         if (al.width[l] == 0) continue;
                         const Label& Ll = bl.labels[l];
                         GemmTask T{};
-                        T.c = handle(3, o1[w * ngl + ga] + g * s1);
+                        T.c = handle(3, o1[w * ngl + ga]);
                         T.cmap = cmap_off[l];
                         T.M = bl.groups[ga].dim;
                         T.N = al.width[l];
@@ -717,7 +709,7 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
                         sg.b_cs = 1;
                         P.A.segs.push_back(sg);
                         P.A.tasks.push_back(T);
-                        P.A.flops += 2.0 * T.M * T.N * sg.K;
+                        P.A.flops += 2.0 * G * T.M * T.N * sg.K;
                     }
                 }
             // phase C: Lnew[u][Gb][lb rows, :] = sum_{la, s: la+q(s)=lb} A[la,s,lb]^T T2[u][Ga(la)][la rows, s cols]
@@ -747,12 +739,12 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
                             sg.a_rs = 1;
                             sg.a_cs = al.width[la];
                             sg.K = La.dim;
-                            sg.b = handle(4, o2[u * ngl + ga] + g * s2 +
+                            sg.b = handle(4, o2[u * ngl + ga] +
                                                  static_cast<int64_t>(La.off - bl.groups[ga].off) * C2.width + C2.col[s]);
                             sg.b_rs = C2.width;
                             sg.b_cs = 1;
                             P.C.segs.push_back(sg);
-                            P.C.flops += 2.0 * T.M * T.N * sg.K;
+                            P.C.flops += 2.0 * G * T.M * T.N * sg.K;
                         }
                         T.nseg = static_cast<int>(P.C.segs.size()) - T.seg0;
                         P.C.tasks.push_back(T);
@@ -761,8 +753,8 @@ void build_left_plan(spmps_t* h, int i, const EnvStore& Lo, const EnvStore& Ln, 
         }
     }
     P.zero_t1 = P.chan.zero_t1;
-    P.tileA_rng[nops * G] = static_cast<int>(P.A.tasks.size());
-    P.tileC_rng[nops * G] = static_cast<int>(P.C.tasks.size());
+    P.tileA_rng[nops] = static_cast<int>(P.A.tasks.size());
+    P.tileC_rng[nops] = static_cast<int>(P.C.tasks.size());
     P.t1_size = t1;
     P.t2_size = t2;
     P.flops = P.A.flops + P.B.flops + P.C.flops;
@@ -778,8 +770,10 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
     const int ngl = static_cast<int>(bl.groups.size()), ngr = static_cast<int>(br.groups.size());
     P.A.clear(); P.B.clear(); P.C.clear();
     P.task_rng_kept = false;
-    P.tileA_rng.assign(nops * G + 1, 0);
-    P.tileC_rng.assign(nops * G + 1, 0);
+    P.per_op = true;
+    P.stride = BetaStride();
+    P.tileA_rng.assign(nops + 1, 0);
+    P.tileC_rng.assign(nops + 1, 0);
     P.flopsB_rng.clear();
     int64_t t1 = 0, t2 = 0;
     P.chan.clear();
@@ -837,11 +831,15 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
         };
         const double fb = comb_add(P.chan, sp);
         P.B.flops += G * fb;
-        for (int g = 0; g < G; ++g) {
-            const int og = op * G + g;
-            P.flopsB_rng.push_back(fb);
-            P.tileA_rng[og] = static_cast<int>(P.A.tasks.size());
-            P.tileC_rng[og] = static_cast<int>(P.C.tasks.size());
+        P.flopsB_rng.insert(P.flopsB_rng.end(), G, fb);
+        P.stride.s[op][3] = s1;
+        P.stride.s[op][4] = s2;
+        P.stride.s[op][6] = Ro.lay[op].size;
+        P.stride.s[op][7] = Rn.lay[op].size;
+        {
+            const int og = op * G;  // beta point 0 stands for all
+            P.tileA_rng[op] = static_cast<int>(P.A.tasks.size());
+            P.tileC_rng[op] = static_cast<int>(P.C.tasks.size());
             // phase A: T1[u][Gb][b, (t, a')] = sum_b' R[u][b, b'] A[a', t, b']
             for (int u = 0; u < dwr; ++u)
                 for (int gb = 0; gb < ngr; ++gb) {
@@ -856,7 +854,7 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                             if (lap < 0 || al.seg_label[lap * 4 + t] != lbp) continue;
                             const Label& Lap = bl.labels[lap];
                             GemmTask T{};
-                            T.c = handle(3, o1[u * ngr + gb] + g * s1 + CL.col[t] + (Lap.off - bl.groups[Lap.group].off));
+                            T.c = handle(3, o1[u * ngr + gb] + CL.col[t] + (Lap.off - bl.groups[Lap.group].off));
                             T.cmap = -1;
                             T.M = br.groups[gb].dim;
                             T.N = Lap.dim;
@@ -873,7 +871,7 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                             sg.b_cs = al.width[lap];
                             P.A.segs.push_back(sg);
                             P.A.tasks.push_back(T);
-                            P.A.flops += 2.0 * T.M * T.N * sg.K;
+                            P.A.flops += 2.0 * G * T.M * T.N * sg.K;
                         }
                     }
                 }
@@ -905,12 +903,12 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
                             sg.a_rs = al.width[la];
                             sg.a_cs = 1;
                             sg.K = Lb.dim;
-                            sg.b = handle(4, o2[w * ngr + gb] + g * s2 +
+                            sg.b = handle(4, o2[w * ngr + gb] +
                                                  static_cast<int64_t>(Lb.off - br.groups[gb].off) * C2.width + C2.col[s]);
                             sg.b_rs = C2.width;
                             sg.b_cs = 1;
                             P.C.segs.push_back(sg);
-                            P.C.flops += 2.0 * T.M * T.N * sg.K;
+                            P.C.flops += 2.0 * G * T.M * T.N * sg.K;
                         }
                         T.nseg = static_cast<int>(P.C.segs.size()) - T.seg0;
                         P.C.tasks.push_back(T);
@@ -919,8 +917,8 @@ void build_right_plan(spmps_t* h, int i, const EnvStore& Ro, const EnvStore& Rn,
         }
     }
     P.zero_t1 = P.chan.zero_t1;
-    P.tileA_rng[nops * G] = static_cast<int>(P.A.tasks.size());
-    P.tileC_rng[nops * G] = static_cast<int>(P.C.tasks.size());
+    P.tileA_rng[nops] = static_cast<int>(P.A.tasks.size());
+    P.tileC_rng[nops] = static_cast<int>(P.C.tasks.size());
     P.t1_size = t1;
     P.t2_size = t2;
     P.flops = P.A.flops + P.B.flops + P.C.flops;
@@ -987,8 +985,13 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
     const int ngl = static_cast<int>(bl.groups.size()), ngr = static_cast<int>(br.groups.size());
     P.A.clear(); P.B.clear(); P.C.clear();
     P.task_rng_kept = false;
-    P.tileA_rng.assign(nops * G + 1, 0);
-    P.tileC_rng.assign(nops * G + 1, 0);
+    // unscreened: the lists hold one beta point per operator; screened: every beta point, its own products
+    P.per_op = !screen;
+    P.stride = BetaStride();
+    const int Gl = screen ? G : 1;
+    const double reps = screen ? 1.0 : G;
+    P.tileA_rng.assign(nops * Gl + 1, 0);
+    P.tileC_rng.assign(nops * Gl + 1, 0);
     P.flopsB_rng.clear();
     for (double& f : P.flops_op) f = 0.0;
     std::vector<int> cmap_off(bl.labels.size(), -1);
@@ -1083,10 +1086,14 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
         P.B.flops += G * fb;
         P.flopsB_op[op] += G * fb;
         const double fa0 = P.A.flops;
-        for (int g = 0; g < G; ++g) {
+        P.flopsB_rng.insert(P.flopsB_rng.end(), G, fb);
+        P.stride.s[op][3] = s1;
+        P.stride.s[op][4] = s3;
+        P.stride.s[op][5] = Le.lay[op].size;
+        P.stride.s[op][6] = Re.lay[op].size;
+        for (int g = 0; g < Gl; ++g) {
             const int og = op * G + g;
-            P.flopsB_rng.push_back(fb);
-            P.tileA_rng[og] = static_cast<int>(P.A.tasks.size());
+            P.tileA_rng[op * Gl + g] = static_cast<int>(P.A.tasks.size());
             // phase A
             for (int w = 0; w < dwl; ++w)
                 for (int ga = 0; ga < ngl; ++ga) {
@@ -1126,7 +1133,7 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
                             sg.b_cs = 1;
                             P.A.segs.push_back(sg);
                             P.A.tasks.push_back(T);
-                            P.A.flops += 2.0 * T.M * T.N * sg.K;
+                            P.A.flops += reps * 2.0 * T.M * T.N * sg.K;
                         }
                     }
                 }
@@ -1164,9 +1171,10 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
                 u_of[q] = u;
             }
         }
-        for (int g = 0; g < G; ++g) {
+        P.stride.s[op][8 + op] = static_cast<int64_t>(ks) * nx;
+        for (int g = 0; g < Gl; ++g) {
             const int og = op * G + g;
-            P.tileC_rng[og] = static_cast<int>(P.C.tasks.size());
+            P.tileC_rng[op * Gl + g] = static_cast<int>(P.C.tasks.size());
             for (int slice = 0; slice < ks; ++slice)
             for (size_t la = 0; la < bl.labels.size(); ++la) {
                 const Label& La = bl.labels[la];
@@ -1211,7 +1219,7 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
                             sg.b_rs = 1;
                             sg.b_cs = K;
                             P.C.segs.push_back(sg);
-                            P.C.flops += 2.0 * T.M * T.N * kl;
+                            P.C.flops += reps * 2.0 * T.M * T.N * kl;
                         }
                     }
                     T.nseg = static_cast<int>(P.C.segs.size()) - T.seg0;
@@ -1225,8 +1233,8 @@ void build_apply_plan(spmps_t* h, int k, const EnvStore& Le, const EnvStore& Re,
         P.bytesC_op[op] = 8.0 * static_cast<double>(G) * (P.chan.stride.t3[op] + Re.lay[op].size + nx);
     }
     P.reduce_nx = nx;
-    P.tileA_rng[nops * G] = static_cast<int>(P.A.tasks.size());
-    P.tileC_rng[nops * G] = static_cast<int>(P.C.tasks.size());
+    P.tileA_rng[nops * Gl] = static_cast<int>(P.A.tasks.size());
+    P.tileC_rng[nops * Gl] = static_cast<int>(P.C.tasks.size());
     P.t1_size = t1;
     P.t2_size = t3;
     P.flops = P.A.flops + P.B.flops + P.C.flops;
@@ -1334,7 +1342,7 @@ spmps_status update_left(spmps_t* h, int i) {
         std::string why;
         if (!validate_plan(P, sz, &why, h->G)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (left update): " + why);
     }
-    st = plan_upload(h, P);
+    st = plan_upload(h, P, h->once);
     if (st != SPMPS_OK) return st;
     Slots S{};
     S.p[0] = h->A[i]->as<double>();
@@ -1344,7 +1352,6 @@ spmps_status update_left(spmps_t* h, int i) {
     S.p[7] = Ln.buf.as<double>();
     st = plan_run(h, P, S, 0, h->ops.n_ops() * h->G, h->stream);
     if (st != SPMPS_OK) return st;
-    CK(cudaStreamSynchronize(h->stream));  // plan buffers are freed on return
     Ln.valid = true;
     Ln.version = ++h->env_counter;
     return SPMPS_OK;
@@ -1368,7 +1375,7 @@ spmps_status update_right(spmps_t* h, int i) {
         std::string why;
         if (!validate_plan(P, sz, &why, h->G)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (right update): " + why);
     }
-    st = plan_upload(h, P);
+    st = plan_upload(h, P, h->once);
     if (st != SPMPS_OK) return st;
     Slots S{};
     S.p[0] = h->A[i]->as<double>();
@@ -1378,7 +1385,6 @@ spmps_status update_right(spmps_t* h, int i) {
     S.p[7] = Rn.buf.as<double>();
     st = plan_run(h, P, S, 0, h->ops.n_ops() * h->G, h->stream);
     if (st != SPMPS_OK) return st;
-    CK(cudaStreamSynchronize(h->stream));
     Rn.valid = true;
     Rn.version = ++h->env_counter;
     return SPMPS_OK;
@@ -1442,7 +1448,7 @@ spmps_status tune_apply_plan(spmps_t* h, int k, Plan& P) {
         spmps_status st = SPMPS_OK;
         for (int c = 0; c < kTileCandidates && st == SPMPS_OK; ++c) {
             P.polA = P.polC = tile_candidate(c);
-            st = plan_upload(h, P);
+            st = plan_upload(h, P, P.lists);
             if (st != SPMPS_OK) break;
             Slots S{};
             S.p[0] = h->tunebuf.as<double>();
@@ -1516,9 +1522,9 @@ spmps_status get_apply_plan(spmps_t* h, int k, Plan** out) {
             st = tune_apply_plan(h, k, *P);
             if (st != SPMPS_OK) return st;
         }
-        st = plan_upload(h, *P);
+        st = plan_upload(h, *P, P->lists);
         if (st != SPMPS_OK) return st;
-        CK(h->work3.ensure(std::max<int64_t>(1, P->partial_size(h->G)) * sizeof(double)));
+        CK(ensure_idle(h->work3, std::max<int64_t>(1, P->partial_size(h->G)) * sizeof(double), h->stream));
         h->apply_plans[k] = std::move(P);
     }
     *out = h->apply_plans[k].get();
@@ -2197,16 +2203,15 @@ spmps_status spmps_two_site(spmps_handle h, int site, double* x) {
         std::string why;
         if (!validate_plan(P, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (two-site): " + why);
     }
-    CK(upload(P.d_tasksA, P.A.tasks, h->stream));
-    CK(upload(P.d_segsA, P.A.segs, h->stream));
-    CK(upload(P.d_tilesA, P.A.tiles, h->stream));
-    CK(upload(P.d_cmapsA, P.A.cmaps, h->stream));
+    Packer K(h->staging);
+    const size_t ot = K.add(P.A.tasks), os = K.add(P.A.segs), oi = K.add(P.A.tiles), oc = K.add(P.A.cmaps);
+    CK(K.put(h->once, h->stream));
     Slots S{};
     S.p[0] = h->A[site]->as<double>();
     S.p[1] = h->A[site + 1]->as<double>();
     S.p[2] = x;
-    CK(launch_gemm_f64(S, P.d_tasksA.as<GemmTask>(), P.d_segsA.as<GemmSeg>(), P.d_tilesA.as<GemmTile>(),
-                       P.d_cmapsA.as<int>(), static_cast<int>(P.A.tiles.size()), h->stream));
+    CK(launch_gemm_f64(S, at<GemmTask>(h->once, ot), at<GemmSeg>(h->once, os), at<GemmTile>(h->once, oi),
+                       at<int>(h->once, oc), static_cast<int>(P.A.tiles.size()), h->stream));
     ++h->launches;
     CK(cudaStreamSynchronize(h->stream));
     return SPMPS_OK;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <memory>
 #include <string>
 #include <vector>
@@ -44,6 +45,61 @@ struct DevMem {
         return cudaSuccess;
     }
     template <class T> T* as() const { return static_cast<T*>(p); }
+};
+
+// Grows a buffer that work queued on `st` may still use: that work is finished first.
+inline cudaError_t ensure_idle(DevMem& m, size_t bytes, cudaStream_t st) {
+    if (bytes > m.bytes && m.p) {
+        const cudaError_t e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return e;
+    }
+    return m.ensure(bytes);
+}
+
+// Host-to-device copies of work lists: an image put together on the host goes through one of two pinned
+// buffers, each reused once its last copy is done.
+struct Staging {
+    std::vector<unsigned char> image;
+    struct Pinned {
+        void* p = nullptr;
+        size_t bytes = 0;
+        cudaEvent_t done = nullptr;
+    } pinned[2];
+    int turn = 0;
+    Staging() = default;
+    Staging(const Staging&) = delete;
+    Staging& operator=(const Staging&) = delete;
+    ~Staging() {
+        for (Pinned& b : pinned) {
+            if (b.done) {
+                cudaEventSynchronize(b.done);
+                cudaEventDestroy(b.done);
+            }
+            if (b.p) cudaFreeHost(b.p);
+        }
+    }
+    cudaError_t copy(void* dst, cudaStream_t st) {
+        if (image.empty()) return cudaSuccess;
+        turn ^= 1;
+        Pinned& b = pinned[turn];
+        cudaError_t e = b.done ? cudaEventSynchronize(b.done) : cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+        if (image.size() > b.bytes) {
+            if (b.p) cudaFreeHost(b.p);
+            b.p = nullptr;
+            b.bytes = 0;
+            const size_t want = image.size() + image.size() / 2 + 65536;
+            e = cudaMallocHost(&b.p, want);
+            if (e != cudaSuccess) {
+                b.p = nullptr;
+                return e;
+            }
+            b.bytes = want;
+        }
+        std::memcpy(b.p, image.data(), image.size());
+        e = cudaMemcpyAsync(dst, b.p, image.size(), cudaMemcpyHostToDevice, st);
+        return e == cudaSuccess ? cudaEventRecord(b.done, st) : e;
+    }
 };
 
 // Doubles of the fixed scratch of spmps_apply_heff_noalloc (32 MiB), and what an action needs of it.
@@ -120,17 +176,29 @@ struct Plan {
     double flops_op[4] = {0, 0, 0, 0};
     double bytesA_op[4] = {0, 0, 0, 0}, bytesB_op[4] = {0, 0, 0, 0}, bytesC_op[4] = {0, 0, 0, 0};
     double flopsA_op[4] = {0, 0, 0, 0}, flopsB_op[4] = {0, 0, 0, 0}, flopsC_op[4] = {0, 0, 0, 0};
-    DevMem d_tasksA, d_segsA, d_tilesA, d_cmapsA, d_outsB, d_termsB, d_tasksC, d_segsC, d_tilesC, d_cmapsC;
-    DevMem d_chan[9];                        // the arrays of chan
+    // The lists of H's and N's plans hold one beta point (range = operator); the kernels add the strides.  The
+    // lists of screened and cross plans hold every beta point (range = op * G + g).
+    bool per_op = false;
+    BetaStride stride;
+    TcPlan stackA, stackC;                   // stacks of all ranges, phases A and C
+    TcUnits tcA, tcC, ozA, ozC, f64C;        // their units for the 3xTF32, split-product and FP64-pipe kernels
+    std::vector<int> warpA_rng, warpC_rng;   // ranges of the mma.sync tiles
+    // every list on the device, in one allocation (filled by plan_upload)
+    DevMem lists;
+    struct Dev {
+        const GemmTask *tasksA, *tasksC;
+        const GemmSeg *segsA, *segsC;
+        const GemmTile *tilesA, *tilesC, *warpA, *warpC;
+        const int *cmapsA, *cmapsC;
+        const CombOut* outsB;
+        const CombTerm* termsB;
+        const TcStack *stacksA, *stacksC;
+        const TcRow *rowsA, *rowsC;
+        const TcSeg *tsegsA, *tsegsC;
+        const uint64_t *atabA, *atabC;
+        const int4 *tcA, *tcC, *ozA, *ozC, *f64C;
+    } dev{};
     CombDev chan_dev{};
-    DevMem d_tcA, d_tcC;                     // tensor-core tile lists
-    std::vector<int> tcA_rng, tcC_rng;       // their ranges per (op, g)
-    TcPlan stA, stC;                         // tcgen05 stacks of the H part, phases A and C
-    DevMem d_stA[5], d_stC[5];               // their stacks, rows, segments, A table, units
-    TcPlan ozA, ozC;                         // stacks of all (op, g) ranges for the FP64-accurate
-    TcPlan f64C;                             // stacks of phase C on the FP64 pipe (actions only)
-    DevMem d_f64C[5];
-    DevMem d_ozA[5], d_ozC[5];               // split-product GEMM (fp64_tensor_cores)
     // diagonal (apply plans only)
     std::vector<DiagBlock> diag_blocks;
     std::vector<DiagTerm> diag_terms;
@@ -189,6 +257,10 @@ struct spmps_t {
     // the integrals of the Hamiltonian (kept for the fragment energies); empty after spmps_set_mpo
     std::vector<double> ints_h1, ints_h2;
     double ints_ecore = 0.0;
+    // device lists of plans that run once (environment updates, two-site tensors, decimations): one
+    // buffer, rewritten in stream order
+    spmps::DevMem once;
+    spmps::Staging staging;
     // autotuner: chosen tile candidate per site for phases A and C (-1 = not tuned yet)
     std::vector<int> tune_a, tune_c;
     spmps::DevMem tunebuf;
@@ -234,9 +306,30 @@ cudaError_t upload(DevMem& m, const std::vector<T>& v, cudaStream_t st) {
     return cudaMemcpyAsync(m.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st);
 }
 
+// Host vectors packed into one device buffer: add() gives each its offset, put() copies them all in stream
+// order.
+struct Packer {
+    Staging& S;
+    explicit Packer(Staging& staging) : S(staging) { S.image.clear(); }
+    template <class T>
+    size_t add(const std::vector<T>& v) {
+        const size_t at = (S.image.size() + 255) / 256 * 256;
+        S.image.resize(at + std::max<size_t>(1, v.size()) * sizeof(T));
+        if (!v.empty()) std::memcpy(S.image.data() + at, v.data(), v.size() * sizeof(T));
+        return at;
+    }
+    cudaError_t put(DevMem& m, cudaStream_t st) {
+        cudaError_t e = ensure_idle(m, std::max<size_t>(1, S.image.size()), st);
+        return e == cudaSuccess ? S.copy(m.p, st) : e;
+    }
+};
+template <class T>
+const T* at(const DevMem& m, size_t off) { return reinterpret_cast<const T*>(static_cast<const char*>(m.p) + off); }
+
 bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why, int G = 1);
-bool validate_gemm(const GemmPlan& G, const int64_t* sizes, std::string* why);
-spmps_status plan_upload(spmps_t* h, Plan& P);
+bool validate_gemm(const GemmPlan& G, const int64_t* sizes, std::string* why, const BetaStride* stride = nullptr,
+                   int op1 = 1 << 30, int copies = 1);
+spmps_status plan_upload(spmps_t* h, Plan& P, DevMem& lists);
 spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t st, cudaEvent_t* ev = nullptr,
                       const SlotsF* split = nullptr);
 spmps_status update_left(spmps_t* h, int i);

@@ -482,7 +482,7 @@ void build_cross_B(spmps_t* h, const LowerState& Ls, int k, const EnvStore& Le, 
 spmps_status run_checked(spmps_t* h, Plan& P, const int64_t* sz, const char* what, Slots S) {
     std::string why;
     if (!validate_plan(P, sz, &why)) return fail(h, SPMPS_ERR_CUDA, std::string("internal plan check (") + what + "): " + why);
-    spmps_status st = plan_upload(h, P);
+    spmps_status st = plan_upload(h, P, h->once);
     if (st != SPMPS_OK) return st;
     S.p[3] = h->work1.as<double>();
     S.p[4] = h->work2.as<double>();
@@ -623,16 +623,15 @@ spmps_status lower_two_site(spmps_t* h, const LowerState& Ls, int k, DevMem& x0,
     std::string why;
     if (!validate_plan(P, sz, &why)) return fail(h, SPMPS_ERR_CUDA, "internal plan check (lower two-site): " + why);
     CK(x0.ensure(std::max<int64_t>(1, xl.size) * sizeof(double)));
-    CK(upload(P.d_tasksA, P.A.tasks, h->stream));
-    CK(upload(P.d_segsA, P.A.segs, h->stream));
-    CK(upload(P.d_tilesA, P.A.tiles, h->stream));
-    CK(upload(P.d_cmapsA, P.A.cmaps, h->stream));
+    Packer K(h->staging);
+    const size_t ot = K.add(P.A.tasks), os = K.add(P.A.segs), oi = K.add(P.A.tiles), oc = K.add(P.A.cmaps);
+    CK(K.put(h->once, h->stream));
     Slots S{};
     S.p[0] = Ls.A[k]->as<double>();
     S.p[1] = Ls.A[k + 1]->as<double>();
     S.p[2] = x0.as<double>();
-    CK(launch_gemm_f64(S, P.d_tasksA.as<GemmTask>(), P.d_segsA.as<GemmSeg>(), P.d_tilesA.as<GemmTile>(),
-                       P.d_cmapsA.as<int>(), static_cast<int>(P.A.tiles.size()), h->stream));
+    CK(launch_gemm_f64(S, at<GemmTask>(h->once, ot), at<GemmSeg>(h->once, os), at<GemmTile>(h->once, oi),
+                       at<int>(h->once, oc), static_cast<int>(P.A.tiles.size()), h->stream));
     ++h->launches;
     CK(cudaStreamSynchronize(h->stream));
     *n0 = xl.size;

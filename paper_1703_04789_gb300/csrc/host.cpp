@@ -145,12 +145,12 @@ int fill_elems(int64_t outputs, int elems) {
     return static_cast<int>(std::min<int64_t>(std::min(elems, 256), std::max<int64_t>(32, (outputs / kFillWarps + 31) / 32 * 32)));
 }
 
-void GemmPlan::add_tiles(const TilePolicy& pol) {
+void GemmPlan::add_tiles(const TilePolicy& pol, int copies) {
     // register-tiled shapes 0..4 (rows x cols per warp); shape 5 = warp block
     static const int shp[5][2] = {{16, 16}, {4, 64}, {64, 4}, {32, 8}, {8, 32}};
     tiles.clear();
     int64_t outputs = 0;
-    for (const GemmTask& T : tasks) outputs += static_cast<int64_t>(T.M) * T.N;
+    for (const GemmTask& T : tasks) outputs += static_cast<int64_t>(T.M) * T.N * copies;
     const int elems = fill_elems(outputs, pol.wb_elems);
     const bool small = outputs < 128 * kFillWarps;
     std::map<std::pair<int, int>, BlockSplit> splits;

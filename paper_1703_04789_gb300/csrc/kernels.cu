@@ -23,13 +23,27 @@ __device__ __forceinline__ void cp_async8(double* dst, const double* src) {
                  "l"(src));
 }
 
+__device__ __forceinline__ double* resolve(double* const* base, uint64_t h) {
+    return base[h >> 56] + static_cast<int64_t>(h & 0x00FFFFFFFFFFFFFFull);
+}
+
+// This warp's base pointers (its beta point and operator) into its row of a shared table.
+__device__ __forceinline__ double* const* warp_bases(const Slots& S, const BetaStride& B, int op, int g,
+                                                     double* (*table)[kMaxSlots]) {
+    const int lane = threadIdx.x & 31;
+    double** mine = table[threadIdx.x >> 5];
+    if (lane < kMaxSlots) mine[lane] = S.p[lane] + g * B.s[op][lane];
+    __syncwarp();
+    return mine;
+}
+
 // ---- grouped FP64 GEMM ----------------------------------------------------------------------
 // Tile shapes (rows x cols per warp; each lane owns RM x CN outputs on a LR x LC lane grid):
 //   0: 16 x 16  (LR 8, LC 4, RM 2, CN 4)      1: 4 x 64  (LR 4, LC 8, RM 1, CN 8)
 //   2: 64 x 4   (LR 8, LC 4, RM 8, CN 1)      3: 32 x 8  (LR 8, LC 4, RM 4, CN 2)
 //   4: 8 x 32   (LR 4, LC 8, RM 2, CN 4)
 template <int LR, int LC, int RM, int CN>
-__device__ __forceinline__ void gemm_tile(const Slots& S, const GemmTask& T, const GemmSeg* __restrict__ segs,
+__device__ __forceinline__ void gemm_tile(double* const* S, const GemmTask& T, const GemmSeg* __restrict__ segs,
                                           const int* __restrict__ cmaps, int m0, int n0, int lane) {
     const int lr = lane / LC, lc = lane % LC;
     int rows[RM], cols[CN];
@@ -94,7 +108,7 @@ constexpr int kWbSlice = 2 * 32 * kWbStride;     // doubles of one stage (A rows
 constexpr int kWbWarpSmem = 2 * kWbSlice;        // per warp
 
 template <int NQ>
-__device__ __forceinline__ void gemm_tile_wb(const Slots& S, const GemmTask& T, const GemmSeg* __restrict__ segs,
+__device__ __forceinline__ void gemm_tile_wb(double* const* S, const GemmTask& T, const GemmSeg* __restrict__ segs,
                                              const int* __restrict__ cmaps, int m0, int n0, int tm, int tn, int lane,
                                              double* __restrict__ sm) {
     const int nout = tm * tn;
@@ -175,15 +189,19 @@ __device__ __forceinline__ void gemm_tile_wb(const Slots& S, const GemmTask& T, 
     }
 }
 
-__global__ void __launch_bounds__(128, 5) k_gemm_f64(Slots S, const GemmTask* __restrict__ tasks,
-                                                  const GemmSeg* __restrict__ segs, const GemmTile* __restrict__ tiles,
-                                                  const int* __restrict__ cmaps, int n_tiles) {
+__global__ void __launch_bounds__(128, 5) k_gemm_f64(const __grid_constant__ Slots P, const __grid_constant__ BetaStride Bs,
+                                                     int n0, int g0, int ng, const GemmTask* __restrict__ tasks,
+                                                     const GemmSeg* __restrict__ segs, const GemmTile* __restrict__ tiles,
+                                                     const int* __restrict__ cmaps, int n_tiles) {
     __shared__ double wb_smem[4 * kWbWarpSmem];
+    __shared__ double* table[4][kMaxSlots];
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (warp >= n_tiles) return;
-    const GemmTile tl = tiles[warp];
+    if (warp >= n_tiles * ng) return;
+    const LaunchItem it = launch_item(warp, n_tiles, n0, ng);
+    const GemmTile tl = tiles[it.entry];
     const GemmTask T = tasks[tl.task];
+    double* const* S = warp_bases(P, Bs, it.op, g0 + it.g, table);
     if (tl.shape == 5) {
         double* sm = wb_smem + (threadIdx.x >> 5) * kWbWarpSmem;
         const int nq = (tl.tm * tl.tn + 31) / 32;
@@ -217,7 +235,7 @@ __global__ void __launch_bounds__(128, 5) k_gemm_f64(Slots S, const GemmTask* __
 // the FP64 pipe.  Measured (GB300, phase C of the middle action of the L = 24, D = 256
 // chain, 494 Mflop): 0.494 ms; one block at a time per warp took 0.647 ms (28 % of the lanes idle).
 template <int NQ>
-__device__ __forceinline__ void stack_tile(const Slots& S, const TcStack& st, const TcRow* __restrict__ rows,
+__device__ __forceinline__ void stack_tile(double* const* S, const TcStack& st, const TcRow* __restrict__ rows,
                                            const TcSeg* __restrict__ segs, const uint64_t* __restrict__ atab,
                                            const int* __restrict__ cmaps, int m0, int n0, int tm, int tn, int lane,
                                            double* __restrict__ sm) {
@@ -300,16 +318,21 @@ __device__ __forceinline__ void stack_tile(const Slots& S, const TcStack& st, co
     }
 }
 
-__global__ void __launch_bounds__(128, 5) k_gemm_f64_stack(Slots S, const TcStack* __restrict__ stacks,
+__global__ void __launch_bounds__(128, 5) k_gemm_f64_stack(const __grid_constant__ Slots P,
+                                                           const __grid_constant__ BetaStride Bs, int n0, int g0, int ng,
+                                                           const TcStack* __restrict__ stacks,
                                                            const TcRow* __restrict__ rows, const TcSeg* __restrict__ segs,
                                                            const uint64_t* __restrict__ atab, const int* __restrict__ cmaps,
-                                                           const int4* __restrict__ units, int n_units) {
+                                                           const int4* __restrict__ units, int u0, int u1) {
     __shared__ double smem[4 * kWbWarpSmem];
-    const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (u >= n_units) return;
-    const int4 U = units[u];
+    __shared__ double* table[4][kMaxSlots];
+    const int id = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (id >= (u1 - u0) * ng) return;
+    const LaunchItem it = launch_item(id, u1 - u0, n0, ng);
+    const int4 U = units[u0 + it.entry];
     const TcStack st = stacks[U.x];
     const int tm = U.w & 0xFFFF, tn = U.w >> 16;
+    double* const* S = warp_bases(P, Bs, it.op, g0 + it.g, table);
     double* sm = smem + (threadIdx.x >> 5) * kWbWarpSmem;
     switch ((tm * tn + 31) / 32) {
         case 1: stack_tile<1>(S, st, rows, segs, atab, cmaps, U.y, U.z, tm, tn, lane, sm); break;
@@ -346,7 +369,7 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__
 }
 
 // ---- block linear combination (MPO legs) ------------------------------------------------------
-__global__ void __launch_bounds__(256) k_comb_f64(Slots S, const CombOut* __restrict__ outs,
+__global__ void __launch_bounds__(256) k_comb_f64(const __grid_constant__ Slots S, const CombOut* __restrict__ outs,
                                                   const CombTerm* __restrict__ terms, int n_outs) {
     const int ob = blockIdx.x;
     if (ob >= n_outs) return;
@@ -365,7 +388,7 @@ __global__ void __launch_bounds__(256) k_comb_f64(Slots S, const CombOut* __rest
 }
 
 // ---- diagonal of the projected operators ------------------------------------------------------
-__global__ void __launch_bounds__(256) k_diag_f64(Slots S, const DiagBlock* __restrict__ blocks,
+__global__ void __launch_bounds__(256) k_diag_f64(const __grid_constant__ Slots S, const DiagBlock* __restrict__ blocks,
                                                   const DiagTerm* __restrict__ terms, int n_blocks, double* dh,
                                                   double* dn) {
     const int bi = blockIdx.x;
@@ -1109,7 +1132,7 @@ __global__ void __launch_bounds__(1024) k_trunc_select(const int64_t* __restrict
 }
 
 // ---- block copies ------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_copy_blocks(Slots S, const CopyBlock* __restrict__ blocks, int n) {
+__global__ void __launch_bounds__(256) k_copy_blocks(const __grid_constant__ Slots S, const CopyBlock* __restrict__ blocks, int n) {
     const int bi = blockIdx.x;
     if (bi >= n) return;
     const CopyBlock b = blocks[bi];
@@ -1150,18 +1173,21 @@ int norm_blocks(int64_t n) { return grid_for(n, 256, kNormBlocks); }
 // ---- launch wrappers ----------------------------------------------------------------------------
 
 cudaError_t launch_gemm_f64(const Slots& slots, const GemmTask* tasks, const GemmSeg* segs, const GemmTile* tiles,
-                            const int* cmaps, int n_tiles, cudaStream_t st) {
+                            const int* cmaps, int n_tiles, cudaStream_t st, const BetaRun& beta) {
     if (n_tiles <= 0) return cudaSuccess;
     const int warps_per_cta = 4;
-    const int grid = (n_tiles + warps_per_cta - 1) / warps_per_cta;
-    k_gemm_f64<<<grid, 32 * warps_per_cta, 0, st>>>(slots, tasks, segs, tiles, cmaps, n_tiles);
+    const int grid = (n_tiles * beta.ng + warps_per_cta - 1) / warps_per_cta;
+    k_gemm_f64<<<grid, 32 * warps_per_cta, 0, st>>>(slots, beta.stride, op0_entries(beta, 0, n_tiles), beta.g0, beta.ng, tasks,
+                                                    segs, tiles, cmaps, n_tiles);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gemm_f64_stack(const Slots& slots, const TcStack* stacks, const TcRow* rows, const TcSeg* segs,
-                                  const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, cudaStream_t st) {
+                                  const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, cudaStream_t st,
+                                  const BetaRun& beta) {
     if (u1 <= u0) return cudaSuccess;
-    k_gemm_f64_stack<<<(u1 - u0 + 3) / 4, 128, 0, st>>>(slots, stacks, rows, segs, atab, cmaps, units + u0, u1 - u0);
+    k_gemm_f64_stack<<<((u1 - u0) * beta.ng + 3) / 4, 128, 0, st>>>(slots, beta.stride, op0_entries(beta, u0, u1 - u0), beta.g0,
+                                                                    beta.ng, stacks, rows, segs, atab, cmaps, units, u0, u1);
     return cudaGetLastError();
 }
 

@@ -8,19 +8,35 @@
 
 namespace spmps {
 
+// Launch item `id` of n list entries (the first n0 operator 0's) times ng beta points: operator 0's entries of
+// every beta point come first, so that the long reductions of H are not left for the end of a launch.
+struct LaunchItem {
+    int entry, g, op;
+};
+__host__ __device__ inline LaunchItem launch_item(int id, int n, int n0, int ng) {
+    const int first = n0 * ng;
+    LaunchItem it;
+    it.op = id >= first ? 1 : 0;
+    const int count = it.op ? n - n0 : n0, rel = id - (it.op ? first : 0);
+    it.g = rel / count;
+    it.entry = rel - it.g * count + (it.op ? n0 : 0);
+    return it;
+}
+// Entries of operator 0 among the n from `from` on.
+inline int op0_entries(const BetaRun& b, int from, int n) {
+    const int k = b.split - from;
+    return k < 0 ? 0 : (k > n ? n : k);
+}
+
 // Grouped FP64 GEMM: one warp per 16x16 output tile of the task list.
 cudaError_t launch_gemm_f64(const Slots& slots, const GemmTask* tasks, const GemmSeg* segs,
-                            const GemmTile* tiles, const int* cmaps, int n_tiles, cudaStream_t st);
+                            const GemmTile* tiles, const int* cmaps, int n_tiles, cudaStream_t st,
+                            const BetaRun& beta = BetaRun());
 
 // out[i] = sum_{g < G} w[g] sum_{k < ks} partial[(g * ks + k) * n + i] (fixed order; w null: 1) for one or
 // two outputs (a null output is left out).
 cudaError_t launch_sum_partials(const double* partial0, const double* partial1, const double* w, int G, int ks0, int ks1,
                                 int64_t n, double* out0, double* out1, cudaStream_t st);
-
-// Same task lists on the tensor cores (m16n8k8 TF32, FP32 accumulation, FP64 in and out);
-// split3 != 0 uses the 3xTF32 split (hi*hi + hi*lo + lo*hi).
-cudaError_t launch_gemm_tf32(const Slots& slots, const GemmTask* tasks, const GemmSeg* segs, const GemmTile* tiles,
-                             const int* cmaps, int n_tiles, int split3, cudaStream_t st);
 
 // Operand buffers in pre-split TF32 form (float2 = (hi, lo) per element), indexed by the same slot
 // handles as the FP64 buffers.
@@ -29,10 +45,12 @@ struct SlotsF {
 };
 // out[i] = (tf32(float(x[i])), tf32(float(x[i]) - hi)).
 cudaError_t launch_split_tf32(const double* x, int64_t n, float2* out, cudaStream_t st);
-// The TF32 / 3xTF32 task lists with every A and B operand read from the pre-split buffers of the
-// same slots (no conversion in the GEMM); C written in FP64 as launch_gemm_tf32.
+// The same task lists on the tensor cores (m16n8k8 TF32, FP32 accumulation; split3 != 0 uses the 3xTF32
+// split hi*hi + hi*lo + lo*hi) with every A and B operand read from the pre-split buffers of the same
+// slots; C written in FP64.
 cudaError_t launch_gemm_tf32s(const Slots& slots, const SlotsF& split, const GemmTask* tasks, const GemmSeg* segs,
-                              const GemmTile* tiles, const int* cmaps, int n_tiles, int split3, cudaStream_t st);
+                              const GemmTile* tiles, const int* cmaps, int n_tiles, int split3, cudaStream_t st,
+                              const BetaRun& beta);
 
 // Linear combination of equally shaped blocks (the MPO-leg contraction).
 cudaError_t launch_comb_f64(const Slots& slots, const CombOut* outs, const CombTerm* terms, int n_outs,

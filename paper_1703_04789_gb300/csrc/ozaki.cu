@@ -44,12 +44,13 @@ constexpr int kOzThreads = 256;  // two threads per tile row
 // row exponent fields of the two K halves at 256
 constexpr int kOffColE = 128;
 constexpr int kOffRowE = 256;
+constexpr int kOffBase = 768;  // kMaxSlots base pointers
 constexpr int kOffPlanesA = 1024;
 constexpr int kOffPlanesB = kOffPlanesA + kSlices * kPlaneA;
 constexpr int kOffRawA = kOffPlanesB + kSlices * kPlaneB;  // FP64 A stage, 128 x 32, swizzled
 constexpr int kOffRawB = kOffRawA + kOzM * kOzK * 8;        // FP64 B stage, 32 x 32, swizzled
 constexpr size_t kOzSmem = kOffRawB + kOzN * kOzK * 8;
-static_assert(kOffRowE + 2 * kOzM * 2 <= kOffPlanesA, "exponent fields overlap the digit planes");
+static_assert(kOffRowE + 2 * kOzM * 2 <= kOffBase && kOffBase + 8 * kMaxSlots <= kOffPlanesA, "control fields overlap");
 
 __device__ __forceinline__ uint32_t saddr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
@@ -143,7 +144,9 @@ __device__ __forceinline__ void pair_signs(const double v[NV], __half2 sg[NV / 2
 // (tile rows) and the column half (K half while splitting) w / 4, so every row has two threads.
 // Two CTAs per SM (shared memory and tensor memory each allow two): one CTA's copies and digit
 // splitting overlap the other's MMAs and combination.
-__global__ void __launch_bounds__(kOzThreads, 2) k_gemm_oz(Slots S, const TcStack* __restrict__ stacks,
+__global__ void __launch_bounds__(kOzThreads, 2) k_gemm_oz(const __grid_constant__ Slots P,
+                                                          const __grid_constant__ BetaStride Bs, int n, int n_op0, int g0, int ng,
+                                                          const TcStack* __restrict__ stacks,
                                                           const TcRow* __restrict__ rows, const TcSeg* __restrict__ segs,
                                                           const uint64_t* __restrict__ atab, const int* __restrict__ cmaps,
                                                           const int4* __restrict__ units, int u0, int* __restrict__ err,
@@ -161,9 +164,13 @@ __global__ void __launch_bounds__(kOzThreads, 2) k_gemm_oz(Slots S, const TcStac
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q = warp & 3, h = warp >> 2;
     const int r = q * 32 + lane;  // tile row of this thread
-    const int4 U = units[u0 + blockIdx.x];
+    const LaunchItem it = launch_item(blockIdx.x, n, n_op0, ng);
+    const int4 U = units[u0 + it.entry];
     const TcStack st = stacks[U.x];
     const int m0 = U.y, n0 = U.z;
+    double** base = reinterpret_cast<double**>(smem + kOffBase);  // base pointers of this beta point and operator
+    if (tid < kMaxSlots)
+        base[tid] = P.p[tid] + static_cast<int64_t>(g0 + it.g) * Bs.s[it.op][tid];
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(tslot)),
                      "r"(kTmemCols));
@@ -186,7 +193,7 @@ __global__ void __launch_bounds__(kOzThreads, 2) k_gemm_oz(Slots S, const TcStac
         const TcSeg sg = segs[st.seg0 + s];
         const int kc = min(kOzK, sg.K - kb);
         const uint64_t ah = rvalid ? atab[st.atab0 + static_cast<int64_t>(row) * st.nseg + s] : kNoOperand;
-        const double* arow = ah == kNoOperand ? nullptr : S.p[ah >> 56] + static_cast<int64_t>(ah & 0x00FFFFFFFFFFFFFFull);
+        const double* arow = ah == kNoOperand ? nullptr : base[ah >> 56] + static_cast<int64_t>(ah & 0x00FFFFFFFFFFFFFFull);
         // A: warp w copies rows 32 q + 16 h .. + 15 (their pointers sit in its own lanes 16 h ..),
         // one row per step with the lanes along K (coalesced)
         for (int j = 0; j < 16; ++j) {
@@ -199,7 +206,7 @@ __global__ void __launch_bounds__(kOzThreads, 2) k_gemm_oz(Slots S, const TcStac
             else
                 *dst = 0.0;
         }
-        const double* B = S.p[sg.b >> 56] + static_cast<int64_t>(sg.b & 0x00FFFFFFFFFFFFFFull);
+        const double* B = base[sg.b >> 56] + static_cast<int64_t>(sg.b & 0x00FFFFFFFFFFFFFFull);
         if (sg.b_ks == 1) {  // columns contiguous along K: lanes along K, warp w takes 4 columns
             for (int c = 0; c < 4; ++c) {
                 const int n = warp * 4 + c;
@@ -385,7 +392,7 @@ __global__ void __launch_bounds__(kOzThreads, 2) k_gemm_oz(Slots S, const TcStac
             if (gr >= st.nrows) break;
             if (lane < ncols_t) {
                 const uint64_t c = rows[st.row0 + gr].c;
-                double* C = S.p[c >> 56] + static_cast<int64_t>(c & 0x00FFFFFFFFFFFFFFull);
+                double* C = base[c >> 56] + static_cast<int64_t>(c & 0x00FFFFFFFFFFFFFFull);
                 const int n = n0 + lane;
                 C[cm ? cm[n] : n] = stage[rr * kOzN + (lane ^ (rr & 31))];
             }
@@ -401,7 +408,7 @@ __global__ void __launch_bounds__(kOzThreads, 2) k_gemm_oz(Slots S, const TcStac
 
 cudaError_t launch_gemm_oz(const Slots& slots, const TcStack* stacks, const TcRow* rows, const TcSeg* segs,
                            const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, int* err,
-                           int wait_polls, cudaStream_t st) {
+                           int wait_polls, cudaStream_t st, const BetaRun& beta) {
     if (u1 <= u0) return cudaSuccess;
     if (wait_polls <= 0) wait_polls = kDefaultWaitPolls;
     static int attr_device = -1;
@@ -413,7 +420,7 @@ cudaError_t launch_gemm_oz(const Slots& slots, const TcStack* stacks, const TcRo
         if (e != cudaSuccess) return e;
         attr_device = dev;
     }
-    k_gemm_oz<<<u1 - u0, kOzThreads, kOzSmem, st>>>(slots, stacks, rows, segs, atab, cmaps, units, u0, err, wait_polls);
+    k_gemm_oz<<<(u1 - u0) * beta.ng, kOzThreads, kOzSmem, st>>>(slots, beta.stride, u1 - u0, op0_entries(beta, u0, u1 - u0), beta.g0, beta.ng, stacks, rows, segs, atab, cmaps, units, u0, err, wait_polls);
     return cudaGetLastError();
 }
 

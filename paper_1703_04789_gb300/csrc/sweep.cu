@@ -741,12 +741,9 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
     CK(A1->ensure(std::max<int64_t>(a1.size, 1) * sizeof(double)));
     CK(cudaMemsetAsync(A0->p, 0, std::max<int64_t>(a0.size, 1) * sizeof(double), h->stream));
     CK(cudaMemsetAsync(A1->p, 0, std::max<int64_t>(a1.size, 1) * sizeof(double), h->stream));
-    DevMem d_tasks, d_segs, d_tiles, d_cmaps, d_copies;
-    CK(upload(d_tasks, W.tasks, h->stream));
-    CK(upload(d_segs, W.segs, h->stream));
-    CK(upload(d_tiles, W.tiles, h->stream));
-    CK(upload(d_cmaps, W.cmaps, h->stream));
-    CK(upload(d_copies, copies, h->stream));
+    Packer K(h->staging);
+    const size_t ot = K.add(W.tasks), os = K.add(W.segs), oi = K.add(W.tiles), oc = K.add(W.cmaps), oy = K.add(copies);
+    CK(K.put(h->once, h->stream));
     Slots S2{};
     S2.p[0] = x;
     S2.p[1] = B.mats.as<double>();
@@ -757,11 +754,11 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
         for (const GemmTask& T : W.tasks)
             for (int q = 0; q < T.nseg; ++q) fl += 2.0 * T.M * T.N * W.segs[T.seg0 + q].K;
         const int rec = h->profile ? prof_begin(h, h->stream, 0, fl) : -1;
-        CK(launch_gemm_f64(S2, d_tasks.as<GemmTask>(), d_segs.as<GemmSeg>(), d_tiles.as<GemmTile>(), d_cmaps.as<int>(),
-                           static_cast<int>(W.tiles.size()), h->stream));
+        CK(launch_gemm_f64(S2, at<GemmTask>(h->once, ot), at<GemmSeg>(h->once, os), at<GemmTile>(h->once, oi),
+                           at<int>(h->once, oc), static_cast<int>(W.tiles.size()), h->stream));
         if (rec >= 0) prof_end(h, h->stream, rec);
     }
-    CK(launch_copy_blocks(S2, d_copies.as<CopyBlock>(), static_cast<int>(copies.size()), h->stream));
+    CK(launch_copy_blocks(S2, at<CopyBlock>(h->once, oy), static_cast<int>(copies.size()), h->stream));
     h->launches += 4;
     CK(cudaStreamSynchronize(h->stream));
     // install

@@ -5,12 +5,10 @@
 
 namespace spmps {
 
-bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ranges, int nt, TcPlan& P) {
+bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ranges, TcPlan& P) {
     P.clear();
-    P.nt = nt;
-    P.unit_rng.assign(n_ranges + 1, 0);
+    P.n_ranges = n_ranges;
     for (int r = 0; r < n_ranges; ++r) {
-        P.unit_rng[r] = static_cast<int>(P.units.size());
         std::map<int, std::vector<int>> by_key;
         for (int t = task_rng[r]; t < task_rng[r + 1]; ++t) by_key[G.tasks[t].key].push_back(t);
         for (const auto& kv : by_key) {
@@ -66,28 +64,39 @@ bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ra
                 }
             }
             S.nrows = static_cast<int>(P.rows.size()) - S.row0;
-            const int si = static_cast<int>(P.stacks.size());
             P.stacks.push_back(S);
             P.stack_range.push_back(r);
-            for (int m0 = 0; m0 < S.nrows; m0 += 128)
-                for (int n0 = 0; n0 < S.N; n0 += nt) P.units.push_back(make_int4(si, m0, n0, 0));
         }
     }
-    P.unit_rng[n_ranges] = static_cast<int>(P.units.size());
     P.ok = true;
     return true;
 }
 
-void stack_units(TcPlan& P, int elems) {
+void tile_units(const TcPlan& P, int nt, TcUnits& U) {
+    U.units.clear();
+    U.rng.assign(P.n_ranges + 1, 0);
+    U.nt = nt;
+    size_t si = 0;
+    for (int r = 0; r < P.n_ranges; ++r) {
+        U.rng[r] = static_cast<int>(U.units.size());
+        for (; si < P.stacks.size() && P.stack_range[si] == r; ++si)
+            for (int m0 = 0; m0 < P.stacks[si].nrows; m0 += 128)
+                for (int n0 = 0; n0 < P.stacks[si].N; n0 += nt) U.units.push_back(make_int4(static_cast<int>(si), m0, n0, 0));
+    }
+    U.rng[P.n_ranges] = static_cast<int>(U.units.size());
+}
+
+void stack_units(const TcPlan& P, int elems, int copies, TcUnits& U) {
     std::map<std::pair<int, int>, BlockSplit> splits;
-    P.units.clear();
+    U.units.clear();
+    U.rng.assign(P.n_ranges + 1, 0);
     int64_t outputs = 0;
     for (const TcStack& st : P.stacks) outputs += static_cast<int64_t>(st.nrows) * st.N;
-    elems = fill_elems(outputs, elems);
+    elems = fill_elems(outputs * copies, elems);
     size_t si = 0;
-    for (size_t r = 0; r + 1 < P.unit_rng.size(); ++r) {
-        P.unit_rng[r] = static_cast<int>(P.units.size());
-        for (; si < P.stacks.size() && P.stack_range[si] == static_cast<int>(r); ++si) {
+    for (int r = 0; r < P.n_ranges; ++r) {
+        U.rng[r] = static_cast<int>(U.units.size());
+        for (; si < P.stacks.size() && P.stack_range[si] == r; ++si) {
             const TcStack& st = P.stacks[si];
             BlockSplit& sp = splits.emplace(std::make_pair(st.nrows, st.N), BlockSplit{0, 0}).first->second;
             if (sp.pm == 0) sp = split_block(st.nrows, st.N, elems);
@@ -95,14 +104,14 @@ void stack_units(TcPlan& P, int elems) {
                 const int tm = st.nrows / sp.pm + (i < st.nrows % sp.pm ? 1 : 0);
                 for (int j = 0, n0 = 0; j < sp.pn; ++j) {
                     const int tn = st.N / sp.pn + (j < st.N % sp.pn ? 1 : 0);
-                    P.units.push_back(make_int4(static_cast<int>(si), m0, n0, tm | (tn << 16)));
+                    U.units.push_back(make_int4(static_cast<int>(si), m0, n0, tm | (tn << 16)));
                     n0 += tn;
                 }
                 m0 += tm;
             }
         }
     }
-    P.unit_rng.back() = static_cast<int>(P.units.size());
+    U.rng[P.n_ranges] = static_cast<int>(U.units.size());
 }
 
 namespace {
@@ -152,7 +161,9 @@ __device__ __forceinline__ uint32_t poll(uint32_t mbar, uint32_t parity, int lim
 }
 
 template <bool SPLIT3>
-__global__ void __launch_bounds__(128, 3) k_gemm_tc(Slots S, SlotsF F, const TcStack* __restrict__ stacks,
+__global__ void __launch_bounds__(128, 3) k_gemm_tc(const __grid_constant__ Slots S, const __grid_constant__ SlotsF F,
+                                                   const __grid_constant__ BetaStride Bs, int split, int g0,
+                                                   const TcStack* __restrict__ stacks,
                                                    const TcRow* __restrict__ rows, const TcSeg* __restrict__ segs,
                                                    const uint64_t* __restrict__ atab, const int* __restrict__ cmaps,
                                                    const int4* __restrict__ units, int u0, int nt,
@@ -172,6 +183,13 @@ __global__ void __launch_bounds__(128, 3) k_gemm_tc(Slots S, SlotsF F, const TcS
     const int4 U = units[u0 + blockIdx.x];
     const TcStack st = stacks[U.x];
     const int m0 = U.y, n0 = U.z;
+    double** dbase = reinterpret_cast<double**>(smem + 256);  // base pointers of this beta point and operator
+    float2** fbase = reinterpret_cast<float2**>(smem + 384);
+    if (tid < kMaxSlots) {
+        const int64_t off = (g0 + static_cast<int64_t>(blockIdx.y)) * Bs.s[static_cast<int>(u0 + blockIdx.x) >= split ? 1 : 0][tid];
+        dbase[tid] = S.p[tid] + off;
+        fbase[tid] = F.p[tid] + off;
+    }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(tslot)), "r"(nt));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -201,8 +219,8 @@ __global__ void __launch_bounds__(128, 3) k_gemm_tc(Slots S, SlotsF F, const TcS
         const int kc = min(kTileK, sg.K - kb);
         const uint64_t ah = rvalid ? atab[st.atab0 + static_cast<int64_t>(row) * st.nseg + s] : kNoOperand;
         const float2* __restrict__ A =
-            ah == kNoOperand ? nullptr : F.p[ah >> 56] + static_cast<int64_t>(ah & 0x00FFFFFFFFFFFFFFull);
-        const float2* __restrict__ B = F.p[sg.b >> 56] + static_cast<int64_t>(sg.b & 0x00FFFFFFFFFFFFFFull);
+            ah == kNoOperand ? nullptr : fbase[ah >> 56] + static_cast<int64_t>(ah & 0x00FFFFFFFFFFFFFFull);
+        const float2* __restrict__ B = fbase[sg.b >> 56] + static_cast<int64_t>(sg.b & 0x00FFFFFFFFFFFFFFull);
 #pragma unroll
         for (int k = 0; k < kTileK; ++k) ra[k] = (A && k < kc) ? A[kb + k] : zero;
         if (sg.b_ks == 1) {  // unit stride along K: lanes along K
@@ -313,7 +331,7 @@ __global__ void __launch_bounds__(128, 3) k_gemm_tc(Slots S, SlotsF F, const TcS
             const int r = m0 + rr;
             if (r >= st.nrows) break;
             const uint64_t c = rows[st.row0 + r].c;
-            double* C = S.p[c >> 56] + static_cast<int64_t>(c & 0x00FFFFFFFFFFFFFFull);
+            double* C = dbase[c >> 56] + static_cast<int64_t>(c & 0x00FFFFFFFFFFFFFFull);
             for (int q = lane; q < ncols; q += 32) {
                 const int n = n0 + q;
                 C[cm ? cm[n] : n] = static_cast<double>(stage[rr * ld + q]);
@@ -335,7 +353,7 @@ __global__ void __launch_bounds__(128, 3) k_gemm_tc(Slots S, SlotsF F, const TcS
 
 cudaError_t launch_gemm_tc(const Slots& slots, const SlotsF& split, const TcStack* stacks, const TcRow* rows,
                            const TcSeg* segs, const uint64_t* atab, const int* cmaps, const int4* units, int u0,
-                           int u1, int nt, int split3, int* err, int wait_polls, cudaStream_t st) {
+                           int u1, int nt, int split3, int* err, int wait_polls, cudaStream_t st, const BetaRun& beta) {
     if (u1 <= u0) return cudaSuccess;
     if (nt != 32 && nt != 64 && nt != 128) return cudaErrorInvalidValue;
     if (wait_polls <= 0) wait_polls = kDefaultWaitPolls;
@@ -352,12 +370,12 @@ cudaError_t launch_gemm_tc(const Slots& slots, const SlotsF& split, const TcStac
         if (e != cudaSuccess) return e;
         attr_device = dev;
     }
-    const int grid = u1 - u0;
+    const dim3 grid(u1 - u0, beta.ng);
     if (split3)
-        k_gemm_tc<true><<<grid, 128, smem, st>>>(slots, split, stacks, rows, segs, atab, cmaps, units, u0, nt, err,
+        k_gemm_tc<true><<<grid, 128, smem, st>>>(slots, split, beta.stride, beta.split, beta.g0, stacks, rows, segs, atab, cmaps, units, u0, nt, err,
                                                  wait_polls);
     else
-        k_gemm_tc<false><<<grid, 128, smem, st>>>(slots, split, stacks, rows, segs, atab, cmaps, units, u0, nt, err,
+        k_gemm_tc<false><<<grid, 128, smem, st>>>(slots, split, beta.stride, beta.split, beta.g0, stacks, rows, segs, atab, cmaps, units, u0, nt, err,
                                                   wait_polls);
     return cudaGetLastError();
 }

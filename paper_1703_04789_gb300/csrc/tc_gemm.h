@@ -41,27 +41,37 @@ struct TcPlan {
     std::vector<TcRow> rows;
     std::vector<TcSeg> segs;
     std::vector<uint64_t> atab;   // A(r, s, k) = A[atab + k], contiguous along K
-    std::vector<int4> units;      // (stack, m0, n0, 0): one CTA each
     std::vector<int> stack_range; // per stack: its range
-    std::vector<int> unit_rng;    // per beta range: units [unit_rng[g], unit_rng[g + 1])
-    int nt = 64;                  // columns per CTA tile (32, 64 or 128)
+    int n_ranges = 0;
     bool ok = false;              // every task of the range could be stacked
     void clear() {
-        stacks.clear(); stack_range.clear(); rows.clear(); segs.clear(); atab.clear(); units.clear(); unit_rng.clear();
+        stacks.clear(); stack_range.clear(); rows.clear(); segs.clear(); atab.clear();
+        n_ranges = 0;
         ok = false;
     }
 };
 
-// Stack the tasks of G (task ranges task_rng[g] .. task_rng[g + 1] for g < n_ranges) by their key;
-// nt = columns per CTA.  Returns false (and leaves P.ok false) when a task does not fit the stacked
-// form (A not contiguous along K).
-bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ranges, int nt, TcPlan& P);
+// A launch's work list over a plan's stacks; units [rng[r], rng[r + 1]) belong to range r.
+struct TcUnits {
+    std::vector<int4> units;
+    std::vector<int> rng;
+    int nt = 0;  // columns per tile (tile_units)
+};
 
-// Units of the FP64 pipe's kernel instead (one warp each: (stack, m0, n0, tm | tn << 16), tm tn <= elems):
-// the even split of every stack that leaves the fewest lanes idle.
-void stack_units(TcPlan& P, int elems);
+// Stack the tasks of G (task ranges task_rng[g] .. task_rng[g + 1] for g < n_ranges) by their key.
+// Returns false (and leaves P.ok false) when a task does not fit the stacked form (A not contiguous
+// along K).
+bool build_tc_plan(const GemmPlan& G, const std::vector<int>& task_rng, int n_ranges, TcPlan& P);
+
+// Units of the tensor-core kernels: tiles (stack, m0, n0, 0) of 128 rows x nt columns (32, 64 or 128), one CTA
+// each.
+void tile_units(const TcPlan& P, int nt, TcUnits& U);
+// Units of the FP64 pipe's kernel: one warp each, (stack, m0, n0, tm | tn << 16) with tm tn <= elems, the even
+// split of every stack that leaves the fewest lanes idle; `copies` beta points run per launch.
+void stack_units(const TcPlan& P, int elems, int copies, TcUnits& U);
 cudaError_t launch_gemm_f64_stack(const Slots& slots, const TcStack* stacks, const TcRow* rows, const TcSeg* segs,
-                                  const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, cudaStream_t st);
+                                  const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, cudaStream_t st,
+                                  const BetaRun& beta);
 
 // One launch over units [u0, u1): C = sum over segments of A B^T for every unit tile, with A and B
 // read from the pre-split (hi, lo) TF32 buffers; split3 != 0 accumulates hi*hi + hi*lo + lo*hi,
@@ -69,10 +79,10 @@ cudaError_t launch_gemm_f64_stack(const Slots& slots, const TcStack* stacks, con
 // waits, with the default limit, for its MMAs in flight and frees its tensor memory).
 cudaError_t launch_gemm_tc(const Slots& slots, const SlotsF& split, const TcStack* stacks, const TcRow* rows,
                            const TcSeg* segs, const uint64_t* atab, const int* cmaps, const int4* units, int u0,
-                           int u1, int nt, int split3, int* err, int wait_polls, cudaStream_t st);
+                           int u1, int nt, int split3, int* err, int wait_polls, cudaStream_t st, const BetaRun& beta);
 
 // FP64-accurate variant over the same stacks (tiles of 128 rows x gemm_oz_columns() columns, so the
-// plan must be built with nt = gemm_oz_columns()): A and B read in FP64, every K stage of 32 split
+// units are tile_units of that width): A and B read in FP64, every K stage of 32 split
 // into seven signed 8-bit digits per entry against per-row and per-column exponents, the digit
 // products summed exactly by tcgen05.mma kind::f16 (FP16 digits, FP32 accumulators in tensor
 // memory, one per level p + q = 2 .. 9, every partial sum an integer below 2^24) and combined in
@@ -80,7 +90,7 @@ cudaError_t launch_gemm_tc(const Slots& slots, const SlotsF& split, const TcStac
 // 32 * 2^-55 max|a_i.| max|b_.j|.  err[0] and wait_polls as for launch_gemm_tc.
 cudaError_t launch_gemm_oz(const Slots& slots, const TcStack* stacks, const TcRow* rows, const TcSeg* segs,
                            const uint64_t* atab, const int* cmaps, const int4* units, int u0, int u1, int* err,
-                           int wait_polls, cudaStream_t st);
+                           int wait_polls, cudaStream_t st, const BetaRun& beta);
 int gemm_oz_columns();
 
 }  // namespace spmps

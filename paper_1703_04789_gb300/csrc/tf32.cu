@@ -16,10 +16,6 @@ namespace spmps {
 
 namespace {
 
-__device__ __forceinline__ double* resolve_t(const Slots& S, uint64_t h) {
-    return S.p[h >> 56] + static_cast<int64_t>(h & 0x00FFFFFFFFFFFFFFull);
-}
-
 __device__ __forceinline__ uint32_t to_tf32(float x) {
     uint32_t r;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -53,98 +49,6 @@ __device__ __forceinline__ void region(const GemmTile& t, int& h, int& w) {
     }
 }
 
-template <bool SPLIT3>
-__global__ void __launch_bounds__(128) k_gemm_tf32(Slots S, const GemmTask* __restrict__ tasks,
-                                                   const GemmSeg* __restrict__ segs, const GemmTile* __restrict__ tiles,
-                                                   const int* __restrict__ cmaps, int n_tiles) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= n_tiles) return;
-    const GemmTile tl = tiles[warp];
-    const GemmTask T = tasks[tl.task];
-    int rh, rw;
-    region(tl, rh, rw);
-    const int rmax = min(T.M, tl.m0 + rh), cmax = min(T.N, tl.n0 + rw);
-    const int g = lane >> 2, q = lane & 3;
-    double* C = resolve_t(S, T.c);
-    const int* cm = T.cmap >= 0 ? cmaps + T.cmap : nullptr;
-    for (int sm0 = tl.m0; sm0 < rmax; sm0 += 32)
-        for (int sn0 = tl.n0; sn0 < cmax; sn0 += 32) {
-            float acc[2][4][4];
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0f;
-            const int mt = (min(32, rmax - sm0) + 15) / 16;  // 1 or 2 row tiles
-            const int nt = (min(32, cmax - sn0) + 7) / 8;    // 1..4 column tiles
-            for (int sgi = 0; sgi < T.nseg; ++sgi) {
-                const GemmSeg sg = segs[T.seg0 + sgi];
-                const double* __restrict__ A = resolve_t(S, sg.a);
-                const double* __restrict__ B = resolve_t(S, sg.b);
-                for (int k0 = 0; k0 < sg.K; k0 += 8) {
-                    uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int r = sm0 + 16 * i + g + ((e & 1) ? 8 : 0);
-                            const int k = k0 + q + ((e & 2) ? 4 : 0);
-                            const double v = (i < mt && r < rmax && k < sg.K)
-                                                 ? __ldg(A + static_cast<int64_t>(r) * sg.a_rs + static_cast<int64_t>(k) * sg.a_cs)
-                                                 : 0.0;
-                            split(v, ah[i][e], al[i][e]);
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int k = k0 + q + (e ? 4 : 0);
-                            const int c = sn0 + 8 * j + g;
-                            const double v = (j < nt && c < cmax && k < sg.K)
-                                                 ? __ldg(B + static_cast<int64_t>(k) * sg.b_rs + static_cast<int64_t>(c) * sg.b_cs)
-                                                 : 0.0;
-                            split(v, bh[j][e], bl[j][e]);
-                        }
-                    }
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        if (i >= mt) continue;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (j >= nt) continue;
-                            mma_tf32(acc[i][j], ah[i], bh[j]);
-                            if (SPLIT3) {
-                                mma_tf32(acc[i][j], ah[i], bl[j]);
-                                mma_tf32(acc[i][j], al[i], bh[j]);
-                            }
-                        }
-                    }
-                }
-            }
-            // D fragment: (row g, cols 2q, 2q+1) and (row g+8, same cols) of each 16 x 8 tile
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                if (i >= mt) continue;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j >= nt) continue;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int r = sm0 + 16 * i + g + ((e & 2) ? 8 : 0);
-                        const int c = sn0 + 8 * j + 2 * q + (e & 1);
-                        if (r < rmax && c < cmax) {
-                            const int64_t cc = cm ? cm[c] : c;
-                            C[static_cast<int64_t>(r) * T.ldc + cc] = static_cast<double>(acc[i][j][e]);
-                        }
-                    }
-                }
-            }
-        }
-}
-
 // ---- pre-split operands -----------------------------------------------------------------------
 // The conversion FP64 -> FP32 -> (hi, lo) runs once per operand buffer (environment after its
 // update, x and the phase-B output once per action) instead of once per fragment load: on this
@@ -159,19 +63,32 @@ __global__ void __launch_bounds__(256) k_split_tf32(const double* __restrict__ x
     }
 }
 
-__device__ __forceinline__ const float2* resolve_s(const SlotsF& F, uint64_t h) {
-    return F.p[h >> 56] + static_cast<int64_t>(h & 0x00FFFFFFFFFFFFFFull);
+template <class T>
+__device__ __forceinline__ T* resolve_t(T* const* base, uint64_t h) {
+    return base[h >> 56] + static_cast<int64_t>(h & 0x00FFFFFFFFFFFFFFull);
 }
 
 template <bool SPLIT3>
-__global__ void __launch_bounds__(128, 4) k_gemm_tf32s(Slots S, SlotsF F, const GemmTask* __restrict__ tasks,
+__global__ void __launch_bounds__(128, 4) k_gemm_tf32s(const __grid_constant__ Slots P, const __grid_constant__ SlotsF PF,
+                                                    const __grid_constant__ BetaStride Bs, int split, int g0,
+                                                    const GemmTask* __restrict__ tasks,
                                                     const GemmSeg* __restrict__ segs, const GemmTile* __restrict__ tiles,
                                                     const int* __restrict__ cmaps, int n_tiles) {
+    __shared__ double* dbase[4][kMaxSlots];
+    __shared__ float2* fbase[4][kMaxSlots];
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= n_tiles) return;
     const GemmTile tl = tiles[warp];
     const GemmTask T = tasks[tl.task];
+    double** S = dbase[threadIdx.x >> 5];
+    float2** F = fbase[threadIdx.x >> 5];
+    if (lane < kMaxSlots) {  // this warp's beta point and operator
+        const int64_t off = (g0 + static_cast<int64_t>(blockIdx.y)) * Bs.s[warp >= split ? 1 : 0][lane];
+        S[lane] = P.p[lane] + off;
+        F[lane] = PF.p[lane] + off;
+    }
+    __syncwarp();
     int rh, rw;
     region(tl, rh, rw);
     const int rmax = min(T.M, tl.m0 + rh), cmax = min(T.N, tl.n0 + rw);
@@ -192,8 +109,8 @@ __global__ void __launch_bounds__(128, 4) k_gemm_tf32s(Slots S, SlotsF F, const 
             const int nt = (min(32, cmax - sn0) + 7) / 8;
             for (int sgi = 0; sgi < T.nseg; ++sgi) {
                 const GemmSeg sg = segs[T.seg0 + sgi];
-                const float2* __restrict__ A = resolve_s(F, sg.a);
-                const float2* __restrict__ B = resolve_s(F, sg.b);
+                const float2* __restrict__ A = resolve_t(F, sg.a);
+                const float2* __restrict__ B = resolve_t(F, sg.b);
                 for (int k0 = 0; k0 < sg.K; k0 += 8) {
                     uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
 #pragma unroll
@@ -259,18 +176,6 @@ __global__ void __launch_bounds__(128, 4) k_gemm_tf32s(Slots S, SlotsF F, const 
 
 }  // namespace
 
-cudaError_t launch_gemm_tf32(const Slots& slots, const GemmTask* tasks, const GemmSeg* segs, const GemmTile* tiles,
-                             const int* cmaps, int n_tiles, int split3, cudaStream_t st) {
-    if (n_tiles <= 0) return cudaSuccess;
-    const int grid = (n_tiles + 3) / 4;
-    if (split3)
-        k_gemm_tf32<true><<<grid, 128, 0, st>>>(slots, tasks, segs, tiles, cmaps, n_tiles);
-    else
-        k_gemm_tf32<false><<<grid, 128, 0, st>>>(slots, tasks, segs, tiles, cmaps, n_tiles);
-    return cudaGetLastError();
-}
-
-
 cudaError_t launch_split_tf32(const double* x, int64_t n, float2* out, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     int64_t blocks = (n + 255) / 256;
@@ -280,13 +185,14 @@ cudaError_t launch_split_tf32(const double* x, int64_t n, float2* out, cudaStrea
 }
 
 cudaError_t launch_gemm_tf32s(const Slots& slots, const SlotsF& split, const GemmTask* tasks, const GemmSeg* segs,
-                              const GemmTile* tiles, const int* cmaps, int n_tiles, int split3, cudaStream_t st) {
+                              const GemmTile* tiles, const int* cmaps, int n_tiles, int split3, cudaStream_t st,
+                              const BetaRun& beta) {
     if (n_tiles <= 0) return cudaSuccess;
-    const int grid = (n_tiles + 3) / 4;
+    const dim3 grid((n_tiles + 3) / 4, beta.ng);
     if (split3)
-        k_gemm_tf32s<true><<<grid, 128, 0, st>>>(slots, split, tasks, segs, tiles, cmaps, n_tiles);
+        k_gemm_tf32s<true><<<grid, 128, 0, st>>>(slots, split, beta.stride, beta.split, beta.g0, tasks, segs, tiles, cmaps, n_tiles);
     else
-        k_gemm_tf32s<false><<<grid, 128, 0, st>>>(slots, split, tasks, segs, tiles, cmaps, n_tiles);
+        k_gemm_tf32s<false><<<grid, 128, 0, st>>>(slots, split, beta.stride, beta.split, beta.g0, tasks, segs, tiles, cmaps, n_tiles);
     return cudaGetLastError();
 }
 
