@@ -34,15 +34,20 @@ __device__ __forceinline__ T wsum(T v) {
     return v;
 }
 
-// c = 1 / sqrt(1 + t^2): the hardware estimate polished to the precision of T, so that the rotation is
-// orthonormal in T (the angle itself may be rounded: the next sweep removes what it leaves).
-__device__ __forceinline__ float rotation_cos(float t) { return rsqrtf(fmaf(t, t, 1.0f)); }
-__device__ __forceinline__ double rotation_cos(double t) {
-    const double w = fma(t, t, 1.0);
-    double y = static_cast<double>(rsqrtf(static_cast<float>(w)));
-    y = y * fma(-0.5 * w, y * y, 1.5);
-    y = y * fma(-0.5 * w, y * y, 1.5);
-    return y;
+// sin(theta) for h = tan(theta / 2): 2 h / (1 + h^2) to the precision of T.  The rotation is applied as three
+// shears x -= h y, y += s x, x -= h y, which is orthonormal for any h as far as s belongs to it; the angle
+// itself may be rounded (the next sweep removes what it leaves).
+__device__ __forceinline__ float shear_sin(float h) { return __fdividef(2.0f * h, fmaf(h, h, 1.0f)); }
+__device__ __forceinline__ double shear_sin(double h) {
+    const double w = h * h;
+    if (fabsf(static_cast<float>(h)) < 1e-3f) {  // 2 h (1 - w + w^2 - w^3): the next term is below 1e-24
+        return 2.0 * h * fma(w, fma(w, 1.0 - w, -1.0), 1.0);
+    }
+    const double d = 1.0 + w;
+    double y = static_cast<double>(__frcp_rn(static_cast<float>(d)));
+    y = y * fma(-d, y, 2.0);
+    y = y * fma(-d, y, 2.0);
+    return 2.0 * h * y;
 }
 
 // One-sided Jacobi on the rows of Z (R x W, row stride W): the first C columns are the block, the rest a
@@ -52,11 +57,13 @@ __device__ __forceinline__ double rotation_cos(double t) {
 // FP64 pipes of 8 SMs share the work.  NCH > 0 keeps the two rows of a pair in registers (W <= 32 NCH)
 // between the product and the update, NCH = 0 reads them twice.  The sweeps end after one that met no
 // relative coupling above `done` (what it leaves is the square of that over the relative gap).
-// Measured (GB300, middle decimation of the L = 24, D = 256 chain, blocks up to 136): see launch_svd.
+// FP64: 3 operations per element for the three shears and 10 for the product and its sum over the warp, with
+// the angle in FP32: a launch of the canonicalisation below takes 0.77 ms on average, 1.16 ms with
+// the four-operation rotation, FP64 square roots and the pairs on the first CTAs of a cluster.
 template <class T, bool SMEM, int NCH>
 __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T done, int* conv, int rank, int ctas) {
     const int lane = threadIdx.x & 31;
-    const int warp = (threadIdx.x >> 5) + rank * (blockDim.x >> 5);
+    const int warp = (threadIdx.x >> 5) * ctas + rank;  // pairs go round the CTAs: the FP64 pipes of all share them
     const int warps = (blockDim.x >> 5) * ctas;
     const int np = (R + 1) & ~1, half = np / 2;
     constexpr bool kF64 = sizeof(T) == 8;
@@ -96,8 +103,9 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T do
         bool rough = false;
         for (int round = 0; round < np - 1; ++round) {
             for (int i = warp; i < half; i += warps) {
-                int p = i == 0 ? 0 : 1 + (i - 1 + round) % (np - 1);
-                int q = 1 + (np - 2 - i + round) % (np - 1);
+                int p = i - 1 + round, q = np - 2 - i + round;  // both below 2 (np - 1)
+                p = i == 0 ? 0 : 1 + (p >= np - 1 ? p - (np - 1) : p);
+                q = 1 + (q >= np - 1 ? q - (np - 1) : q);
                 if (p > q) {
                     const int t = p;
                     p = q;
@@ -130,28 +138,33 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T do
                 if (g2 > done * done * ab && a > null2 && b > null2) rough = true;
                 const float zeta = static_cast<float>((b - a) * inv_all) / (2.0f * static_cast<float>(g * inv_all));
                 const float tf = copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
-                const T t = static_cast<T>(tf);
-                const T cs = rotation_cos(t), sn = cs * t;
+                const T hh = static_cast<T>(tf / (1.0f + sqrtf(fmaf(tf, tf, 1.0f))));
+                const T sn = shear_sin(hh);
+                auto turn = [&](T& u, T& v) {
+                    u -= hh * v;
+                    v += sn * u;
+                    u -= hh * v;
+                };
                 if constexpr (NCH > 0) {
 #pragma unroll
                     for (int k = 0; k < NCH; ++k) {
                         const int c = lane + 32 * k;
                         if (c < W) {
-                            stg(zp + c, cs * x[k] - sn * y[k]);
-                            stg(zq + c, sn * x[k] + cs * y[k]);
+                            turn(x[k], y[k]);
+                            stg(zp + c, x[k]);
+                            stg(zq + c, y[k]);
                         }
                     }
                 } else {
                     for (int c = lane; c < W; c += 32) {
-                        const T u = ld(zp + c), v = ld(zq + c);
-                        stg(zp + c, cs * u - sn * v);
-                        stg(zq + c, sn * u + cs * v);
+                        T u = ld(zp + c), v = ld(zq + c);
+                        turn(u, v);
+                        stg(zp + c, u);
+                        stg(zq + c, v);
                     }
                 }
-                if (lane == 0) {
-                    // |p'|^2 = c^2 a - 2 c s g + s^2 b
-                    const T na = cs * cs * a - T(2) * cs * sn * g + sn * sn * b;
-                    const T nb = sn * sn * a + T(2) * cs * sn * g + cs * cs * b;
+                if (lane == 0) {  // |p|^2 and |q|^2 move by tan(theta) g (summed anew at every sweep)
+                    const T d = static_cast<T>(tf) * g, na = a - d, nb = b + d;
                     stg(nrm2 + p, na > T(0) ? na : T(0));
                     stg(nrm2 + q, nb > T(0) ? nb : T(0));
                 }
@@ -197,8 +210,10 @@ __device__ void osj32_block(const SvdBlock& B, const double* __restrict__ zraw, 
         __syncthreads();
     else
         cgx::this_cluster().sync();
-    if (W <= 256 && !SMEM)
-        osj_sweeps<float, SMEM, SMEM ? 0 : 8>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
+    if (W <= 128)
+        osj_sweeps<float, SMEM, 4>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
+    else if (W <= 256)
+        osj_sweeps<float, SMEM, 8>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
     else
         osj_sweeps<float, SMEM, 0>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
     for (int e = rank * blockDim.x + threadIdx.x; e < R * R; e += blockDim.x * ctas) {
@@ -273,7 +288,7 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
     else
         osj_sweeps<double, false, 0>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     // exact norms of the final rows, then the vectors by descending norm (ties by row)
-    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) + rank * (blockDim.x >> 5);
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) * kOsjC + rank;
     const int warps = (blockDim.x >> 5) * kOsjC;
     for (int r = warp; r < R; r += warps) {
         double t = 0.0;
@@ -466,10 +481,9 @@ double* SvdPlan::z_buffer(void* ws) const {
                                      up(blocks.size() * 2 * kSvdConv * sizeof(int)));
 }
 
-// Measured (GB300, with the parallel k_trunc_*): loading, canonicalising and measuring a random L = 24,
-// D = 256 triplet state (blocks up to 52 rows) takes 104.8 ms, 398.5 ms with the two-sided FP64 Jacobi on
-// X X^T and the one-thread truncation; a two-site step at the middle of the L = 24, D = 256 chain (blocks
-// up to 150 rows) 96.2 ms, 108.8 ms before.
+// Measured (GB300): the decimations of one canonicalisation (random L = 24, D = 256 triplet state, 23 of them,
+// blocks up to 52 rows) take 33.6 ms, the middle decimation of the L = 24, D = 256 chain (blocks up to 150 rows)
+// 7.6 ms; two-sided FP64 Jacobi on X X^T with a one-thread truncation took 308 and 22 ms.
 cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, cudaStream_t st) {
     const int nb = static_cast<int>(P.blocks.size());
     if (nb == 0) return cudaSuccess;
