@@ -34,20 +34,45 @@ __device__ __forceinline__ T wsum(T v) {
     return v;
 }
 
+// FP32 <-> FP64 by integer instructions: a conversion instruction runs on the FP64 pipe.  to_f32 truncates,
+// divides by 2^shift first and clamps to [0, FLT_MAX]; to_f64 is exact (zero for subnormals).
+__device__ __forceinline__ float to_f32(float v, int) { return v; }
+__device__ __forceinline__ float to_f32(double v, int shift) {
+    const int hi = __double2hiint(v), t = (hi & 0x7FFFFFFF) - ((896 + shift) << 20);
+    const unsigned m = t < (1 << 20) ? 0u : (t >= (255 << 20) ? 0x7F7FFFFFu : __funnelshift_l(__double2loint(v), t, 3));
+    return __uint_as_float(m | (static_cast<unsigned>(hi) & 0x80000000u));
+}
+__device__ __forceinline__ double to_f64(float v) {
+    const unsigned u = __float_as_uint(v), m = u & 0x7FFFFFFFu;
+    const unsigned hi = m < 0x00800000u ? 0u : (m >> 3) + (896u << 20);
+    return __hiloint2double(static_cast<int>(hi | (u & 0x80000000u)), m < 0x00800000u ? 0 : static_cast<int>(m << 29));
+}
+
+// tan(theta) of the rotation that uncouples two rows: d the difference of their squared norms, g their product.
+// For rows of very different norms it has to be right down to g / d, far below FP32's epsilon.
+__device__ __forceinline__ float rotation_tan(float d, float g) {
+    const float zeta = __fdividef(d, 2.0f * g), z = fabsf(zeta), q = fmaf(z, z, 1.0f);
+    return z > 1e8f ? __fdividef(g, d) : copysignf(__fdividef(1.0f, fmaf(q, rsqrtf(q), z)), zeta);
+}
+__device__ __forceinline__ float half_tan(float t) {
+    const float q = fmaf(t, t, 1.0f);
+    return __fdividef(t, 1.0f + q * rsqrtf(q));
+}
+
 // sin(theta) for h = tan(theta / 2): 2 h / (1 + h^2) to the precision of T.  The rotation is applied as three
-// shears x -= h y, y += s x, x -= h y, which is orthonormal for any h as far as s belongs to it; the angle
-// itself may be rounded (the next sweep removes what it leaves).
-__device__ __forceinline__ float shear_sin(float h) { return __fdividef(2.0f * h, fmaf(h, h, 1.0f)); }
-__device__ __forceinline__ double shear_sin(double h) {
-    const double w = h * h;
-    if (fabsf(static_cast<float>(h)) < 1e-3f) {  // 2 h (1 - w + w^2 - w^3): the next term is below 1e-24
-        return 2.0 * h * fma(w, fma(w, 1.0 - w, -1.0), 1.0);
-    }
-    const double d = 1.0 + w;
-    double y = static_cast<double>(__frcp_rn(static_cast<float>(d)));
-    y = y * fma(-d, y, 2.0);
-    y = y * fma(-d, y, 2.0);
-    return 2.0 * h * y;
+// shears x -= h y, y += s x, x -= h y, which is orthonormal for any h as far as s belongs to it (an error e
+// of s leaves h e); the angle itself may be rounded (the next sweep removes what it leaves).
+__device__ __forceinline__ float shear_sin(float hf, float) { return __fdividef(2.0f * hf, fmaf(hf, hf, 1.0f)); }
+__device__ __forceinline__ double shear_sin(float hf, double h) {
+    const double h2 = to_f64(2.0f * hf);
+    const float m = fabsf(hf);
+    if (m < 4e-5f) return h2;                     // h e = 2 h^4 < 6e-18
+    if (m < 1e-3f) return fma(-h2, h * h, h2);    // h e = 2 h^6 < 2e-18
+    const double d = fma(h, h, 1.0);
+    double y = to_f64(__fdividef(1.0f, fmaf(hf, hf, 1.0f)));
+    y = fma(y, fma(-d, y, 1.0), y);
+    y = fma(y, fma(-d, y, 1.0), y);
+    return h2 * y;
 }
 
 // One-sided Jacobi on the rows of Z (R x W, row stride W): the first C columns are the block, the rest a
@@ -57,20 +82,25 @@ __device__ __forceinline__ double shear_sin(double h) {
 // FP64 pipes of 8 SMs share the work.  NCH > 0 keeps the two rows of a pair in registers (W <= 32 NCH)
 // between the product and the update, NCH = 0 reads them twice.  The sweeps end after one that met no
 // relative coupling above `done` (what it leaves is the square of that over the relative gap).
-// FP64: 3 operations per element for the three shears and 10 for the product and its sum over the warp, with
-// the angle in FP32: a launch of the canonicalisation below takes 0.77 ms on average, 1.16 ms with
-// the four-operation rotation, FP64 square roots and the pairs on the first CTAs of a cluster.
+// FP64: an instruction of a warp occupies its sub-partition's FP64 pipe for 64 cycles whether its lanes hold
+// one number or 32, so a pair issues 3 per 32 elements for the shears, one for the product, 5 for its sum
+// over the warp, 2 for the norms and at most 7 for the sine; comparisons, conversions and the angle are
+// FP32 and integer instructions.  Measured (GB300): a launch
+// of the canonicalisation below 0.63 ms on average, the middle decimation of L = 24, D = 256 2.0 ms; 0.81 and 2.7 ms
+// with the comparisons, conversions and the angle's operands in FP64.
 template <class T, bool SMEM, int NCH>
-__device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T done, int* conv, int rank, int ctas) {
+__device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, float done, int* conv, int rank, int ctas) {
     const int lane = threadIdx.x & 31;
     const int warp = (threadIdx.x >> 5) * ctas + rank;  // pairs go round the CTAs: the FP64 pipes of all share them
     const int warps = (blockDim.x >> 5) * ctas;
     const int np = (R + 1) & ~1, half = np / 2;
     constexpr bool kF64 = sizeof(T) == 8;
-    const T tol = kF64 ? T(1e-15) : T(3e-7);
-    const T floor_abs = kF64 ? T(0) : norm2_all * T(1e-12);  // FP32: the noise of the block's largest rows
-    const T null2 = norm2_all * (kF64 ? T(kNullRel * kNullRel) : T(1e-13));
-    const T inv_all = norm2_all > T(0) ? T(1) / norm2_all : T(0);  // keeps the angle's FP32 operands in range
+    constexpr float tol = kF64 ? 1e-15f : 3e-7f;
+    constexpr float floor_abs = kF64 ? 0.0f : 1e-12f;  // FP32: the noise of the block's largest rows
+    constexpr float null2 = kF64 ? static_cast<float>(kNullRel * kNullRel) : 1e-13f;
+    // squared norms and products as FP32 numbers relative to the block's squared norm (to a factor of 2)
+    int shift = 0;
+    if constexpr (kF64) shift = norm2_all > T(0) ? ((__double2hiint(norm2_all) >> 20) & 2047) - 1023 : 0;
     auto barrier = [&]() {
         if constexpr (SMEM)
             __syncthreads();
@@ -115,7 +145,8 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T do
                 T* zp = Z + static_cast<int64_t>(p) * W;
                 T* zq = Z + static_cast<int64_t>(q) * W;
                 const T a = ld(nrm2 + p), b = ld(nrm2 + q);
-                if (!(a > null2) && !(b > null2)) continue;
+                const float af = to_f32(a, shift), bf = to_f32(b, shift);
+                if (!(af > null2) && !(bf > null2)) continue;
                 T x[NCH > 0 ? NCH : 1], y[NCH > 0 ? NCH : 1];
                 T g = T(0);
                 if constexpr (NCH > 0) {
@@ -132,14 +163,16 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T do
                     for (int c = lane; c < C; c += 32) g += ld(zp + c) * ld(zq + c);
                 }
                 g = wsum(g);
-                // |g| <= tol sqrt(a b), compared by the squares
-                const T g2 = g * g, ab = a * b;
-                if (!(g2 > tol * tol * ab) || !(fabs(g) > floor_abs)) continue;
-                if (g2 > done * done * ab && a > null2 && b > null2) rough = true;
-                const float zeta = static_cast<float>((b - a) * inv_all) / (2.0f * static_cast<float>(g * inv_all));
-                const float tf = copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
-                const T hh = static_cast<T>(tf / (1.0f + sqrtf(fmaf(tf, tf, 1.0f))));
-                const T sn = shear_sin(hh);
+                const float gf = to_f32(g, shift), gm = fabsf(gf), root = sqrtf(af) * sqrtf(bf);
+                if (!(gm > tol * root) || !(gm > floor_abs)) continue;
+                if (gm > done * root && af > null2 && bf > null2) rough = true;
+                const float tf = rotation_tan(to_f32(b - a, shift), gf), hf = half_tan(tf);
+                T hh;
+                if constexpr (kF64)
+                    hh = to_f64(hf);
+                else
+                    hh = hf;
+                const T sn = shear_sin(hf, hh);
                 auto turn = [&](T& u, T& v) {
                     u -= hh * v;
                     v += sn * u;
@@ -163,11 +196,14 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, T do
                         stg(zq + c, v);
                     }
                 }
-                if (lane == 0) {  // |p|^2 and |q|^2 move by tan(theta) g (summed anew at every sweep)
-                    const T d = static_cast<T>(tf) * g, na = a - d, nb = b + d;
-                    stg(nrm2 + p, na > T(0) ? na : T(0));
-                    stg(nrm2 + q, nb > T(0) ? nb : T(0));
-                }
+                // |p|^2 and |q|^2 move by tan(theta) g (summed anew at every sweep)
+                T tl;
+                if constexpr (kF64)
+                    tl = to_f64(lane == 0 ? -tf : tf);
+                else
+                    tl = lane == 0 ? -tf : tf;
+                const T moved = fma(tl, g, lane == 0 ? a : b);
+                if (lane < 2) stg(nrm2 + (lane == 0 ? p : q), moved > T(0) ? moved : T(0));
             }
             barrier();
         }
@@ -280,7 +316,7 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
     cgx::this_cluster().sync();  // every CTA has read Z before any rotates it
     int* cv = conv + (b * 2 + 1) * kSvdConv;
     // the companion is orthonormal by construction; normalised rows only as far as they are uncoupled
-    const double done = B.companion ? 1e-11 : 1e-13;
+    const float done = B.companion ? 1e-11f : 1e-13f;
     if (W <= 160)
         osj_sweeps<double, false, 5>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     else if (W <= 320)
