@@ -21,6 +21,7 @@ namespace {
 namespace cgx = cooperative_groups;
 
 constexpr int kOsjC = 8;             // CTAs per block of the global-memory form
+constexpr int kOsj32Threads = 640;   // shared-memory form: 80 pairs at once with up to 102 registers a thread
 constexpr int kMaxSweeps = 40;
 constexpr double kNullRel = 1e-9;    // rows below this fraction of the block's norm are not separated further
 
@@ -77,8 +78,7 @@ __device__ __forceinline__ double shear_sin(float hf, double h) {
 
 // One-sided Jacobi on the rows of Z (R x W, row stride W): the first C columns are the block, the rest a
 // companion that receives the same rotations.  Round-robin pairs, one warp per pair and round.
-// SMEM: one CTA per block with the rows in shared memory (a round costs a __syncthreads); otherwise a
-// cluster of kOsjC CTAs with the rows in global memory (L2), a cluster barrier per round: in FP64 the
+// A cluster of kOsjC CTAs with the rows in global memory (L2), a cluster barrier per round: in FP64 the
 // FP64 pipes of 8 SMs share the work.  NCH > 0 keeps the two rows of a pair in registers (W <= 32 NCH)
 // between the product and the update, NCH = 0 reads them twice.  The sweeps end after one that met no
 // relative coupling above `done` (what it leaves is the square of that over the relative gap).
@@ -88,7 +88,7 @@ __device__ __forceinline__ double shear_sin(float hf, double h) {
 // FP32 and integer instructions.  Measured (GB300): a launch
 // of the canonicalisation below 0.63 ms on average, the middle decimation of L = 24, D = 256 2.0 ms; 0.81 and 2.7 ms
 // with the comparisons, conversions and the angle's operands in FP64.
-template <class T, bool SMEM, int NCH>
+template <class T, int NCH>
 __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, float done, int* conv, int rank, int ctas) {
     const int lane = threadIdx.x & 31;
     const int warp = (threadIdx.x >> 5) * ctas + rank;  // pairs go round the CTAs: the FP64 pipes of all share them
@@ -101,24 +101,9 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
     // squared norms and products as FP32 numbers relative to the block's squared norm (to a factor of 2)
     int shift = 0;
     if constexpr (kF64) shift = norm2_all > T(0) ? ((__double2hiint(norm2_all) >> 20) & 2047) - 1023 : 0;
-    auto barrier = [&]() {
-        if constexpr (SMEM)
-            __syncthreads();
-        else
-            cgx::this_cluster().sync();
-    };
-    auto ld = [&](const T* p) -> T {
-        if constexpr (SMEM)
-            return *p;
-        else
-            return ldc(p);
-    };
-    auto stg = [&](T* p, T v) {
-        if constexpr (SMEM)
-            *p = v;
-        else
-            __stcg(p, v);
-    };
+    auto barrier = [&]() { cgx::this_cluster().sync(); };
+    auto ld = [&](const T* p) -> T { return ldc(p); };
+    auto stg = [&](T* p, T v) { __stcg(p, v); };
     for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
         for (int r = warp; r < R; r += warps) {
             T s = T(0);
@@ -208,22 +193,121 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
             barrier();
         }
         if (rough && lane == 0) atomicOr(conv + sweep, 1);
-        if constexpr (!SMEM) __threadfence();
+        __threadfence();
         barrier();
         if (!*reinterpret_cast<volatile int*>(conv + sweep)) break;  // uniform: read after the barrier
     }
 }
 
-// FP32 start: [Z | I] of a block scaled to norm 1; J (R x R) leaves in FP64.
-template <bool SMEM>
-__device__ void osj32_block(const SvdBlock& B, const double* __restrict__ zraw, float* work, float* nrm2, double* J,
-                            int* conv, int rank, int ctas) {
+// The FP32 start in one CTA's shared memory: 8 lanes per pair and four elements per access, so that a warp
+// computes four angles and four sums at once.  The scheduler's issue slots bound it (a round of 26 pairs was
+// 1200 of them per sub-partition with a warp per pair, half for the angle and the sum); measured (GB300): the
+// middle decimation of L = 24, D = 256 3.3 ms and 0.37 ms on average in the canonicalisation below, 5.0 and 0.52 ms before.
+__device__ __forceinline__ float sum8(float v) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ float dot4(float4 a, float4 b) { return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w))); }
+__device__ __forceinline__ void turn4(float4& x, float4& y, float h, float s) {
+    auto turn = [&](float& u, float& v) {
+        u = fmaf(-h, v, u);
+        v = fmaf(s, u, v);
+        u = fmaf(-h, v, u);
+    };
+    turn(x.x, y.x);
+    turn(x.y, y.y);
+    turn(x.z, y.z);
+    turn(x.w, y.w);
+}
+
+// Rows of V vectors of four, the first CV of them the block; NV > 0 keeps a pair in registers (V <= 8 NV).
+template <int NV>
+__device__ void osj32_sweeps(float4* Z, float* nrm2, int R, int CV, int V) {
+    constexpr float tol = 3e-7f, floor_abs = 1e-12f, null2 = 1e-13f, done = 1e-3f;
+    const int gl = threadIdx.x & 7, group = threadIdx.x >> 3, groups = blockDim.x >> 3;
+    const int np = (R + 1) & ~1, half = np / 2;
+    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+        for (int base = 0; base < R; base += groups) {
+            const int r = base + group;
+            float s = 0.0f;
+            if (r < R)
+                for (int v = gl; v < CV; v += 8) s += dot4(Z[r * V + v], Z[r * V + v]);
+            s = sum8(s);
+            if (r < R && gl == 0) nrm2[r] = s;
+        }
+        __syncthreads();
+        int rough = 0;
+        for (int round = 0; round < np - 1; ++round) {
+            for (int base = 0; base < half; base += groups) {
+                const int i = base + group;
+                int p = i - 1 + round, q = np - 2 - i + round;
+                p = i == 0 ? 0 : 1 + (p >= np - 1 ? p - (np - 1) : p);
+                q = 1 + (q >= np - 1 ? q - (np - 1) : q);
+                if (p > q) {
+                    const int t = p;
+                    p = q;
+                    q = t;
+                }
+                bool on = i < half && q < R;
+                const float a = on ? nrm2[p] : 0.0f, b = on ? nrm2[q] : 0.0f;
+                on = on && (a > null2 || b > null2);
+                float4* zp = Z + p * V;
+                float4* zq = Z + q * V;
+                const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                float4 x[NV > 0 ? NV : 1], y[NV > 0 ? NV : 1];
+                float g = 0.0f;
+                if constexpr (NV > 0) {
+#pragma unroll
+                    for (int k = 0; k < NV; ++k) {
+                        const int v = gl + 8 * k;
+                        x[k] = on && v < V ? zp[v] : zero;
+                        y[k] = on && v < V ? zq[v] : zero;
+                    }
+#pragma unroll
+                    for (int k = 0; k < NV; ++k)
+                        if (gl + 8 * k < CV) g += dot4(x[k], y[k]);
+                } else {
+                    for (int v = gl; on && v < CV; v += 8) g += dot4(zp[v], zq[v]);
+                }
+                g = sum8(g);
+                const float root = sqrtf(a) * sqrtf(b), gm = fabsf(g);
+                if (on && gm > tol * root && gm > floor_abs) {
+                    if (gm > done * root && a > null2 && b > null2) rough = 1;
+                    const float t = rotation_tan(b - a, g), h = half_tan(t), s = shear_sin(h, 0.0f);
+                    if constexpr (NV > 0) {
+#pragma unroll
+                        for (int k = 0; k < NV; ++k) {
+                            const int v = gl + 8 * k;
+                            if (v < V) {
+                                turn4(x[k], y[k], h, s);
+                                zp[v] = x[k];
+                                zq[v] = y[k];
+                            }
+                        }
+                    } else {
+                        for (int v = gl; v < V; v += 8) {
+                            float4 u = zp[v], w = zq[v];
+                            turn4(u, w, h, s);
+                            zp[v] = u;
+                            zq[v] = w;
+                        }
+                    }
+                    if (gl < 2) nrm2[gl == 0 ? p : q] = fmaxf(fmaf(gl == 0 ? -t : t, g, gl == 0 ? a : b), 0.0f);
+                }
+            }
+            __syncthreads();
+        }
+        if (!__syncthreads_or(rough)) break;
+    }
+}
+
+// 1 / norm of a block, by all threads of a CTA.
+__device__ double block_scale(const double* __restrict__ Z, int n) {
     __shared__ double red[32];
     __shared__ double tot;
-    const int R = B.R, C = B.C, W = C + R;
-    const double* Zr = zraw + B.z_off;
     double s = 0.0;
-    for (int e = threadIdx.x; e < R * C; e += blockDim.x) s = fma(Zr[e], Zr[e], s);
+    for (int e = threadIdx.x; e < n; e += blockDim.x) s = fma(Z[e], Z[e], s);
     s = wsum(s);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -233,55 +317,62 @@ __device__ void osj32_block(const SvdBlock& B, const double* __restrict__ zraw, 
         tot = t;
     }
     __syncthreads();
-    const double scale = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
-    for (int e = rank * blockDim.x + threadIdx.x; e < R * W; e += blockDim.x * ctas) {
-        const int r = e / W, c = e - r * W;
-        const float v = c < C ? static_cast<float>(Zr[static_cast<int64_t>(r) * C + c] * scale) : (c - C == r ? 1.0f : 0.0f);
-        if constexpr (SMEM)
-            work[e] = v;
-        else
-            __stcg(work + e, v);
-    }
-    if constexpr (SMEM)
-        __syncthreads();
-    else
-        cgx::this_cluster().sync();
-    if (W <= 128)
-        osj_sweeps<float, SMEM, 4>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
-    else if (W <= 256)
-        osj_sweeps<float, SMEM, 8>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
-    else
-        osj_sweeps<float, SMEM, 0>(work, nrm2, R, C, W, 1.0f, 1e-3f, conv, rank, ctas);
-    for (int e = rank * blockDim.x + threadIdx.x; e < R * R; e += blockDim.x * ctas) {
-        const int r = e / R, c = e - r * R;
-        const float* p = work + static_cast<int64_t>(r) * W + C + c;
-        float v;
-        if constexpr (SMEM)
-            v = *p;
-        else
-            v = __ldcg(p);
-        J[B.j_off + e] = static_cast<double>(v);
-    }
+    return tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
 }
 
-__global__ void __launch_bounds__(1024) k_osj32_smem(const SvdBlock* __restrict__ blocks, const double* __restrict__ zraw,
-                                                    double* __restrict__ J, int* __restrict__ conv, int smem_floats) {
-    extern __shared__ float sm32[];
+// FP32 start: [Z | I] of a block scaled to norm 1; J (R x R) leaves in FP64.
+__global__ void __launch_bounds__(kOsj32Threads) k_osj32_smem(const SvdBlock* __restrict__ blocks, const double* __restrict__ zraw,
+                                                              double* __restrict__ J, int smem_floats) {
+    extern __shared__ float4 sm32[];
     const SvdBlock B = blocks[blockIdx.x];
     if (B.R <= 0 || B.C <= 0 || B.smem == 0) return;
-    const int need = B.R * (B.C + B.R) + B.R;
-    if (need > smem_floats) return;  // never: the host marks only blocks that fit
-    osj32_block<true>(B, zraw, sm32, sm32 + B.R * (B.C + B.R), J, conv + blockIdx.x * 2 * kSvdConv, 0, 1);
+    const int R = B.R, C = B.C, CV = (C + 3) / 4, V = CV + (R + 3) / 4, W = 4 * V;
+    if (R * W + R > smem_floats) return;  // never: the host marks only blocks that fit
+    const double* Zr = zraw + B.z_off;
+    const double scale = block_scale(Zr, R * C);
+    float* work = reinterpret_cast<float*>(sm32);
+    for (int e = threadIdx.x; e < R * W; e += blockDim.x) {
+        const int r = e / W, c = e - r * W;
+        work[e] = c < C ? static_cast<float>(Zr[r * C + c] * scale) : (c - 4 * CV == r ? 1.0f : 0.0f);
+    }
+    __syncthreads();
+    float* nrm2 = work + R * W;
+    if (V <= 32)
+        osj32_sweeps<4>(sm32, nrm2, R, CV, V);
+    else if (V <= 56)
+        osj32_sweeps<7>(sm32, nrm2, R, CV, V);
+    else
+        osj32_sweeps<0>(sm32, nrm2, R, CV, V);
+    for (int e = threadIdx.x; e < R * R; e += blockDim.x) {
+        const int r = e / R, c = e - r * R;
+        J[B.j_off + e] = static_cast<double>(work[r * W + 4 * CV + c]);
+    }
 }
 
 __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
-    k_osj32_global(const SvdBlock* __restrict__ blocks, const double* __restrict__ zraw, float* __restrict__ work,
+    k_osj32_global(const SvdBlock* __restrict__ blocks, const double* __restrict__ zraw, float* __restrict__ works,
                    float* __restrict__ nrm, double* __restrict__ J, int* __restrict__ conv) {
-    const int b = blockIdx.x / kOsjC;
+    const int b = blockIdx.x / kOsjC, rank = static_cast<int>(cgx::this_cluster().block_rank());
     const SvdBlock B = blocks[b];
     if (B.R <= 0 || B.C <= 0 || B.smem != 0) return;  // uniform over the cluster
-    osj32_block<false>(B, zraw, work + B.w_off, nrm + B.n_off, J, conv + b * 2 * kSvdConv,
-                       static_cast<int>(cgx::this_cluster().block_rank()), kOsjC);
+    const int R = B.R, C = B.C, W = C + R;
+    const double* Zr = zraw + B.z_off;
+    float* work = works + B.w_off;
+    const double scale = block_scale(Zr, R * C);
+    for (int e = rank * blockDim.x + threadIdx.x; e < R * W; e += blockDim.x * kOsjC) {
+        const int r = e / W, c = e - r * W;
+        __stcg(work + e, c < C ? static_cast<float>(Zr[static_cast<int64_t>(r) * C + c] * scale) : (c - C == r ? 1.0f : 0.0f));
+    }
+    cgx::this_cluster().sync();
+    int* cv = conv + b * kSvdConv;
+    if (W <= 256)
+        osj_sweeps<float, 8>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC);
+    else
+        osj_sweeps<float, 0>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC);
+    for (int e = rank * blockDim.x + threadIdx.x; e < R * R; e += blockDim.x * kOsjC) {
+        const int r = e / R, c = e - r * R;
+        J[B.j_off + e] = static_cast<double>(__ldcg(work + static_cast<int64_t>(r) * W + C + c));
+    }
 }
 
 // FP64 finish on Z' (R x W, W = C, or C + R with the companion J): singular values squared, sorted
@@ -314,15 +405,15 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
         tot = t;
     }
     cgx::this_cluster().sync();  // every CTA has read Z before any rotates it
-    int* cv = conv + (b * 2 + 1) * kSvdConv;
+    int* cv = conv + (gridDim.x / kOsjC + b) * kSvdConv;
     // the companion is orthonormal by construction; normalised rows only as far as they are uncoupled
     const float done = B.companion ? 1e-11f : 1e-13f;
     if (W <= 160)
-        osj_sweeps<double, false, 5>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
+        osj_sweeps<double, 5>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     else if (W <= 320)
-        osj_sweeps<double, false, 10>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
+        osj_sweeps<double, 10>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     else
-        osj_sweeps<double, false, 0>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
+        osj_sweeps<double, 0>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
     // exact norms of the final rows, then the vectors by descending norm (ties by row)
     const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) * kOsjC + rank;
     const int warps = (blockDim.x >> 5) * kOsjC;
@@ -458,7 +549,7 @@ void SvdPlan::build(const std::vector<SvdShape>& shapes, int smem_dim) {
         f_size += static_cast<int64_t>(B.R) * (B.C + (B.companion ? B.R : 0));
         B.n_off = n_size;
         n_size += B.R;
-        const int64_t fl = static_cast<int64_t>(B.R) * (B.C + B.R) + B.R;
+        const int64_t fl = static_cast<int64_t>(B.R) * ((B.C + 3) / 4 * 4 + (B.R + 3) / 4 * 4) + B.R;
         // shared memory while it fits and the caller's limit on the dimension allows it
         B.smem = (s.dim <= smem_dim || smem_dim >= kSvdSmemDefault) && fl <= kSvdSmemFloats ? 1 : 0;
         B.w_off = w_size;
@@ -551,8 +642,8 @@ cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, 
         e = cudaFuncSetAttribute(k_osj32_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kSvdSmemFloats * static_cast<int>(sizeof(float)));
         if (e != cudaSuccess) return e;
-        const int threads = std::min(1024, std::max(64, 32 * ((P.max_rows + 1) / 2)));  // a warp per pair
-        k_osj32_smem<<<nb, threads, bytes, st>>>(blocks, z, j0, conv, P.smem_floats);
+        const int threads = std::min(kOsj32Threads, std::max(64, ((P.max_rows + 1) / 2 * 8 + 31) / 32 * 32));  // 8 per pair
+        k_osj32_smem<<<nb, threads, bytes, st>>>(blocks, z, j0, P.smem_floats);
     }
     if (P.any_global) k_osj32_global<<<nb * kOsjC, 256, 0, st>>>(blocks, z, w, n32, j0, conv);
     auto gemm = [&](int step, const double* a, const double* b, double* c) {
