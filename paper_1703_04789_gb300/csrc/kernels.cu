@@ -1099,7 +1099,12 @@ __global__ void __launch_bounds__(1024) k_trunc_select(const int64_t* __restrict
     for (int r = tid; r < total; r += nt) {
         const int cs = start[r], i = order[r];
         int before = 0;
-        for (int j = cs; j < total && start[j] == cs; ++j) before += order[j] < i ? 1 : 0;
+        // a cluster of dropped values needs no order (the null directions of all labels are one: hundreds of
+        // dependent loads a thread, TRUNCFIG)
+        if (sorted[cs] < drop_abs)
+            before = r - cs;
+        else
+            for (int j = cs; j < total && start[j] == cs; ++j) before += order[j] < i ? 1 : 0;
         order2[cs + before] = i;
         sig2[cs + before] = sorted[r];
     }

@@ -451,52 +451,51 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
 }
 
 // Grouped FP64 products of the Newton-Schulz steps and of Z' = J Z: C = alpha A op(B) + diag 1, one CTA
-// per 32 x 32 tile (the FP64 pipes of all SMs), K staged through shared memory in chunks of 16.
+// per 16 x 16 tile, K staged through shared memory in chunks of 32.  The FP64 pipe of an SM (2 FMA per clock)
+// bounds a tile, so blocks of some tens of rows need tiles small enough for all SMs; a launch of the
+// canonicalisation below takes 12 us (30 us with 32 x 32 tiles), of the middle decimation of L = 24, D = 256 26 us (66 us).
+constexpr int kGemmTile = 16;
 __global__ void __launch_bounds__(128) k_block_gemm(const double* __restrict__ a, const double* __restrict__ bm,
                                                     double* __restrict__ cm, const SvdGemm* __restrict__ gs,
                                                     const int3* __restrict__ tiles) {
-    __shared__ double As[16][34], Bs[16][34];
+    constexpr int KC = 32;
+    __shared__ double As[KC][kGemmTile + 1], Bs[KC][kGemmTile + 1];
     const int3 tl = tiles[blockIdx.x];
     const SvdGemm G = gs[tl.x];
     const int m0 = tl.y, n0 = tl.z, tid = threadIdx.x;
     const double* A = a + G.a;
     const double* Bp = bm + G.b;
-    const int tr = tid >> 3, tc = tid & 7;  // 16 x 8 threads, 2 x 4 outputs each
-    double acc[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
-    for (int k0 = 0; k0 < G.K; k0 += 16) {
-        for (int e = tid; e < 512; e += 128) {
-            const int r = e >> 4, k = e & 15;
+    const int tr = tid >> 3, tc = tid & 7;  // 16 x 8 threads, 1 x 2 outputs each
+    double acc[2] = {0.0, 0.0};
+    for (int k0 = 0; k0 < G.K; k0 += KC) {
+#pragma unroll
+        for (int e = tid; e < KC * kGemmTile; e += 128) {
+            const int r = e / KC, k = e % KC;
             As[k][r] = (m0 + r < G.M && k0 + k < G.K) ? A[static_cast<int64_t>(m0 + r) * G.lda + k0 + k] : 0.0;
             if (G.transb) Bs[k][r] = (n0 + r < G.N && k0 + k < G.K) ? Bp[static_cast<int64_t>(n0 + r) * G.ldb + k0 + k] : 0.0;
         }
-        if (!G.transb)
-            for (int e = tid; e < 512; e += 128) {
-                const int k = e >> 5, c = e & 31;
+        if (!G.transb) {
+#pragma unroll
+            for (int e = tid; e < KC * kGemmTile; e += 128) {
+                const int k = e / kGemmTile, c = e % kGemmTile;
                 Bs[k][c] = (n0 + c < G.N && k0 + k < G.K) ? Bp[static_cast<int64_t>(k0 + k) * G.ldb + n0 + c] : 0.0;
             }
+        }
         __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            double x[2], y[4];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) x[i] = As[k][tr + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) y[j] = Bs[k][tc + 8 * j];
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
+#pragma unroll 8
+        for (int k = 0; k < min(KC, G.K - k0); ++k) {
+            const double x = As[k][tr];
+            acc[0] = fma(x, Bs[k][tc], acc[0]);
+            acc[1] = fma(x, Bs[k][tc + 8], acc[1]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = m0 + tr + 16 * i, c = n0 + tc + 8 * j;
-            if (r < G.M && c < G.N)
-                cm[G.c + static_cast<int64_t>(r) * G.ldc + c] = G.alpha * acc[i][j] + (r == c ? G.diag : 0.0);
-        }
+    for (int j = 0; j < 2; ++j) {
+        const int r = m0 + tr, c = n0 + tc + 8 * j;
+        if (r < G.M && c < G.N)
+            cm[G.c + static_cast<int64_t>(r) * G.ldc + c] = G.alpha * acc[j] + (r == c ? G.diag : 0.0);
+    }
 }
 
 // The companion columns of Z' of the blocks that keep J.
@@ -588,8 +587,8 @@ void SvdPlan::build(const std::vector<SvdShape>& shapes, int smem_dim) {
                 G.c = B.f_off;
                 G.ldc = B.C + (B.companion ? B.R : 0);
             }
-            for (int m0 = 0; m0 < G.M; m0 += 32)
-                for (int n0 = 0; n0 < G.N; n0 += 32) tiles.push_back(make_int3(static_cast<int>(gemms.size()), m0, n0));
+            for (int m0 = 0; m0 < G.M; m0 += kGemmTile)
+                for (int n0 = 0; n0 < G.N; n0 += kGemmTile) tiles.push_back(make_int3(static_cast<int>(gemms.size()), m0, n0));
             gemms.push_back(G);
         }
         gemm_rng.push_back(static_cast<int>(tiles.size()));
