@@ -1100,7 +1100,7 @@ __global__ void __launch_bounds__(1024) k_trunc_select(const int64_t* __restrict
         const int cs = start[r], i = order[r];
         int before = 0;
         // a cluster of dropped values needs no order (the null directions of all labels are one: hundreds of
-        // dependent loads a thread, TRUNCFIG)
+        // dependent loads a thread, 49 us a launch of the L = 24, D = 256 canonicalisation, 8 us without)
         if (sorted[cs] < drop_abs)
             before = r - cs;
         else
