@@ -772,7 +772,8 @@ __device__ void jacobi_cta_f32(float*& a, float*& v, float*& a2, float*& v2, int
                 const float apq = a[lo * kRitzLd + hi];
                 if (!(fabsf(apq) > tiny)) return;
                 const float z = __fdividef(a[hi * kRitzLd + hi] - a[lo * kRitzLd + lo], 2.0f * apq);
-                const float t = copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f)));
+                const float w = fminf(fabsf(z), 1e18f), q2 = fmaf(w, w, 1.0f);
+                const float t = copysignf(__fdividef(1.0f, fmaf(q2, rsqrtf(q2), w)), z);
                 c = rsqrtf(fmaf(t, t, 1.0f));
                 s = i == lo ? -t * c : t * c;
             };

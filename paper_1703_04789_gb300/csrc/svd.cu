@@ -35,6 +35,26 @@ __device__ __forceinline__ T wsum(T v) {
     return v;
 }
 
+// The rows of [0, R) whose squared norm is above `least`, ascending, by the first warp of a CTA (R <= kMaxRows).
+// Rows beyond a block's rank shrink to the rounding noise of the large rows within two sweeps; without them a
+// sweep has as many rounds as the block has rank.
+constexpr int kMaxRows = 1024;
+constexpr int kFullSweeps = 2;
+template <class Norm>
+__device__ __forceinline__ void list_rows(unsigned short* list, int* count, int R, bool all, Norm above) {
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    int n = 0;
+    for (int base = 0; base < R; base += 32) {
+        const int r = base + lane;
+        const bool in = r < R && (all || above(r));
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (in) list[n + __popc(m & ((1u << lane) - 1u))] = static_cast<unsigned short>(r);
+        n += __popc(m);
+    }
+    if (lane == 0) *count = n;
+}
+
 // FP32 <-> FP64 by integer instructions: a conversion instruction runs on the FP64 pipe.  to_f32 truncates,
 // divides by 2^shift first and clamps to [0, FLT_MAX]; to_f64 is exact (zero for subnormals).
 __device__ __forceinline__ float to_f32(float v, int) { return v; }
@@ -93,11 +113,13 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
     const int lane = threadIdx.x & 31;
     const int warp = (threadIdx.x >> 5) * ctas + rank;  // pairs go round the CTAs: the FP64 pipes of all share them
     const int warps = (blockDim.x >> 5) * ctas;
-    const int np = (R + 1) & ~1, half = np / 2;
+    __shared__ unsigned short list[kMaxRows];
+    __shared__ int count;
     constexpr bool kF64 = sizeof(T) == 8;
     constexpr float tol = kF64 ? 1e-15f : 3e-7f;
     constexpr float floor_abs = kF64 ? 0.0f : 1e-12f;  // FP32: the noise of the block's largest rows
     constexpr float null2 = kF64 ? static_cast<float>(kNullRel * kNullRel) : 1e-13f;
+    constexpr float least = kF64 ? 1e-28f : null2;
     // squared norms and products as FP32 numbers relative to the block's squared norm (to a factor of 2)
     int shift = 0;
     if constexpr (kF64) shift = norm2_all > T(0) ? ((__double2hiint(norm2_all) >> 20) & 2047) - 1023 : 0;
@@ -115,6 +137,9 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
             if (lane == 0) stg(nrm2 + r, s);
         }
         barrier();
+        list_rows(list, &count, R, sweep < kFullSweeps, [&](int r) { return to_f32(ld(nrm2 + r), shift) > least; });
+        barrier();  // every CTA has its list before a rotation moves a norm
+        const int np = (count + 1) & ~1, half = np / 2, rows = count;
         bool rough = false;
         for (int round = 0; round < np - 1; ++round) {
             for (int i = warp; i < half; i += warps) {
@@ -126,7 +151,9 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
                     p = q;
                     q = t;
                 }
-                if (q >= R) continue;
+                if (q >= rows) continue;
+                p = list[p];
+                q = list[q];
                 T* zp = Z + static_cast<int64_t>(p) * W;
                 T* zq = Z + static_cast<int64_t>(q) * W;
                 const T a = ld(nrm2 + p), b = ld(nrm2 + q);
@@ -226,7 +253,8 @@ template <int NV>
 __device__ void osj32_sweeps(float4* Z, float* nrm2, int R, int CV, int V) {
     constexpr float tol = 3e-7f, floor_abs = 1e-12f, null2 = 1e-13f, done = 1e-3f;
     const int gl = threadIdx.x & 7, group = threadIdx.x >> 3, groups = blockDim.x >> 3;
-    const int np = (R + 1) & ~1, half = np / 2;
+    __shared__ unsigned short list[kMaxRows];
+    __shared__ int count;
     for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
         for (int base = 0; base < R; base += groups) {
             const int r = base + group;
@@ -237,6 +265,9 @@ __device__ void osj32_sweeps(float4* Z, float* nrm2, int R, int CV, int V) {
             if (r < R && gl == 0) nrm2[r] = s;
         }
         __syncthreads();
+        list_rows(list, &count, R, sweep < kFullSweeps, [&](int r) { return nrm2[r] > null2; });
+        __syncthreads();
+        const int np = (count + 1) & ~1, half = np / 2, rows = count;
         int rough = 0;
         for (int round = 0; round < np - 1; ++round) {
             for (int base = 0; base < half; base += groups) {
@@ -249,7 +280,11 @@ __device__ void osj32_sweeps(float4* Z, float* nrm2, int R, int CV, int V) {
                     p = q;
                     q = t;
                 }
-                bool on = i < half && q < R;
+                bool on = i < half && q < rows;
+                if (on) {
+                    p = list[p];
+                    q = list[q];
+                }
                 const float a = on ? nrm2[p] : 0.0f, b = on ? nrm2[q] : 0.0f;
                 on = on && (a > null2 || b > null2);
                 float4* zp = Z + p * V;
