@@ -55,6 +55,18 @@ __device__ __forceinline__ void list_rows(unsigned short* list, int* count, int 
     if (lane == 0) *count = n;
 }
 
+// Place of row r among R rows by descending norm (ties by row), by a warp.
+template <class Norm>
+__device__ __forceinline__ int row_rank(int R, int r, Norm norm) {
+    const auto v = norm(r);
+    int before = 0;
+    for (int j = threadIdx.x & 31; j < R; j += 32) {
+        const auto o = norm(j);
+        before += (o > v || (o == v && j < r)) ? 1 : 0;
+    }
+    return __reduce_add_sync(0xffffffffu, before);
+}
+
 // FP32 <-> FP64 by integer instructions: a conversion instruction runs on the FP64 pipe.  to_f32 truncates,
 // divides by 2^shift first and clamps to [0, FLT_MAX]; to_f64 is exact (zero for subnormals).
 __device__ __forceinline__ float to_f32(float v, int) { return v; }
@@ -378,9 +390,10 @@ __global__ void __launch_bounds__(kOsj32Threads) k_osj32_smem(const SvdBlock* __
         osj32_sweeps<7>(sm32, nrm2, R, CV, V);
     else
         osj32_sweeps<0>(sm32, nrm2, R, CV, V);
-    for (int e = threadIdx.x; e < R * R; e += blockDim.x) {
-        const int r = e / R, c = e - r * R;
-        J[B.j_off + e] = static_cast<double>(work[r * W + 4 * CV + c]);
+    for (int r = threadIdx.x >> 5; r < R; r += blockDim.x >> 5) {
+        const int to = row_rank(R, r, [&](int j) { return nrm2[j]; });
+        for (int c = threadIdx.x & 31; c < R; c += 32)
+            J[B.j_off + static_cast<int64_t>(to) * R + c] = static_cast<double>(work[r * W + 4 * CV + c]);
     }
 }
 
@@ -404,9 +417,10 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
         osj_sweeps<float, 8>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC);
     else
         osj_sweeps<float, 0>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC);
-    for (int e = rank * blockDim.x + threadIdx.x; e < R * R; e += blockDim.x * kOsjC) {
-        const int r = e / R, c = e - r * R;
-        J[B.j_off + e] = static_cast<double>(__ldcg(work + static_cast<int64_t>(r) * W + C + c));
+    for (int r = (threadIdx.x >> 5) * kOsjC + rank; r < R; r += (blockDim.x >> 5) * kOsjC) {
+        const int to = row_rank(R, r, [&](int j) { return __ldcg(nrm + B.n_off + j); });
+        for (int c = threadIdx.x & 31; c < R; c += 32)
+            J[B.j_off + static_cast<int64_t>(to) * R + c] = static_cast<double>(__ldcg(work + static_cast<int64_t>(r) * W + C + c));
     }
 }
 

@@ -48,6 +48,25 @@ def test_canonical_form_is_isometric_and_keeps_the_state(K, N, twoM, D, smem_max
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("K,D,smem_max", [(7, 24, 0), (8, 90, 0), (8, 90, 8)])
+def test_graded_states_stay_isometric(K, D, smem_max):
+    """Singular values over twelve decades, most of a block's rows far below the largest: the rotation of two
+    rows of very different norms, rows at the rounding noise, and values dropped below 1e-7."""
+    require_gpu()
+    from paper_1703_04789_gb300 import Spmps
+    labels, tens = inputs.random_mps(K, 6, 0, D, 3)
+    for i in (1, 2, 4):
+        tens[i] = tens[i] * 10.0 ** -((7 * np.arange(tens[i].shape[2])) % 13)
+    dev = Spmps(K, 6, 0, 0, 4, D, jacobi_smem_max=smem_max)
+    dev.set_hubbard(1.0, 4.0)
+    dev.set_mps(labels, tens, center=0)
+    dev.canonicalize()
+    lab, ts, _ = dev.get_mps()
+    assert _deviation(lab, ts) < 1e-12
+    dev.close()
+
+
+@pytest.mark.gpu
 def test_blocks_beyond_shared_memory_in_both_directions():
     """Blocks of up to 272 x 272, whose [Z | I] no longer fits one CTA's shared memory: canonicalisation
     (vectors of the right side), then steps to the right with one Davidson iteration each (the Ritz
