@@ -118,8 +118,9 @@ __device__ __forceinline__ double shear_sin(float hf, double h) {
 // one number or 32, so a pair issues 3 per 32 elements for the shears, one for the product, 5 for its sum
 // over the warp, 2 for the norms and at most 7 for the sine; comparisons, conversions and the angle are
 // FP32 and integer instructions.  Measured (GB300): a launch
-// of the canonicalisation below 0.63 ms on average, the middle decimation of L = 24, D = 256 2.0 ms; 0.81 and 2.7 ms
-// with the comparisons, conversions and the angle's operands in FP64.
+// of the canonicalisation below 0.38 ms on average, the middle decimation of L = 24, D = 256 2.0 ms; 0.81 and 2.7 ms
+// with the comparisons, conversions and the angle's operands in FP64, 0.63 ms without the next two.  Rows beyond the
+// block's rank leave the rounds after two sweeps (0.57 ms), and the FP32 start hands its rows over by descending norm.
 template <class T, int NCH>
 __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, float done, int* conv, int rank, int ctas) {
     const int lane = threadIdx.x & 31;
@@ -241,7 +242,8 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
 // The FP32 start in one CTA's shared memory: 8 lanes per pair and four elements per access, so that a warp
 // computes four angles and four sums at once.  The scheduler's issue slots bound it (a round of 26 pairs was
 // 1200 of them per sub-partition with a warp per pair, half for the angle and the sum); measured (GB300): the
-// middle decimation of L = 24, D = 256 3.3 ms and 0.37 ms on average in the canonicalisation below, 5.0 and 0.52 ms before.
+// middle decimation of L = 24, D = 256 3.1 ms and 0.31 ms on average in the canonicalisation below, 5.0 and 0.52 ms
+// before.  The pairs of a sweep follow the order of the norms (3.4 and 0.34 ms by row).
 __device__ __forceinline__ float sum8(float v) {
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -278,6 +280,11 @@ __device__ void osj32_sweeps(float4* Z, float* nrm2, int R, int CV, int V) {
         }
         __syncthreads();
         list_rows(list, &count, R, sweep < kFullSweeps, [&](int r) { return nrm2[r] > null2; });
+        __syncthreads();
+        for (int r = threadIdx.x >> 5; r < R; r += blockDim.x >> 5) {
+            const int to = row_rank(R, r, [&](int j) { return nrm2[j]; });
+            if ((threadIdx.x & 31) == 0 && to < count) list[to] = static_cast<unsigned short>(r);
+        }
         __syncthreads();
         const int np = (count + 1) & ~1, half = np / 2, rows = count;
         int rough = 0;
@@ -657,8 +664,8 @@ double* SvdPlan::z_buffer(void* ws) const {
 }
 
 // Measured (GB300): the decimations of one canonicalisation (random L = 24, D = 256 triplet state, 23 of them,
-// blocks up to 52 rows) take 33.6 ms, the middle decimation of the L = 24, D = 256 chain (blocks up to 150 rows)
-// 7.6 ms; two-sided FP64 Jacobi on X X^T with a one-thread truncation took 308 and 22 ms.
+// blocks up to 100 rows) take 17.5 ms, the middle decimation of the L = 24, D = 256 chain (blocks up to 126 rows)
+// 5.3 ms; two-sided FP64 Jacobi on X X^T with a one-thread truncation took 308 and 22 ms.
 cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, cudaStream_t st) {
     const int nb = static_cast<int>(P.blocks.size());
     if (nb == 0) return cudaSuccess;
