@@ -683,7 +683,8 @@ constexpr int kRitzMax = 32;
 // pipe for 64 clocks.  The FP64 products of vectors of 32 run on four warps, one per sub-partition, each
 // taking a quarter of the sum; every thread of the CTA owns two elements of the FP32 matrices, so a Jacobi
 // round (the two rotations of an element's row and column, recomputed by each thread) is one barrier.
-// Measured (GB300, ncu, L = 16, D = 64 step, subspaces up to 20): 48 us; one warp took 93 us.
+// Measured (GB300, ncu, L = 16, D = 64 step, subspaces up to 20): 46 us (49 us with IEEE division and root in the
+// Jacobi rotations); one warp took 93 us.
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
