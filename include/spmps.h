@@ -217,6 +217,8 @@ spmps_status spmps_x_layout(spmps_handle h, int site, int64_t* n_x, int* n_block
  * x, y, z are DEVICE pointers in the row-block layout (n_x doubles each, x read-only; y or z
  * may be NULL to skip that output).  stream is a cudaStream_t (NULL: the handle's stream);
  * the call is asynchronous with respect to the host except when environments must be built.
+ * Actions on several streams share the handle's workspaces: each waits, on the device, for the
+ * previous one, and so does all later work of the handle.
  * The H part uses the handle's precision option (FP64, TF32 or 3xTF32 block products); z is FP64. */
 spmps_status spmps_apply_heff(spmps_handle h, int site, const double* x, double* y, double* z,
                               void* stream);
@@ -266,10 +268,10 @@ spmps_status spmps_device_tf32_peak(int device, int kind, int sms, double* tflop
  * call for that site builds them, and allocates); otherwise SPMPS_ERR_STATE.  All calls share the
  * array, which keeps the last call's contents (the call zeroes what must start at zero): calls
  * that overlap on the GPU race and must be serialised.  When `stream` is not the handle's stream,
- * the call orders it after the work already queued on the handle's stream (an event; the first
- * such call on a handle creates it).  The first call on each device looks up the array's address
- * (cudaGetSymbolAddress).  The per-launch profiler (spmps_profile) does not record this call.
- * Arguments as in spmps_apply_heff. */
+ * the call orders it after the work already queued on the handle's stream, and the handle's later
+ * work after it (two events; the first such call on a handle creates them).  The first call on each
+ * device looks up the array's address (cudaGetSymbolAddress).  The per-launch profiler
+ * (spmps_profile) does not record this call.  Arguments as in spmps_apply_heff. */
 spmps_status spmps_apply_heff_noalloc(spmps_handle h, int site, const double* x, double* y, double* z,
                                       void* stream);
 

@@ -1727,7 +1727,7 @@ spmps_status spmps_create(int K, int N, int twoM, int twoS, int n_beta, int D, c
     h->K = K; h->N = N; h->twoM = twoM; h->twoS = twoS; h->G = n_beta; h->D = D;
     h->opt = o;
     h->device = o.device;
-    if (cudaSetDevice(h->device) != cudaSuccess || cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess) {
+    if (cudaSetDevice(h->device) != cudaSuccess || cudaStreamCreateWithFlags(&h->stream.raw, cudaStreamNonBlocking) != cudaSuccess) {
         delete h;
         return fail(nullptr, SPMPS_ERR_CUDA, "cannot create a stream on the device");
     }
@@ -1764,7 +1764,7 @@ spmps_status spmps_create(int K, int N, int twoM, int twoS, int n_beta, int D, c
 spmps_status spmps_destroy(spmps_handle h) {
     if (!h) return SPMPS_OK;
     cudaSetDevice(h->device);
-    if (h->stream) cudaStreamSynchronize(h->stream);
+    if (h->stream.raw) cudaStreamSynchronize(h->stream);
     for (auto& r : h->timers_live) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto& r : h->timers_free) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     h->apply_plans.clear();
@@ -1778,7 +1778,8 @@ spmps_status spmps_destroy(spmps_handle h) {
     if (h->aux_fork) cudaEventDestroy(h->aux_fork);
     if (h->aux_join) cudaEventDestroy(h->aux_join);
     if (h->noalloc_order) cudaEventDestroy(h->noalloc_order);
-    if (h->stream) cudaStreamDestroy(h->stream);
+    if (h->stream.foreign) cudaEventDestroy(h->stream.foreign);
+    if (h->stream.raw) cudaStreamDestroy(h->stream.raw);
     delete h;
     return SPMPS_OK;
 }
@@ -2044,17 +2045,21 @@ spmps_status spmps_apply_heff(spmps_handle h, int site, const double* x, double*
     if (site < 0 || site > h->K - 2) return fail(h, SPMPS_ERR_BAD_INPUT, "site out of range");
     if (!x || (!y && !z)) return fail(h, SPMPS_ERR_BAD_INPUT, "x and one of y, z are required");
     if (cudaSetDevice(h->device) != cudaSuccess) return fail(h, SPMPS_ERR_CUDA, "cudaSetDevice");
-    cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : h->stream;
-    if (s != h->stream) {
-        // environments are built on the handle's stream; order the caller's stream after it
+    const bool foreign = stream && static_cast<cudaStream_t>(stream) != h->stream.raw;
+    const cudaStream_t s = foreign ? static_cast<cudaStream_t>(stream) : h->stream;
+    if (foreign) {
+        // environments are built on the handle's stream; order the caller's stream after it, and after
+        // an action on another caller's stream (the workspaces are the same)
         Plan* P = nullptr;
         st = get_apply_plan(h, site, &P);
         if (st != SPMPS_OK) return st;
-        CK(cudaStreamSynchronize(h->stream));
+        CK(cudaStreamSynchronize(h->stream.raw));
+        CK(h->stream.enter(s));
     }
     h->apply_precision = h->opt.precision;
     st = do_apply(h, site, x, y, z, s);
     h->apply_precision = 0;
+    if (foreign) CK(h->stream.leave(s));
     return st;
 }
 
@@ -2313,7 +2318,7 @@ spmps_status spmps_get_mps(spmps_handle h, int* bond_dims, int* labels, double* 
 
 spmps_status spmps_stream(spmps_handle h, void** stream) {
     if (!h || !stream) return fail(h, SPMPS_ERR_BAD_INPUT, "NULL argument");
-    *stream = h->stream;
+    *stream = h->stream.raw;
     return SPMPS_OK;
 }
 

@@ -237,17 +237,55 @@ struct MlpState {
     spmps::DevMem h_idx, h_feat, h_x, h_norm, h_dots;  // per solve
 };
 
+// The handle's own stream.  An action on a caller's stream uses the handle's workspaces, environments and
+// work lists and returns before it has run: leave() records an event behind it, and the next use of the
+// handle's stream (every use goes through the conversion) or of another caller's stream (enter()) waits
+// for that event on the device.
+struct OwnStream {
+    cudaStream_t raw = nullptr;
+    cudaEvent_t foreign = nullptr;  // behind the last action on a caller's stream
+    bool pending = false;           // which the own stream does not wait for yet
+    operator cudaStream_t() {
+        if (pending) {
+            pending = false;
+            cudaStreamWaitEvent(raw, foreign, 0);
+        }
+        return raw;
+    }
+    // A captured action runs when the caller launches its graph: the caller orders that.
+    static cudaError_t captured(cudaStream_t s, bool* yes) {
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(s, &status);
+        *yes = status != cudaStreamCaptureStatusNone;
+        return e;
+    }
+    cudaError_t enter(cudaStream_t s) const {
+        bool skip = false;
+        const cudaError_t e = captured(s, &skip);
+        return e != cudaSuccess || skip || !pending ? e : cudaStreamWaitEvent(s, foreign, 0);
+    }
+    cudaError_t leave(cudaStream_t s) {
+        bool skip = false;
+        cudaError_t e = captured(s, &skip);
+        if (e != cudaSuccess || skip) return e;
+        if (!foreign) e = cudaEventCreateWithFlags(&foreign, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(foreign, s);
+        pending = pending || e == cudaSuccess;
+        return e;
+    }
+};
+
 struct spmps_t {
     int K = 0, N = 0, twoM = 0, twoS = 0, G = 0, D = 0;
     spmps_options opt{};
     std::string err;
     int device = 0;
-    cudaStream_t stream = nullptr;
+    OwnStream stream;
     // second stream of the mixed-precision action: the FP64 N_eff products run on it while the
     // tensor-core H products run on the action's stream (created on first use)
     cudaStream_t aux_stream = nullptr;
     cudaEvent_t aux_fork = nullptr, aux_join = nullptr;
-    // orders a caller's stream after the handle's stream in spmps_apply_heff_noalloc
+    // orders a caller's stream after the handle's stream in spmps_apply_heff_noalloc (OwnStream: the reverse)
     cudaEvent_t noalloc_order = nullptr;
     spmps::DevMem tc_err;  // set by the stacked tensor-core GEMM when a bounded wait gave up
     std::vector<LowerState> lower;  // lower states of an excited-state optimisation (Eq. orthoB)

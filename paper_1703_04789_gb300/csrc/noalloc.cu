@@ -19,8 +19,9 @@
 //     and allocated, by a previous spmps_apply_heff or spmps_energy call for that site and MPS);
 //     otherwise the call returns SPMPS_ERR_STATE without doing anything.
 //   - The first call on each device looks up the array's device address (cudaGetSymbolAddress,
-//     with that device current), and the first call on each handle creates one CUDA event (no
-//     device memory) that orders the caller's stream after the handle's stream.
+//     with that device current), and the first call on each handle creates two CUDA events (no
+//     device memory) that order the caller's stream after the handle's stream and later calls on the
+//     handle after this one.
 //   - The H part always runs in FP64, whatever the handle's precision option: the pre-split TF32
 //     operands of the reduced-precision forms would need room of their own in the array.
 //   - The library's per-launch profiler (spmps_profile) is not used by this call.
@@ -76,16 +77,18 @@ extern "C" spmps_status spmps_apply_heff_noalloc(spmps_handle h, int site, const
     double* base = nullptr;
     e = scratch_address(h->device, &base);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaGetSymbolAddress");
-    cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : h->stream;
-    if (s != h->stream) {
+    const bool foreign = stream && static_cast<cudaStream_t>(stream) != h->stream.raw;
+    const cudaStream_t s = foreign ? static_cast<cudaStream_t>(stream) : h->stream;
+    if (foreign) {
         // environments are built on the handle's stream: order the caller's stream after the
         // work queued there so far (no host synchronisation)
         if (!h->noalloc_order) {
             e = cudaEventCreateWithFlags(&h->noalloc_order, cudaEventDisableTiming);
             if (e != cudaSuccess) { h->noalloc_order = nullptr; return cuda_fail(h, e, "cudaEventCreate"); }
         }
-        e = cudaEventRecord(h->noalloc_order, h->stream);
+        e = cudaEventRecord(h->noalloc_order, h->stream.raw);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->noalloc_order, 0);
+        if (e == cudaSuccess) e = h->stream.enter(s);
         if (e != cudaSuccess) return cuda_fail(h, e, "ordering the caller's stream after the handle's");
     }
     Slots S{};
@@ -111,6 +114,11 @@ extern "C" spmps_status spmps_apply_heff_noalloc(spmps_handle h, int site, const
     else st = plan_run(h, *P, S, G, 2 * G, s);
     h->apply_precision = prec_saved;
     h->profile = prof_saved;
+    // it reads the environments and the plan's lists, which the handle's stream may rewrite next
+    if (foreign) {
+        e = h->stream.leave(s);
+        if (e != cudaSuccess) return cuda_fail(h, e, "ordering the handle's stream after the caller's");
+    }
     if (st != SPMPS_OK) return st;
     ++h->applies;
     return SPMPS_OK;
