@@ -289,7 +289,7 @@ double comb_add(CombChan& C, const CombSpec& sp) {
                 K.ncoef = static_cast<int>(C.coefs.size()) - K.coef0;
             }
             const Class& K = it->second;
-            if (K.outs.empty()) continue;
+            if (K.outs.empty() && K.share_in < 0) continue;  // operator 1 may have outputs where this one has none
             CombPair P{};
             P.op = sp.op;
             P.rows = sp.row->groups[ga].dim;

@@ -1,0 +1,53 @@
+"""Actions of operators and bonds outside the usual: H without an output where N has one.
+
+The bounds are those of the other FP64 parity tests: 1e-10 of the largest entry (the forms differ from the
+oracle only in summation order).
+"""
+import numpy as np
+import pytest
+
+from oracle import mps as S
+from paper_1703_04789_gb300 import inputs
+from tests.gpu_util import masked_random_two_site, require_gpu
+
+
+def _three_body():
+    """T + T^T on four orbitals, T moving three electrons from the right half to the left one: the middle bond
+    has channels of charge +3 and -3 only."""
+    one, z = np.eye(2), np.diag([1.0, -1.0])
+    up = np.array([[0.0, 0.0], [1.0, 0.0]])
+    ca, cb = np.kron(up, one), np.kron(z, up)
+    pair, par = ca @ cb, np.kron(z, z)
+    W = [np.zeros((1, 2, 4, 4)), np.zeros((2, 2, 4, 4)), np.zeros((2, 2, 4, 4)), np.zeros((2, 1, 4, 4))]
+    W[0][0, 0], W[0][0, 1] = pair, pair.T
+    W[1][0, 0], W[1][1, 1] = ca @ par, par @ ca.T
+    W[2][0, 0], W[2][1, 1] = ca.T, ca
+    W[3][0, 0], W[3][1, 0] = pair.T, pair
+    return W
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("opts", [{}, {"fp64_tensor_cores": True}, {"batched": False}])
+def test_channels_of_charge_three_only(opts):
+    require_gpu()
+    from paper_1703_04789_gb300 import Spmps
+    K, N, twoM, twoS, D, G = 4, 4, 0, 0, 16, 3
+    sites = _three_body()
+    labels, tens = inputs.random_mps(K, N, twoM, D, 4)
+    P = S.prepare(labels, tens, sites, twoS, twoM, G)
+    dev = Spmps(K, N, twoM, twoS, G, D, **opts)
+    dev.set_mpo(sites)
+    dev.set_mps(P.mps.labels, P.mps.A, center=0)
+    P.build_left(K - 2)
+    rng = np.random.default_rng(1)
+    for k in range(K - 1):
+        ql, qr = P.mps.labels[k], P.mps.labels[k + 2]
+        lay = dev.x_layout(k)
+        x = masked_random_two_site(ql, qr, rng)
+        y_ref, z_ref = P.apply(x, k)
+        # another vector first: what an output that is not formed would hold
+        dev.apply_heff_host(k, rng.standard_normal(lay["n_x"]))
+        y, z = dev.apply_heff_host(k, dev.pack(x, lay, ql, qr))
+        assert np.abs(dev.unpack(z, lay, ql, qr) - z_ref).max() <= 1e-10 * max(1.0, np.abs(z_ref).max())
+        assert np.abs(dev.unpack(y, lay, ql, qr) - y_ref).max() <= 1e-10 * max(1.0, np.abs(y_ref).max())
+    dev.close()
