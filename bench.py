@@ -276,11 +276,11 @@ def run_ours(args):
         d.close()
     dtc = _handle("fast", hs[0]["twoM"], hs[0]["twoS"])
     dtc.set_mps(*hs[0]["ckpt"][:2], center=hs[0]["ckpt"][2])
-    phase_tc, (fl_op, by_op) = middle_site_phases(dtc, with_z=False)
+    phase_tc, (_, by_op) = middle_site_phases(dtc, with_z=False)
     dtc.close()
     doz = _handle("fast_fp64_tc", hs[0]["twoM"], hs[0]["twoS"])
     doz.set_mps(*hs[0]["ckpt"][:2], center=hs[0]["ckpt"][2])
-    phase_oz, _ = middle_site_phases(doz, with_z=True)
+    phase_oz, (fl_op, _) = middle_site_phases(doz, with_z=True)  # the products that an FP64 action runs
     doz.close()
     d64 = _handle("fast_fp64", hs[0]["twoM"], hs[0]["twoS"])
     d64.set_mps(*hs[0]["ckpt"][:2], center=hs[0]["ckpt"][2])

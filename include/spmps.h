@@ -230,11 +230,14 @@ spmps_status spmps_apply_heff_timed(spmps_handle h, int site, const double* x, d
                                     void* stream, double* phase_ms);
 
 /* Algorithmic flops of one call of spmps_apply_heff at `site`, split as [A, B, C] (symmetry-
- * allowed block products only: 2*m*n*k per block GEMM, 2*rows*cols per MPO-leg term). */
+ * allowed block products only: 2*m*n*k per block GEMM, 2*rows*cols per MPO-leg term), H's and N's
+ * each counted by itself, as in an action of that operator alone. */
 spmps_status spmps_apply_flops(spmps_handle h, int site, double* flops3);
 
 /* Algorithmic flops and bytes of one call of spmps_apply_heff at `site`, per operator (op 0 = H,
- * 1 = N) and phase (index 3*op + phase, phase 0 = A, 1 = B, 2 = C).  Flops as spmps_apply_flops.
+ * 1 = N) and phase (index 3*op + phase, phase 0 = A, 1 = B, 2 = C), of what a call with both outputs
+ * runs: N's phase A is 0 where N's T1 is part of H's (FP64 or fp64_tensor_cores, batched, an operator
+ * with a channel of identities up to `site`, no screening).  Flops otherwise as spmps_apply_flops.
  * Bytes, 8 per element: phase A reads the op's left environment and x and writes T1, each once
  * per beta point; phase B reads T1 and writes T3; phase C reads T3 and the op's right environment
  * and writes the per-beta partial outputs (the HBM roofline numerators).  Either pointer may be
@@ -329,8 +332,9 @@ spmps_status spmps_seniority(spmps_handle h, double* value);
 /* Statistics: counts[0] = Davidson iterations of the last sweep, counts[1] = projected applies
  * issued, counts[2] = kernel launches issued by the library since the handle was created;
  * values[0] = algorithmic flops of one projected apply at the last site applied (symmetry-
- * allowed block products only), values[1] = discarded weight of the last sweep, values[2] =
- * algorithmic flops of every projected apply issued since the handle was created.  Either
+ * allowed block products only, as spmps_apply_flops), values[1] = discarded weight of the last
+ * sweep, values[2] = algorithmic flops of every projected apply issued since the handle was created,
+ * without the products that an apply did not run (spmps_apply_costs).  Either
  * pointer may be NULL (counts holds 3, values 3). */
 spmps_status spmps_stats(spmps_handle h, int64_t* counts, double* values);
 

@@ -320,7 +320,7 @@ class Spmps:
 
     def apply_costs(self, site: int):
         """Algorithmic (flops, bytes), each [[A, B, C] of H, [A, B, C] of N], of one projected
-        action at `site`."""
+        action at `site` with both outputs (N's phase A is 0 where it is part of H's)."""
         fl, by = np.zeros(6), np.zeros(6)
         self._check(self.lib.spmps_apply_costs(self._h, site, fl.ctypes.data_as(C.POINTER(C.c_double)),
                                                by.ctypes.data_as(C.POINTER(C.c_double))))

@@ -344,7 +344,7 @@ spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t
     const int G = h->G;
     // both operators in one launch per phase: N's phase A is part of H's where the operator allows it
     // (its T1 is H's channel of identities; in FP64 only, N never runs in reduced precision)
-    const bool shared = batched && prec == 0 && P.chan.shares && r0 == 0 && r1 == 2 * G;
+    const bool shared = prec == 0 && shares_t1(h, P) && r0 == 0 && r1 == 2 * G;
     // ranges and beta points of the (op, g) range [a, b): whole operators, or beta points of one
     struct Part {
         int lo, hi, g0, ng;
@@ -1590,6 +1590,7 @@ spmps_status do_apply(spmps_t* h, int k, const double* x, double* y, double* z, 
     ++h->applies;
     h->last_apply_flops = P->flops;
     h->apply_flops_total += (y ? P->flops_op[0] : 0.0) + (z ? P->flops_op[1] : 0.0);
+    if (y && z && h->apply_precision == 0 && shares_t1(h, *P)) h->apply_flops_total -= P->flopsA_op[1];
     return SPMPS_OK;
 }
 
@@ -2099,14 +2100,15 @@ spmps_status spmps_apply_costs(spmps_handle h, int site, double* flops6, double*
     Plan* P = nullptr;
     st = get_apply_plan(h, site, &P);
     if (st != SPMPS_OK) return st;
+    const bool shared = h->opt.precision == 0 && shares_t1(h, *P);  // N's phase A is not run
     for (int op = 0; op < 2; ++op) {
         if (flops6) {
-            flops6[3 * op + 0] = P->flopsA_op[op];
+            flops6[3 * op + 0] = op == 1 && shared ? 0.0 : P->flopsA_op[op];
             flops6[3 * op + 1] = P->flopsB_op[op];
             flops6[3 * op + 2] = P->flopsC_op[op];
         }
         if (bytes6) {
-            bytes6[3 * op + 0] = P->bytesA_op[op];
+            bytes6[3 * op + 0] = op == 1 && shared ? 0.0 : P->bytesA_op[op];
             bytes6[3 * op + 1] = P->bytesB_op[op];
             bytes6[3 * op + 2] = P->bytesC_op[op];
         }

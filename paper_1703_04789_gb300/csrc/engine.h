@@ -367,6 +367,8 @@ const T* at(const DevMem& m, size_t off) { return reinterpret_cast<const T*>(sta
 bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why, int G = 1);
 bool validate_gemm(const GemmPlan& G, const int64_t* sizes, std::string* why, const BetaStride* stride = nullptr,
                    int op1 = 1 << 30, int copies = 1);
+// Whether an FP64 action that wants both outputs takes N's T1 out of H's (N's phase A is then not run).
+inline bool shares_t1(const spmps_t* h, const Plan& P) { return h->opt.batched != 0 && P.chan.shares; }
 spmps_status plan_upload(spmps_t* h, Plan& P, DevMem& lists);
 spmps_status plan_run(spmps_t* h, Plan& P, Slots S, int r0, int r1, cudaStream_t st, cudaEvent_t* ev = nullptr,
                       const SlotsF* split = nullptr);

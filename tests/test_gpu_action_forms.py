@@ -51,3 +51,30 @@ def test_channels_of_charge_three_only(opts):
         assert np.abs(dev.unpack(z, lay, ql, qr) - z_ref).max() <= 1e-10 * max(1.0, np.abs(z_ref).max())
         assert np.abs(dev.unpack(y, lay, ql, qr) - y_ref).max() <= 1e-10 * max(1.0, np.abs(y_ref).max())
     dev.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("opts", [{}, {"fp64_tensor_cores": True}, {"batched": False}, {"m_screen": 1e-3}])
+def test_costs_are_those_of_the_launches(opts):
+    """The flops that the costs and the statistics report for an action are those of the kernels it ran."""
+    require_gpu()
+    import torch
+    from paper_1703_04789_gb300 import Spmps
+    labels, tens = inputs.random_mps(8, 8, 0, 32, 1)
+    dev = Spmps(8, 8, 0, 0, 5, 32, **opts)
+    dev.set_hubbard(1.0, 4.0)
+    dev.set_mps(labels, tens, center=0)
+    x = torch.ones(dev.x_layout(3)["n_x"], dtype=torch.float64, device="cuda")
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    dev.apply_heff(3, x, y, z)
+    costs, bytes_ = dev.apply_costs(3)
+    for outs, want in (((y, z), costs.sum()), ((y, None), dev.apply_costs(3)[0][0].sum())):
+        before = dev.stats()["apply_flops_total"]
+        dev.profile(True)
+        dev.apply_heff(3, x, *outs)
+        ran = sum(dev.kernel_stats(kind)["flops"] for kind in (0, 1, 8, 9))
+        dev.profile(False)
+        assert abs(ran - want) <= 1e-12 * want
+        assert abs(dev.stats()["apply_flops_total"] - before - ran) <= 1e-12 * dev.stats()["apply_flops_total"]
+    assert (costs[1][0] == 0) == (bytes_[1][0] == 0)
+    dev.close()
