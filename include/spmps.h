@@ -89,7 +89,9 @@ typedef struct {
     int autotune;       /* 1: the first projected-action plan of each site times the candidate
                            tile policies of the block GEMMs (phases A and C separately, CUDA
                            events, a few actions on scratch vectors) and keeps the fastest for
-                           that site; 0 (default): the fixed least-padding policy. */
+                           that site; policies that give the same work lists are timed once, and
+                           none where the lists do not depend on them (small launches, split
+                           products); 0 (default): the fixed least-padding policy. */
     int metric_max_dim; /* precond == 4: largest metric block that is factorised (0 = default 3072) */
     int tc_wait_polls;  /* polls of the bounded mbarrier wait for the tensor-core MMAs of the learned
                            correction before it gives up with SPMPS_ERR_TIMEOUT (0 = default 2^24,

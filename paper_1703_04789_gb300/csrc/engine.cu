@@ -208,6 +208,19 @@ bool validate_plan(const Plan& P, const int64_t* sizes, std::string* why, int G)
 
 // ---- plan upload and launch -------------------------------------------------------------------
 
+// The lists that the tile policies shape: none where the split products take both phases.
+void policy_lists(Plan& P, int copies) {
+    P.A.tiles.clear();
+    P.C.tiles.clear();
+    P.f64C = TcUnits();
+    if (P.ozA.rng.empty()) P.A.add_tiles(P.polA, copies);
+    if (!P.ozC.rng.empty()) return;
+    if (P.stackC.ok)
+        stack_units(P.stackC, std::min(256, P.polC.wb_elems), copies, P.f64C);
+    else
+        P.C.add_tiles(P.polC, copies);
+}
+
 // Work lists of the plan's kernels, packed into `lists` (the plan's own buffer, or the handle's for plans that
 // run once) with one copy.  Only the lists that the handle's options can launch are made.
 spmps_status plan_upload(spmps_t* h, Plan& P, DevMem& lists) {
@@ -247,15 +260,10 @@ spmps_status plan_upload(spmps_t* h, Plan& P, DevMem& lists) {
             CK(h->tc_err.ensure(sizeof(int)));
             CK(cudaMemsetAsync(h->tc_err.p, 0, sizeof(int), h->stream));
         }
-    } else if (P.stackC.ok) {
-        stack_units(P.stackC, std::min(256, P.polC.wb_elems), copies, P.f64C);
     }
-    P.A.tiles.clear();
-    P.C.tiles.clear();
+    policy_lists(P, copies);
     P.A.tc_tiles.clear();
     P.C.tc_tiles.clear();
-    if (P.ozA.rng.empty()) P.A.add_tiles(P.polA, copies);
-    if (P.ozC.rng.empty() && P.f64C.rng.empty()) P.C.add_tiles(P.polC, copies);
     if (reduced && P.tcA.rng.empty()) {
         P.A.add_tc_tiles();
         P.C.add_tc_tiles();
@@ -1422,7 +1430,40 @@ void invalidate_all(spmps_t* h) {
     excited_invalidate(h);
 }
 
-// Autotuner: time every tile candidate for phases A and C of the site's action plan (one warm-up
+// The tile candidates whose list for phase A or C is not that of an earlier one; returns their number.  (A
+// launch too small to fill the chip has the same tiles under all of them, phase C's stacks depend on wb_elems
+// alone, and the split products on none.)  P has been uploaded: its stacks exist.
+int distinct_candidates(spmps_t* h, Plan& P, bool* new_a, bool* new_c) {
+    auto same_tiles = [](const std::vector<GemmTile>& x, const std::vector<GemmTile>& y) {
+        return std::equal(x.begin(), x.end(), y.begin(), y.end(), [](const GemmTile& u, const GemmTile& v) {
+            return u.task == v.task && u.m0 == v.m0 && u.n0 == v.n0 && u.tm == v.tm && u.tn == v.tn && u.shape == v.shape;
+        });
+    };
+    auto same_units = [](const std::vector<int4>& x, const std::vector<int4>& y) {
+        return std::equal(x.begin(), x.end(), y.begin(), y.end(), [](const int4& u, const int4& v) {
+            return u.x == v.x && u.y == v.y && u.z == v.z && u.w == v.w;
+        });
+    };
+    std::vector<GemmTile> a[kTileCandidates], c[kTileCandidates];
+    std::vector<int4> units[kTileCandidates];
+    int distinct = 0;
+    for (int i = 0; i < kTileCandidates; ++i) {
+        P.polA = P.polC = tile_candidate(i);
+        policy_lists(P, P.per_op ? h->G : 1);
+        a[i] = P.A.tiles;
+        c[i] = P.C.tiles;
+        units[i] = P.f64C.units;
+        new_a[i] = new_c[i] = true;
+        for (int j = 0; j < i; ++j) {
+            new_a[i] = new_a[i] && !same_tiles(a[j], a[i]);
+            new_c[i] = new_c[i] && !(same_tiles(c[j], c[i]) && same_units(units[j], units[i]));
+        }
+        distinct += new_a[i] || new_c[i] ? 1 : 0;
+    }
+    return distinct;
+}
+
+// Autotuner: time the distinct tile candidates for phases A and C of the site's action plan (one warm-up
 // and two timed actions each on zero scratch vectors, CUDA events around the phases) and keep
 // the fastest per phase; the choice is cached per site for the life of the handle.
 spmps_status tune_apply_plan(spmps_t* h, int k, Plan& P) {
@@ -1445,8 +1486,11 @@ spmps_status tune_apply_plan(spmps_t* h, int k, Plan& P) {
         for (auto& e : ev) CK(cudaEventCreate(&e));
         float best_a = INFINITY, best_c = INFINITY;
         int ia = 0, ic = 0;
-        spmps_status st = SPMPS_OK;
-        for (int c = 0; c < kTileCandidates && st == SPMPS_OK; ++c) {
+        spmps_status st = plan_upload(h, P, P.lists);
+        bool new_a[kTileCandidates], new_c[kTileCandidates];
+        const int n_cand = st == SPMPS_OK && distinct_candidates(h, P, new_a, new_c) > 1 ? kTileCandidates : 0;
+        for (int c = 0; c < n_cand && st == SPMPS_OK; ++c) {
+            if (!new_a[c] && !new_c[c]) continue;
             P.polA = P.polC = tile_candidate(c);
             st = plan_upload(h, P, P.lists);
             if (st != SPMPS_OK) break;
@@ -1472,8 +1516,8 @@ spmps_status tune_apply_plan(spmps_t* h, int k, Plan& P) {
                 ta += a;
                 tc += cc;
             }
-            if (ta < best_a) { best_a = ta; ia = c; }
-            if (tc < best_c) { best_c = tc; ic = c; }
+            if (new_a[c] && ta < best_a) { best_a = ta; ia = c; }
+            if (new_c[c] && tc < best_c) { best_c = tc; ic = c; }
         }
         for (auto& e : ev) cudaEventDestroy(e);
         if (st != SPMPS_OK) return st;

@@ -78,3 +78,30 @@ def test_costs_are_those_of_the_launches(opts):
         assert abs(dev.stats()["apply_flops_total"] - before - ran) <= 1e-12 * dev.stats()["apply_flops_total"]
     assert (costs[1][0] == 0) == (bytes_[1][0] == 0)
     dev.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K,D,G,opts,choice", [
+    (8, 32, 5, {}, False),
+    (8, 32, 5, {"fp64_tensor_cores": True}, False),    # no tiles
+    (16, 200, 5, {}, False),                           # 51 outputs a warp of the chip
+    (16, 200, 24, {}, True),                           # 244: 256 and 128 outputs a warp differ
+    (16, 200, 24, {"fp64_tensor_cores": True}, False),
+])
+def test_autotuner_times_only_what_differs(K, D, G, opts, choice):
+    """Launches of the first action at a site with and without the autotuner: the same number where no policy
+    changes a work list (a launch of up to 128 outputs of phase C per warp that the chip holds; split products)."""
+    require_gpu()
+    from paper_1703_04789_gb300 import Spmps
+    labels, tens = inputs.random_mps(K, K, 0, D, 1)
+    launches, z = [], []
+    for tuned in (False, True):
+        dev = Spmps(K, K, 0, 0, G, D, autotune=tuned, **opts)
+        dev.set_hubbard(1.0, 4.0)
+        dev.set_mps(labels, tens, center=0)
+        x = np.random.default_rng(3).standard_normal(dev.x_layout(K // 2 - 1)["n_x"])
+        z.append(dev.apply_heff_host(K // 2 - 1, x)[1])
+        launches.append(dev.stats()["launches"])
+        dev.close()
+    assert (launches[1] > launches[0]) == choice and launches[1] - launches[0] <= 72
+    assert np.abs(z[1] - z[0]).max() <= 1e-12 * max(1.0, np.abs(z[0]).max())
