@@ -35,10 +35,9 @@ __device__ __forceinline__ T wsum(T v) {
     return v;
 }
 
-// The rows of [0, R) whose squared norm is above `least`, ascending, by the first warp of a CTA (R <= kMaxRows).
+// The rows of [0, R) whose squared norm is above `least`, ascending, by the first warp of a CTA (R <= kSvdMaxRows).
 // Rows beyond a block's rank shrink to the rounding noise of the large rows within two sweeps; without them a
 // sweep has as many rounds as the block has rank.
-constexpr int kMaxRows = 1024;
 constexpr int kFullSweeps = 2;
 template <class Norm>
 __device__ __forceinline__ void list_rows(unsigned short* list, int* count, int R, bool all, Norm above) {
@@ -126,7 +125,7 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
     const int lane = threadIdx.x & 31;
     const int warp = (threadIdx.x >> 5) * ctas + rank;  // pairs go round the CTAs: the FP64 pipes of all share them
     const int warps = (blockDim.x >> 5) * ctas;
-    __shared__ unsigned short list[kMaxRows];
+    __shared__ unsigned short list[kSvdMaxRows];
     __shared__ int count;
     constexpr bool kF64 = sizeof(T) == 8;
     constexpr float tol = kF64 ? 1e-15f : 3e-7f;
@@ -267,7 +266,7 @@ template <int NV>
 __device__ void osj32_sweeps(float4* Z, float* nrm2, int R, int CV, int V) {
     constexpr float tol = 3e-7f, floor_abs = 1e-12f, null2 = 1e-13f, done = 1e-3f;
     const int gl = threadIdx.x & 7, group = threadIdx.x >> 3, groups = blockDim.x >> 3;
-    __shared__ unsigned short list[kMaxRows];
+    __shared__ unsigned short list[kSvdMaxRows];
     __shared__ int count;
     for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
         for (int base = 0; base < R; base += groups) {
@@ -582,7 +581,7 @@ void SvdPlan::build(const std::vector<SvdShape>& shapes, int smem_dim) {
     tiles.clear();
     gemm_rng.assign(1, 0);
     z_size = j_size = f_size = w_size = n_size = 0;
-    smem_floats = max_rows = 0;
+    smem_floats = max_rows = most_rows = 0;
     any_smem = any_global = any_companion = false;
     int64_t m_off = 0, e_off = 0;
     for (const SvdShape& s : shapes) {
@@ -596,6 +595,7 @@ void SvdPlan::build(const std::vector<SvdShape>& shapes, int smem_dim) {
         B.dim = s.dim;
         B.R = B.companion ? s.dim : s.other;
         B.C = B.companion ? s.other : s.dim;
+        most_rows = std::max(most_rows, B.R);
         B.z_off = z_size;
         z_size += static_cast<int64_t>(B.R) * B.C;
         B.j_off = j_size;
@@ -669,6 +669,7 @@ double* SvdPlan::z_buffer(void* ws) const {
 cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, cudaStream_t st) {
     const int nb = static_cast<int>(P.blocks.size());
     if (nb == 0) return cudaSuccess;
+    if (P.most_rows > kSvdMaxRows) return cudaErrorInvalidValue;
     char* p = static_cast<char*>(ws);
     auto take = [&](size_t bytes) {
         char* q = p;
