@@ -288,14 +288,15 @@ spmps_status spmps_apply_heff_host(spmps_handle h, int site, const double* x, do
 spmps_status spmps_two_site(spmps_handle h, int site, double* x);
 
 /* Canonicalise the loaded MPS on the device: right-canonical sites 1..K-1, centre on site 0,
- * norm 1.  Labels whose rank is zero are removed (bond dimensions may shrink). */
+ * norm 1.  Labels whose rank is zero are removed (bond dimensions may shrink).  Returns
+ * SPMPS_ERR_NOT_CONVERGED (after finishing) when the singular vectors of a block did not settle. */
 spmps_status spmps_canonicalize(spmps_handle h);
 
 /* n_sweeps two-site sweeps (left-to-right steps k = 0..K-3, then right-to-left k = K-2..0;
  * centre must be on site 0).  Per step: generalised Davidson for H_eff x = theta N_eff x,
  * SVD decimation to D (Sec. 2.3.1), environment update.  energies[s] (may be NULL) receives the
- * energy after sweep s.  Returns SPMPS_ERR_NOT_CONVERGED if any Davidson hit its cap (the
- * sweep still completes). */
+ * energy after sweep s.  Returns SPMPS_ERR_NOT_CONVERGED if any Davidson hit its cap or the
+ * singular vectors of a block did not settle (the sweep still completes). */
 spmps_status spmps_sweep(spmps_handle h, int n_sweeps, double* energies);
 
 /* One two-site step at sites (site, site+1) with the centre inside the pair: generalised
@@ -303,7 +304,8 @@ spmps_status spmps_sweep(spmps_handle h, int n_sweeps, double* energies);
  * move_right != 0 leaves site `site` left-canonical and the centre on site+1; otherwise site+1
  * becomes right-canonical and the centre moves to `site`.  theta (may be NULL) receives the
  * lowest generalised eigenvalue, iterations (may be NULL) the Davidson iteration count.
- * Returns SPMPS_ERR_NOT_CONVERGED (after finishing the step) when Davidson hit its cap. */
+ * Returns SPMPS_ERR_NOT_CONVERGED (after finishing the step) when Davidson hit its cap or the
+ * singular vectors of a block did not settle. */
 spmps_status spmps_optimize_step(spmps_handle h, int site, int move_right, double* theta, int* iterations);
 
 /* Energy functional (Eq. efunctional) and <Psi|P|Psi> at the current centre. */

@@ -22,7 +22,7 @@ namespace cgx = cooperative_groups;
 
 constexpr int kOsjC = 8;             // CTAs per block of the global-memory form
 constexpr int kOsj32Threads = 640;   // shared-memory form: 80 pairs at once with up to 102 registers a thread
-constexpr int kMaxSweeps = 40;
+constexpr int kFp32Sweeps = 40;      // most sweeps of the FP32 start
 constexpr double kNullRel = 1e-9;    // rows below this fraction of the block's norm are not separated further
 
 template <class T>
@@ -112,7 +112,8 @@ __device__ __forceinline__ double shear_sin(float hf, double h) {
 // A cluster of kOsjC CTAs with the rows in global memory (L2), a cluster barrier per round: in FP64 the
 // FP64 pipes of 8 SMs share the work.  NCH > 0 keeps the two rows of a pair in registers (W <= 32 NCH)
 // between the product and the update, NCH = 0 reads them twice.  The sweeps end after one that met no
-// relative coupling above `done` (what it leaves is the square of that over the relative gap).
+// relative coupling above `done` (what it leaves is the square of that over the relative gap), or after `sweeps` of
+// them with the result false.
 // FP64: an instruction of a warp occupies its sub-partition's FP64 pipe for 64 cycles whether its lanes hold
 // one number or 32, so a pair issues 3 per 32 elements for the shears, one for the product, 5 for its sum
 // over the warp, 2 for the norms and at most 7 for the sine; comparisons, conversions and the angle are
@@ -121,7 +122,8 @@ __device__ __forceinline__ double shear_sin(float hf, double h) {
 // with the comparisons, conversions and the angle's operands in FP64, 0.63 ms without the next two.  Rows beyond the
 // block's rank leave the rounds after two sweeps (0.57 ms), and the FP32 start hands its rows over by descending norm.
 template <class T, int NCH>
-__device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, float done, int* conv, int rank, int ctas) {
+__device__ bool osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, float done, int* conv, int rank, int ctas,
+                           int sweeps) {
     const int lane = threadIdx.x & 31;
     const int warp = (threadIdx.x >> 5) * ctas + rank;  // pairs go round the CTAs: the FP64 pipes of all share them
     const int warps = (blockDim.x >> 5) * ctas;
@@ -138,7 +140,7 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
     auto barrier = [&]() { cgx::this_cluster().sync(); };
     auto ld = [&](const T* p) -> T { return ldc(p); };
     auto stg = [&](T* p, T v) { __stcg(p, v); };
-    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+    for (int sweep = 0; sweep < sweeps; ++sweep) {
         for (int r = warp; r < R; r += warps) {
             T s = T(0);
             for (int c = lane; c < C; c += 32) {
@@ -234,8 +236,9 @@ __device__ void osj_sweeps(T* Z, T* nrm2, int R, int C, int W, T norm2_all, floa
         if (rough && lane == 0) atomicOr(conv + sweep, 1);
         __threadfence();
         barrier();
-        if (!*reinterpret_cast<volatile int*>(conv + sweep)) break;  // uniform: read after the barrier
+        if (!*reinterpret_cast<volatile int*>(conv + sweep)) return true;  // uniform: read after the barrier
     }
+    return false;
 }
 
 // The FP32 start in one CTA's shared memory: 8 lanes per pair and four elements per access, so that a warp
@@ -268,7 +271,7 @@ __device__ void osj32_sweeps(float4* Z, float* nrm2, int R, int CV, int V) {
     const int gl = threadIdx.x & 7, group = threadIdx.x >> 3, groups = blockDim.x >> 3;
     __shared__ unsigned short list[kSvdMaxRows];
     __shared__ int count;
-    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+    for (int sweep = 0; sweep < kFp32Sweeps; ++sweep) {
         for (int base = 0; base < R; base += groups) {
             const int r = base + group;
             float s = 0.0f;
@@ -373,7 +376,8 @@ __device__ double block_scale(const double* __restrict__ Z, int n) {
     return tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
 }
 
-// FP32 start: [Z | I] of a block scaled to norm 1; J (R x R) leaves in FP64.
+// FP32 start: [Z | I] of a block scaled to norm 1; J (R x R) leaves in FP64.  However its sweeps end, the FP64
+// finish takes what they leave.
 __global__ void __launch_bounds__(kOsj32Threads) k_osj32_smem(const SvdBlock* __restrict__ blocks, const double* __restrict__ zraw,
                                                               double* __restrict__ J, int smem_floats) {
     extern __shared__ float4 sm32[];
@@ -420,9 +424,9 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
     cgx::this_cluster().sync();
     int* cv = conv + b * kSvdConv;
     if (W <= 256)
-        osj_sweeps<float, 8>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC);
+        osj_sweeps<float, 8>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC, kFp32Sweeps);
     else
-        osj_sweeps<float, 0>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC);
+        osj_sweeps<float, 0>(work, nrm + B.n_off, R, C, W, 1.0f, 1e-3f, cv, rank, kOsjC, kFp32Sweeps);
     for (int r = (threadIdx.x >> 5) * kOsjC + rank; r < R; r += (blockDim.x >> 5) * kOsjC) {
         const int to = row_rank(R, r, [&](int j) { return __ldcg(nrm + B.n_off + j); });
         for (int c = threadIdx.x & 31; c < R; c += 32)
@@ -435,7 +439,7 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
 // mats (dim x dim): the companion's rows, or the normalised rows of Z'.
 __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
     k_osj64(const SvdBlock* __restrict__ blocks, double* __restrict__ z, double* __restrict__ nrm, int* __restrict__ conv,
-            double* __restrict__ mats, double* __restrict__ evals) {
+            double* __restrict__ mats, double* __restrict__ evals, int max_sweeps, int* __restrict__ unsettled) {
     __shared__ double red[32];
     __shared__ double tot;
     const int b = blockIdx.x / kOsjC;
@@ -463,12 +467,14 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
     int* cv = conv + (gridDim.x / kOsjC + b) * kSvdConv;
     // the companion is orthonormal by construction; normalised rows only as far as they are uncoupled
     const float done = B.companion ? 1e-11f : 1e-13f;
+    bool settled;
     if (W <= 160)
-        osj_sweeps<double, 5>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
+        settled = osj_sweeps<double, 5>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC, max_sweeps);
     else if (W <= 320)
-        osj_sweeps<double, 10>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
+        settled = osj_sweeps<double, 10>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC, max_sweeps);
     else
-        osj_sweeps<double, 0>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC);
+        settled = osj_sweeps<double, 0>(Z, nr, R, C, W, tot, done, cv, rank, kOsjC, max_sweeps);
+    if (!settled && rank == 0 && threadIdx.x == 0) *unsettled = 1;
     // exact norms of the final rows, then the vectors by descending norm (ties by row)
     const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) * kOsjC + rank;
     const int warps = (blockDim.x >> 5) * kOsjC;
@@ -666,10 +672,10 @@ double* SvdPlan::z_buffer(void* ws) const {
 // Measured (GB300): the decimations of one canonicalisation (random L = 24, D = 256 triplet state, 23 of them,
 // blocks up to 100 rows) take 17.5 ms, the middle decimation of the L = 24, D = 256 chain (blocks up to 126 rows)
 // 5.3 ms; two-sided FP64 Jacobi on X X^T with a one-thread truncation took 308 and 22 ms.
-cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, cudaStream_t st) {
+cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, int* unsettled, cudaStream_t st) {
     const int nb = static_cast<int>(P.blocks.size());
     if (nb == 0) return cudaSuccess;
-    if (P.most_rows > kSvdMaxRows) return cudaErrorInvalidValue;
+    if (P.most_rows > kSvdMaxRows || P.max_sweeps > kSvdConv) return cudaErrorInvalidValue;
     char* p = static_cast<char*>(ws);
     auto take = [&](size_t bytes) {
         char* q = p;
@@ -712,7 +718,7 @@ cudaError_t launch_svd(const SvdPlan& P, void* ws, double* mats, double* evals, 
     gemm(3, t0, j1, j0);
     gemm(4, j0, z, f);
     if (P.any_companion) k_companion<<<nb, 256, 0, st>>>(blocks, j0, f);
-    k_osj64<<<nb * kOsjC, 256, 0, st>>>(blocks, f, n64, conv, mats, evals);
+    k_osj64<<<nb * kOsjC, 256, 0, st>>>(blocks, f, n64, conv, mats, evals, P.max_sweeps, unsettled);
     return cudaGetLastError();
 }
 

@@ -36,6 +36,7 @@ constexpr double kTieRtol = 1e-10;   // relative gap below which singular values
 constexpr double kDropAbs = 1e-7;
 constexpr double kEpsMetric = 1e-12;
 constexpr double kClamp = 1e-4;
+constexpr const char* kUnsettled = "decimation: the singular vectors of a block did not settle";
 
 struct DavidsonOut {
     double theta = 0.0, resid = 0.0;
@@ -494,8 +495,10 @@ bool copies_in_range(const std::vector<CopyBlock>& copies, const int64_t* sizes)
 
 // Decimate the two-site tensor x (row-block layout at sites (k, k+1), device) into new site
 // tensors k and k+1 with at most Dmax states on the middle bond; move_right selects the
-// canonical side (left-canonical A[k] when true, right-canonical A[k+1] otherwise).
-spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, DecBuffers& B, double* discarded) {
+// canonical side (left-canonical A[k] when true, right-canonical A[k+1] otherwise).  *settled becomes false
+// where the singular vectors of a block were still coupled after the last sweep (the tensors are kept).
+spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, DecBuffers& B, double* discarded,
+                      bool* settled) {
     const Bond& bl = h->bonds[k];
     const Bond& br = h->bonds[k + 2];
     const RowBlockLayout xl = make_row_block_layout(bl, br, 16);
@@ -601,21 +604,23 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
     for (MidLabel* M : list) vo.push_back(M->val_off);
     const int nm = static_cast<int>(list.size());
     CK(upload(B.val_off, vo, h->stream));
-    CK(B.keep.ensure(std::max(nm, 1) * sizeof(int)));
+    CK(B.keep.ensure((nm + 1) * sizeof(int)));  // and whether a block did not settle
+    int* unsettled = B.keep.as<int>() + nm;
+    CK(cudaMemsetAsync(unsettled, 0, sizeof(int), h->stream));
     CK(B.keep_total.ensure(sizeof(int)));
     CK(B.disc.ensure(sizeof(double)));
     CK(B.sidx.ensure(std::max(3 * total, 1) * sizeof(int)));
     CK(B.sval.ensure(std::max(2 * total, 1) * sizeof(double)));
     const int rec_eig = h->profile ? prof_begin(h, h->stream, 4, 0.0) : -1;
     CK(launch_copy_blocks(S, B.gather.as<CopyBlock>(), static_cast<int>(gather.size()), h->stream));
-    CK(launch_svd(SP, B.svd.p, B.mats.as<double>(), B.evals.as<double>(), h->stream));
+    CK(launch_svd(SP, B.svd.p, B.mats.as<double>(), B.evals.as<double>(), unsettled, h->stream));
     CK(launch_truncate(B.evals.as<double>(), B.val_off.as<int64_t>(), nm, total, Dmax, kTieRtol, kDropAbs, B.keep.as<int>(),
                        B.keep_total.as<int>(), B.disc.as<double>(), B.sidx.as<int>(), B.sval.as<double>(), h->stream));
     if (rec_eig >= 0) prof_end(h, h->stream, rec_eig);
     h->launches += 11;
-    std::vector<int> keep(std::max(nm, 1));
+    std::vector<int> keep(nm + 1);
     double disc = 0.0;
-    CK(cudaMemcpyAsync(keep.data(), B.keep.p, std::max(nm, 1) * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(keep.data(), B.keep.p, (nm + 1) * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(&disc, B.disc.p, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     if (discarded) *discarded = disc;
@@ -761,6 +766,7 @@ spmps_status decimate(spmps_t* h, int k, double* x, int Dmax, bool move_right, D
     CK(launch_copy_blocks(S2, at<CopyBlock>(h->once, oy), static_cast<int>(copies.size()), h->stream));
     h->launches += 4;
     CK(cudaStreamSynchronize(h->stream));
+    if (keep[nm]) *settled = false;
     // install
     h->bonds[k + 1] = nb;
     h->alay[k] = a0;
@@ -785,16 +791,18 @@ spmps_status spmps_canonicalize(spmps_handle h) {
     if (cudaSetDevice(h->device) != cudaSuccess) return fail(h, SPMPS_ERR_CUDA, "cudaSetDevice");
     DecBuffers B;
     DevMem xb;
+    bool settled = true;
     for (int k = h->K - 2; k >= 0; --k) {
         const int64_t n = x_size(h, k);
         CK(xb.ensure(std::max<int64_t>(n, 1) * sizeof(double)));
         st = spmps_two_site(h, k, xb.as<double>());
         if (st != SPMPS_OK) return st;
-        st = decimate(h, k, xb.as<double>(), h->D, false, B, nullptr);
+        st = decimate(h, k, xb.as<double>(), h->D, false, B, nullptr, &settled);
         if (st != SPMPS_OK) return st;
     }
     invalidate_all(h);
     h->center = 0;
+    if (!settled) return fail(h, SPMPS_ERR_NOT_CONVERGED, kUnsettled);
     return SPMPS_OK;
 }
 
@@ -815,7 +823,8 @@ spmps_status spmps_optimize_step(spmps_handle h, int site, int move_right, doubl
     st = davidson(h, site, x0.as<double>(), DB, &out);
     if (st != SPMPS_OK) return st;
     double disc = 0.0;
-    st = decimate(h, site, DB.x.as<double>(), h->D, move_right != 0, EB, &disc);
+    bool settled = true;
+    st = decimate(h, site, DB.x.as<double>(), h->D, move_right != 0, EB, &disc, &settled);
     if (st != SPMPS_OK) return st;
     h->last_discarded = disc;
     if (move_right) {
@@ -831,6 +840,7 @@ spmps_status spmps_optimize_step(spmps_handle h, int site, int move_right, doubl
     if (theta) *theta = out.theta;
     if (iterations) *iterations = out.iters;
     if (!out.converged) return fail(h, SPMPS_ERR_NOT_CONVERGED, "Davidson reached its iteration cap");
+    if (!settled) return fail(h, SPMPS_ERR_NOT_CONVERGED, kUnsettled);
     return SPMPS_OK;
 }
 
@@ -847,7 +857,7 @@ spmps_status spmps_sweep(spmps_handle h, int n_sweeps, double* energies) {
     DavBuffers DB;
     DecBuffers EB;
     DevMem x0;
-    bool all_converged = true;
+    bool all_converged = true, settled = true;
     h->dav_iters = 0;
     h->refine_iters = 0;
     double disc_total = 0.0;
@@ -868,7 +878,7 @@ spmps_status spmps_sweep(spmps_handle h, int n_sweeps, double* energies) {
             all_converged = all_converged && out.converged;
             theta = out.theta;
             double disc = 0.0;
-            st = decimate(h, k, DB.x.as<double>(), h->D, mr, EB, &disc);
+            st = decimate(h, k, DB.x.as<double>(), h->D, mr, EB, &disc, &settled);
             if (st != SPMPS_OK) return st;
             disc_total += disc;
             if (mr) {
@@ -886,6 +896,7 @@ spmps_status spmps_sweep(spmps_handle h, int n_sweeps, double* energies) {
     }
     h->last_discarded = disc_total;
     if (!all_converged) return fail(h, SPMPS_ERR_NOT_CONVERGED, "a Davidson solve reached its iteration cap");
+    if (!settled) return fail(h, SPMPS_ERR_NOT_CONVERGED, kUnsettled);
     return SPMPS_OK;
 }
 

@@ -1,8 +1,13 @@
-"""One block of the decimation's singular vectors: limits that are refused."""
+"""One block of the decimation's singular vectors: limits that are refused, sweeps that end too early.
+
+Singular values of a block of norm 1 are FP64 rounding of it: 1e-14 for some hundreds of rows (a few n eps); the
+vectors' orthonormality 1e-12, as in the tests of the canonical form.
+"""
 import ctypes as C
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 from paper_1703_04789_gb300 import build as B
@@ -20,8 +25,42 @@ def lib(tmp_path_factory):
     return C.CDLL(out)
 
 
-@pytest.mark.parametrize("dim,other", [(1025, 1025), (2000, 4000)])
-def test_blocks_beyond_the_limits_are_refused(lib, dim, other):
+@pytest.mark.parametrize("dim,other,sweeps", [(1025, 1025, 250), (2000, 4000, 250), (8, 8, 257)])
+def test_blocks_beyond_the_limits_are_refused(lib, dim, other, sweeps):
     if gpu_available():
         pytest.skip("shown without a device: a launch would need one")
-    assert lib.svd_launch_empty(dim, other) == INVALID_VALUE
+    assert lib.svd_launch_empty(dim, other, sweeps) == INVALID_VALUE
+
+
+def _block(lib, x, sweeps=250):
+    dim, other = x.shape
+    ev, vec, flag = np.empty(dim), np.empty((dim, dim)), C.c_int(-1)
+    ptr = lambda a: a.ctypes.data_as(C.POINTER(C.c_double))
+    assert lib.svd_block(dim, other, sweeps, ptr(x), ptr(ev), ptr(vec), C.byref(flag)) == 0
+    return np.sqrt(np.maximum(ev, 0.0)), vec, flag.value
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dim,other", [(1, 3), (9, 9), (100, 25), (25, 100), (130, 150), (300, 300)])
+def test_block_reports_whether_it_settled(lib, dim, other):
+    if not gpu_available():
+        pytest.skip("needs a CUDA device")
+    x = np.random.default_rng(dim).standard_normal((dim, other))
+    x /= np.linalg.norm(x)
+    k = min(dim, other)
+    # one sweep leaves couplings where two rows or more have a norm (a single row has none)
+    assert _block(lib, x, 1)[2] == (1 if k > 1 else 0)
+    values, vec, flag = _block(lib, x)
+    assert flag == 0
+    assert np.abs(values[:k] - np.linalg.svd(x, compute_uv=False)).max() < 1e-14
+    assert np.abs(vec[:, :k].T @ vec[:, :k] - np.eye(k)).max() < 1e-12
+
+
+@pytest.mark.gpu
+def test_slowest_blocks_settle(lib):
+    """Rows that differ little beside a few large columns need the most sweeps."""
+    if not gpu_available():
+        pytest.skip("needs a CUDA device")
+    rng = np.random.default_rng(0)
+    x = rng.standard_normal((400, 500)) * 10.0 ** -rng.uniform(0, 14, 400)[:, None]
+    assert _block(lib, x / np.linalg.norm(x))[2] == 0
