@@ -92,14 +92,16 @@ __device__ __forceinline__ float half_tan(float t) {
 }
 
 // sin(theta) for h = tan(theta / 2): 2 h / (1 + h^2) to the precision of T.  The rotation is applied as three
-// shears x -= h y, y += s x, x -= h y, which is orthonormal for any h as far as s belongs to it (an error e
-// of s leaves h e); the angle itself may be rounded (the next sweep removes what it leaves).
+// shears x -= h y, y += s x, x -= h y, which is orthonormal for any h as far as s belongs to it: an error e of s
+// leaves e between the two rows, so it has to be rounding of s itself; the angle may be rounded (the next sweep
+// removes what it leaves).
 __device__ __forceinline__ float shear_sin(float hf, float) { return __fdividef(2.0f * hf, fmaf(hf, hf, 1.0f)); }
 __device__ __forceinline__ double shear_sin(float hf, double h) {
     const double h2 = to_f64(2.0f * hf);
     const float m = fabsf(hf);
-    if (m < 4e-5f) return h2;                     // h e = 2 h^4 < 6e-18
-    if (m < 1e-3f) return fma(-h2, h * h, h2);    // h e = 2 h^6 < 2e-18
+    if (m < 7e-9f) return h2;                         // relative error h^2 < 5e-17
+    const double q = h * h;
+    if (m < 2e-3f) return fma(h2, fma(q, q, -q), h2);  // h^6 < 7e-17
     const double d = fma(h, h, 1.0);
     double y = to_f64(__fdividef(1.0f, fmaf(hf, hf, 1.0f)));
     y = fma(y, fma(-d, y, 1.0), y);

@@ -64,3 +64,18 @@ def test_slowest_blocks_settle(lib):
     rng = np.random.default_rng(0)
     x = rng.standard_normal((400, 500)) * 10.0 ** -rng.uniform(0, 14, 400)[:, None]
     assert _block(lib, x / np.linalg.norm(x))[2] == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dim,other", [(8, 40), (20, 40), (60, 100), (126, 250), (180, 300)])
+def test_vectors_are_orthonormal_to_rounding(lib, dim, other):
+    """Blocks whose vectors are the accumulated rotations, singular values over 14 decades: a rotation moves the
+    product of two rows by at most four roundings, and a row takes part in dim rotations of each of up to 20 sweeps."""
+    if not gpu_available():
+        pytest.skip("needs a CUDA device")
+    rng = np.random.default_rng(dim)
+    u, v = (np.linalg.qr(rng.standard_normal((n, dim)))[0] for n in (dim, other))
+    x = (u * 10.0 ** -np.linspace(0, 14, dim)) @ v.T
+    _, vec, flag = _block(lib, x / np.linalg.norm(x))
+    assert flag == 0
+    assert np.abs(vec.T @ vec - np.eye(dim)).max() < 4 * 2.0 ** -53 * np.sqrt(20 * dim)
