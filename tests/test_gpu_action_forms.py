@@ -1,4 +1,5 @@
-"""Actions of operators and bonds outside the usual: H without an output where N has one.
+"""Actions of operators and bonds outside the usual: H without an output where N has one, groups of many
+labels, blocks of many elements; what an action reports and what its tuner times.
 
 The bounds are those of the other FP64 parity tests: 1e-10 of the largest entry (the forms differ from the
 oracle only in summation order).
@@ -6,7 +7,7 @@ oracle only in summation order).
 import numpy as np
 import pytest
 
-from oracle import mps as S
+from oracle import mpo as M, mps as S
 from paper_1703_04789_gb300 import inputs
 from tests.gpu_util import masked_random_two_site, require_gpu
 
@@ -105,3 +106,67 @@ def test_autotuner_times_only_what_differs(K, D, G, opts, choice):
         dev.close()
     assert (launches[1] > launches[0]) == choice and launches[1] - launches[0] <= 72
     assert np.abs(z[1] - z[0]).max() <= 1e-12 * max(1.0, np.abs(z[0]).max())
+
+
+def _one_electron_per_site(K, seed):
+    """A raw state with one electron on every site and every spin label a bond can have, dimension 1 each: bond i
+    has the labels (i, 2m) of one particle number, up to K / 2 + 1 of them."""
+    rng = np.random.default_rng(seed)
+    half = K // 2
+    labels = [np.array([(i, 2 * na - i) for na in range(max(0, half - (K - i)), min(i, half) + 1)], dtype=np.int64)
+              for i in range(K + 1)]
+    tens = [np.where(S.site_mask(labels[i], labels[i + 1]),
+                     rng.uniform(0.5, 1.5, (labels[i].shape[0], 4, labels[i + 1].shape[0])), 0.0) for i in range(K)]
+    return labels, tens
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("opts", [{}, {"fp64_tensor_cores": True}, {"batched": False}])
+def test_groups_of_more_labels_than_mask_bits(opts):
+    """67 labels of one particle number: those from the 64th on share a bit, and T1 starts at zero."""
+    require_gpu()
+    from paper_1703_04789_gb300 import Spmps
+    K, G, k = 132, 2, 64
+    labels, tens = _one_electron_per_site(K, 5)
+    sites = M.hubbard_mpo(K, 1.0, 4.0)
+    P = S.prepare(labels, tens, sites, 0, 0, G)
+    ql, qr = P.mps.labels[k], P.mps.labels[k + 2]
+    assert qr.shape[0] == 67
+    dev = Spmps(K, K, 0, 0, G, 80, **opts)
+    dev.set_mpo(sites)
+    dev.set_mps(P.mps.labels, P.mps.A, center=0)
+    P.build_left(k)
+    lay = dev.x_layout(k)
+    x = masked_random_two_site(ql, qr, np.random.default_rng(1))
+    y_ref, z_ref = P.apply(x, k)
+    dev.apply_heff_host(k, np.full(lay["n_x"], 1e3))  # what a column that is not written would hold
+    y, z = dev.apply_heff_host(k, dev.pack(x, lay, ql, qr))
+    assert np.abs(dev.unpack(y, lay, ql, qr) - y_ref).max() <= 1e-10 * np.abs(y_ref).max()
+    assert np.abs(dev.unpack(z, lay, ql, qr) - z_ref).max() <= 1e-10 * np.abs(z_ref).max()
+    dev.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D,site", [(40, 3), (150, 3), (150, 1)])
+def test_separate_combination_over_several_passes(D, site):
+    """Active-space operator on eight orbitals: too many inputs for the fused form; at D = 150 the blocks have
+    more elements than a CTA takes in one pass (512), at D = 40 fewer."""
+    require_gpu()
+    from paper_1703_04789_gb300 import Spmps, mpo_from_integrals
+    K, N, G = 8, 8, 3
+    h1, eri, _ = inputs.synthetic_active_space(K, 7)
+    sites = mpo_from_integrals(h1, eri, 0.0)
+    labels, tens = inputs.random_mps(K, N, 0, D, 4)
+    P = S.prepare(labels, tens, sites, 0, 0, G)
+    dev = Spmps(K, N, 0, 0, G, D)
+    dev.set_mpo(sites)
+    dev.set_mps(P.mps.labels, P.mps.A, center=0)
+    P.build_left(site)
+    ql, qr = P.mps.labels[site], P.mps.labels[site + 2]
+    lay = dev.x_layout(site)
+    x = masked_random_two_site(ql, qr, np.random.default_rng(1))
+    y_ref, z_ref = P.apply(x, site)
+    y, z = dev.apply_heff_host(site, dev.pack(x, lay, ql, qr))
+    assert np.abs(dev.unpack(y, lay, ql, qr) - y_ref).max() <= 1e-10 * max(1.0, np.abs(y_ref).max())
+    assert np.abs(dev.unpack(z, lay, ql, qr) - z_ref).max() <= 1e-10 * max(1.0, np.abs(z_ref).max())
+    dev.close()
