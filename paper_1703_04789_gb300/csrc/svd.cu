@@ -466,6 +466,10 @@ __global__ void __cluster_dims__(kOsjC, 1, 1) __launch_bounds__(256)
         tot = t;
     }
     cgx::this_cluster().sync();  // every CTA has read Z before any rotates it
+    if (!(tot < INFINITY)) {  // the block overflowed (the same sum in every CTA): no values, none of them is kept
+        for (int rk = rank * blockDim.x + threadIdx.x; rk < B.dim; rk += blockDim.x * kOsjC) evals[B.e_off + rk] = 0.0;
+        return;
+    }
     int* cv = conv + (gridDim.x / kOsjC + b) * kSvdConv;
     // the companion is orthonormal by construction; normalised rows only as far as they are uncoupled
     const float done = B.companion ? 1e-11f : 1e-13f;

@@ -79,3 +79,31 @@ def test_vectors_are_orthonormal_to_rounding(lib, dim, other):
     _, vec, flag = _block(lib, x / np.linalg.norm(x))
     assert flag == 0
     assert np.abs(vec.T @ vec - np.eye(dim)).max() < 4 * 2.0 ** -53 * np.sqrt(20 * dim)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("dim,other", [(60, 100), (100, 60), (160, 200)])
+def test_block_that_overflowed_has_no_values(lib, bad, dim, other):
+    if not gpu_available():
+        pytest.skip("needs a CUDA device")
+    x = np.random.default_rng(dim).standard_normal((dim, other))
+    x[dim // 2, other // 3] = bad
+    values, _, flag = _block(lib, x)
+    assert flag == 0 and not values.any()
+
+
+@pytest.mark.gpu
+def test_state_that_overflows_is_an_error():
+    if not gpu_available():
+        pytest.skip("needs a CUDA device")
+    from paper_1703_04789_gb300 import Spmps, SpmpsError, inputs
+    labels, tens = inputs.random_mps(6, 6, 0, 16, 1)
+    dev = Spmps(6, 6, 0, 0, 4, 16)
+    dev.set_hubbard(1.0, 4.0)
+    dev.set_mps(labels, tens, center=0)
+    dev.canonicalize()
+    dev.set_mps(labels, tens[:4] + [tens[4] * 1e200, tens[5] * 1e200], center=0)
+    with pytest.raises(SpmpsError):
+        dev.canonicalize()
+    dev.close()
