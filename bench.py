@@ -360,8 +360,8 @@ def _roofline(phase_oz, phase_tc, phase64, fl_op, by_op, hbm, tf32_peaks, fp64_p
     (k_gemm_oz: every FP64-accurate block product of phases A and C, H and N).  Its arithmetic is
     FP16 tensor-core MMAs, DIGIT_PRODUCTS digit products per FP64 multiply-add, so its roofline is
     the FP16 dense tensor peak (the measured BF16 burst; FP16 has the same nominal dense rate):
-    achieved = DIGIT_PRODUCTS x the algorithmic FP64 flops of phases A and C of the middle-site action
-    / their CUDA-event time.  Beside it, the same algorithmic FP64 flops per second against the
+    achieved = DIGIT_PRODUCTS x the algorithmic FP64 flops of phases A and C that the middle-site action
+    runs / their CUDA-event time.  Beside it, the same algorithmic FP64 flops per second against the
     measured FP64 pipe (what an FP64 GEMM could reach), the FP64 pipe kernel on the same action, and
     the 3xTF32 products of the H part (k_gemm_tc) against the HBM bandwidth and the tcgen05
     kind::tf32 peak."""
@@ -398,7 +398,7 @@ def _roofline(phase_oz, phase_tc, phase64, fl_op, by_op, hbm, tf32_peaks, fp64_p
                             "frac_of_fp64_pipe": round(fp64_eq / fp64_peak, 4) if fp64_peak else None,
                             "peak_source": "measured: FP64 FMA-chain kernel on all SMs (spmps_device_fp64_peak)"},
         "fp64_pipe_kernel": {
-            "kernel": "k_gemm_f64 on the same action (the fast_fp64 form)", "bound": "alu",
+            "kernel": "k_gemm_f64 (phase A) and k_gemm_f64_stack (phase C) on the same action (the fast_fp64 form)", "bound": "alu",
             "achieved_tflops": round(ach64, 4), "peak_tflops": round(fp64_peak, 4),
             "frac": round(ach64 / fp64_peak, 4) if fp64_peak else None,
             "phase_ms": [round(float(v), 4) for v in phase64],

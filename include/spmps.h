@@ -153,9 +153,8 @@ spmps_status spmps_set_hubbard(spmps_handle h, double t, double U);
  * couple only nearest neighbours (h1) and single orbitals ((pp|pp)) get the bond-dimension-6
  * Hubbard-like MPO; all others the general MPO (Eq. sumH / Eq. Wfac): every term placed with
  * complementary-operator channels, bond dimension 2 + 2 n_L + 2 n_R + O(min(n_L, n_R)^2) at a
- * cut with n_L / n_R spin-orbitals on its sides.  The MPO site tensors live on the host (one
- * copy per beta point); when they would need more than 4 GB the call returns
- * SPMPS_ERR_UNSUPPORTED. */
+ * cut with n_L / n_R spin-orbitals on its sides.  The MPO site tensors live on the host; when
+ * n_beta + 1 times their size is more than 4 GB the call returns SPMPS_ERR_UNSUPPORTED. */
 spmps_status spmps_set_hamiltonian(spmps_handle h, const double* h1, const double* h2, double ecore);
 
 /* Hamiltonian given directly as an MPO on spatial sites (an alternative to the integrals):
@@ -360,8 +359,9 @@ spmps_status spmps_stream(spmps_handle h, void** stream);
  * enable != 0 switches it on and clears the counters; enable == 0 switches it off. */
 spmps_status spmps_profile(spmps_handle h, int enable);
 
-/* Counters of the profiler for `kind`: 0 = k_gemm_f64 launches, 1 = k_comb_f64 launches (their
- * algorithmic flops, same rule as spmps_apply_flops), 2 = the Davidson Ritz step (k_ritz),
+/* Counters of the profiler for `kind`: 0 = FP64-pipe block-GEMM launches (k_gemm_f64,
+ * k_gemm_f64_stack), 1 = the MPO-leg combinations (k_comb_pair, or k_comb_rotate and k_comb_list; k_comb_f64
+ * in the plans of excited states; their algorithmic flops, same rule as spmps_apply_flops), 2 = the Davidson Ritz step (k_ritz),
  * 3 = the rest of each Davidson iteration outside the projected action (dots, gemv, residual,
  * Gram-Schmidt), 4 = the decimation eigen-solve and truncation, 5 = host time spent building and
  * uploading contraction plans (ms of host clock, launches = plans built), 6 = assembly and

@@ -1875,7 +1875,8 @@ spmps_status check_integrals(spmps_t* h, int K, const double* h1, const double* 
     return SPMPS_OK;
 }
 
-// the library's MPO site tensors (one copy per beta point) are held on the host: keep them within this size
+// Operators are refused by n_beta + 1 times the host memory of their site tensors.  The plans keep one copy of them;
+// the limit dates from a form with one per beta point and stays, since what it refuses has never been run.
 constexpr double kMaxMpoHostBytes = 4.0e9;
 
 bool mpo_fits(const MPO& m, int copies, std::string* why) {

@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(256) k_normalise(double* __restrict__ y, int64
         y[i] *= s;
 }
 
-// out = v / (diag H - theta diag N), the denominator clamped as in k_residual_diag
+// out = v / (diag H - theta diag N), the denominator clamped as in k_ritz_vectors
 __global__ void __launch_bounds__(256) k_precond_apply(const double* __restrict__ v, const double* __restrict__ dh,
                                                        const double* __restrict__ dn,
                                                        const double* __restrict__ scal, double clamp, int64_t n,

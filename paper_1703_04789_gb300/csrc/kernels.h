@@ -28,7 +28,7 @@ inline int op0_entries(const BetaRun& b, int from, int n) {
     return k < 0 ? 0 : (k > n ? n : k);
 }
 
-// Grouped FP64 GEMM: one warp per 16x16 output tile of the task list.
+// Grouped FP64 GEMM: one warp per tile of the task list (register tiles of 256 outputs, warp blocks of up to 256).
 cudaError_t launch_gemm_f64(const Slots& slots, const GemmTask* tasks, const GemmSeg* segs,
                             const GemmTile* tiles, const int* cmaps, int n_tiles, cudaStream_t st,
                             const BetaRun& beta = BetaRun());
