@@ -98,3 +98,29 @@ def test_calls_on_several_streams_equal_serial_calls(opts):
     got, scalars2 = calls([torch.cuda.Stream(), None, torch.cuda.Stream(), torch.cuda.Stream()])
     assert all(np.array_equal(a, b) for a, b in zip(serial, got))
     assert scalars == scalars2
+
+
+@pytest.mark.gpu
+def test_captured_action_replays():
+    """Capture on a caller's stream (relaxed mode: the call waits on the host for the handle's own stream), with an
+    earlier action on that stream that the handle has not waited for yet."""
+    require_gpu()
+    import torch
+    dev = _handle()
+    x, y, z = _vectors(dev, 3, 1)
+    s = torch.cuda.Stream()
+    dev.apply_heff(3, x, y, z, stream=s)
+    torch.cuda.synchronize()
+    want = y.clone(), z.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s, capture_error_mode="relaxed"):
+        dev.apply_heff(3, x, y, z, stream=s)
+    x2, y2, z2 = _vectors(dev, 3, 2)
+    torch.cuda.synchronize()
+    dev.apply_heff(3, x2, y2, z2)
+    y.zero_(), z.zero_()
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, want[0]) and torch.equal(z, want[1])
+    dev.close()
